@@ -216,13 +216,13 @@ void carve_rep(Rep &r, Carver &cv)
         r.psis = cv.take<float>(P);
         r.E = cv.take<float>(N);
     }
-    if (r.p.integrator == FLB_RK4 && r.dim == 3) r.Dn = cv.take<float>(N);
-    if (r.dim == 2 || general_path(r.p)) {  // the per-site path keeps mu*, the noise increment and the FV flux in HBM
+    if (r.p.integrator == FLB_RK4) r.Dn = cv.take<float>(N);
+    if (general_path(r.p)) {  // the per-site path keeps mu*, the noise increment and the FV flux in HBM
         r.eta = cv.take<float>(N);
         if (r.p.integrator != FLB_EULER) r.mus = cv.take<float>(P);
         if (r.p.psi_scheme == FLB_FV) r.J = cv.take<float>((size_t)r.dim * P);
     }
-    if (r.p.force_grad == FLB_FORCE_STRESS) r.sig = cv.take<float>((size_t)(r.dim == 3 ? 6 : 3) * P);
+    if (r.p.force_grad == FLB_FORCE_STRESS && r.dim == 3) r.sig = cv.take<float>(6 * P);
     r.Kx = axis_K(g.nx, r.p.sq_kmax);
     r.Ky = axis_K(g.ny, r.p.sq_kmax);
     r.Kz = r.dim == 3 ? axis_K(g.nz, r.p.sq_kmax) : 1;
@@ -503,14 +503,15 @@ LBArgs lb_args(const Rep &r, float *psi_n)
         la.rq[0] = (float)(4.5 * (1.0 - ws));
         la.rq[1] = (float)(4.5 * ws);
         la.rq[2] = (float)(4.5 * cs);
-        la.rq[3] = (float)(1.5 * (wb - ws));
-        la.rq[4] = (float)(3.0 * (cb - cs));
+        la.rq[3] = (float)(4.5 / r.dim * (wb - ws));
+        la.rq[4] = (float)(9.0 / r.dim * (cb - cs));
         la.iso = r.omega_s != r.omega_b;
         la.k3T = (float)(3.0 * p.kT);
         // Q = 4.5 B takes the stress noise at 4.5 x (2/9, 1/9); the ghosts G10-G12,
         // G16 are g/3 and G17, G18 are g/2
         const double sc[15] = {1, 1, 1, 0.5, 0.5, 0.5, 1.0 / 3, 1.0 / 3, 1.0 / 3, 1, 1, 1, 1.0 / 3, 0.5, 0.5};
-        for (int t = 0; t < 15; ++t) la.nq[t] = (float)(sc[t] * (double)r.namp[t]);
+        const double sc2[6] = {1, 1, 0.5, 1.0 / 3, 1.0 / 3, 2.0 / 9};  // D2Q9: Qxy, h6, h7, h8
+        for (int t = 0; t < 15; ++t) la.nq[t] = (float)((r.dim == 3 ? sc[t] : t < 6 ? sc2[t] : 0.0) * (double)r.namp[t]);
     }
     la.coupling = p.coupling;
     const bool fv_grad =
@@ -610,11 +611,73 @@ int step_rep3(flb_handle *h, Rep &r)
     return FLB_OK;
 }
 
+// 2D step: the collide-stream with its force, then one launch per Runge-Kutta
+// stage of psi, the first of which forms the velocity of the new fluid state.
+int step_rep2(flb_handle *h, Rep &r)
+{
+    const flb_params &p = r.p;
+    cudaStream_t st = h->st;
+    float *psi_n = r.psi[r.pcur], *psi_np1 = r.psi[r.pcur ^ 1];
+    const LBArgs la = lb_args(r, psi_n);
+    Psi2Args pa;
+    pa.g = r.g;
+    pa.psi = psi_n;
+    pa.f = la.fout;
+    pa.u = r.u;
+    pa.out = p.integrator == FLB_EULER ? psi_np1 : r.psis;
+    pa.E = r.E;
+    pa.eta = r.Dn;
+    pa.base = psi_n;
+    pa.A = (float)p.A;
+    pa.B = (float)p.B;
+    pa.K = (float)p.K;
+    pa.M = (float)p.M;
+    pa.rho0 = (float)p.rho0;
+    pa.lw = lap_weights(2, p.laplacian);
+    pa.amp[0] = sqrtf(2.f * (float)p.kT * pa.M);
+    pa.amp[1] = sqrtf(2.f * (float)p.kT * pa.M * pa.lw.c1);
+    pa.amp[2] = sqrtf(2.f * (float)p.kT * pa.M * pa.lw.c2);
+    pa.coupling = p.coupling;
+    pa.force_kind = la.force_kind;
+    pa.scheme = p.psi_scheme;
+    pa.integrator = p.integrator;
+    pa.stage = 1;
+    pa.key = la.key;
+    pa.step = r.step;
+    const bool noisy = p.kT > 0 && p.M > 0;
+    cudaEvent_t e1 = mark(h);
+    {
+        const Range range("collide-stream");
+        FLB_TRY(launch_lb2(la, pa, p.storage, st));
+    }
+    cudaEvent_t e2 = mark(h);
+    const int64_t l2 = h->launches;
+    {
+        const Range range("psi");
+        FLB_TRY(launch_psi2(pa, p.storage, noisy, st));
+        // stages 2.. alternate between psi* and the spare psi buffer
+        for (int s = 2; s <= (p.integrator == FLB_RK4 ? 4 : p.integrator == FLB_HEUN ? 2 : 1); ++s) {
+            pa.psi = s % 2 == 0 ? r.psis : psi_np1;
+            pa.out = s % 2 == 0 ? psi_np1 : r.psis;
+            pa.stage = s;
+            FLB_TRY(launch_psi2(pa, p.storage, false, st));
+        }
+    }
+    cudaEvent_t e3 = mark(h);
+    span(h, 0, e1, e2, 1);
+    span(h, 1, e2, e3, (int)(h->launches - l2));
+    r.cur ^= 1;
+    r.pcur ^= 1;
+    r.step += 1;
+    return FLB_OK;
+}
+
 int step_rep(flb_handle *h, Rep &r)
 {
-    if (r.dim == 3 && !general_path(r.p)) return step_rep3(h, r);
+    if (r.dim == 2) return step_rep2(h, r);
+    if (!general_path(r.p)) return step_rep3(h, r);
     const Range range("step (per-site kernels)");
-    // one-thread-per-site path: 2D, and the 3D combinations of general_path()
+    // one-thread-per-site path: the combinations of general_path()
     const Geom &g = r.g;
     const flb_params &p = r.p;
     cudaStream_t st = h->st;
@@ -623,19 +686,15 @@ int step_rep(flb_handle *h, Rep &r)
     const int64_t l0 = h->launches;
     cudaEvent_t e0 = mark(h);
     FLB_TRY(launch_mu(g, psi_n, r.mu, (float)p.A, (float)p.B, (float)p.K, lw, st));
-    if ((p.coupling & FLB_COUPLE_FORCE) && p.force_grad == FLB_FORCE_STRESS) {
-        if (r.dim == 3) FLB_TRY(launch_sigma3(g, psi_n, r.sig, (float)p.A, (float)p.B, (float)p.K, st));
-        else FLB_TRY(launch_sigma2(g, psi_n, r.sig, (float)p.A, (float)p.B, (float)p.K, st));
-    }
+    if ((p.coupling & FLB_COUPLE_FORCE) && p.force_grad == FLB_FORCE_STRESS)
+        FLB_TRY(launch_sigma3(g, psi_n, r.sig, (float)p.A, (float)p.B, (float)p.K, st));
     cudaEvent_t e1 = mark(h);
 
     const LBArgs la = lb_args(r, psi_n);
-    if (r.dim == 3) FLB_TRY(r.q == 15 ? launch_lb15(la, p.storage, st) : launch_lb3d(la, p.storage, st));
-    else FLB_TRY(launch_lb(la, r.q, p.storage, st));
+    FLB_TRY(r.q == 15 ? launch_lb15(la, p.storage, st) : launch_lb3d(la, p.storage, st));
     cudaEvent_t e2 = mark(h);
     const int64_t l2 = h->launches;
-    if (r.dim == 3) FLB_TRY(r.q == 15 ? launch_vel15(la, p.storage, st) : launch_vel3(la, p.storage, st));
-    else FLB_TRY(launch_vel2(la, p.storage, st));
+    FLB_TRY(r.q == 15 ? launch_vel15(la, p.storage, st) : launch_vel3(la, p.storage, st));
 
     const bool noisy = p.kT > 0 && p.M > 0;
     if (noisy) {

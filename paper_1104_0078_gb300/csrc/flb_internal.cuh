@@ -181,6 +181,15 @@ constexpr Tables make_tables()
 // one copy per translation unit, read through the read-only cache
 static __device__ const bm::Tables kBM = bm::make_tables();
 
+// 1/sqrt(x) of a positive normal x: rsqrtf without its steps for subnormals (the same
+// approximation and bits)
+__device__ __forceinline__ float rsqrt_normal(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // Box-Muller on V::L independent words at once, one per lane (F2: two words in
 // Blackwell's packed FP32 registers): lane l turns word w[l] into
 // g0 = r cos 2 pi v, g1 = r sin 2 pi v (u, v and r as above).
@@ -221,7 +230,7 @@ __device__ __forceinline__ void bm_eval(const uint32_t *w, V sc, V &g0, V &g1)
     const V e2 = vfma(d, p, vfma(em, V::bc(-2.0f * 0.693147180559945f), vmake<V>(l2r)));  // >= 9.5e-7
     float rs[L];
 #pragma unroll
-    for (int l = 0; l < L; ++l) rs[l] = rsqrtf(e2.lane(l));
+    for (int l = 0; l < L; ++l) rs[l] = rsqrt_normal(e2.lane(l));
     V rad = e2 * vmake<V>(rs);
     if (SCALED) rad = rad * sc;
     // sin, cos of 2 pi v by angle addition
@@ -325,6 +334,31 @@ __device__ __forceinline__ void cp_async4(float *dst, const float *src, int src_
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
+
+// Programmatic dependent launch: a kernel of the step issues pdl_trigger at its
+// start, so that the next one's blocks may be scheduled as soon as its own leave
+// room, and pdl_wait before its first access to global memory, which returns when
+// the kernels before it in the stream have completed and their writes are visible.
+// What stands before pdl_wait (index arithmetic, random numbers) touches registers and
+// the block's own shared memory only.  A kernel that triggers also waits, so
+// completion stays in stream order however many launches overlap.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
 
 // ---------------------------------------------------------------------------
 // Geometry.  Populations: SoA planes [q][N], N = nx*ny*nz, unpadded, periodic
@@ -435,9 +469,9 @@ struct LBArgs {
     float gamma_g;             // ghost relaxation factor
     float kT;
     float namp[16];            // sqrt((1 - gamma_k^2)/b_k) of the noisy modes, in noise order
-    // D3Q19 collide-stream, in the units of its scaled stress Q = 4.5 B and scaled
-    // ghosts: rq = 4.5 (1 - ws), 4.5 ws, 4.5 cs (cs = 1 - ws/2), 1.5 (wb - ws),
-    // 3 (cb - cs); iso: wb != ws; k3T = kT / c_s^2; nq: the noise amplitudes
+    // D3Q19 and D2Q9 collide-streams, in the units of their scaled stress Q = 4.5 B
+    // and scaled ghosts: rq = 4.5 (1 - ws), 4.5 ws, 4.5 cs (cs = 1 - ws/2), 4.5/d (wb - ws),
+    // 9/d (cb - cs); iso: wb != ws; k3T = kT / c_s^2; nq: the noise amplitudes
     // namp scaled to those units
     float rq[5];
     int iso;
@@ -475,6 +509,23 @@ struct PsiArgs {
     int scheme;
     int stage;             // 1 or 2 (RK4: 1 to 4)
     int integrator;
+};
+
+// One Runge-Kutta stage of psi on the plane (flb_step2d.cu).
+struct Psi2Args {
+    Geom g;
+    const float *psi;      // padded stage input
+    const void *f;         // stage 1: the populations of the new fluid state [9][N]
+    float *u;              // padded velocity: written by stage 1, read by the later ones
+    float *out;            // padded stage output
+    float *E, *eta;        // [N] accumulator; RK4: the noise increment
+    const float *base;     // RK4: padded psi^n
+    float A, B, K, M, rho0;
+    float amp[3];          // noise: sqrt(2 kT M), sqrt(2 kT M a_l) of the axis and diagonal half-links
+    LapW lw;
+    int coupling, force_kind, scheme, integrator, stage;
+    PhiloxKey key;
+    int64_t step;
 };
 
 struct NoiseArgs {
@@ -643,20 +694,22 @@ void persist_tasks(std::vector<PTask> &v, int rep, int ph, const Geom &g, int zc
 cudaError_t launch_persist(const PersistArgs &a, bool q15, cudaStream_t st);  // q15: D3Q15 replicas
 
 // host launchers (flb_lb.cu, flb_psi.cu, flb_obs.cu)
-cudaError_t launch_lb(const LBArgs &a, int q, int storage, cudaStream_t s);
+// D2Q9: the collide-stream with the force formed from psi (p: A, B, K and the
+// Laplacian), and one stage of psi (flb_step2d.cu)
+cudaError_t launch_lb2(const LBArgs &a, const Psi2Args &p, int storage, cudaStream_t s);
+cudaError_t launch_psi2(const Psi2Args &a, int storage, bool noise, cudaStream_t s);
 // D3Q19 collide-stream that computes mu and the force itself from psi (flb_lb3d.cu)
 cudaError_t launch_lb3d(const LBArgs &a, int storage, cudaStream_t s);
-// order-parameter stress sigma on the interior + 1 ghost layer (flb_aux3d.cu, flb_psi.cu)
+// order-parameter stress sigma on the interior + 1 ghost layer (flb_aux3d.cu)
 cudaError_t launch_sigma3(const Geom &g, const float *psi, float *sig, float A, float B, float K, cudaStream_t st);
-cudaError_t launch_sigma2(const Geom &g, const float *psi, float *sig, float A, float B, float K, cudaStream_t st);
-// velocity of the streamed state after a step, written to a.u (flb_aux3d.cu, flb_lb.cu)
+// velocity of the streamed state after a step, written to a.u (flb_aux3d.cu)
 cudaError_t launch_vel3(const LBArgs &a, int storage, cudaStream_t s);
 cudaError_t launch_lb15(const LBArgs &a, int storage, cudaStream_t s);   // D3Q15 collide-stream
 cudaError_t launch_vel15(const LBArgs &a, int storage, cudaStream_t s);  // D3Q15 velocity of the new state
 // batched mu and velocity over the work lists (flb_aux3d.cu)
 cudaError_t launch_mu3_batch(const BatchLists &L, cudaStream_t st);
 cudaError_t launch_vel3_batch(const BatchLists &L, int storage, bool force, cudaStream_t st);
-cudaError_t launch_vel2(const LBArgs &a, int storage, cudaStream_t s);
+cudaError_t launch_vel2(const LBArgs &a, int storage, cudaStream_t s);  // of a D2Q9 start, without a force (flb_lb.cu)
 // one fused Runge-Kutta stage of psi on a 3D box (flb_psi3d.cu); q: the lattice
 // of the FV operators (19 or 15); mu_in: the mu of the stage input on the
 // interior and 2 ghost layers, or null (stage 1 then forms it)

@@ -87,82 +87,6 @@ __global__ void mu_kernel(const Geom g, const float *__restrict__ psi, float *__
     mu[g.pidx(x, y, z)] = A * p + B * p * p * p - K * lap_w(psi, g, x, y, z, lw);
 }
 
-// Order-parameter stress (Sec. IV, Eq. muf) in 2D on the interior + 1 ghost
-// layer: planes xx, yy, xy of sigma_ab = K g_a g_b + delta_ab [A/2 psi^2
-// + 3B/4 psi^4 - K psi lap_SO psi - K/2 |g|^2], g the central difference.
-__global__ void sigma2_kernel(const Geom g, const float *__restrict__ psi, float *__restrict__ sig, float A, float B,
-                              float K)
-{
-    const int ex = g.nx + 2, ey = g.ny + 2;
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)ex * ey) return;
-    const int x = (int)(i % ex) - 1, y = (int)(i / ex) - 1;
-    const float p = psi[g.pidx(x, y, 0)];
-    const float gx = 0.5f * (psi[g.pidx(x + 1, y, 0)] - psi[g.pidx(x - 1, y, 0)]);
-    const float gy = 0.5f * (psi[g.pidx(x, y + 1, 0)] - psi[g.pidx(x, y - 1, 0)]);
-    const float p2 = p * p;
-    const LapW so{-3.f, 0.5f, 0.25f, 0.f};  // the planar SO stencil (the stress form runs with SO only)
-    const float iso = 0.5f * A * p2 + 0.75f * B * p2 * p2 - K * p * lap_w(psi, g, x, y, 0, so) - 0.5f * K * (gx * gx + gy * gy);
-    const long long o = g.pidx(x, y, 0);
-    sig[o] = K * gx * gx + iso;
-    sig[o + g.pn] = K * gy * gy + iso;
-    sig[o + 2 * g.pn] = K * gx * gy;
-}
-
-// Noise increment eta of one 2D step (Sec. V), held fixed over the step's
-// Runge-Kutta stages.  A block of 32 x 16 threads first draws, once per point,
-// the four normals of every point of its tile and a one-point halo into shared
-// memory (counter: the point's site id, Philox stream 1, block 0), then
-//   FD: eta(r) = sum_l sqrt(2 kT M a_l) [zeta_l(r - c_l) - zeta_l(r)] over the
-//       half-links (1,0), (0,1), (1,1), (1,-1), a_l the Laplacian's axis and
-//       diagonal coefficients (SO: 1/2, 1/4);
-//   FV: eta(r) = (2/c_s^2) sum_i w_i c_i . (xi(r) + xi(r + c_i)) / 2, xi_a the
-//       first two normals times sqrt(2 kT M);
-//   naive (Sec. III): eta(r) = (1/2) sum_a [xi_a(r + e_a) - xi_a(r - e_a)].
-__global__ void __launch_bounds__(512) noise2_kernel(const NoiseArgs a)
-{
-    constexpr int TX = 32, TY = 16, HX = TX + 2, HY = TY + 2;
-    __shared__ float zs[4][HY][HX];
-    const Geom &g = a.g;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    const int t = threadIdx.x + TX * threadIdx.y;
-    for (int k = t; k < HX * HY; k += TX * TY) {
-        const int lx = k % HX, ly = k / HX;
-        const int gx = ((x0 - 1 + lx) % g.nx + g.nx) % g.nx, gy = ((y0 - 1 + ly) % g.ny + g.ny) % g.ny;
-        float G[4];
-        normals<2>(a.key, a.step, (uint32_t)(gx + g.nx * gy), 1u, 0u, G);
-        zs[0][ly][lx] = G[0];
-        zs[1][ly][lx] = G[1];
-        zs[2][ly][lx] = G[2];
-        zs[3][ly][lx] = G[3];
-    }
-    __syncthreads();
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-    if (x >= g.nx || y >= g.ny) return;
-    const int lx = threadIdx.x + 1, ly = threadIdx.y + 1;
-    float eta;
-    if (a.scheme == FLB_FD) {
-        const float s1 = sqrtf(2.f * a.kT * a.M * a.lw.c1), s2 = sqrtf(2.f * a.kT * a.M * a.lw.c2);  // sqrt(2 kT M a_l)
-        eta = s1 * ((zs[0][ly][lx - 1] - zs[0][ly][lx]) + (zs[1][ly - 1][lx] - zs[1][ly][lx])) +
-              s2 * ((zs[2][ly - 1][lx - 1] - zs[2][ly][lx]) + (zs[3][ly + 1][lx - 1] - zs[3][ly][lx]));
-    } else if (a.scheme == FLB_NAIVE) {
-        const float sd = sqrtf(2.f * a.kT * a.M);
-        eta = 0.5f * sd * ((zs[0][ly][lx + 1] - zs[0][ly][lx - 1]) + (zs[1][ly + 1][lx] - zs[1][ly - 1][lx]));
-    } else {
-        const float sd = sqrtf(2.f * a.kT * a.M);
-        const float ox = zs[0][ly][lx], oy = zs[1][ly][lx];
-        // axis links (w = 1/9) and diagonal links (w = 1/36), c . (xi(r) + xi(r + c))
-        const float ax = ((ox + zs[0][ly][lx + 1]) - (ox + zs[0][ly][lx - 1])) +
-                         ((oy + zs[1][ly + 1][lx]) - (oy + zs[1][ly - 1][lx]));
-        const float dg = ((ox + zs[0][ly + 1][lx + 1]) + (oy + zs[1][ly + 1][lx + 1])) -
-                         ((ox + zs[0][ly - 1][lx - 1]) + (oy + zs[1][ly - 1][lx - 1])) +
-                         ((ox + zs[0][ly - 1][lx + 1]) - (oy + zs[1][ly - 1][lx + 1])) -
-                         ((ox + zs[0][ly + 1][lx - 1]) - (oy + zs[1][ly + 1][lx - 1]));
-        eta = 3.f * sd * ((1.f / 9.f) * ax + (1.f / 36.f) * dg);
-    }
-    a.eta[x + g.nx * y] = eta;
-}
-
 // Noise increment eta of one 3D step for the one-thread-per-site path (other
 // Laplacians, the naive scheme, FV on D3Q15).  A block of 16 x 8 x 4 threads
 // draws, once per point, the normals of its tile and a one-point halo (18 x 10
@@ -331,25 +255,13 @@ cudaError_t launch_mu(const Geom &g, const float *psi, float *mu, float A, float
     return cudaGetLastError();
 }
 
-cudaError_t launch_sigma2(const Geom &g, const float *psi, float *sig, float A, float B, float K, cudaStream_t s)
-{
-    const long long ext = (long long)(g.nx + 2) * (g.ny + 2);
-    sigma2_kernel<<<blocks_for(ext, 256), 256, 0, s>>>(g, psi, sig, A, B, K);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_noise(const NoiseArgs &a, cudaStream_t s)
 {
-    if (a.g.dim == 3) {
-        const int smem = (a.scheme == FLB_FD ? 13 : 3) * N3P * (int)sizeof(float);
-        const cudaError_t e = cudaFuncSetAttribute(noise3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        const dim3 grid((a.g.nx + N3X - 1) / N3X, (a.g.ny + N3Y - 1) / N3Y, (a.g.nz + N3Z - 1) / N3Z);
-        noise3_kernel<<<grid, dim3(N3X, N3Y, N3Z), smem, s>>>(a);
-        return cudaGetLastError();
-    }
-    const dim3 grid((a.g.nx + 31) / 32, (a.g.ny + 15) / 16);
-    noise2_kernel<<<grid, dim3(32, 16), 0, s>>>(a);
+    const int smem = (a.scheme == FLB_FD ? 13 : 3) * N3P * (int)sizeof(float);
+    const cudaError_t e = cudaFuncSetAttribute(noise3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((a.g.nx + N3X - 1) / N3X, (a.g.ny + N3Y - 1) / N3Y, (a.g.nz + N3Z - 1) / N3Z);
+    noise3_kernel<<<grid, dim3(N3X, N3Y, N3Z), smem, s>>>(a);
     return cudaGetLastError();
 }
 
