@@ -80,9 +80,9 @@ struct Rep {
     int cur = 0;
     float *psi[2] = {nullptr, nullptr};
     int pcur = 0;
-    float *psis = nullptr, *mu = nullptr, *mus = nullptr, *u = nullptr, *J = nullptr, *eta = nullptr, *E = nullptr;
-    float *sig = nullptr;  // stress-form force: sigma planes (3D xx, yy, zz, xy, xz, yz; 2D xx, yy, xy)
-    float *Dn = nullptr;   // RK4 (3D): the step's noise increment per site
+    float *psis = nullptr, *mu = nullptr, *u = nullptr, *E = nullptr;
+    float *sig = nullptr;  // 3D stress-form force: sigma planes xx, yy, zz, xy, xz, yz
+    float *Dn = nullptr;   // RK4: the step's noise increment per site
     double *sq = nullptr, *hsq = nullptr;
     int Kx = 0, Ky = 0, Kz = 0;
     int64_t sq_n = 0, h_n = 0;
@@ -94,6 +94,8 @@ struct Rep {
     float omega_s = 0, omega_b = 0, gamma_g = 0;
     float namp[16] = {0};
     int zc = PS_ZC;  // planes per psi block (3D), set by flb_set_tuning / flb_autotune
+    bool tuned = false;  // whether it was set (else auto_depth chooses)
+    bool cube = false;   // tuned: the small-tile kernels were faster than any chunk
     int fused = 0;   // single-pass Heun psi step (flb_set_psi_fused)
 };
 
@@ -141,14 +143,9 @@ bool valid(const flb_params &p)
     return true;
 }
 
-// 3D combinations outside the tiled kernels (another Laplacian, the naive
-// scheme) run the one-thread-per-site kernels of the 2D path.
-bool general_path(const flb_params &p)
-{
-    // the tiled 3D kernels take the FD scheme with any Laplacian (class weights)
-    // and the FV scheme with the SO Laplacian
-    return p.dim == 3 && (p.psi_scheme == FLB_NAIVE || (p.laplacian != FLB_LAP_SO && p.psi_scheme != FLB_FD));
-}
+// 3D replicas whose psi stages may take the z-marching kernel: the FV scheme with the
+// SO Laplacian.  The others run the small-tile kernels at every size.
+bool marching(const flb_params &p) { return p.dim == 3 && p.psi_scheme == FLB_FV && p.laplacian == FLB_LAP_SO; }
 
 // Class weights of the App. A Laplacians (faces, edges, corners; 2D axes and
 // diagonals), the centre weight closing the sum to zero.
@@ -176,13 +173,48 @@ LapW lap_weights(int dim, int kind)
     return w;
 }
 
-// The class weights of a 3D replica's App. A Laplacian on the tiled FD path
-// (stored in w), or null for the SO Laplacian of the tiled kernels.
+// The class weights of a 3D replica's App. A Laplacian (stored in w), or null for SO.
 const LapW *app_a_weights(const Rep &r, LapW &w)
 {
-    if (r.dim != 3 || r.p.laplacian == FLB_LAP_SO || r.p.psi_scheme != FLB_FD) return nullptr;
+    if (r.dim != 3 || r.p.laplacian == FLB_LAP_SO) return nullptr;
     w = lap_weights(3, r.p.laplacian);
     return &w;
+}
+
+// Planes per block of the z-marching psi kernel where neither the caller nor the
+// tuner has chosen, or 0 for the small-tile kernels.  Those are the faster ones up to
+// about 110^3 (a Heun step at 96^3: 123 against 132 us with the best chunk, at 128^3 239
+// against 230 us).  Above, the even split of the depth that costs least with two
+// blocks on each of 152 SMs, a chunk of zc planes taking zc + 8 plane times (its
+// pipeline fills): 128^3 16 planes, 160^3 27, 256 x 256 x 64 32, 512^3 64 (what the
+// tuner finds there); with 64 planes throughout those took 1.6, 1.16, 1.16 times as long.
+int auto_depth(const Geom &g)
+{
+    if (g.n < 1300000) return 0;
+    const double cols = (double)((g.nx + PS_TX - 1) / PS_TX) * ((g.ny + PS_TY - 1) / PS_TY);
+    int best = PS_ZC;
+    double cbest = 0.0;
+    for (int k = 1; k <= g.nz; ++k) {
+        const int zc = (g.nz + k - 1) / k;
+        if (zc > PS_ZC) continue;
+        if (zc < 8) break;
+        double waves = cols * ((g.nz + zc - 1) / zc) / 304.0;
+        if (waves < 4.0) waves = std::ceil(waves);
+        const double cost = waves * (zc + 8);
+        if (cbest == 0.0 || cost < cbest) {
+            cbest = cost;
+            best = zc;
+        }
+    }
+    return best;
+}
+
+// The same as it stands for replica r now.
+int psi_depth(const Rep &r)
+{
+    if (!marching(r.p)) return 0;
+    if (!r.tuned) return auto_depth(r.g);
+    return r.cube ? 0 : r.zc;
 }
 
 Geom make_geom(const flb_params &p)
@@ -217,11 +249,6 @@ void carve_rep(Rep &r, Carver &cv)
         r.E = cv.take<float>(N);
     }
     if (r.p.integrator == FLB_RK4) r.Dn = cv.take<float>(N);
-    if (general_path(r.p)) {  // the per-site path keeps mu*, the noise increment and the FV flux in HBM
-        r.eta = cv.take<float>(N);
-        if (r.p.integrator != FLB_EULER) r.mus = cv.take<float>(P);
-        if (r.p.psi_scheme == FLB_FV) r.J = cv.take<float>((size_t)r.dim * P);
-    }
     if (r.p.force_grad == FLB_FORCE_STRESS && r.dim == 3) r.sig = cv.take<float>(6 * P);
     r.Kx = axis_K(g.nx, r.p.sq_kmax);
     r.Ky = axis_K(g.ny, r.p.sq_kmax);
@@ -540,6 +567,7 @@ int launch_psi_stages(flb_handle *h, Rep &r)
     const bool heun = p.integrator == FLB_HEUN;
     const int advect = (p.coupling & FLB_COUPLE_ADVECT) ? 1 : 0;
     const PhiloxKey key = philox_key(p.seed);
+    const int zc = psi_depth(r);
     if (p.integrator == FLB_RK4) {
         // stage inputs and outputs alternate between psi* and the spare psi buffer
         const float *in[4] = {psi_n, r.psis, psi_np1, r.psis};
@@ -547,7 +575,7 @@ int launch_psi_stages(flb_handle *h, Rep &r)
         for (int s = 0; s < 4; ++s)
             FLB_TRY(launch_psi3(r.g, p.psi_scheme, r.q, s == 0 ? 1 : 2, s == 0 && noisy, in[s], r.u, out[s], r.E,
                                 (float)p.A, (float)p.B, (float)p.K, (float)p.M, (float)p.kT, advect, 0, key, r.step,
-                                r.zc, s + 1, psi_n, r.Dn, s == 0 ? mu_n : nullptr, h->status, st, lw));
+                                zc, s + 1, psi_n, r.Dn, s == 0 ? mu_n : nullptr, h->status, st, lw));
         return FLB_OK;
     }
     if (r.fused && heun) {  // both stages in one launch (flb_set_psi_fused)
@@ -556,11 +584,11 @@ int launch_psi_stages(flb_handle *h, Rep &r)
         return FLB_OK;
     }
     FLB_TRY(launch_psi3(r.g, p.psi_scheme, r.q, 1, noisy, psi_n, r.u, heun ? r.psis : psi_np1, r.E, (float)p.A,
-                        (float)p.B, (float)p.K, (float)p.M, (float)p.kT, advect, heun ? 1 : 0, key, r.step, r.zc, 0,
+                        (float)p.B, (float)p.K, (float)p.M, (float)p.kT, advect, heun ? 1 : 0, key, r.step, zc, 0,
                         nullptr, nullptr, mu_n, h->status, st, lw));
     if (heun)
         FLB_TRY(launch_psi3(r.g, p.psi_scheme, r.q, 2, false, r.psis, r.u, psi_np1, r.E, (float)p.A, (float)p.B,
-                            (float)p.K, (float)p.M, (float)p.kT, advect, 1, key, r.step, r.zc, 0, nullptr, nullptr,
+                            (float)p.K, (float)p.M, (float)p.kT, advect, 1, key, r.step, zc, 0, nullptr, nullptr,
                             nullptr, h->status, st, lw));
     return FLB_OK;
 }
@@ -672,102 +700,7 @@ int step_rep2(flb_handle *h, Rep &r)
     return FLB_OK;
 }
 
-int step_rep(flb_handle *h, Rep &r)
-{
-    if (r.dim == 2) return step_rep2(h, r);
-    if (!general_path(r.p)) return step_rep3(h, r);
-    const Range range("step (per-site kernels)");
-    // one-thread-per-site path: the combinations of general_path()
-    const Geom &g = r.g;
-    const flb_params &p = r.p;
-    cudaStream_t st = h->st;
-    const LapW lw = lap_weights(r.dim, p.laplacian);
-    float *psi_n = r.psi[r.pcur], *psi_np1 = r.psi[r.pcur ^ 1];
-    const int64_t l0 = h->launches;
-    cudaEvent_t e0 = mark(h);
-    FLB_TRY(launch_mu(g, psi_n, r.mu, (float)p.A, (float)p.B, (float)p.K, lw, st));
-    if ((p.coupling & FLB_COUPLE_FORCE) && p.force_grad == FLB_FORCE_STRESS)
-        FLB_TRY(launch_sigma3(g, psi_n, r.sig, (float)p.A, (float)p.B, (float)p.K, st));
-    cudaEvent_t e1 = mark(h);
-
-    const LBArgs la = lb_args(r, psi_n);
-    FLB_TRY(r.q == 15 ? launch_lb15(la, p.storage, st) : launch_lb3d(la, p.storage, st));
-    cudaEvent_t e2 = mark(h);
-    const int64_t l2 = h->launches;
-    FLB_TRY(r.q == 15 ? launch_vel15(la, p.storage, st) : launch_vel3(la, p.storage, st));
-
-    const bool noisy = p.kT > 0 && p.M > 0;
-    if (noisy) {
-        NoiseArgs na;
-        na.g = g;
-        na.eta = r.eta;
-        na.kT = (float)p.kT;
-        na.M = (float)p.M;
-        na.scheme = p.psi_scheme;
-        na.q = r.q;
-        na.lw = lw;
-        na.key = philox_key(p.seed);
-        na.step = r.step;
-        FLB_TRY(launch_noise(na, st));
-    }
-    if (p.psi_scheme == FLB_FV) FLB_TRY(launch_flux(g, r.q, psi_n, r.mu, r.u, r.J, (float)p.M, p.coupling, st));
-    PsiArgs pa;
-    pa.g = g;
-    pa.lw = lw;
-    pa.q = r.q;
-    pa.psi = psi_n;
-    pa.mu = r.mu;
-    pa.u = r.u;
-    pa.J = r.J;
-    pa.eta = noisy ? r.eta : nullptr;
-    pa.psi0 = nullptr;
-    pa.out = p.integrator == FLB_EULER ? psi_np1 : r.psis;
-    pa.acc = r.E;
-    pa.base = psi_n;
-    pa.A = (float)p.A;
-    pa.B = (float)p.B;
-    pa.K = (float)p.K;
-    pa.M = (float)p.M;
-    pa.coupling = p.coupling;
-    pa.scheme = p.psi_scheme;
-    pa.stage = 1;
-    pa.integrator = p.integrator;
-    FLB_TRY(launch_psi_update(pa, r.q, st));
-    if (p.integrator == FLB_RK4) {  // stages 2-4 alternate between psi* and the spare psi buffer
-        float *in[3] = {r.psis, psi_np1, r.psis};
-        float *out[3] = {psi_np1, r.psis, psi_np1};
-        for (int s = 0; s < 3; ++s) {
-            FLB_TRY(launch_mu(g, in[s], r.mus, (float)p.A, (float)p.B, (float)p.K, lw, st));
-            if (p.psi_scheme == FLB_FV)
-                FLB_TRY(launch_flux(g, r.q, in[s], r.mus, r.u, r.J, (float)p.M, p.coupling, st));
-            pa.psi = in[s];
-            pa.mu = r.mus;
-            pa.out = out[s];
-            pa.stage = s + 2;
-            FLB_TRY(launch_psi_update(pa, r.q, st));
-        }
-    }
-    if (p.integrator == FLB_HEUN) {
-        FLB_TRY(launch_mu(g, r.psis, r.mus, (float)p.A, (float)p.B, (float)p.K, lw, st));
-        if (p.psi_scheme == FLB_FV)
-            FLB_TRY(launch_flux(g, r.q, r.psis, r.mus, r.u, r.J, (float)p.M, p.coupling, st));
-        pa.psi = r.psis;
-        pa.mu = r.mus;
-        pa.psi0 = r.E;
-        pa.out = psi_np1;
-        pa.stage = 2;
-        FLB_TRY(launch_psi_update(pa, r.q, st));
-    }
-    cudaEvent_t e3 = mark(h);
-    span(h, 0, e1, e2, 1);
-    span(h, 1, e0, e1, 1);
-    span(h, 1, e2, e3, (int)(h->launches - l2));
-    (void)l0;
-    r.cur ^= 1;
-    r.pcur ^= 1;
-    r.step += 1;
-    return FLB_OK;
-}
+int step_rep(flb_handle *h, Rep &r) { return r.dim == 2 ? step_rep2(h, r) : step_rep3(h, r); }
 
 int sample_rep(flb_handle *h, Rep &r, int mask)
 {
@@ -1683,11 +1616,17 @@ int flb_set_tuning(flb_handle *h, int32_t rep, int32_t psi_zchunk)
 {
     if (!h || psi_zchunk < PS_ZC_MIN || psi_zchunk > 4096) return FLB_EINVAL;
     if (rep == -1) {
-        for (Rep &r : h->reps) r.zc = psi_zchunk;
+        for (Rep &r : h->reps) {
+            r.zc = psi_zchunk;
+            r.tuned = true;
+            r.cube = false;
+        }
     } else {
         Rep *r = get_rep(h, rep);
         if (!r) return FLB_EINVAL;
         r->zc = psi_zchunk;
+        r->tuned = true;
+        r->cube = false;
     }
     batch_reset(h);
     return FLB_OK;
@@ -1780,34 +1719,44 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
             }
         }
     } else {
-        std::map<std::string, int> done;
+        std::map<std::string, std::pair<int, bool>> done;
         for (Rep &r : h->reps) {
-            if (r.dim != 3 || general_path(r.p)) continue;
+            if (!marching(r.p)) continue;
             const std::string key = "plain|" + dk + "|" + rep_key(r);
             auto d = done.find(key);
-            if (d != done.end()) {
-                r.zc = d->second;
-                continue;
-            }
             const auto it = cache.find(key);
-            if (it != cache.end()) {
+            if (d != done.end()) {
+                r.zc = d->second.first;
+                r.cube = d->second.second;
+            } else if (it != cache.end()) {
                 r.zc = it->second;
+                r.cube = auto_depth(r.g) == 0;
             } else {
                 float tbest = 0.f;
                 int best = PS_ZC;
+                auto timed = [&](float &t) {
+                    t = time_launches(h, [&]() { return launch_psi_stages(h, r); }, reps);
+                    return t >= 0.f;
+                };
+                r.tuned = true;
+                r.cube = false;
+                float t;
                 for (int zc : zc_candidates(r.g.nz)) {
                     r.zc = zc;
-                    const float t = time_launches(h, [&]() { return launch_psi_stages(h, r); }, reps);
-                    if (t < 0.f) return FLB_ECUDA;
+                    if (!timed(t)) return FLB_ECUDA;
                     if (tbest == 0.f || t < tbest) {
                         tbest = t;
                         best = zc;
                     }
                 }
                 r.zc = best;
+                r.cube = true;  // the small tiles, where they are faster than any chunk
+                if (!timed(t)) return FLB_ECUDA;
+                r.cube = t < tbest;
                 append_cache(cache_path, key, best);
             }
-            done[key] = r.zc;
+            r.tuned = true;
+            done[key] = {r.zc, r.cube};
         }
     }
     batch_reset(h);

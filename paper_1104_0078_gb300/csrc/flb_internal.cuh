@@ -344,8 +344,16 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 // completion stays in stream order however many launches overlap.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Each block's wait drops its SM's L1 contents, which a grid of many short blocks
+// pays for over and over (a 512^3 step took 13.2 ms with every launch so made
+// and 10.2 ms with none), so a grid above max_blocks is launched in plain stream order (both
+// instructions then return at once).  16 blocks per SM is where a step of 64^3 to
+// 128^3 gains most (64^3: 59.0 -> 49.1 us); the 2D kernels, which read little twice,
+// gain up to larger grids (2048^2, 8192 blocks: 244 -> 233 us).
+constexpr long long PDL_BLOCKS = 16 * 152;
 template <class... P, class... A>
-inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              long long max_blocks, A &&...args)
 {
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -356,7 +364,7 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
     c.dynamicSmemBytes = smem;
     c.stream = st;
     c.attrs = at;
-    c.numAttrs = 1;
+    c.numAttrs = (long long)grid.x * grid.y * grid.z <= max_blocks ? 1 : 0;
     return cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 
@@ -491,26 +499,6 @@ struct LapW {
     float c0, c1, c2, c3;
 };
 
-struct PsiArgs {
-    Geom g;
-    LapW lw;               // FD / naive: the Laplacian of mu and of M lap mu
-    int q;                 // FV: the lattice of the gradient and divergence (9, 15 or 19)
-    const float *psi;      // padded psi at the stage input
-    const float *mu;       // padded mu of that psi, valid to halo 2
-    const float *u;        // padded u, valid to halo 1
-    const float *J;        // FV: padded deterministic node flux, valid to halo 1
-    const float *eta;      // noise increment per site [N]
-    const float *psi0;     // stage 2: Heun accumulator E [N]
-    float *out;            // padded psi output (images to the full frame)
-    float *acc;            // stage 1 of Heun: E = psi + D/2 + eta [N]; RK4: the running sum
-    const float *base;     // RK4: padded psi^n
-    float A, B, K, M;
-    int coupling;
-    int scheme;
-    int stage;             // 1 or 2 (RK4: 1 to 4)
-    int integrator;
-};
-
 // One Runge-Kutta stage of psi on the plane (flb_step2d.cu).
 struct Psi2Args {
     Geom g;
@@ -524,17 +512,6 @@ struct Psi2Args {
     float amp[3];          // noise: sqrt(2 kT M), sqrt(2 kT M a_l) of the axis and diagonal half-links
     LapW lw;
     int coupling, force_kind, scheme, integrator, stage;
-    PhiloxKey key;
-    int64_t step;
-};
-
-struct NoiseArgs {
-    Geom g;
-    float *eta;            // [N]
-    float kT, M;
-    int scheme;
-    int q;                 // FV: lattice of the noise divergence
-    LapW lw;               // FD: link weights are the Laplacian's class coefficients
     PhiloxKey key;
     int64_t step;
 };
@@ -693,7 +670,7 @@ void persist_tiles(const Geom &g, int zc, int coupling, int heun, int counts[PH_
 void persist_tasks(std::vector<PTask> &v, int rep, int ph, const Geom &g, int zc, int need);
 cudaError_t launch_persist(const PersistArgs &a, bool q15, cudaStream_t st);  // q15: D3Q15 replicas
 
-// host launchers (flb_lb.cu, flb_psi.cu, flb_obs.cu)
+// host launchers (flb_lb.cu, flb_obs.cu)
 // D2Q9: the collide-stream with the force formed from psi (p: A, B, K and the
 // Laplacian), and one stage of psi (flb_step2d.cu)
 cudaError_t launch_lb2(const LBArgs &a, const Psi2Args &p, int storage, cudaStream_t s);
@@ -710,9 +687,11 @@ cudaError_t launch_vel15(const LBArgs &a, int storage, cudaStream_t s);  // D3Q1
 cudaError_t launch_mu3_batch(const BatchLists &L, cudaStream_t st);
 cudaError_t launch_vel3_batch(const BatchLists &L, int storage, bool force, cudaStream_t st);
 cudaError_t launch_vel2(const LBArgs &a, int storage, cudaStream_t s);  // of a D2Q9 start, without a force (flb_lb.cu)
-// one fused Runge-Kutta stage of psi on a 3D box (flb_psi3d.cu); q: the lattice
-// of the FV operators (19 or 15); mu_in: the mu of the stage input on the
-// interior and 2 ghost layers, or null (stage 1 then forms it)
+// one fused Runge-Kutta stage of psi on a 3D box: zc planes per z-marching block
+// (flb_psi3d.cu; FV with SO's Laplacian), or small tiles with zc 0 (flb_psi3c.cu;
+// every scheme and Laplacian); q: the lattice of the FV operators
+// (19 or 15); mu_in: the mu of the stage input on the interior and 2 ghost layers,
+// or null (stage 1 then forms it)
 cudaError_t launch_psi3(const Geom &g, int scheme, int q, int stage, bool noise, const float *psi, const float *u,
                         float *out, float *E, float A, float B, float K, float M, float kT, int advect, int heun,
                         const PhiloxKey &key, int64_t step, int zc, int rk4, const float *base, float *Dn,
@@ -723,8 +702,6 @@ cudaError_t launch_mu3(const Geom &g, const float *psi, float *mu, float A, floa
                        const LapW *lw = nullptr);
 cudaError_t launch_init_eq(const Geom &g, int q, int storage, const float *rho, const float *u, float rho0, void *f,
                            cudaStream_t st);
-cudaError_t launch_mu(const Geom &g, const float *psi, float *mu, float A, float B, float K, const LapW &lw,
-                      cudaStream_t s);
 // both Heun stages of the FV psi step in one launch by halo recompute (flb_heun1.cu)
 cudaError_t launch_psi3_heun1(const Geom &g, int scheme, const float *psi, const float *u, float *out, float A, float B,
                               float K, float M, float kT, int advect, bool noise, const PhiloxKey &key, int64_t step,
@@ -735,9 +712,5 @@ cudaError_t launch_psi3_heun1(const Geom &g, int scheme, const float *psi, const
 cudaError_t launch_equilibrium_start(const Geom &g, int q, int storage, const LapW &lw, double rho0, double kT,
                                      double A, double K, uint64_t seed, void *f, void *spare, float *psi,
                                      cudaStream_t st);
-cudaError_t launch_noise(const NoiseArgs &a, cudaStream_t s);
-cudaError_t launch_flux(const Geom &g, int q, const float *psi, const float *mu, const float *u, float *J, float M,
-                        int coupling, cudaStream_t s);
-cudaError_t launch_psi_update(const PsiArgs &a, int q, cudaStream_t s);
 
 }  // namespace flb

@@ -13,7 +13,6 @@ constexpr int PS_NT = PS_TX * PS_TY;
 constexpr int H3X = PS_TX + 6, H3Y = PS_TY + 6, H3N = H3X * H3Y;  // psi: tile + 3
 constexpr int H2X = PS_TX + 4, H2Y = PS_TY + 4, H2N = H2X * H2Y;  // mu: tile + 2
 constexpr int H1X = PS_TX + 2, H1Y = PS_TY + 2, H1N = H1X * H1Y;  // flux / noise: tile + 1
-constexpr int S3 = (H3N + PS_NT - 1) / PS_NT, S2 = (H2N + PS_NT - 1) / PS_NT, S1 = (H1N + PS_NT - 1) / PS_NT;
 
 struct Psi3Args {
     Geom g;
@@ -29,43 +28,13 @@ struct Psi3Args {
     float *Dn;         // RK4: [N] noise increment, written in stage 1, read in stages 2, 3
     PhiloxKey key;
     int64_t step;
-    LapW lw;           // FD: the class weights of an App. A Laplacian when lap_w (else SO's)
+    LapW lw;           // the class weights of an App. A Laplacian when lap_w (else SO's)
     int lap_w;
 };
 
-// Output of a Runge-Kutta stage at interior site (x, y, z), site index si: pv the
-// stage input there (stage 1), D the deterministic increment, eta the noise
-// increment (generated in stage 1; Sec. V holds it fixed over the step).
-//   Euler / Heun (Sec. V): stage 1 psi + D + eta (Heun also E = psi + D/2 + eta),
-//     stage 2 E + D/2.
-//   RK4: k_s = D_s + eta; stage 1 writes psi + k1/2 and E = psi + eta + D1/6 and
-//     keeps eta; stages 2, 3 write psi^n + k2/2, psi^n + k3 and add D_s/3 to E;
-//     stage 4 writes E + D4/6 = psi^n + (k1 + 2 k2 + 2 k3 + k4)/6.
-//   RK false compiles the RK4 branches out (only for launches with a.rk4 == 0).
-template <int STAGE, bool COH, bool RK = true>
-__device__ __forceinline__ float rk_stage_out(const Psi3Args &a, int x, int y, int z, int si, float pv, float D,
-                                              float eta)
-{
-    if (RK && a.rk4) {
-        constexpr float sixth = 1.f / 6.f, third = 1.f / 3.f;
-        if (a.rk4 == 1) {
-            a.E[si] = pv + eta + sixth * D;
-            a.Dn[si] = eta;
-            return pv + 0.5f * (D + eta);
-        }
-        const float e = COH ? __ldcg(a.E + si) : a.E[si];
-        if (a.rk4 == 4) return e + sixth * D;
-        const float n = COH ? __ldcg(a.Dn + si) : a.Dn[si];
-        const float b = COH ? __ldcg(a.base + a.g.pidx32(x, y, z)) : a.base[a.g.pidx32(x, y, z)];
-        a.E[si] = e + third * D;
-        return a.rk4 == 2 ? b + 0.5f * (D + n) : b + D + n;
-    }
-    if (STAGE == 1) {
-        if (a.heun) a.E[si] = pv + 0.5f * D + eta;
-        return pv + D + eta;
-    }
-    return (COH ? __ldcg(a.E + si) : a.E[si]) + 0.5f * D;
-}
+// One stage by small tiles (flb_psi3c.cu).
+cudaError_t launch_psi3_cube(const Psi3Args &a, int scheme, int q, bool first, bool noise, const float *mu_in,
+                             cudaStream_t st);
 
 // Point k of a W x H region (W >= 32): rows' first 32 columns first, then the
 // W - 32 remaining columns of every row.

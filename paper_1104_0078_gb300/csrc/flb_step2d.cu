@@ -452,6 +452,7 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
 // Tiles: 32 x 16 where two blocks per SM of them cover the chip, else 16 x 8: a
 // small box then has four times the blocks, each with one point per thread, and its
 // latency is what a step costs.
+constexpr long long PDL_BLOCKS2 = 108 * 152;  // see launch_pdl
 bool small_box2(const Geom &g) { return (long long)g.nx * g.ny < 304LL * 512; }
 
 template <int TX, int TY, int NT, typename T, bool FV, bool FIRST, bool NOISE>
@@ -462,7 +463,7 @@ cudaError_t go_psi2(const Psi2Args &a, cudaStream_t st)
     const bool stress = FIRST && (a.coupling & FLB_COUPLE_FORCE) && a.force_kind == 2;
     const size_t smem = sizeof(float) * (size_t)(NP + NM + (2 + (NOISE ? (FV ? 2 : 4) : 0)) * N1 + (stress ? 3 * NM : 0));
     const dim3 grid((a.g.nx + TX - 1) / TX, (a.g.ny + TY - 1) / TY);
-    return launch_pdl(psi2_kernel<TX, TY, NT, T, FV, FIRST, NOISE>, grid, NT, smem, st, a);
+    return launch_pdl(psi2_kernel<TX, TY, NT, T, FV, FIRST, NOISE>, grid, NT, smem, st, PDL_BLOCKS2, a);
 }
 
 template <typename T, bool FV, bool FIRST, bool NOISE>
@@ -488,10 +489,10 @@ cudaError_t go_lb2(const LBArgs &a, const Psi2Args &p, int storage, cudaStream_t
     const dim3 grid((a.g.nx + TX - 1) / TX, (a.g.ny + TY - 1) / TY);
     const bool gr = a.gamma_g != 0.0f;
     if (storage == FLB_F16_DEV)
-        return gr ? launch_pdl(lb2_kernel<TX, TY, V, __half, true>, grid, NT, 0, st, a, p)
-                  : launch_pdl(lb2_kernel<TX, TY, V, __half, false>, grid, NT, 0, st, a, p);
-    return gr ? launch_pdl(lb2_kernel<TX, TY, V, float, true>, grid, NT, 0, st, a, p)
-              : launch_pdl(lb2_kernel<TX, TY, V, float, false>, grid, NT, 0, st, a, p);
+        return gr ? launch_pdl(lb2_kernel<TX, TY, V, __half, true>, grid, NT, 0, st, PDL_BLOCKS2, a, p)
+                  : launch_pdl(lb2_kernel<TX, TY, V, __half, false>, grid, NT, 0, st, PDL_BLOCKS2, a, p);
+    return gr ? launch_pdl(lb2_kernel<TX, TY, V, float, true>, grid, NT, 0, st, PDL_BLOCKS2, a, p)
+              : launch_pdl(lb2_kernel<TX, TY, V, float, false>, grid, NT, 0, st, PDL_BLOCKS2, a, p);
 }
 
 }  // namespace
