@@ -31,6 +31,8 @@ struct PlanesStride32 {
 template <typename T, bool FORCE>
 __global__ void __launch_bounds__(LB_BX *LB_BY, 10) vel3_kernel(const LBArgs a)
 {
+    pdl_trigger();
+    pdl_wait();
     const Geom &g = a.g;
     const int x = blockIdx.x * LB_BX + threadIdx.x;
     const int y = blockIdx.y * LB_BY + threadIdx.y;
@@ -65,6 +67,8 @@ __device__ __forceinline__ void mu3_block(const Geom &g, const float *__restrict
 __global__ void __launch_bounds__(MU_BX *MU_BY) sigma3_kernel(const Geom g, const float *__restrict__ psi,
                                                              float *__restrict__ sig, float A, float B, float K)
 {
+    pdl_trigger();
+    pdl_wait();
     const int x = blockIdx.x * MU_BX + (int)threadIdx.x - 1;
     const int y = blockIdx.y * MU_BY + (int)threadIdx.y - 1;
     const int zb = blockIdx.z * MU_ZC - 1;
@@ -78,6 +82,8 @@ template <bool W>
 __global__ void __launch_bounds__(MU_BX *MU_BY) mu3_kernel(const Geom g, const float *__restrict__ psi,
                                                           float *__restrict__ mu, float A, float B, float K, const LapW lw)
 {
+    pdl_trigger();
+    pdl_wait();
     mu3_block<MU3_HALO>(g, psi, mu, A, B, K, blockIdx.x, blockIdx.y, blockIdx.z, W ? &lw : nullptr);
 }
 
@@ -89,14 +95,19 @@ __global__ void __launch_bounds__(MU_BX *MU_BY) mu3_kernel(const Geom g, const f
 // the same sums in the same order (mu_so), so the field is bitwise that of the
 // batched and persistent kernels.  Points x < -2 or x >= nx + 2 are not written,
 // and the side cells they alone would need are not read.
-constexpr int MV_TX = 16, MV_TY = 8, MV_ZC = 16;
+// A block marches zc planes: 16, or 4 where that leaves fewer than four 128-thread blocks
+// per SM (64^3 has 90 blocks of 16 planes).
+constexpr int MV_TX = 16, MV_TY = 8, MV_ZC = 16, MV_ZC_SMALL = 4;
 
 __global__ void __launch_bounds__(MV_TX *MV_TY) mu3_vec_kernel(const Geom g, const float *__restrict__ psi,
-                                                             float *__restrict__ mu, float A, float B, float K)
+                                                             float *__restrict__ mu, float A, float B, float K,
+                                                             int zc)
 {
+    pdl_trigger();
+    pdl_wait();
     const int xs = -4 + 4 * (int)(blockIdx.x * MV_TX + threadIdx.x);
     const int y = (int)(blockIdx.y * MV_TY + threadIdx.y) - MU3_HALO;
-    const int zb = (int)blockIdx.z * MV_ZC - MU3_HALO, ze = min(zb + MV_ZC, g.nz + MU3_HALO);
+    const int zb = (int)blockIdx.z * zc - MU3_HALO, ze = min(zb + zc, g.nz + MU3_HALO);
     const int xl = g.nx + MU3_HALO;  // one past the last output column
     if (xs + 3 < -MU3_HALO || xs >= xl || y >= g.ny + MU3_HALO || zb >= ze) return;
     const bool lo = xs - 1 >= -MU3_HALO - 1, hi = xs + 4 <= xl;  // side cells some point needs
@@ -168,23 +179,22 @@ cudaError_t launch_mu3(const Geom &g, const float *psi, float *mu, float A, floa
     constexpr int E = 2 * MU3_HALO;
     if (!lw && g.dim == 3) {  // threads for x = -4 .. nx + 1 in fours
         const int nxt = (g.nx + 2 + 4 + 3) / 4;
-        const dim3 vgrid((nxt + MV_TX - 1) / MV_TX, (g.ny + E + MV_TY - 1) / MV_TY, (g.nz + E + MV_ZC - 1) / MV_ZC);
-        mu3_vec_kernel<<<vgrid, dim3(MV_TX, MV_TY, 1), 0, st>>>(g, psi, mu, A, B, K);
-        return cudaGetLastError();
+        const int cols = ((nxt + MV_TX - 1) / MV_TX) * ((g.ny + E + MV_TY - 1) / MV_TY);
+        const int zc = cols * ((g.nz + E + MV_ZC - 1) / MV_ZC) < 4 * 152 ? MV_ZC_SMALL : MV_ZC;
+        const dim3 vgrid((nxt + MV_TX - 1) / MV_TX, (g.ny + E + MV_TY - 1) / MV_TY, (g.nz + E + zc - 1) / zc);
+        return launch_pdl(mu3_vec_kernel, vgrid, dim3(MV_TX, MV_TY, 1), 0, st, PDL_BLOCKS, g, psi, mu, A, B, K, zc);
     }
     const dim3 block(MU_BX, MU_BY, 1);
     const dim3 grid((g.nx + E + MU_BX - 1) / MU_BX, (g.ny + E + MU_BY - 1) / MU_BY, (g.nz + E + MU_ZC - 1) / MU_ZC);
-    if (lw) mu3_kernel<true><<<grid, block, 0, st>>>(g, psi, mu, A, B, K, *lw);
-    else mu3_kernel<false><<<grid, block, 0, st>>>(g, psi, mu, A, B, K, LapW{0.f, 0.f, 0.f, 0.f});
-    return cudaGetLastError();
+    return lw ? launch_pdl(mu3_kernel<true>, grid, block, 0, st, PDL_BLOCKS, g, psi, mu, A, B, K, *lw)
+              : launch_pdl(mu3_kernel<false>, grid, block, 0, st, PDL_BLOCKS, g, psi, mu, A, B, K, LapW{0.f, 0.f, 0.f, 0.f});
 }
 
 cudaError_t launch_sigma3(const Geom &g, const float *psi, float *sig, float A, float B, float K, cudaStream_t st)
 {
     const dim3 block(MU_BX, MU_BY, 1);
     const dim3 grid((g.nx + 2 + MU_BX - 1) / MU_BX, (g.ny + 2 + MU_BY - 1) / MU_BY, (g.nz + 2 + MU_ZC - 1) / MU_ZC);
-    sigma3_kernel<<<grid, block, 0, st>>>(g, psi, sig, A, B, K);
-    return cudaGetLastError();
+    return launch_pdl(sigma3_kernel, grid, block, 0, st, PDL_BLOCKS, g, psi, sig, A, B, K);
 }
 
 cudaError_t launch_vel3(const LBArgs &a, int storage, cudaStream_t st)
@@ -192,14 +202,11 @@ cudaError_t launch_vel3(const LBArgs &a, int storage, cudaStream_t st)
     const dim3 block(LB_BX, LB_BY, 1);
     const dim3 grid((a.g.nx + LB_BX - 1) / LB_BX, (a.g.ny + LB_BY - 1) / LB_BY, (a.g.nz + LB_BZ - 1) / LB_BZ);
     const bool force = (a.coupling & FLB_COUPLE_FORCE) != 0;
-    if (storage == FLB_F16_DEV) {
-        if (force) vel3_kernel<__half, true><<<grid, block, 0, st>>>(a);
-        else vel3_kernel<__half, false><<<grid, block, 0, st>>>(a);
-    } else {
-        if (force) vel3_kernel<float, true><<<grid, block, 0, st>>>(a);
-        else vel3_kernel<float, false><<<grid, block, 0, st>>>(a);
-    }
-    return cudaGetLastError();
+    if (storage == FLB_F16_DEV)
+        return force ? launch_pdl(vel3_kernel<__half, true>, grid, block, 0, st, PDL_BLOCKS, a)
+                     : launch_pdl(vel3_kernel<__half, false>, grid, block, 0, st, PDL_BLOCKS, a);
+    return force ? launch_pdl(vel3_kernel<float, true>, grid, block, 0, st, PDL_BLOCKS, a)
+                 : launch_pdl(vel3_kernel<float, false>, grid, block, 0, st, PDL_BLOCKS, a);
 }
 
 cudaError_t launch_mu3_batch(const BatchLists &L, cudaStream_t st)

@@ -14,6 +14,8 @@ namespace {
 template <typename T, bool GHOST_RELAX, bool FORCE>
 __global__ void __launch_bounds__(LB_BX *LB_BY, 7) lb15_kernel(const LBArgs a, const __grid_constant__ PlaneTable<T> P)
 {
+    pdl_trigger();
+    pdl_wait();
     const Geom &g = a.g;
     const int x = blockIdx.x * LB_BX + threadIdx.x;
     const int y = blockIdx.y * LB_BY + threadIdx.y;
@@ -31,6 +33,8 @@ __global__ void __launch_bounds__(LB_BX *LB_BY, 7) lb15_kernel(const LBArgs a, c
 template <typename T, bool FORCE>
 __global__ void __launch_bounds__(LB_BX *LB_BY *LB_BZ) vel15_kernel(const LBArgs a)
 {
+    pdl_trigger();
+    pdl_wait();
     const Geom &g = a.g;
     const int x = blockIdx.x * LB_BX + threadIdx.x;
     const int y = blockIdx.y * LB_BY + threadIdx.y;
@@ -104,7 +108,7 @@ cudaError_t launch_lb15(const LBArgs &a, int storage, cudaStream_t st)
     const dim3 grid((a.g.nx + LB_BX - 1) / LB_BX, (a.g.ny + LB_BY - 1) / LB_BY, (a.g.nz + LB_BZ - 1) / LB_BZ);
     const bool gr = a.gamma_g != 0.0f;
     const bool force = (a.coupling & FLB_COUPLE_FORCE) != 0;
-#define FLB_LB15(T, G, F) lb15_kernel<T, G, F><<<grid, block, 0, st>>>(a, plane_table<T>(a.fin, a.fout, a.g.n, 15))
+#define FLB_LB15(T, G, F) return launch_pdl(lb15_kernel<T, G, F>, grid, block, 0, st, PDL_BLOCKS, a, plane_table<T>(a.fin, a.fout, a.g.n, 15))
     if (storage == FLB_F16_DEV) {
         if (gr) { if (force) FLB_LB15(__half, true, true); else FLB_LB15(__half, true, false); }
         else { if (force) FLB_LB15(__half, false, true); else FLB_LB15(__half, false, false); }
@@ -113,7 +117,6 @@ cudaError_t launch_lb15(const LBArgs &a, int storage, cudaStream_t st)
         else { if (force) FLB_LB15(float, false, true); else FLB_LB15(float, false, false); }
     }
 #undef FLB_LB15
-    return cudaGetLastError();
 }
 
 cudaError_t launch_vel15(const LBArgs &a, int storage, cudaStream_t st)
@@ -122,13 +125,12 @@ cudaError_t launch_vel15(const LBArgs &a, int storage, cudaStream_t st)
     const dim3 grid((a.g.nx + LB_BX - 1) / LB_BX, (a.g.ny + LB_BY - 1) / LB_BY, (a.g.nz + LB_BZ - 1) / LB_BZ);
     const bool force = (a.coupling & FLB_COUPLE_FORCE) != 0;
     if (storage == FLB_F16_DEV) {
-        if (force) vel15_kernel<__half, true><<<grid, block, 0, st>>>(a);
-        else vel15_kernel<__half, false><<<grid, block, 0, st>>>(a);
+        if (force) return launch_pdl(vel15_kernel<__half, true>, grid, block, 0, st, PDL_BLOCKS, a);
+        else return launch_pdl(vel15_kernel<__half, false>, grid, block, 0, st, PDL_BLOCKS, a);
     } else {
-        if (force) vel15_kernel<float, true><<<grid, block, 0, st>>>(a);
-        else vel15_kernel<float, false><<<grid, block, 0, st>>>(a);
+        if (force) return launch_pdl(vel15_kernel<float, true>, grid, block, 0, st, PDL_BLOCKS, a);
+        else return launch_pdl(vel15_kernel<float, false>, grid, block, 0, st, PDL_BLOCKS, a);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace flb

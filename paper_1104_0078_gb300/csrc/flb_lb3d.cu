@@ -28,6 +28,8 @@ template <typename T, bool GHOST_RELAX, bool FORCE>
 __global__ void __launch_bounds__(LB_BX *LB_BY, 7)
     lb3_kernel(const LBArgs a, const __grid_constant__ PlaneTable<T> P)
 {
+    pdl_trigger();
+    pdl_wait();
     const Geom &g = a.g;
     const int x = blockIdx.x * LB_BX + threadIdx.x;
     const int y = blockIdx.y * LB_BY + threadIdx.y;
@@ -83,7 +85,7 @@ cudaError_t launch_lb3d(const LBArgs &a, int storage, cudaStream_t st)
     const dim3 grid((a.g.nx + LB_BX - 1) / LB_BX, (a.g.ny + LB_BY - 1) / LB_BY, (a.g.nz + LB_BZ - 1) / LB_BZ);
     const bool gr = a.gamma_g != 0.0f;
     const bool force = (a.coupling & FLB_COUPLE_FORCE) != 0;
-#define FLB_LB3(T, G, F) lb3_kernel<T, G, F><<<grid, block, 0, st>>>(a, plane_table<T>(a.fin, a.fout, a.g.n, 19))
+#define FLB_LB3(T, G, F) return launch_pdl(lb3_kernel<T, G, F>, grid, block, 0, st, PDL_BLOCKS, a, plane_table<T>(a.fin, a.fout, a.g.n, 19))
     if (storage == FLB_F16_DEV) {
         if (gr) { if (force) FLB_LB3(__half, true, true); else FLB_LB3(__half, true, false); }
         else { if (force) FLB_LB3(__half, false, true); else FLB_LB3(__half, false, false); }
@@ -92,7 +94,6 @@ cudaError_t launch_lb3d(const LBArgs &a, int storage, cudaStream_t st)
         else { if (force) FLB_LB3(float, false, true); else FLB_LB3(float, false, false); }
     }
 #undef FLB_LB3
-    return cudaGetLastError();
 }
 
 }  // namespace flb
