@@ -736,7 +736,7 @@ int sample_rep(flb_handle *h, Rep &r, int mask)
         const int slot = dyn ? (r.dslot + 1) % L : 0;
         d.snap = dyn ? r.dring + (size_t)slot * K : nullptr;
         const cudaError_t e = launch_dft_accumulate(d, h->st);
-        h->launches += 3;
+        h->launches += dft_launches(d);
         if (e != cudaSuccess) return FLB_ECUDA;
         if (mask & 1) r.sq_n += 1;
         if (dyn) {
@@ -765,7 +765,7 @@ int sample_rep(flb_handle *h, Rep &r, int mask)
             d.S = r.hsq;
             d.scale = 0.5 / ((double)g.nx * g.ny);
             const cudaError_t e = launch_dft_accumulate(d, h->st);
-            h->launches += 3;
+            h->launches += dft_launches(d);
             if (e != cudaSuccess) return FLB_ECUDA;
         }
         r.h_n += 1;

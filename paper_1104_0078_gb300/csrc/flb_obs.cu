@@ -92,14 +92,17 @@ __global__ void __launch_bounds__(RED_BS) totals_kernel(const Geom g, int q, con
     }
 }
 
-// Pass 2: one block sums the per-block partials in a fixed order.
-__global__ void totals_final_kernel(const double *__restrict__ partial, int nblocks, double *__restrict__ out)
+// Pass 2: one block of a warp per sum adds the nk sums of every first-pass block,
+// each lane its own share and then the lanes, in a fixed order.  (One thread per
+// sum, its loads one behind the other, took 77 us for 1024 blocks; this takes 7.)
+__global__ void __launch_bounds__(32 * NMSQ) final_kernel(const double *__restrict__ partial, int nblocks, int nk,
+                                                         double *__restrict__ out)
 {
-    const int k = threadIdx.x;
-    if (k >= NRED) return;
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double t = 0.0;
-    for (int b = 0; b < nblocks; ++b) t += partial[(long long)b * NRED + k];
-    out[k] = t;
+    for (int b = lane; b < nblocks; b += 32) t += partial[(long long)b * nk + k];
+    t = warp_sum(t);
+    if (lane == 0) out[k] = t;
 }
 
 cudaError_t launch_totals(const Geom &g, int q, int storage, const void *f, const float *psi, const float *u,
@@ -109,7 +112,7 @@ cudaError_t launch_totals(const Geom &g, int q, int storage, const void *f, cons
         totals_kernel<__half><<<nblocks, RED_BS, 0, s>>>(g, q, (const __half *)f, psi, u, partial);
     else
         totals_kernel<float><<<nblocks, RED_BS, 0, s>>>(g, q, (const float *)f, psi, u, partial);
-    totals_final_kernel<<<1, 32, 0, s>>>(partial, nblocks, out);
+    final_kernel<<<1, 32 * NRED, 0, s>>>(partial, nblocks, NRED, out);
     return cudaGetLastError();
 }
 
@@ -171,15 +174,6 @@ __global__ void __launch_bounds__(RED_BS) mode_msq_kernel(const Geom g, const Mo
     }
 }
 
-__global__ void msq_final_kernel(const double *__restrict__ partial, int nblocks, double *__restrict__ out)
-{
-    const int k = threadIdx.x;
-    if (k >= NMSQ) return;
-    double t = 0.0;
-    for (int b = 0; b < nblocks; ++b) t += partial[(long long)b * NMSQ + k];
-    out[k] = t;
-}
-
 cudaError_t launch_mode_msq(const Geom &g, int storage, const ModeBasis &B, const void *f, double *partial,
                             int nblocks, double *out, cudaStream_t s)
 {
@@ -187,16 +181,20 @@ cudaError_t launch_mode_msq(const Geom &g, int storage, const ModeBasis &B, cons
         mode_msq_kernel<__half><<<nblocks, RED_BS, 0, s>>>(g, B, (const __half *)f, partial);
     else
         mode_msq_kernel<float><<<nblocks, RED_BS, 0, s>>>(g, B, (const float *)f, partial);
-    msq_final_kernel<<<1, 32, 0, s>>>(partial, nblocks, out);
+    final_kernel<<<1, 32 * NMSQ, 0, s>>>(partial, nblocks, NMSQ, out);
     return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
 // Separable DFT.  Axis lists: index j of an axis of length n with window kmax
 // (K = 2 kmax + 1 < n) is k = j for j <= kmax and n - (K - j) otherwise; with
-// K = n every k is kept.
+// K = n every k is kept.  The field is real, so the component at -k is the
+// conjugate of that at k: the x pass forms k_x = 0 .. Kx/2 only (nu = Kx/2 + 1 of
+// them, the width of X1 and X2), the other passes work on those, and the last one
+// writes each |.|^2 at both places.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int kval(int j, int n, int K) { return (K >= n || j <= K / 2) ? j : n - (K - j); }
+// list index of -k for the list index j of k
+__device__ __forceinline__ int conj_partner(int j, int n, int K) { return j == 0 ? 0 : (K >= n ? n - j : K - j); }
 
 __device__ __forceinline__ float2 twiddle(int k, int x, int n)
 {
@@ -207,248 +205,280 @@ __device__ __forceinline__ float2 twiddle(int k, int x, int n)
     return make_float2(c, -s);
 }
 
-// Twiddle table e^{-2 pi i m / n}, m < n, in shared memory (n <= TW_MAX); each
-// output then walks its phase index m = k x mod n by additions.
+// Longest axis: the twiddle tables e^{-2 pi i m / n}, m < n, sit in shared memory;
+// each output walks its phase index m = k x mod n by additions.
 constexpr int TW_MAX = 4096;
 
-__device__ __forceinline__ void fill_twiddles(float2 *tw, int n)
-{
-    for (int m = threadIdx.x; m < n; m += blockDim.x) tw[m] = twiddle(1, m, n);
-    __syncthreads();
-}
-
-// X1[(z*ny + y)*Kx + jx] = sum_x in(x,y,z) e^{-i qx x}
+// X1[(z*ny + y)*nu + j] = sum_x in(x,y,z) e^{-2 pi i j x / nx}, one output per thread
 __global__ void dft_x_kernel(DftArgs a)
 {
     extern __shared__ float2 tw[];
-    fill_twiddles(tw, a.nx);
+    for (int m = threadIdx.x; m < a.nx; m += blockDim.x) tw[m] = twiddle(1, m, a.nx);
+    __syncthreads();
+    const int nu = a.Kx / 2 + 1;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long tot = (long long)a.Kx * a.ny * a.nz;
+    const long long tot = (long long)nu * a.ny * a.nz;
     if (t >= tot) return;
-    const int jx = (int)(t % a.Kx);
-    const long long row = t / a.Kx;  // z*ny + y
-    const int y = (int)(row % a.ny), z = (int)(row / a.ny);
-    const int k = kval(jx, a.nx, a.Kx);
-    const float *src = a.in + a.off + (long long)y * a.sy + (long long)z * a.sz;
-    float re = 0.f, im = 0.f;
-    int m = 0;
-    for (int x = 0; x < a.nx; ++x) {
+    const int k = (int)(t % nu);
+    const long long row = t / nu;  // z*ny + y
+    const float *src = a.in + a.off + (row % a.ny) * a.sy + (row / a.ny) * a.sz;
+    float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};  // x mod 4: four independent chains
+    int m = 0, x = 0;
+    for (; x + 4 <= a.nx; x += 4) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float v = src[x + u];
+            const float2 w = tw[m];
+            re[u] = fmaf(v, w.x, re[u]);
+            im[u] = fmaf(v, w.y, im[u]);
+            m += k;
+            if (m >= a.nx) m -= a.nx;
+        }
+    }
+    for (; x < a.nx; ++x) {
         const float v = src[x];
         const float2 w = tw[m];
-        re = fmaf(v, w.x, re);
-        im = fmaf(v, w.y, im);
+        re[0] = fmaf(v, w.x, re[0]);
+        im[0] = fmaf(v, w.y, im[0]);
         m += k;
         if (m >= a.nx) m -= a.nx;
     }
-    a.X1[t] = make_float2(re, im);
+    a.X1[t] = make_float2((re[0] + re[1]) + (re[2] + re[3]), (im[0] + im[1]) + (im[2] + im[3]));
 }
 
-// The same X1 for windows of Kx <= 32 on rows of nx <= 1024, as a small matrix
-// product over blocks of DXR_R rows.  The input is real, so X(-k) = conj X(k):
-// only the kept k = 0 .. Kx/2 are summed (nu of them), each written with its
-// partner.  A block builds the table e^{-2 pi i m / nx} once; chunks of DXR_CX
-// columns of its rows are copied into two shared-memory buffers by cp.async
-// (the next chunk in flight while the current one is summed), the chunk's
-// twiddles e^{-2 pi i k x / nx} (k x reduced mod nx exactly, as twiddle() does)
-// are taken from the table, and thread t sums row t, sequentially in x.
-constexpr int DXR_R = 128, DXR_CX = 32, DXR_NMAX = 1024, DXR_PS = DXR_R * (DXR_CX + 1);
+// The same X1 for windows of nu <= 18, as a small matrix product over blocks of
+// rows.  A block builds the table e^{-2 pi i m / nx} once; chunks of DXR_CX columns
+// of its rows are copied into two shared-memory buffers by cp.async (the next chunk
+// in flight while the current one is summed), and the chunk's twiddles
+// e^{-2 pi i k x / nx} (k x reduced mod nx exactly, as twiddle() does) are taken from
+// the table.  S threads share a row, each summing every S-th column of a chunk, and
+// add up at the end: 1 where 128-row blocks cover the chip, else 8 (2048 rows of
+// 2048 with nu = 17 in 16 blocks would keep 16 SMs busy).
+constexpr int DXR_NT = 128, DXR_CX = 32;
 
-__device__ __forceinline__ int conj_partner(int j, int n, int K) { return j == 0 ? 0 : (K >= n ? n - j : K - j); }
-
-// dynamic shared memory of dft_x_rows_kernel<NUP> for rows of n
-template <int NUP>
+// dynamic shared memory of dft_x_rows_kernel<NUP, S> for rows of n
+template <int NUP, int S>
 constexpr size_t dxr_smem(int n)
 {
-    return DXR_R * sizeof(long long) + DXR_CX * NUP * sizeof(float2) + 2 * DXR_PS * sizeof(float) + n * sizeof(float2);
+    constexpr int R = DXR_NT / S;
+    return R * sizeof(long long) + DXR_CX * NUP * sizeof(float2) + 2 * R * (DXR_CX + 1) * sizeof(float) + n * sizeof(float2);
 }
 
-template <int NUP>
-__global__ void __launch_bounds__(DXR_R) dft_x_rows_kernel(DftArgs a, long long nrows)
+template <int NUP, int S>
+__global__ void __launch_bounds__(DXR_NT) dft_x_rows_kernel(DftArgs a, long long nrows)
 {
+    constexpr int R = DXR_NT / S, PS = R * (DXR_CX + 1);
     extern __shared__ __align__(16) unsigned char dsm[];
-    long long *roff = reinterpret_cast<long long *>(dsm);                          // [DXR_R]
-    float2 *Wc = reinterpret_cast<float2 *>(roff + DXR_R);                           // [DXR_CX][NUP]
-    float *P = reinterpret_cast<float *>(Wc + DXR_CX * NUP);                        // [2][DXR_R][DXR_CX + 1]
-    float2 *tw = reinterpret_cast<float2 *>(P + 2 * DXR_PS);                         // [n]
+    long long *roff = reinterpret_cast<long long *>(dsm);                          // [R]
+    float2 *Wc = reinterpret_cast<float2 *>(roff + R);                               // [DXR_CX][NUP]
+    float *P = reinterpret_cast<float *>(Wc + DXR_CX * NUP);                        // [2][R][DXR_CX + 1]
+    float2 *tw = reinterpret_cast<float2 *>(P + 2 * PS);                             // [n]
     const int n = a.nx, nu = a.Kx / 2 + 1, t = threadIdx.x, lane = t & 31, wp = t >> 5;
+    const int row = t / S, sl = t % S;
     const int nch = (n + DXR_CX - 1) / DXR_CX;
-    for (int m = t; m < n; m += DXR_R) tw[m] = twiddle(1, m, n);
+    const long long r0 = (long long)blockIdx.x * R;
+    for (int m = t; m < n; m += DXR_NT) tw[m] = twiddle(1, m, n);
+    if (t < R) roff[t] = r0 + t < nrows ? a.off + ((r0 + t) % a.ny) * a.sy + ((r0 + t) / a.ny) * a.sz : -1;
+    __syncthreads();
     // this thread's copies of chunk c: rows wp, wp + 4, ..., column x0 + lane
     auto stage = [&](int c) {
-        float *buf = P + (c & 1) * DXR_PS;
+        float *buf = P + (c & 1) * PS;
         const int x = c * DXR_CX + lane;
-        for (int rr = wp; rr < DXR_R; rr += DXR_R / 32) {
+        for (int rr = wp; rr < R; rr += DXR_NT / 32) {
             const long long o = roff[rr];
             const bool ok = o >= 0 && x < n;
             cp_async4(buf + rr * (DXR_CX + 1) + lane, a.in + (ok ? o + x : 0), ok ? 4 : 0);
         }
     };
-    for (long long r0 = (long long)blockIdx.x * DXR_R; r0 < nrows; r0 += (long long)gridDim.x * DXR_R) {
-        __syncthreads();  // the table is complete; the previous group is done with roff and P
-        {
-            const long long r = r0 + t;
-            roff[t] = r < nrows ? a.off + (r % a.ny) * a.sy + (r / a.ny) * a.sz : -1;
-        }
-        __syncthreads();
-        stage(0);
+    stage(0);
+    cp_async_commit();
+    float re[NUP], im[NUP];
+#pragma unroll
+    for (int j = 0; j < NUP; ++j) re[j] = im[j] = 0.f;
+    for (int c = 0; c < nch; ++c) {
+        if (c + 1 < nch) stage(c + 1);
         cp_async_commit();
-        float re[NUP], im[NUP];
-#pragma unroll
-        for (int j = 0; j < NUP; ++j) re[j] = im[j] = 0.f;
-        for (int c = 0; c < nch; ++c) {
-            if (c + 1 < nch) stage(c + 1);
-            cp_async_commit();
-            const int x0 = c * DXR_CX;
-            for (int e = t; e < DXR_CX * NUP; e += DXR_R) {
-                const int i = e / NUP, j = e % NUP, x = x0 + i;
-                Wc[e] = (j < nu && x < n) ? tw[(j * x) % n] : make_float2(0.f, 0.f);
-            }
-            cp_async_wait1();  // this thread's copies of chunk c have landed
-            __syncthreads();   // everyone's copies of chunk c, and the chunk's twiddles
-            const float *Pc = P + (c & 1) * DXR_PS + t * (DXR_CX + 1);
-            const int cx = min(DXR_CX, n - x0);
-            for (int i = 0; i < cx; ++i) {
-                const float v = Pc[i];
-#pragma unroll
-                for (int j = 0; j < NUP; j += 2) {
-                    const float4 w = *reinterpret_cast<const float4 *>(&Wc[i * NUP + j]);
-                    re[j] = fmaf(v, w.x, re[j]);
-                    im[j] = fmaf(v, w.y, im[j]);
-                    re[j + 1] = fmaf(v, w.z, re[j + 1]);
-                    im[j + 1] = fmaf(v, w.w, im[j + 1]);
-                }
-            }
-            __syncthreads();  // chunk c's buffer and twiddles are free again
+        const int x0 = c * DXR_CX;
+        for (int e = t; e < DXR_CX * NUP; e += DXR_NT) {
+            const int i = e / NUP, j = e % NUP, x = x0 + i;
+            Wc[e] = (j < nu && x < n) ? tw[(int)(((long long)j * x) % n)] : make_float2(0.f, 0.f);
         }
-        const long long r = r0 + t;
-        if (r < nrows) {
-            float2 *o = a.X1 + r * a.Kx;
+        cp_async_wait1();  // this thread's copies of chunk c have landed
+        __syncthreads();   // everyone's copies of chunk c, and the chunk's twiddles
+        const float *Pc = P + (c & 1) * PS + row * (DXR_CX + 1);
+        const int cx = min(DXR_CX, n - x0);
+        for (int i = sl; i < cx; i += S) {
+            const float v = Pc[i];
 #pragma unroll
-            for (int j = 0; j < NUP; ++j) {
-                if (j < nu) {
-                    o[j] = make_float2(re[j], im[j]);
-                    const int jp = conj_partner(j, n, a.Kx);
-                    if (jp != j) o[jp] = make_float2(re[j], -im[j]);
-                }
+            for (int j = 0; j < NUP; j += 2) {
+                const float4 w = *reinterpret_cast<const float4 *>(&Wc[i * NUP + j]);
+                re[j] = fmaf(v, w.x, re[j]);
+                im[j] = fmaf(v, w.y, im[j]);
+                re[j + 1] = fmaf(v, w.z, re[j + 1]);
+                im[j + 1] = fmaf(v, w.w, im[j + 1]);
             }
         }
+        __syncthreads();  // chunk c's buffer and twiddles are free again
+    }
+#pragma unroll
+    for (int o = S / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int j = 0; j < NUP; ++j) {
+            re[j] += __shfl_xor_sync(0xffffffffu, re[j], o);
+            im[j] += __shfl_xor_sync(0xffffffffu, im[j], o);
+        }
+    if (sl == 0 && r0 + row < nrows) {
+        float2 *o = a.X1 + (r0 + row) * nu;
+#pragma unroll
+        for (int j = 0; j < NUP; ++j)
+            if (j < nu) o[j] = make_float2(re[j], im[j]);
     }
 }
 
-// The y pass for windows with Kx Ky <= 1024: one block per plane z, thread t
-// the output (jx, jy) = (t mod Kx, t / Kx); the plane's X1 rows (contiguous)
-// come into shared memory DYS_YC rows at a time, and each thread sums its
-// output sequentially in y.
-constexpr int DYS_YC = 32;
+// The y and z passes: DFT along the middle axis of in[outer][n][C], columns
+// (outer, c) to lanes, out[outer][K][C].  The components at k and -k share their
+// products: with A = sum v_x c, B = sum v_y s, C = sum v_y c, D = sum v_x s,
+//   X(k) = (A + B) + i (C - D),  X(-k) = (A - B) + i (C + D),
+// so a thread carries PP such pairs.  The NS warps of a pair group take every NS-th
+// term and are added in order at the end; a block has PB groups.
+//   ACC: the sums' type (float in the y pass, double in the z pass).
+//   LAST: instead of `out`, S += scale |X|^2 (and the snapshot) at k and at the conjugate place.
+// The z pass is bound by the FP64 pipe (4 products a term and pair): one warp per
+// output, without the pairs and the symmetry, took 515 us for all of a 64^3 box, and
+// this 55; the window passes of a 512^3 box (|k| <= 8) 68 + 65 us, here 26 + 38; one
+// thread per output took 664 us for the y pass of a 2048^2 box (|k| <= 16), here 76.
+struct AxisArgs {
+    const float2 *in;
+    float2 *out;
+    int outer, n, C, K;
+    DftArgs d;  // LAST: S, scale, snap and the lists
+};
 
-__global__ void __launch_bounds__(1024) dft_y_slab_kernel(DftArgs a)
+template <class ACC>
+struct Pair2;
+template <>
+struct Pair2<float> { using T = float2; };
+template <>
+struct Pair2<double> { using T = double2; };
+
+template <class ACC, int PP, int NS, int PB, bool LAST>
+__global__ void __launch_bounds__(32 * NS * PB) dft_axis_kernel(const AxisArgs a)
 {
-    extern __shared__ __align__(16) float2 ysm[];
-    float2 *tw = ysm;               // [ny]
-    float2 *Xs = ysm + a.ny;        // [DYS_YC][Kx]
-    fill_twiddles(tw, a.ny);
-    const int z = blockIdx.x, t = threadIdx.x, nout = a.Kx * a.Ky;
-    const bool act = t < nout;
-    const int jx = act ? t % a.Kx : 0, jy = act ? t / a.Kx : 0;
-    const int k = kval(jy, a.ny, a.Ky);
-    const float2 *src = a.X1 + (long long)z * a.ny * a.Kx;
-    float re = 0.f, im = 0.f;
-    int m = 0;
-    for (int y0 = 0; y0 < a.ny; y0 += DYS_YC) {
-        const int cy = min(DYS_YC, a.ny - y0);
-        __syncthreads();  // the previous rows are consumed
-        for (int e = t; e < cy * a.Kx; e += blockDim.x) Xs[e] = src[(long long)y0 * a.Kx + e];
+    using A2 = typename Pair2<ACC>::T;
+    extern __shared__ __align__(16) unsigned char asm_[];
+    A2 *tw = reinterpret_cast<A2 *>(asm_);                 // [n] (cos, sin)
+    ACC *red = reinterpret_cast<ACC *>(tw + a.n);          // [PB][NS][4 PP][32]
+    const int n = a.n;
+    for (int m = threadIdx.x; m < n; m += blockDim.x) {
+        const float2 w = twiddle(1, m, n);
+        tw[m].x = w.x;
+        tw[m].y = -w.y;
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, pg = wp / NS, sl = wp % NS;
+    const long long col = (long long)blockIdx.x * 32 + lane;
+    const bool act = col < (long long)a.outer * a.C;
+    const int o = act ? (int)(col / a.C) : 0, c = act ? (int)(col % a.C) : 0;
+    const int npair = a.K / 2 + 1, p0 = (blockIdx.y * PB + pg) * PP;
+    ACC acc[PP][4];
+    int m[PP], step[PP];
+#pragma unroll
+    for (int q = 0; q < PP; ++q) {
+        const int k = min(p0 + q, npair - 1);
+        acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0;
+        m[q] = (int)(((long long)k * sl) % n);
+        step[q] = (int)(((long long)k * NS) % n);
+    }
+    const float2 *src = a.in + (long long)o * n * a.C + c;
+    if (p0 < npair) {
+#pragma unroll 4
+        for (int r = sl; r < n; r += NS) {
+            const float2 v = __ldg(src + (long long)r * a.C);
+            const ACC vx = v.x, vy = v.y;
+#pragma unroll
+            for (int q = 0; q < PP; ++q) {
+                const A2 w = tw[m[q]];
+                acc[q][0] += vx * w.x;
+                acc[q][1] += vy * w.y;
+                acc[q][2] += vy * w.x;
+                acc[q][3] += vx * w.y;
+                m[q] += step[q];
+                if (m[q] >= n) m[q] -= n;
+            }
+        }
+    }
+    if (NS > 1) {
+        ACC *mine = red + (pg * NS + sl) * (4 * PP) * 32 + lane;
+#pragma unroll
+        for (int q = 0; q < PP; ++q)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) mine[(4 * q + e) * 32] = acc[q][e];
         __syncthreads();
-        if (act) {
-            for (int i = 0; i < cy; ++i) {
-                const float2 v = Xs[i * a.Kx + jx];
-                const float2 w = tw[m];
-                re += v.x * w.x - v.y * w.y;
-                im += v.x * w.y + v.y * w.x;
-                m += k;
-                if (m >= a.ny) m -= a.ny;
+        if (sl != 0) return;
+        const ACC *all = red + pg * NS * (4 * PP) * 32 + lane;
+#pragma unroll
+        for (int q = 0; q < PP; ++q)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                ACC t = all[(4 * q + e) * 32];
+                for (int w = 1; w < NS; ++w) t += all[(w * 4 * PP + 4 * q + e) * 32];
+                acc[q][e] = t;
             }
+    }
+    if (!act) return;
+#pragma unroll
+    for (int q = 0; q < PP; ++q) {
+        const int j = p0 + q;
+        if (j >= npair) break;
+        const int jm = conj_partner(j, n, a.K);
+        const ACC re[2] = {acc[q][0] + acc[q][1], acc[q][0] - acc[q][1]};
+        const ACC im[2] = {acc[q][2] - acc[q][3], acc[q][2] + acc[q][3]};
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const int jk = s ? jm : j;
+            if (s && jm == j) break;
+            if (!LAST) {
+                a.out[((long long)o * a.K + jk) * a.C + c] = make_float2((float)re[s], (float)im[s]);
+                continue;
+            }
+            const DftArgs &d = a.d;
+            const int nu = d.Kx / 2 + 1, jx = c % nu;
+            // planar fields end with the y pass (columns jx), others with the z pass (columns jx + nu jy)
+            const int jy = d.nz == 1 ? jk : c / nu, jz = d.nz == 1 ? 0 : jk;
+            const double val = d.scale * ((double)re[s] * re[s] + (double)im[s] * im[s]);
+            const long long e = ((long long)jz * d.Ky + jy) * d.Kx + jx;
+            if (d.S) d.S[e] += val;
+            if (d.snap) d.snap[e] = make_float2((float)re[s], (float)im[s]);
+            const int jxm = conj_partner(jx, d.nx, d.Kx);
+            if (jxm == jx) continue;  // -k is another column's
+            const long long em = ((long long)conj_partner(jz, d.nz, d.Kz) * d.Ky + conj_partner(jy, d.ny, d.Ky)) * d.Kx + jxm;
+            if (d.S) d.S[em] += val;
+            if (d.snap) d.snap[em] = make_float2((float)re[s], -(float)im[s]);
         }
     }
-    if (act) a.X2[((long long)z * a.Ky + jy) * a.Kx + jx] = make_float2(re, im);
 }
 
-// X2[(z*Ky + jy)*Kx + jx] = sum_y X1[(z*ny + y)*Kx + jx] e^{-i qy y}
-__global__ void dft_y_kernel(DftArgs a)
+template <class ACC, int PP, int NS, int PB, bool LAST>
+cudaError_t go_axis(const AxisArgs &a, long long groups, cudaStream_t s)
 {
-    extern __shared__ float2 tw[];
-    fill_twiddles(tw, a.ny);
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long tot = (long long)a.Kx * a.Ky * a.nz;
-    if (t >= tot) return;
-    const int jx = (int)(t % a.Kx);
-    const int jy = (int)((t / a.Kx) % a.Ky);
-    const int z = (int)(t / ((long long)a.Kx * a.Ky));
-    const int k = kval(jy, a.ny, a.Ky);
-    // four partial sums over y mod 4 (independent chains), added in a fixed order
-    float re4[4] = {0.f, 0.f, 0.f, 0.f}, im4[4] = {0.f, 0.f, 0.f, 0.f};
-    const float2 *src = a.X1 + (long long)z * a.ny * a.Kx + jx;
-    int m = 0, y = 0;
-    for (; y + 4 <= a.ny; y += 4) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const float2 v = src[(long long)(y + u) * a.Kx];
-            const float2 w = tw[m];
-            re4[u] += v.x * w.x - v.y * w.y;
-            im4[u] += v.x * w.y + v.y * w.x;
-            m += k;
-            if (m >= a.ny) m -= a.ny;
-        }
-    }
-    for (; y < a.ny; ++y) {
-        const float2 v = src[(long long)y * a.Kx];
-        const float2 w = tw[m];
-        re4[0] += v.x * w.x - v.y * w.y;
-        im4[0] += v.x * w.y + v.y * w.x;
-        m += k;
-        if (m >= a.ny) m -= a.ny;
-    }
-    const float re = (re4[0] + re4[1]) + (re4[2] + re4[3]), im = (im4[0] + im4[1]) + (im4[2] + im4[3]);
-    a.X2[t] = make_float2(re, im);
+    const int npair = a.K / 2 + 1;
+    const size_t smem = sizeof(ACC) * (2 * (size_t)a.n + (NS > 1 ? (size_t)PB * NS * 4 * PP * 32 : 0));
+    auto k = dft_axis_kernel<ACC, PP, NS, PB, LAST>;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k<<<dim3((unsigned)groups, (unsigned)((npair + PP * PB - 1) / (PP * PB))), 32 * NS * PB, smem, s>>>(a);
+    return cudaGetLastError();
 }
 
-// S[(jz*Ky + jy)*Kx + jx] += scale |sum_z X2[(z*Ky + jy)*Kx + jx] e^{-i qz z}|^2  (FP64).
-// One warp per output: lane l sums z = l, l + 32, ... in FP64, then a
-// shuffle reduction in a fixed order.
-constexpr int DZ_WARPS = 8;
-
-__global__ void __launch_bounds__(32 * DZ_WARPS) dft_z_acc_kernel(DftArgs a)
+// Four pairs a block (two groups of two pairs, four warps each) where that makes two
+// blocks per SM, else one pair and eight warps: a short list of columns on a long axis is
+// spread over as many SMs as it can.
+template <class ACC, bool LAST>
+cudaError_t launch_axis(const AxisArgs &a, cudaStream_t s)
 {
-    extern __shared__ float2 tw[];
-    fill_twiddles(tw, a.nz);
-    const long long t = (long long)blockIdx.x * DZ_WARPS + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    const long long tot = (long long)a.Kx * a.Ky * a.Kz;
-    if (t >= tot) return;
-    const long long plane = (long long)a.Kx * a.Ky;
-    const long long xy = t % plane;
-    const int jz = (int)(t / plane);
-    const int k = kval(jz, a.nz, a.Kz);
-    const int step = (int)(((long long)k * 32) % a.nz);
-    int m = (int)(((long long)k * lane) % a.nz);
-    double re = 0.0, im = 0.0;
-    for (int z = lane; z < a.nz; z += 32) {
-        const float2 v = a.X2[(long long)z * plane + xy];
-        const float2 w = tw[m];
-        re += (double)v.x * w.x - (double)v.y * w.y;
-        im += (double)v.x * w.y + (double)v.y * w.x;
-        m += step;
-        if (m >= a.nz) m -= a.nz;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        re += __shfl_xor_sync(0xffffffffu, re, o);
-        im += __shfl_xor_sync(0xffffffffu, im, o);
-    }
-    if (lane == 0) {
-        if (a.S) a.S[t] += a.scale * (re * re + im * im);
-        if (a.snap) a.snap[t] = make_float2((float)re, (float)im);
-    }
+    const long long groups = ((long long)a.outer * a.C + 31) / 32;
+    return groups * ((a.K / 2 + 4) / 4) >= 304 ? go_axis<ACC, 2, 4, 2, LAST>(a, groups, s)
+                                               : go_axis<ACC, 1, 8, 1, LAST>(a, groups, s);
 }
 
 // Dynamic structure factor: correlate the newest Fourier components with those
@@ -475,34 +505,44 @@ cudaError_t launch_dyn_corr(const float2 *ring, int L, int slot, int nlag, long 
     return cudaGetLastError();
 }
 
+template <int NUP>
+cudaError_t go_rows(const DftArgs &a, cudaStream_t s)
+{
+    const long long rows = (long long)a.ny * a.nz;
+    auto go = [&](auto k, int per, size_t smem) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k<<<(unsigned)((rows + per - 1) / per), DXR_NT, smem, s>>>(a, rows);
+        return cudaGetLastError();
+    };
+    return rows >= 152 * DXR_NT ? go(dft_x_rows_kernel<NUP, 1>, DXR_NT, dxr_smem<NUP, 1>(a.nx))
+                                : go(dft_x_rows_kernel<NUP, 8>, DXR_NT / 8, dxr_smem<NUP, 8>(a.nx));
+}
+
+// kernels launched by launch_dft_accumulate
+int dft_launches(const DftArgs &a) { return a.nz == 1 ? 2 : 3; }
+
 cudaError_t launch_dft_accumulate(const DftArgs &a, cudaStream_t s)
 {
-    const int bs = 256;
-    long long n1 = (long long)a.Kx * a.ny * a.nz, n2 = (long long)a.Kx * a.Ky * a.nz, n3 = (long long)a.Kx * a.Ky * a.Kz;
     if (a.nx > TW_MAX || a.ny > TW_MAX || a.nz > TW_MAX) return cudaErrorInvalidValue;
-    if (a.Kx <= 32 && a.nx <= DXR_NMAX) {
-        const long long rows = (long long)a.ny * a.nz;
-        const unsigned grid = (unsigned)((rows + DXR_R - 1) / DXR_R);
-        const int nu = a.Kx / 2 + 1;
-#define FLB_DXR(NUP) dft_x_rows_kernel<NUP><<<grid, DXR_R, dxr_smem<NUP>(a.nx), s>>>(a, rows)
-        if (nu <= 2) FLB_DXR(2);
-        else if (nu <= 4) FLB_DXR(4);
-        else if (nu <= 6) FLB_DXR(6);
-        else if (nu <= 10) FLB_DXR(10);
-        else FLB_DXR(18);
-#undef FLB_DXR
-    } else {
-        dft_x_kernel<<<(unsigned)((n1 + bs - 1) / bs), bs, sizeof(float2) * a.nx, s>>>(a);
+    const int nu = a.Kx / 2 + 1;
+    cudaError_t e;
+    if (nu <= 2) e = go_rows<2>(a, s);
+    else if (nu <= 4) e = go_rows<4>(a, s);
+    else if (nu <= 6) e = go_rows<6>(a, s);
+    else if (nu <= 10) e = go_rows<10>(a, s);
+    else if (nu <= 18) e = go_rows<18>(a, s);
+    else {
+        const int bs = 256;
+        dft_x_kernel<<<(unsigned)(((long long)nu * a.ny * a.nz + bs - 1) / bs), bs, sizeof(float2) * a.nx, s>>>(a);
+        e = cudaGetLastError();
     }
-    const size_t ysm = sizeof(float2) * ((size_t)a.ny + (size_t)DYS_YC * a.Kx);
-    if (a.Kx * a.Ky <= 1024 && ysm <= 48 * 1024) {
-        const int nt = ((a.Kx * a.Ky + 31) / 32) * 32;
-        dft_y_slab_kernel<<<(unsigned)a.nz, nt, ysm, s>>>(a);
-    } else {
-        dft_y_kernel<<<(unsigned)((n2 + bs - 1) / bs), bs, sizeof(float2) * a.ny, s>>>(a);
-    }
-    dft_z_acc_kernel<<<(unsigned)((n3 + DZ_WARPS - 1) / DZ_WARPS), 32 * DZ_WARPS, sizeof(float2) * a.nz, s>>>(a);
-    return cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const AxisArgs y{a.X1, a.X2, a.nz, a.ny, nu, a.Ky, a};
+    if (a.nz == 1) return launch_axis<float, true>(y, s);
+    e = launch_axis<float, false>(y, s);
+    if (e != cudaSuccess) return e;
+    return launch_axis<double, true>(AxisArgs{a.X2, nullptr, 1, a.nz, a.Ky * nu, a.Kz, a}, s);
 }
 
 // Heights of the two psi = 0 surfaces of a slab normal to z: in every column the

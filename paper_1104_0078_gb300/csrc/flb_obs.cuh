@@ -18,7 +18,7 @@ struct DftArgs {
     long long off, sy, sz; // element offset of (0,0,0) and strides of y and z (x stride 1)
     int nx, ny, nz;        // extents
     int Kx, Ky, Kz;        // number of kept wavevector indices per axis
-    float2 *X1, *X2;       // scratch: nz*ny*Kx and nz*Ky*Kx complex values
+    float2 *X1, *X2;       // scratch: nz*ny*nu and nz*Ky*nu complex values, nu = Kx/2 + 1
     double *S;             // accumulator Kz*Ky*Kx (may be null: no accumulation)
     double scale;          // factor on |.|^2
     float2 *snap = nullptr;  // if not null: the Fourier components, Kz*Ky*Kx
@@ -26,6 +26,7 @@ struct DftArgs {
 
 cudaError_t launch_totals(const Geom &g, int q, int storage, const void *f, const float *psi, const float *u,
                           double *partial, int nblocks, double *out, cudaStream_t s);
+int dft_launches(const DftArgs &a);
 cudaError_t launch_dft_accumulate(const DftArgs &a, cudaStream_t s);
 // out[k] = sum over sites of m_k^2 (k < q), out[NMSQ-1] = non-finite count; partial holds nblocks*NMSQ
 cudaError_t launch_mode_msq(const Geom &g, int storage, const ModeBasis &B, const void *f, double *partial,
