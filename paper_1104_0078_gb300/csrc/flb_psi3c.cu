@@ -31,44 +31,46 @@ namespace flb {
 
 namespace {
 
-// A block's tile of sites; two threads per output column, each CZ/2 planes.
+// A block's tile of sites.
 template <int X_, int Y_, int Z_>
 struct Tile3 {
-    static constexpr int CX = X_, CY = Y_, CZ = Z_, CNT = 2 * CX * CY;
+    static constexpr int CX = X_, CY = Y_, CZ = Z_, NT = 2 * CX * CY;  // NT: threads, two per output column, each CZ/2 planes
     static constexpr int CW1 = CX + 2, CH1 = CY + 2, CP1 = CW1 * CH1;  // flux and noise columns: tile + 1
     static constexpr int CW2 = CX + 4, CH2 = CY + 4;                   // FV mu columns: tile + 2
-    
 };
-#define FLB_TILE3(T)                                                                                          \
-    constexpr int CX = T::CX, CY = T::CY, CZ = T::CZ, CNT = T::CNT, CW1 = T::CW1, CH1 = T::CH1, CP1 = T::CP1, \
-                  CW2 = T::CW2, CH2 = T::CH2;                                                                 \
-    (void)CX, (void)CY, (void)CZ, (void)CNT, (void)CW1, (void)CH1, (void)CP1, (void)CW2, (void)CH2
+#define FLB_TILE3(T)                                                                                        \
+    constexpr int CX = T::CX, CY = T::CY, CZ = T::CZ, NT = T::NT, CW1 = T::CW1, CH1 = T::CH1, CP1 = T::CP1, \
+                  CW2 = T::CW2, CH2 = T::CH2;                                                               \
+    (void)CX, (void)CY, (void)CZ, (void)NT, (void)CW1, (void)CH1, (void)CP1, (void)CW2, (void)CH2
 
 struct CubeArgs {
     Psi3Args a;
     const float *mu;  // MU_IN: mu of the stage input, 2 ghost layers
     int naive;        // the naive noise (Sec. III) instead of FD's link noise
     float s1, s2, s3; // FD: sqrt(2 kT M a_l) of the face, edge and corner half-links
-    float sd;         // FV, naive: sqrt(2 kT M)
+    float sd;         // naive: sqrt(2 kT M)
 };
 
-// Sums of one plane of a field at c (row pitch Y): the centre, the four in-plane
-// faces, the four in-plane diagonals.
-struct Plane3 {
-    F1 a, b, d;
-};
+// The value at p (global memory through the read-only path, or shared memory).
 template <bool GLOBAL>
 __device__ __forceinline__ F1 rd(const float *p)
 {
     return F1{GLOBAL ? __ldg(p) : *p};
 }
+
+// Sums of one plane of a field at p (row pitch Y): the centre, the four in-plane faces,
+// the four in-plane diagonals.
+struct Plane3 {
+    F1 a, b, d;
+};
 template <bool GLOBAL>
 __device__ __forceinline__ Plane3 plane3(const float *p, int Y)
 {
+    auto at = [&](int o) { return rd<GLOBAL>(p + o); };
     Plane3 r;
-    r.a = rd<GLOBAL>(p);
-    r.b = (rd<GLOBAL>(p - 1) + rd<GLOBAL>(p + 1)) + (rd<GLOBAL>(p - Y) + rd<GLOBAL>(p + Y));
-    r.d = (rd<GLOBAL>(p - 1 - Y) + rd<GLOBAL>(p + 1 - Y)) + (rd<GLOBAL>(p - 1 + Y) + rd<GLOBAL>(p + 1 + Y));
+    r.a = at(0);
+    r.b = (at(-1) + at(1)) + (at(-Y) + at(Y));
+    r.d = (at(-1 - Y) + at(1 - Y)) + (at(-1 + Y) + at(1 + Y));
     return r;
 }
 
@@ -79,6 +81,7 @@ __device__ __forceinline__ void form_mu(const Psi3Args &a, int x0, int y0, int z
 {
     FLB_TILE3(T);
     constexpr int WX = CX + 2 * H, WY = CY + 2 * H;
+    static_assert(WX * WY <= NT, "one thread per column of the region");
     const Geom &g = a.g;
     const int k = threadIdx.x, lx = k % WX, ly = k / WX;
     const int x = x0 - H + lx, y = y0 - H + ly;
@@ -142,22 +145,23 @@ struct Div3 {
     F1 lo, mid, hi;
 };
 template <class T, bool Q15>
-__device__ __forceinline__ Div3 div3(const float *vx, const float *vy, const float *vz, int c)
+__device__ __forceinline__ Div3 div3(const float *v, int JN, int c)
 {
-    auto at = [](const float *v, int o) { return F1{v[o]}; };
     constexpr int Y = T::CW1;
-    const F1 hxy = (at(vx, c + 1) - at(vx, c - 1)) + (at(vy, c + Y) - at(vy, c - Y));
-    const F1 dg = ((at(vx, c + 1 + Y) + at(vy, c + 1 + Y)) - (at(vx, c - 1 - Y) + at(vy, c - 1 - Y))) +
-                  ((at(vx, c + 1 - Y) - at(vy, c + 1 - Y)) - (at(vx, c - 1 + Y) - at(vy, c - 1 + Y)));
-    const F1 zc = at(vz, c);
+    auto X = [&](int o) { return F1{v[c + o]}; };
+    auto Yv = [&](int o) { return F1{v[JN + c + o]}; };
+    auto Zv = [&](int o) { return F1{v[2 * JN + c + o]}; };
+    const F1 hxy = (X(1) - X(-1)) + (Yv(Y) - Yv(-Y));
+    const F1 dg = ((X(1 + Y) + Yv(1 + Y)) - (X(-1 - Y) + Yv(-1 - Y))) + ((X(1 - Y) - Yv(1 - Y)) - (X(-1 + Y) - Yv(-1 + Y)));
+    const F1 zc = Zv(0);
     Div3 r;
     if (Q15) {
-        const F1 c4 = (at(vz, c + 1 + Y) + at(vz, c + 1 - Y)) + (at(vz, c - 1 + Y) + at(vz, c - 1 - Y));
+        const F1 c4 = (Zv(1 + Y) + Zv(1 - Y)) + (Zv(-1 + Y) + Zv(-1 - Y));
         r.lo = vfma(zc, 8.f, dg) + c4;
         r.mid = hxy;
         r.hi = vfma(zc, -8.f, dg - c4);
     } else {
-        const F1 z4 = (at(vz, c + 1) + at(vz, c - 1)) + (at(vz, c + Y) + at(vz, c - Y));
+        const F1 z4 = (Zv(1) + Zv(-1)) + (Zv(Y) + Zv(-Y));
         r.lo = vfma(zc, 2.f, hxy) + z4;
         r.mid = vfma(hxy, 2.f, dg);
         r.hi = vfma(zc, -2.f, hxy - z4);
@@ -171,55 +175,67 @@ __device__ __forceinline__ F1 div_sum(const Div3 &below, const Div3 &own, const 
     return (Q15 ? vfma(own.mid, 8.f, below.hi) : below.hi + own.mid) + above.lo;
 }
 
-template <class T, bool FIRST, bool NOISE, bool MU_IN, bool Q15, bool W>
-__global__ void __launch_bounds__(T::CNT) psi3_fv_cube_kernel(const CubeArgs ca)
+// shared memory of a block (floats)
+template <class T, bool NOISE, bool MU_IN>
+__host__ __device__ constexpr int cube_fv_floats()
+{
+    return (T::CZ + 2) * T::CP1 * (NOISE ? 6 : 3) + (MU_IN ? 0 : (T::CZ + 4) * T::CW2 * T::CH2);
+}
+
+// The noise of the block's nodes (tile + 1) into sX, [3][CZ + 2][CH1][CW1].
+template <class T>
+__device__ __forceinline__ void cube_fv_noise(const Psi3Args &a, int x0, int y0, int z0, float *sX)
 {
     FLB_TILE3(T);
     constexpr int JN = (CZ + 2) * CP1;
-    extern __shared__ float csm[];
-    float *sJ = csm, *sX = sJ + 3 * JN, *smu = sX + (NOISE ? 3 * JN : 0);  // smu: [CZ + 4][CH2][CW2] unless MU_IN
-    const Psi3Args &a = ca.a;
     const Geom &g = a.g;
-    const int x0 = blockIdx.x * CX, y0 = blockIdx.y * CY, z0 = blockIdx.z * CZ;
-    const int nzt = min(CZ, g.nz - z0);
-    pdl_trigger();
-    if (NOISE) {
-        for (int k = threadIdx.x; k < JN; k += CNT) {
-            const int lx = k % CW1, ly = (k / CW1) % CH1, lz = k / CP1;
-            const int x = x0 - 1 + lx, y = y0 - 1 + ly, z = z0 - 1 + lz;
-            if (x > g.nx || y > g.ny || z > g.nz) continue;
-            float G[4];
-            const uint32_t id = (uint32_t)(wrapi(x, g.nx) + g.nx * (wrapi(y, g.ny) + g.ny * wrapi(z, g.nz)));
-            normals<2, false, true>(a.key, a.step, id, 1u, 0u, G, ca.sd);
-            sX[k] = G[0];
-            sX[JN + k] = G[1];
-            sX[2 * JN + k] = G[2];
-        }
+    const float sdx = sqrtf(2.0f * a.kT * a.M);
+    for (int k = threadIdx.x; k < JN; k += NT) {
+        const int lx = k % CW1, ly = (k / CW1) % CH1, lz = k / CP1;
+        const int x = x0 - 1 + lx, y = y0 - 1 + ly, z = z0 - 1 + lz;
+        if (x > g.nx || y > g.ny || z > g.nz) continue;
+        float G[4];
+        const uint32_t id = (uint32_t)(wrapi(x, g.nx) + g.nx * (wrapi(y, g.ny) + g.ny * wrapi(z, g.nz)));
+        normals<2, false, true>(a.key, a.step, id, 1u, 0u, G, sdx);
+        sX[k] = G[0];
+        sX[JN + k] = G[1];
+        sX[2 * JN + k] = G[2];
     }
-    pdl_wait();
+}
+
+// The rest of a stage on the tile at (x0, y0, z0); the noise, if any, is in sX.
+template <class T, bool FIRST, bool NOISE, bool MU_IN, bool Q15, bool W>
+__device__ __forceinline__ void cube_fv_stage(const Psi3Args &a, const float *mu, int x0, int y0, int z0, float *sJ,
+                                              const float *sX, float *smu)
+{
+    FLB_TILE3(T);
+    constexpr int JN = (CZ + 2) * CP1;
+    const Geom &g = a.g;
+    const int nzt = min(CZ, g.nz - z0);
     if (!MU_IN) {
         form_mu<T, 2, W>(a, x0, y0, z0, nzt, smu);
         __syncthreads();
     }
     {  // flux columns
+        static_assert(CP1 <= NT, "one thread per flux column");
         const int k = threadIdx.x, lx = k % CW1, ly = k / CW1, x = x0 - 1 + lx, y = y0 - 1 + ly;
         if (k < CP1 && x <= g.nx && y <= g.ny) {
             const int Y = MU_IN ? g.px : CW2, Z = MU_IN ? g.px * g.py : CW2 * CH2;
             const int pi = g.pidx32(x, y, z0 - 1), pz = g.px * g.py;
-            const float *m0 = MU_IN ? ca.mu + (pi - pz) : smu + (lx + 1) + CW2 * (ly + 1);
+            const float *m0 = MU_IN ? mu + (pi - pz) : smu + (lx + 1) + CW2 * (ly + 1);
             const float mg = a.M * (Q15 ? 1.0f / 24.0f : 1.0f / 12.0f);
             F1 G0[3], G1[3];
 #pragma unroll
             for (int j = 0; j < CZ + 4; ++j) {
                 const float *m = m0 + (MU_IN ? min(j, nzt + 3) : j) * Z;
-                const F1 mxp = rd<MU_IN>(m + 1), mxm = rd<MU_IN>(m - 1), myp = rd<MU_IN>(m + Y), mym = rd<MU_IN>(m - Y);
-                const F1 mpp = rd<MU_IN>(m + 1 + Y), mpm = rd<MU_IN>(m + 1 - Y);
-                const F1 mmp = rd<MU_IN>(m - 1 + Y), mmm = rd<MU_IN>(m - 1 - Y);
+                auto at = [&](int o) { return rd<MU_IN>(m + o); };
+                const F1 mxp = at(1), mxm = at(-1), myp = at(Y), mym = at(-Y);
+                const F1 mpp = at(1 + Y), mpm = at(1 - Y), mmp = at(-1 + Y), mmm = at(-1 - Y);
                 const F1 ex = mxp - mxm, ey = myp - mym;
                 const F1 Dx = (mpp + mpm) - (mmp + mmm), Dy = (mpp + mmp) - (mpm + mmm);
                 F1 gx, gy, gz;
                 if (Q15) {
-                    const F1 Zq = vfma(rd<MU_IN>(m), 8.f, (mpp + mpm) + (mmp + mmm));
+                    const F1 Zq = vfma(at(0), 8.f, (mpp + mpm) + (mmp + mmm));
                     if (j >= 2) {
                         gx = G0[0] + Dx;
                         gy = G0[1] + Dy;
@@ -234,7 +250,7 @@ __global__ void __launch_bounds__(T::CNT) psi3_fv_cube_kernel(const CubeArgs ca)
                     G1[1] = Dy;
                     G1[2] = Zq * -1.0f;
                 } else {
-                    const F1 Zp = vfma(rd<MU_IN>(m), 2.f, (mxp + mxm) + (myp + mym));
+                    const F1 Zp = vfma(at(0), 2.f, (mxp + mxm) + (myp + mym));
                     if (j >= 2) {
                         gx = G0[0] + ex;
                         gy = G0[1] + ey;
@@ -253,10 +269,10 @@ __global__ void __launch_bounds__(T::CNT) psi3_fv_cube_kernel(const CubeArgs ca)
                     F1 jx = gx * mg, jy = gy * mg, jz = gz * mg;
                     if (a.advect) {
                         const int o = pi + min(j - 2, nzt + 1) * pz;
-                        const F1 npv = F1{__ldg(a.psi + o)} * -1.0f;
-                        jx = vfma(F1{__ldg(a.u + o)}, npv, jx);
-                        jy = vfma(F1{__ldg(a.u + g.pn + o)}, npv, jy);
-                        jz = vfma(F1{__ldg(a.u + 2 * g.pn + o)}, npv, jz);
+                        const F1 npv = rd<true>(a.psi + o) * -1.0f;
+                        jx = vfma(rd<true>(a.u + o), npv, jx);
+                        jy = vfma(rd<true>(a.u + g.pn + o), npv, jy);
+                        jz = vfma(rd<true>(a.u + 2 * g.pn + o), npv, jz);
                     }
                     float *J = sJ + (j - 2) * CP1 + k;
                     J[0] = jx.v;
@@ -274,21 +290,21 @@ __global__ void __launch_bounds__(T::CNT) psi3_fv_cube_kernel(const CubeArgs ca)
         constexpr float DIV = Q15 ? 1.0f / 24.0f : 1.0f / 12.0f;
         int c = (tx + 1) + CW1 * (ty + 1) + CP1 * zh;
         Div3 d0, d1, n0, n1;
-        d0 = div3<T, Q15>(sJ, sJ + JN, sJ + 2 * JN, c);
-        d1 = div3<T, Q15>(sJ, sJ + JN, sJ + 2 * JN, c + CP1);
+        d0 = div3<T, Q15>(sJ, JN, c);
+        d1 = div3<T, Q15>(sJ, JN, c + CP1);
         if (NOISE) {
-            n0 = div3<T, Q15>(sX, sX + JN, sX + 2 * JN, c);
-            n1 = div3<T, Q15>(sX, sX + JN, sX + 2 * JN, c + CP1);
+            n0 = div3<T, Q15>(sX, JN, c);
+            n1 = div3<T, Q15>(sX, JN, c + CP1);
         }
         c += 2 * CP1;
 #pragma unroll
         for (int j = 0; j < CZ / 2; ++j, c += CP1) {
             const int z = z0 + zh + j;
-            const Div3 d2 = div3<T, Q15>(sJ, sJ + JN, sJ + 2 * JN, c);
+            const Div3 d2 = div3<T, Q15>(sJ, JN, c);
             const F1 D = vmul_sep(div_sum<Q15>(d0, d1, d2), DIV);
-            F1 eta{0.f};
+            F1 eta = F1{0.f};
             if (NOISE) {
-                const Div3 n2 = div3<T, Q15>(sX, sX + JN, sX + 2 * JN, c);
+                const Div3 n2 = div3<T, Q15>(sX, JN, c);
                 eta = vmul_sep(div_sum<Q15>(n0, n1, n2), DIV);
                 n0 = n1;
                 n1 = n2;
@@ -302,6 +318,19 @@ __global__ void __launch_bounds__(T::CNT) psi3_fv_cube_kernel(const CubeArgs ca)
     }
 }
 
+template <class T, bool FIRST, bool NOISE, bool MU_IN, bool Q15, bool W>
+__global__ void __launch_bounds__(T::NT) psi3_fv_cube_kernel(const CubeArgs ca)
+{
+    constexpr int JN = (T::CZ + 2) * T::CP1;
+    extern __shared__ float csm[];
+    float *sJ = csm, *sX = sJ + 3 * JN, *smu = sX + (NOISE ? 3 * JN : 0);  // smu: [CZ + 4][CH2][CW2] unless MU_IN
+    const int x0 = blockIdx.x * T::CX, y0 = blockIdx.y * T::CY, z0 = blockIdx.z * T::CZ;
+    pdl_trigger();
+    if (NOISE) cube_fv_noise<T>(ca.a, x0, y0, z0, sX);
+    pdl_wait();
+    cube_fv_stage<T, FIRST, NOISE, MU_IN, Q15, W>(ca.a, ca.mu, x0, y0, z0, sJ, sX, smu);
+}
+
 // ---------------------------------------------------------------------------
 // Finite difference and the naive contrast: D = M lap mu - div_CD(u psi).
 // ---------------------------------------------------------------------------
@@ -312,7 +341,7 @@ __device__ constexpr int8_t kCubeL[13][3] = {{1, 0, 0},  {0, 1, 0},  {0, 0, 1}, 
                                              {1, 1, -1}, {1, -1, 1}, {1, -1, -1}};
 
 template <class T, bool FIRST, bool NOISE, bool MU_IN, bool W>
-__global__ void __launch_bounds__(T::CNT) psi3_fd_cube_kernel(const CubeArgs ca)
+__global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
 {
     FLB_TILE3(T);
     constexpr int ZN = (CZ + 2) * CP1;
@@ -325,7 +354,7 @@ __global__ void __launch_bounds__(T::CNT) psi3_fd_cube_kernel(const CubeArgs ca)
     const int nzt = min(CZ, g.nz - z0);
     pdl_trigger();
     if (NOISE) {
-        for (int k = threadIdx.x; k < ZN; k += CNT) {
+        for (int k = threadIdx.x; k < ZN; k += NT) {
             const int lx = k % CW1, ly = (k / CW1) % CH1, lz = k / CP1;
             const int x = x0 - 1 + lx, y = y0 - 1 + ly, z = z0 - 1 + lz;
             if (x > g.nx || y > g.ny || z > g.nz) continue;
@@ -402,14 +431,13 @@ template <class T, bool FIRST, bool NOISE, bool MU_IN, bool W>
 cudaError_t go_fd(const CubeArgs &ca, dim3 grid, cudaStream_t st)
 {
     const int zn = (T::CZ + 2) * T::CP1;
-    return go(psi3_fd_cube_kernel<T, FIRST, NOISE, MU_IN, W>, ca, grid, T::CNT,
+    return go(psi3_fd_cube_kernel<T, FIRST, NOISE, MU_IN, W>, ca, grid, T::NT,
               zn * ((MU_IN ? 0 : 1) + (NOISE ? (ca.naive ? 3 : 13) : 0)), st);
 }
 template <class T, bool FIRST, bool NOISE, bool MU_IN, bool Q15, bool W>
 cudaError_t go_fv(const CubeArgs &ca, dim3 grid, cudaStream_t st)
 {
-    return go(psi3_fv_cube_kernel<T, FIRST, NOISE, MU_IN, Q15, W>, ca, grid, T::CNT,
-              (T::CZ + 2) * T::CP1 * (NOISE ? 6 : 3) + (MU_IN ? 0 : (T::CZ + 4) * T::CW2 * T::CH2), st);
+    return go(psi3_fv_cube_kernel<T, FIRST, NOISE, MU_IN, Q15, W>, ca, grid, T::NT, cube_fv_floats<T, NOISE, MU_IN>(), st);
 }
 
 template <class T, bool W>
