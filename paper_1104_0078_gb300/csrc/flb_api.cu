@@ -96,6 +96,8 @@ struct Rep {
     int zc = PS_ZC;  // planes per psi block (3D), set by flb_set_tuning / flb_autotune
     bool tuned = false;  // whether it was set (else auto_depth chooses)
     bool cube = false;   // tuned: the small-tile kernels were faster than any chunk
+    bool btuned = false; // whether it was set for the batched and persistent modes
+    int bzc = PS_ZC;     // planes per psi block in those modes: zc when set, else batch_depths()
     int fused = 0;   // single-pass Heun psi step (flb_set_psi_fused)
 };
 
@@ -792,8 +794,44 @@ bool batch_supported(const flb_handle *h)
     return !h->reps.empty();
 }
 
+// Planes per psi block of every replica in the batched and persistent modes: the
+// caller's or the tuner's, else even splits of the boxes' depths near one target, the one that
+// costs least when the whole list runs on two blocks for each of 152 SMs, a chunk of
+// zc planes taking zc + 8 plane times.  With 64 planes throughout, 25 replicas of
+// 32^3 ran 50 blocks (232 us a step, 131 with the 6 planes this gives); lists of many
+// blocks keep whole depths (256 replicas of 16^3 to 48^3).
+void batch_depths(flb_handle *h)
+{
+    auto split = [](int nz, int target) {
+        const int k = (nz + target - 1) / target;
+        return (nz + k - 1) / k;
+    };
+    int best = PS_ZC;
+    double cbest = 0.0;
+    for (int target : {4, 6, 8, 11, 13, 16, 22, 26, 32, 48, 64}) {
+        double blocks = 0.0, planes = 0.0, longest = 0.0;
+        for (const Rep &r : h->reps) {
+            const Geom &g = r.g;
+            const int zc = split(g.nz, target);
+            const double n = (double)((g.nx + PS_TX - 1) / PS_TX) * ((g.ny + PS_TY - 1) / PS_TY) * ((g.nz + zc - 1) / zc);
+            blocks += n;
+            planes += n * (zc + 8);
+            longest = std::max(longest, zc + 8.0);
+        }
+        double waves = blocks / 304.0;
+        if (waves < 4.0) waves = std::ceil(waves);
+        const double cost = std::max(waves * planes / blocks, longest);
+        if (cbest == 0.0 || cost < cbest) {
+            cbest = cost;
+            best = target;
+        }
+    }
+    for (Rep &r : h->reps) r.bzc = r.btuned ? r.zc : split(r.g.nz, best);
+}
+
 int batch_upload_lists(flb_handle *h)
 {
+    batch_depths(h);
     std::vector<BatchBlock> &v = h->b_blocks_host;
     v.clear();
     for (int r = 0; r < (int)h->reps.size(); ++r) {
@@ -810,7 +848,7 @@ int batch_upload_lists(flb_handle *h)
     const size_t nlb = v.size() - nmu;
     for (int r = 0; r < (int)h->reps.size(); ++r) {
         const Geom &g = h->reps[(size_t)r].g;
-        const int zc = h->reps[(size_t)r].zc;
+        const int zc = h->reps[(size_t)r].bzc;
         for (int bz = 0; bz < (g.nz + zc - 1) / zc; ++bz)
             for (int by = 0; by < (g.ny + PS_TY - 1) / PS_TY; ++by)
                 for (int bx = 0; bx < (g.nx + PS_TX - 1) / PS_TX; ++bx) v.push_back({r, bx, by, bz});
@@ -820,7 +858,7 @@ int batch_upload_lists(flb_handle *h)
     // blocks instead of starting a long one last
     auto planes = [&](const BatchBlock &b) {
         const Rep &r = h->reps[(size_t)b.rep];
-        return std::min(r.zc, r.g.nz - b.bz * r.zc);
+        return std::min(r.bzc, r.g.nz - b.bz * r.bzc);
     };
     std::stable_sort(v.begin() + (std::ptrdiff_t)(nmu + nlb), v.end(),
                      [&](const BatchBlock &a, const BatchBlock &b) { return planes(a) > planes(b); });
@@ -860,7 +898,7 @@ int batch_upload_table(flb_handle *h)
         d.noise = r.p.kT > 0 && r.p.M > 0;
         d.mu_in = (r.p.coupling & FLB_COUPLE_FORCE) && r.p.force_grad != FLB_FORCE_STRESS;
         d.q15 = r.q == 15;
-        d.zc = r.zc;
+        d.zc = r.bzc;
         d.pstep_tasks = k < h->p_pstep.size() ? h->p_pstep[k] : 0;
         const uint64_t pd[3] = {(uint64_t)g.px, (uint64_t)g.py, (uint64_t)g.pz};
         const uint64_t ps[2] = {(uint64_t)g.px * 4, (uint64_t)g.px * g.py * 4};
@@ -995,6 +1033,7 @@ bool persist_supported(const flb_handle *h)
 // need of a task counts the tasks of its replica listed before it.
 int persist_build(flb_handle *h)
 {
+    batch_depths(h);
     std::vector<PTask> v;
     const size_t nr = h->reps.size();
     std::vector<int> need(nr, 0);
@@ -1002,9 +1041,9 @@ int persist_build(flb_handle *h)
         for (size_t k = 0; k < nr; ++k) {
             const Rep &r = h->reps[k];
             int c[PH_COUNT];
-            persist_tiles(r.g, r.zc, r.p.coupling, r.p.integrator == FLB_HEUN ? 1 : 0, c);
+            persist_tiles(r.g, r.bzc, r.p.coupling, r.p.integrator == FLB_HEUN ? 1 : 0, c);
             if (c[ph] == 0) continue;
-            persist_tasks(v, (int)k, ph, r.g, r.zc, need[k]);
+            persist_tasks(v, (int)k, ph, r.g, r.bzc, need[k]);
             need[k] += c[ph];
         }
     if (v.size() > h->p_cap) return FLB_EINVAL;
@@ -1618,14 +1657,14 @@ int flb_set_tuning(flb_handle *h, int32_t rep, int32_t psi_zchunk)
     if (rep == -1) {
         for (Rep &r : h->reps) {
             r.zc = psi_zchunk;
-            r.tuned = true;
+            r.tuned = r.btuned = true;
             r.cube = false;
         }
     } else {
         Rep *r = get_rep(h, rep);
         if (!r) return FLB_EINVAL;
         r->zc = psi_zchunk;
-        r->tuned = true;
+        r->tuned = r->btuned = true;
         r->cube = false;
     }
     batch_reset(h);
@@ -1661,6 +1700,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
         for (const Rep &r : h->reps) depths.push_back(r.g.nz);
         std::sort(depths.begin(), depths.end(), std::greater<int>());
         depths.erase(std::unique(depths.begin(), depths.end()), depths.end());
+        for (Rep &r : h->reps) r.btuned = true;
         auto set_depth = [&](int nz, int zc) {
             for (Rep &r : h->reps)
                 if (r.g.nz == nz) r.zc = zc;
