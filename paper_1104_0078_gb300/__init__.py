@@ -240,14 +240,14 @@ class Solver:
         _check(self.lib.flb_set_populations(self.h, rep, _dp(a)), "flb_set_populations")
 
     def get_psi_u(self, rep=0):
-        psi = np.zeros(self.n(rep))
-        u = np.zeros((self.params[rep].dim, self.n(rep)))
+        psi = np.empty(self.n(rep))
+        u = np.empty((self.params[rep].dim, self.n(rep)))
         _check(self.lib.flb_get_psi_u(self.h, rep, _dp(psi), _dp(u)), "flb_get_psi_u")
         return psi, u
 
     def get_psi(self, rep=0):
         """psi [N] alone (flb_get_psi_u with no velocity)."""
-        psi = np.zeros(self.n(rep))
+        psi = np.empty(self.n(rep))
         _check(self.lib.flb_get_psi_u(self.h, rep, _dp(psi), None), "flb_get_psi_u")
         return psi
 
