@@ -754,6 +754,7 @@ int sample_rep(flb_handle *h, Rep &r, int mask)
         for (int part = 0; part < 2; ++part) {
             DftArgs d;
             d.in = h->heights;
+            d.ordered = true;
             d.off = (long long)part * g.nx * g.ny;
             d.sy = g.nx;
             d.sz = 0;

@@ -209,7 +209,9 @@ __device__ __forceinline__ float2 twiddle(int k, int x, int n)
 // each output walks its phase index m = k x mod n by additions.
 constexpr int TW_MAX = 4096;
 
-// X1[(z*ny + y)*nu + j] = sum_x in(x,y,z) e^{-2 pi i j x / nx}, one output per thread
+// X1[(z*ny + y)*nu + j] = sum_x in(x,y,z) e^{-2 pi i j x / nx}, one output per thread,
+// in NP partial sums over x mod NP (independent chains).
+template <int NP>
 __global__ void dft_x_kernel(DftArgs a)
 {
     extern __shared__ float2 tw[];
@@ -222,12 +224,13 @@ __global__ void dft_x_kernel(DftArgs a)
     const int k = (int)(t % nu);
     const long long row = t / nu;  // z*ny + y
     const float *src = a.in + a.off + (row % a.ny) * a.sy + (row / a.ny) * a.sz;
-    float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};  // x mod 4: four independent chains
+    float re[NP] = {}, im[NP] = {};
     int m = 0, x = 0;
-    for (; x + 4 <= a.nx; x += 4) {
+#pragma unroll 8 / NP
+    for (; x + NP <= a.nx; x += NP) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const float v = src[x + u];
+        for (int u = 0; u < NP; ++u) {
+            const float v = __ldg(src + x + u);
             const float2 w = tw[m];
             re[u] = fmaf(v, w.x, re[u]);
             im[u] = fmaf(v, w.y, im[u]);
@@ -236,14 +239,15 @@ __global__ void dft_x_kernel(DftArgs a)
         }
     }
     for (; x < a.nx; ++x) {
-        const float v = src[x];
+        const float v = __ldg(src + x);
         const float2 w = tw[m];
         re[0] = fmaf(v, w.x, re[0]);
         im[0] = fmaf(v, w.y, im[0]);
         m += k;
         if (m >= a.nx) m -= a.nx;
     }
-    a.X1[t] = make_float2((re[0] + re[1]) + (re[2] + re[3]), (im[0] + im[1]) + (im[2] + im[3]));
+    a.X1[t] = NP == 4 ? make_float2((re[0] + re[1]) + (re[2] + re[NP - 1]), (im[0] + im[1]) + (im[2] + im[NP - 1]))
+                      : make_float2(re[0], im[0]);
 }
 
 // The same X1 for windows of nu <= 18, as a small matrix product over blocks of
@@ -505,6 +509,50 @@ cudaError_t launch_dyn_corr(const float2 *ring, int L, int slot, int nlag, long 
     return cudaGetLastError();
 }
 
+// The y pass of a planar field in a fixed order of summation, one output (j, jy) per
+// thread in NP partial sums over y mod NP: S += scale |X|^2 at k and at its conjugate place.  For
+// the interface heights: their mean is 10^3 times what the spectrum shows, so its small
+// components carry the rounding of this order, which is therefore part of the result.
+template <int NP>
+__global__ void __launch_bounds__(128) dft_y_planar_kernel(DftArgs a)
+{
+    extern __shared__ float2 tw[];
+    for (int m = threadIdx.x; m < a.ny; m += blockDim.x) tw[m] = twiddle(1, m, a.ny);
+    __syncthreads();
+    const int nu = a.Kx / 2 + 1, t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= nu * a.Ky) return;
+    const int jx = t % nu, jy = t / nu;
+    const int k = (a.Ky >= a.ny || jy <= a.Ky / 2) ? jy : a.ny - (a.Ky - jy);
+    const float2 *src = a.X1 + jx;
+    float re4[NP] = {}, im4[NP] = {};
+    int m = 0, y = 0;
+    auto add = [&](int u, float2 v) {
+        const float2 w = tw[m];
+        re4[u] += v.x * w.x - v.y * w.y;
+        im4[u] += v.x * w.y + v.y * w.x;
+        m += k;
+        if (m >= a.ny) m -= a.ny;
+    };
+    constexpr int B = 16;  // loads in flight
+    for (; y + B <= a.ny; y += B) {
+        float2 v[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) v[u] = __ldg(src + (long long)(y + u) * nu);
+#pragma unroll
+        for (int u = 0; u < B; ++u) add(u % NP, v[u]);
+    }
+    for (; y + NP <= a.ny; y += NP)
+#pragma unroll
+        for (int u = 0; u < NP; ++u) add(u, __ldg(src + (long long)(y + u) * nu));
+    for (; y < a.ny; ++y) add(0, __ldg(src + (long long)y * nu));
+    const double re = NP == 4 ? (re4[0] + re4[1]) + (re4[2] + re4[NP - 1]) : re4[0];
+    const double im = NP == 4 ? (im4[0] + im4[1]) + (im4[2] + im4[NP - 1]) : im4[0];
+    const double val = a.scale * (re * re + im * im);
+    a.S[(long long)jy * a.Kx + jx] += val;
+    const int jxm = conj_partner(jx, a.nx, a.Kx);
+    if (jxm != jx) a.S[(long long)conj_partner(jy, a.ny, a.Ky) * a.Kx + jxm] += val;
+}
+
 template <int NUP>
 cudaError_t go_rows(const DftArgs &a, cudaStream_t s)
 {
@@ -515,7 +563,7 @@ cudaError_t go_rows(const DftArgs &a, cudaStream_t s)
         k<<<(unsigned)((rows + per - 1) / per), DXR_NT, smem, s>>>(a, rows);
         return cudaGetLastError();
     };
-    return rows >= 152 * DXR_NT ? go(dft_x_rows_kernel<NUP, 1>, DXR_NT, dxr_smem<NUP, 1>(a.nx))
+    return rows >= 152 * DXR_NT || a.ordered ? go(dft_x_rows_kernel<NUP, 1>, DXR_NT, dxr_smem<NUP, 1>(a.nx))
                                 : go(dft_x_rows_kernel<NUP, 8>, DXR_NT / 8, dxr_smem<NUP, 8>(a.nx));
 }
 
@@ -534,10 +582,18 @@ cudaError_t launch_dft_accumulate(const DftArgs &a, cudaStream_t s)
     else if (nu <= 18) e = go_rows<18>(a, s);
     else {
         const int bs = 256;
-        dft_x_kernel<<<(unsigned)(((long long)nu * a.ny * a.nz + bs - 1) / bs), bs, sizeof(float2) * a.nx, s>>>(a);
+        const unsigned grid = (unsigned)(((long long)nu * a.ny * a.nz + bs - 1) / bs);
+        if (a.ordered) dft_x_kernel<1><<<grid, bs, sizeof(float2) * a.nx, s>>>(a);
+        else dft_x_kernel<4><<<grid, bs, sizeof(float2) * a.nx, s>>>(a);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) return e;
+    if (a.ordered) {  // planar; one chain for small windows, four for others
+        const unsigned grid = (unsigned)((nu * a.Ky + 127) / 128);
+        if (a.Kx * a.Ky <= 1024) dft_y_planar_kernel<1><<<grid, 128, sizeof(float2) * a.ny, s>>>(a);
+        else dft_y_planar_kernel<4><<<grid, 128, sizeof(float2) * a.ny, s>>>(a);
+        return cudaGetLastError();
+    }
     const AxisArgs y{a.X1, a.X2, a.nz, a.ny, nu, a.Ky, a};
     if (a.nz == 1) return launch_axis<float, true>(y, s);
     e = launch_axis<float, false>(y, s);

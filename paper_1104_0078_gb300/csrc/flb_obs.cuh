@@ -21,6 +21,7 @@ struct DftArgs {
     float2 *X1, *X2;       // scratch: nz*ny*nu and nz*Ky*nu complex values, nu = Kx/2 + 1
     double *S;             // accumulator Kz*Ky*Kx (may be null: no accumulation)
     double scale;          // factor on |.|^2
+    bool ordered = false;    // planar fields with a large mean: one fixed order of summation
     float2 *snap = nullptr;  // if not null: the Fourier components, Kz*Ky*Kx
 };
 
