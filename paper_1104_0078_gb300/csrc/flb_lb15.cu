@@ -24,8 +24,19 @@ __global__ void __launch_bounds__(LB_BX *LB_BY, 7) lb15_kernel(const LBArgs a, c
     const int nl = z + 1 < g.nz ? 2 : 1;
     const int zl[2] = {z, z + nl - 1};
     F2 Fx = F2::bc(0.f), Fy = F2::bc(0.f), Fz = F2::bc(0.f);
-    if (FORCE) force3v<false>(a, x, y, zl, Fx, Fy, Fz);
-    lb15_sites<F2, T, GHOST_RELAX>(a, P, x, y, zl, nl, Fx, Fy, Fz);
+    if (FORCE) force3v<false, F2, true>(a, x, y, zl, Fx, Fy, Fz);
+    const bool inner = y > 0 && y < g.ny - 1 && z > 0 && z < g.nz - 2;  // the same for the whole warp
+    lb15_sites_on<F2, T, GHOST_RELAX, false>(a, P, x, y, zl, nl, Fx, Fy, Fz, [&](F2 *f) {
+        if (inner) {
+            pull_inner<T, 15>(P, g, x, y, z, f);
+            return;
+        }
+        float f0[15], f1[15];
+        pull15<T>(P, g, x, y, zl[0], f0);
+        pull15<T>(P, g, x, y, zl[1], f1);
+#pragma unroll
+        for (int i = 0; i < 15; ++i) f[i] = F2{make_float2(f0[i], f1[i])};
+    });
 }
 
 // u of the streamed state, one thread per site (plane addresses formed from
@@ -54,7 +65,7 @@ __global__ void __launch_bounds__(LBB_NT, 7) lb15_batch_kernel(const BatchLists 
     int x, y, zl[2], nl;
     if (!packed_pair<LBB_NT>(sa.g, b.bx, b.by, b.bz, threadIdx.x, x, y, zl, nl)) return;
     F2 Fx = F2::bc(0.f), Fy = F2::bc(0.f), Fz = F2::bc(0.f);
-    if (FORCE && (sa.coupling & FLB_COUPLE_FORCE)) force3v<false>(sa, x, y, zl, Fx, Fy, Fz);
+    if (FORCE && (sa.coupling & FLB_COUPLE_FORCE)) force3v<false, F2, true>(sa, x, y, zl, Fx, Fy, Fz);
     lb15_sites<F2, T, GHOST_RELAX, false, true>(sa, PlanesFromBase<T>{(const T *)sa.fin, (T *)sa.fout, sa.g.n}, x, y,
                                                 zl, nl, Fx, Fy, Fz);
 }
@@ -108,7 +119,7 @@ cudaError_t launch_lb15(const LBArgs &a, int storage, cudaStream_t st)
     const dim3 grid((a.g.nx + LB_BX - 1) / LB_BX, (a.g.ny + LB_BY - 1) / LB_BY, (a.g.nz + LB_BZ - 1) / LB_BZ);
     const bool gr = a.gamma_g != 0.0f;
     const bool force = (a.coupling & FLB_COUPLE_FORCE) != 0;
-#define FLB_LB15(T, G, F) return launch_pdl(lb15_kernel<T, G, F>, grid, block, 0, st, PDL_BLOCKS, a, plane_table<T>(a.fin, a.fout, a.g.n, 15))
+#define FLB_LB15(T, G, F) return launch_pdl(lb15_kernel<T, G, F>, grid, block, 0, st, PDL_BLOCKS, a, plane_table<T>(a.fin, a.fout, a.g, 15))
     if (storage == FLB_F16_DEV) {
         if (gr) { if (force) FLB_LB15(__half, true, true); else FLB_LB15(__half, true, false); }
         else { if (force) FLB_LB15(__half, false, true); else FLB_LB15(__half, false, false); }

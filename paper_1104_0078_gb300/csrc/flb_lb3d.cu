@@ -11,8 +11,14 @@
 //
 // Indices are 32-bit (N and the padded planes are < 2^31); population plane i
 // of N sites starts at fin + i*N.  The plain kernel runs seven 128-thread blocks
-// per SM (72 registers, no spills): 4.08 ms at 512^3; six blocks (80 registers)
-// and eight (64, spilling) measured slower.  Noise order: bulk, 3c_x^2-c^2, c_y^2-c_z^2,
+// per SM (72 registers, no spills; six blocks at 80 registers and eight at 64,
+// spilling, measured slower): 3.71 ms at 512^3, 5.5 TB/s on its 152 B/site.  It is bound by
+// instruction issue and by the L1's wavefronts together: 4.01 ms before sites away from
+// the box's y and z faces took one index for all planes (of pre-shifted plane
+// pointers) and the pair of sites the planes of mu between them once (3.82), and
+// before the angle of Box-Muller came from polynomials instead of gathers (3.71).
+// Marching z with the populations fetched one pair of planes ahead by cp.async took
+// 4.69 ms: latency is not what bounds it.  Noise order: bulk, 3c_x^2-c^2, c_y^2-c_z^2,
 // xy, yz, zx, three c^2 c_a ghosts, three c_a(c_b^2-c_g^2) ghosts, c^4,
 // c^2(3c_x^2-c^2), c^2(c_y^2-c_z^2).
 #include "flb_site3d.cuh"
@@ -38,8 +44,12 @@ __global__ void __launch_bounds__(LB_BX *LB_BY, 7)
     const int nl = z + 1 < g.nz ? 2 : 1;
     const int zl[2] = {z, z + nl - 1};  // a lane past the box repeats lane 0's site
     F2 Fx = F2::bc(0.f), Fy = F2::bc(0.f), Fz = F2::bc(0.f);
-    if (FORCE && (a.coupling & FLB_COUPLE_FORCE)) force3v<false>(a, x, y, zl, Fx, Fy, Fz);
-    lb_sites<F2, T, GHOST_RELAX, false, false>(a, P, x, y, zl, nl, Fx, Fy, Fz);
+    if (FORCE && (a.coupling & FLB_COUPLE_FORCE)) force3v<false, F2, true>(a, x, y, zl, Fx, Fy, Fz);
+    const bool inner = y > 0 && y < g.ny - 1 && z > 0 && z < g.nz - 2;  // the same for the whole warp
+    lb_sites_on<F2, T, GHOST_RELAX, false>(a, P, x, y, zl, nl, Fx, Fy, Fz, [&](F2 *f) {
+        if (inner) pull_inner<T, 19>(P, g, x, y, z, f);
+        else pullv<T, false>(P, g, x, y, zl, f);
+    });
 }
 
 // ---- batched variant: block b of the launch works on the row-packed entry L.lb[b]
@@ -53,7 +63,7 @@ __global__ void __launch_bounds__(LBB_NT, 7) lb3_batch_kernel(const BatchLists L
     int x, y, zl[2], nl;
     if (!packed_pair<LBB_NT>(sa.g, b.bx, b.by, b.bz, threadIdx.x, x, y, zl, nl)) return;
     F2 Fx = F2::bc(0.f), Fy = F2::bc(0.f), Fz = F2::bc(0.f);
-    if (FORCE && (sa.coupling & FLB_COUPLE_FORCE)) force3v<false>(sa, x, y, zl, Fx, Fy, Fz);
+    if (FORCE && (sa.coupling & FLB_COUPLE_FORCE)) force3v<false, F2, true>(sa, x, y, zl, Fx, Fy, Fz);
     lb_sites<F2, T, GHOST_RELAX, false, true>(sa, PlanesFromBase<T>{(const T *)sa.fin, (T *)sa.fout, sa.g.n}, x, y,
                                               zl, nl, Fx, Fy, Fz);
 }
@@ -85,7 +95,7 @@ cudaError_t launch_lb3d(const LBArgs &a, int storage, cudaStream_t st)
     const dim3 grid((a.g.nx + LB_BX - 1) / LB_BX, (a.g.ny + LB_BY - 1) / LB_BY, (a.g.nz + LB_BZ - 1) / LB_BZ);
     const bool gr = a.gamma_g != 0.0f;
     const bool force = (a.coupling & FLB_COUPLE_FORCE) != 0;
-#define FLB_LB3(T, G, F) return launch_pdl(lb3_kernel<T, G, F>, grid, block, 0, st, PDL_BLOCKS, a, plane_table<T>(a.fin, a.fout, a.g.n, 19))
+#define FLB_LB3(T, G, F) return launch_pdl(lb3_kernel<T, G, F>, grid, block, 0, st, PDL_BLOCKS, a, plane_table<T>(a.fin, a.fout, a.g, 19))
     if (storage == FLB_F16_DEV) {
         if (gr) { if (force) FLB_LB3(__half, true, true); else FLB_LB3(__half, true, false); }
         else { if (force) FLB_LB3(__half, false, true); else FLB_LB3(__half, false, false); }

@@ -72,32 +72,19 @@ __device__ __forceinline__ void moments15(const float f[15], float sp[8], float 
 // The second moment is carried as Q = 9/2 B, with the relaxation coefficients
 // a.rq of the D3Q19 kernel (they do not depend on the lattice); the ghost
 // amplitudes g_k stay in the units above.
-// P: the planes it pulls from (P.in) and stores to (P.out).  COH: loads through
-// L2 (fields written in the same launch); KEY_R0: round keys formed from round
-// 0's (arguments in shared memory).
-template <class V, typename T, bool GHOST_RELAX, bool COH = false, bool KEY_R0 = false, class PL>
-__device__ __forceinline__ void lb15_sites(const LBArgs &a, const PL &P, int x, int y, const int *zl, int nl, V Fx,
-                                           V Fy, V Fz)
+// P: the planes it stores to (P.out); pull(f) gives the streamed populations; KEY_R0:
+// round keys formed from round 0's (arguments in shared memory).
+template <class V, typename T, bool GHOST_RELAX, bool KEY_R0, class PL, class PULL>
+__device__ __forceinline__ void lb15_sites_on(const LBArgs &a, const PL &P, int x, int y, const int *zl, int nl, V Fx,
+                                              V Fy, V Fz, PULL &&pull)
 {
     constexpr int L = V::L;
     const Geom &g = a.g;
     int s[L];
+#pragma unroll
+    for (int l = 0; l < L; ++l) s[l] = x + g.nx * (y + g.ny * zl[l]);
     V f[15];
-    {
-        float fl[L][15];
-#pragma unroll
-        for (int l = 0; l < L; ++l) {
-            s[l] = x + g.nx * (y + g.ny * zl[l]);
-            pull15<T, COH>(P, g, x, y, zl[l], fl[l]);
-        }
-#pragma unroll
-        for (int i = 0; i < 15; ++i) {
-            float t[L];
-#pragma unroll
-            for (int l = 0; l < L; ++l) t[l] = fl[l][i];
-            f[i] = vmake<V>(t);
-        }
-    }
+    pull(f);
     V sp[8], dp[8];
 #pragma unroll
     for (int p = 1; p <= 7; ++p) {
@@ -255,6 +242,27 @@ __device__ __forceinline__ void vel15_site_on(const LBArgs &a, const PL &P, int 
     store_padded(a.u, g, x, y, z, (jx + 0.5f * Fx) * irho, 1);
     store_padded(a.u + g.pn, g, x, y, z, (jy + 0.5f * Fy) * irho, 1);
     store_padded(a.u + 2 * g.pn, g, x, y, z, (jz + 0.5f * Fz) * irho, 1);
+}
+
+// The same with the populations pulled from the planes P.in (COH: loads through L2,
+// fields written in the same launch).
+template <class V, typename T, bool GHOST_RELAX, bool COH = false, bool KEY_R0 = false, class PL>
+__device__ __forceinline__ void lb15_sites(const LBArgs &a, const PL &P, int x, int y, const int *zl, int nl, V Fx,
+                                           V Fy, V Fz)
+{
+    constexpr int L = V::L;
+    lb15_sites_on<V, T, GHOST_RELAX, KEY_R0>(a, P, x, y, zl, nl, Fx, Fy, Fz, [&](V *f) {
+        float fl[L][15];
+#pragma unroll
+        for (int l = 0; l < L; ++l) pull15<T, COH>(P, a.g, x, y, zl[l], fl[l]);
+#pragma unroll
+        for (int i = 0; i < 15; ++i) {
+            float t[L];
+#pragma unroll
+            for (int l = 0; l < L; ++l) t[l] = fl[l][i];
+            f[i] = vmake<V>(t);
+        }
+    });
 }
 
 // One site's collide-stream on the planes of a.fin and a.fout (the persistent

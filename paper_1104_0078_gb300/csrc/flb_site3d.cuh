@@ -59,19 +59,38 @@ struct PlanesFromBase {
 template <typename T>
 struct PlaneTable {
     const T *in_[19];
+    const T *up_[19];  // in_[i] - (c_i as a site offset): where population i of site s streams from, away from the box's faces
     T *out_[19];
     __device__ __forceinline__ const T *in(int i) const { return in_[i]; }
+    __device__ __forceinline__ const T *up(int i) const { return up_[i]; }
     __device__ __forceinline__ T *out(int i) const { return out_[i]; }
 };
 
 // The table of q planes of n sites from the buffers in and out (either may be
 // null) (host).
-template <typename T>
-inline PlaneTable<T> plane_table(const void *in, void *out, long long n, int q)
+inline const int8_t (*stream_vectors(int q))[3]  // c_i in plane order
 {
+    static const int8_t c19[19][3] = {{0, 0, 0},  {1, 0, 0},   {-1, 0, 0}, {0, 1, 0},  {0, -1, 0},
+                                      {0, 0, 1},  {0, 0, -1},  {1, 1, 0},  {-1, -1, 0}, {1, -1, 0},
+                                      {-1, 1, 0}, {1, 0, 1},   {-1, 0, -1}, {1, 0, -1}, {-1, 0, 1},
+                                      {0, 1, 1},  {0, -1, -1}, {0, 1, -1}, {0, -1, 1}};
+    static const int8_t c15[15][3] = {{0, 0, 0},  {1, 0, 0},   {-1, 0, 0},   {0, 1, 0},  {0, -1, 0},
+                                      {0, 0, 1},  {0, 0, -1},  {1, 1, 1},    {-1, -1, -1}, {1, 1, -1},
+                                      {-1, -1, 1}, {1, -1, 1}, {-1, 1, -1},  {1, -1, -1}, {-1, 1, 1}};
+    return q == 15 ? c15 : c19;
+}
+template <typename T>
+inline PlaneTable<T> plane_table(const void *in, void *out, const Geom &g, int q)
+{
+    const long long n = g.n;
     PlaneTable<T> P{};
     for (int i = 0; i < q; ++i) {
         P.in_[i] = in ? (const T *)in + i * n : nullptr;
+        if (in) {
+            const int8_t *c = stream_vectors(q)[i];
+            const long long off = c[0] + (long long)g.nx * (c[1] + (long long)g.ny * c[2]);
+            P.up_[i] = (const T *)((uintptr_t)P.in_[i] - (uintptr_t)(off * (long long)sizeof(T)));
+        }
         P.out_[i] = out ? (T *)out + i * n : nullptr;
     }
     return P;
@@ -125,10 +144,36 @@ __device__ __forceinline__ void pullv(const PL &P, const Geom &g, int x, int y, 
 #undef FLB_PULL
 }
 
+// The same for two lanes (x, y, z) and (x, y, z + 1) that touch no face of the box in y
+// or z: population i of site s comes from P.up(i)[s], but for the columns x = 0 and
+// x = nx - 1, whose neighbours beyond the face are a row's length on.
+template <typename T, int Q, class PL>
+__device__ __forceinline__ void pull_inner(const PL &P, const Geom &g, int x, int y, int z, F2 f[Q])
+{
+    int s0[2], sm[2], sp[2];
+    s0[0] = x + g.nx * (y + g.ny * z);
+    s0[1] = s0[0] + g.nx * g.ny;
+    const int wm = x == 0 ? g.nx : 0, wp = x == g.nx - 1 ? -g.nx : 0;
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        sm[l] = s0[l] + wm;
+        sp[l] = s0[l] + wp;
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const bool xi = i == 1 || i == 2 || (i >= 7 && i <= 14);  // c_x = +1 for the odd ones, -1 for the even (both lattices)
+        const int *s = !xi ? s0 : (i & 1) ? sm : sp;
+        const float t[2] = {ld3<false>(P.up(i), s[0]), ld3<false>(P.up(i), s[1])};
+        f[i] = vmake<F2>(t);
+    }
+}
+
 // Force density of Sec. IV at the lanes' interior sites (x, y, zl[l]):
 // F = -psi grad mu with the central difference or the FV gradient of mu, or
-// F = -div sigma (stress form).
-template <bool COH, class V>
+// F = -div sigma (stress form).  PAIR: lane 1 is the site above lane 0's (on the last
+// plane of an odd box a ghost site, whose value is not used), so that the two share
+// the loads of the planes between them.
+template <bool COH, class V, bool PAIR = false>
 __device__ __forceinline__ void force3v(const LBArgs &a, int x, int y, const int *zl, V &Fx, V &Fy, V &Fz)
 {
     constexpr int L = V::L;
@@ -136,7 +181,7 @@ __device__ __forceinline__ void force3v(const LBArgs &a, int x, int y, const int
     const int sy = g.px, sz = g.px * g.py;
     int pi[L];
 #pragma unroll
-    for (int l = 0; l < L; ++l) pi[l] = g.pidx32(x, y, zl[l]);
+    for (int l = 0; l < L; ++l) pi[l] = PAIR ? g.pidx32(x, y, zl[0]) + l * sz : g.pidx32(x, y, zl[l]);
     auto LD = [&](const float *base, int off) {
         float t[L];
 #pragma unroll
@@ -246,10 +291,10 @@ __device__ __forceinline__ void batch_lb_args(const BatchLists &L, const BatchRe
 // ghosts] needs no further scale factors; a.rq and a.nq carry the relaxation
 // and noise coefficients in these units.
 // KEY_R0: the arguments sit in shared memory (batched and persistent kernels).
-// P: the planes it pulls from (P.in) and stores to (P.out).
-template <class V, typename T, bool GHOST_RELAX, bool COH, bool KEY_R0, class PL>
-__device__ __forceinline__ void lb_sites(const LBArgs &a, const PL &P, int x, int y, const int *zl, int nl, V Fx,
-                                         V Fy, V Fz)
+// P: the planes it stores to (P.out); pull(f) gives the streamed populations.
+template <class V, typename T, bool GHOST_RELAX, bool KEY_R0, class PL, class PULL>
+__device__ __forceinline__ void lb_sites_on(const LBArgs &a, const PL &P, int x, int y, const int *zl, int nl, V Fx,
+                                            V Fy, V Fz, PULL &&pull)
 {
     constexpr int L = V::L;
     const Geom &g = a.g;
@@ -258,7 +303,7 @@ __device__ __forceinline__ void lb_sites(const LBArgs &a, const PL &P, int x, in
     for (int l = 0; l < L; ++l) s[l] = x + g.nx * y + g.nx * g.ny * zl[l];
 
     V f[19];
-    pullv<T, COH>(P, g, x, y, zl, f);
+    pull(f);
 
     V sp[10], dp[10];
 #pragma unroll
@@ -417,6 +462,15 @@ __device__ __forceinline__ void lb_sites(const LBArgs &a, const PL &P, int x, in
         store(17, (E17 + O17) * w2);
         store(18, (E17 - O17) * w2);
     }
+}
+
+// The same with the populations pulled from the planes P.in.
+template <class V, typename T, bool GHOST_RELAX, bool COH, bool KEY_R0, class PL>
+__device__ __forceinline__ void lb_sites(const LBArgs &a, const PL &P, int x, int y, const int *zl, int nl, V Fx,
+                                         V Fy, V Fz)
+{
+    lb_sites_on<V, T, GHOST_RELAX, KEY_R0>(a, P, x, y, zl, nl, Fx, Fy, Fz,
+                                           [&](V *f) { pullv<T, COH>(P, a.g, x, y, zl, f); });
 }
 
 // One site on the planes of a.fin and a.fout (the persistent kernel, one site per thread).
