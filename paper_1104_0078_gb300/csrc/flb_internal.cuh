@@ -71,7 +71,7 @@ __device__ __forceinline__ u32x4 philox4x32_10_r0(u32x4 c, uint32_t a, uint32_t 
     return c;
 }
 
-// ---- Box-Muller by table lookup --------------------------------------------
+// ---- Box-Muller ---------------------------------------------------------------
 // One Philox word w makes one Box-Muller pair: its top 20 bits give the radius
 // uniform u = ((w >> 12) + 1/2) 2^-20 and its low 12 bits the angle uniform
 // v = ((w & 0xFFF) + 1/2) 2^-12, both exact in binary32, so a block of four
@@ -79,78 +79,31 @@ __device__ __forceinline__ u32x4 philox4x32_10_r0(u32x4 c, uint32_t a, uint32_t 
 // r = sqrt(-2 ln u): its radius stops at sqrt(42 ln 2) = 5.40 (the pair falls
 // beyond it with probability 4.8e-7) and the 4096 equally spaced angles make
 // every moment of (cos, sin) of order below 4096 the continuous one.
-// The two transcendental steps are specialised to these uniforms and
-// evaluated from small tables, to single-precision accuracy with fewer
-// instructions than the general logf and sincospif:
-//  * ln u, u = (2k+1) 2^-21: the table-driven method of P. T. P. Tang (ACM
-//    TOMS 16(4), 1990).  2k+1 = 2^e f with f in [sqrt(1/2), sqrt(2)); the bits
-//    of f select one of 32 cells; ln f = -ln r_j + ln(1 + d) with d = f r_j - 1
-//    formed by one FMA (|d| < 1/64) and ln(1 + d) by its series to d^5 (error
-//    < 3e-12).  r_j is near 1/(cell centre) and exactly 1 in the cell holding 1,
-//    where d = f - 1 is exact, so u near 1 keeps its relative accuracy.  The
-//    radius needs -2 ln u: the series and the table carry the factor -2, which
-//    is exact in binary arithmetic.
-//  * sin, cos of 2 pi v, v = (m + 1/2) 2^-12: v = x or x + 1/2 with x in (-1/4, 1/4), exact in
+// The two transcendental steps are specialised to these uniforms, to
+// single-precision accuracy, without a branch or a memory access:
+//  * ln u, u = (2k+1) 2^-21: 2k+1 = 2^e f with f in [sqrt(1/2), sqrt(2)), and
+//    -2 ln f = d P(d) with d = f - 1 exact and P of degree 9, interpolating
+//    -2 ln(1 + d)/d at the Chebyshev nodes of that interval (in 64 bits, rounded) with
+//    P(0) = -2, so u near 1 keeps its relative accuracy; (e - 21) times a 19-bit
+//    part of -2 ln 2 is exact, and the rest is added last.  Over the 2^20 radius
+//    uniforms -2 ln u is off by 1.2e-7 of itself at most, 3.1e-8 rms, and its root by 2.2e-7 at
+//    most, 1.9e-8 rms (Tang's method with a 32-cell table: 1.3e-7, 3.6e-8, 2.3e-7, 2.6e-8).
+//  * sin, cos of 2 pi v: v = x or x + 1/2 with x in (-1/4, 1/4), exact in
 //    binary32, the half turn negating both; then polynomials in y = x^2, interpolating
 //    sin(2 pi x)/x and cos 2 pi x at the Chebyshev nodes of [0, 1/16] (in 64 bits, rounded;
 //    their own error < 1e-9), the sine's leading 2 pi as the rounded constant and the
 //    rest.  Over the 4096 angles the sine is off by 7.9e-8 at most and 1.8e-8 rms, the cosine by
 //    7.8e-8 and 2.2e-8 (a 64-entry table with angle addition: 8.0e-8 and 2.4e-8 both).
-//    As many instructions as that table, whose gathers cost the L1 eight wavefronts a
-//    word: 64 of the 136 of a site's collide-stream, at 59% of the L1's rate.
-// The logarithm's table is computed at compile time in double precision from its series
-// and rounded to float.
+// As many instructions as with those tables, whose gathers cost the L1 ten wavefronts
+// a word, 80 of the 136 of a site's collide-stream at 59% of the L1's rate: 512^3
+// collide-stream 3.82 ms with both tables, 3.71 with the logarithm's, 3.62 with
+// none; the FD step at 160^3 467, 441 and 427 us.  (Fewer integer steps, funnel shifts
+// in place of the conversion and a mask: 3.63 ms, no gain.)
 namespace bm {
-
-struct alignas(8) LogCell {
-    float r, l2r;  // r_j and 2 ln r_j
-};
-struct Tables {
-    LogCell lg[32];
-};
 
 constexpr uint32_t kSqrtHalfBits = 0x3F3504F3u;  // bits of sqrt(1/2) in binary32
 
-// ln x for x in [0.5, 2] as 2 atanh((x - 1)/(x + 1)) (|s| <= 1/3; 40 terms)
-constexpr double series_log(double x)
-{
-    const double s = (x - 1.0) / (x + 1.0);
-    double p = s, sum = 0.0;
-    for (int n = 0; n < 40; ++n) {
-        sum += p / (2.0 * n + 1.0);
-        p *= s * s;
-    }
-    return 2.0 * sum;
-}
-// the binary32 value with bits b, for b in [0x3F000000, 0x40000000)
-constexpr double f32_of_bits(uint32_t b)
-{
-    return b < 0x3F800000u ? 0.5 * (1.0 + (double)(b - 0x3F000000u) / 8388608.0)
-                           : 1.0 + (double)(b - 0x3F800000u) / 8388608.0;
-}
-constexpr Tables make_tables()
-{
-    Tables T{};
-    const int one = (int)((0x3F800000u - kSqrtHalfBits) >> 18);  // the cell holding 1
-    for (int j = 0; j < 32; ++j) {
-        if (j == one) {
-            T.lg[j].r = 1.0f;
-            T.lg[j].l2r = 0.0f;
-            continue;
-        }
-        const double lo = f32_of_bits(kSqrtHalfBits + ((uint32_t)j << 18));
-        const double hi = f32_of_bits(kSqrtHalfBits + ((uint32_t)(j + 1) << 18));
-        const float r = (float)(2.0 / (lo + hi));
-        T.lg[j].r = r;
-        T.lg[j].l2r = -2.0f * (float)(-series_log((double)r));  // -2 x (the binary32 -ln r_j)
-    }
-    return T;
-}
-
 }  // namespace bm
-
-// one copy per translation unit, read through the read-only cache
-static __device__ const bm::Tables kBM = bm::make_tables();
 
 // 1/sqrt(x) of a positive normal x: rsqrtf without its steps for subnormals (the same
 // approximation and bits)
@@ -165,38 +118,39 @@ __device__ __forceinline__ float rsqrt_normal(float x)
 // Blackwell's packed FP32 registers): lane l turns word w[l] into
 // g0 = r cos 2 pi v, g1 = r sin 2 pi v (u, v and r as above).
 // SCALED: r is multiplied by sc first (lane-wise), so the outputs come scaled.
-// The integer steps, table loads and the reciprocal square root run per lane;
+// The integer steps and the reciprocal square root run per lane;
 // every FP32 step is one lane-generic operation, so a word gets the same bits
 // in either lane type.
 template <class V, bool SCALED = false>
 __device__ __forceinline__ void bm_eval(const uint32_t *w, V sc, V &g0, V &g1)
 {
     constexpr int L = V::L;
-    float f[L], lr[L], l2r[L], eb[L], xm[L];
+    float f[L], eb[L], xm[L];
     uint32_t half[L];
 #pragma unroll
     for (int l = 0; l < L; ++l) {
         const float fn = __uint2float_rn((w[l] >> 11) | 1u);  // 2k+1 < 2^21, exact
         const int bits = __float_as_int(fn);
-        const int t = bits - (int)bm::kSqrtHalfBits;
-        const int e = t >> 23;                                // 2k+1 = 2^e f
+        const int e = (bits - (int)bm::kSqrtHalfBits) >> 23;  // 2k+1 = 2^e f
         f[l] = __int_as_float(bits - (e << 23));              // f in [sqrt(1/2), sqrt(2))
-        const float2 C = __ldg(reinterpret_cast<const float2 *>(&kBM.lg[(t >> 18) & 31]));  // (r_j, 2 ln r_j)
-        lr[l] = C.x;
-        l2r[l] = C.y;
         eb[l] = __int_as_float(0x4B400000 + e - 21);          // 1.5 2^23 + (e - 21), exact
         const uint32_t n = w[l] + 1024u;                      // v + 1/4 in units of 2^-12, less 1/2
         xm[l] = __uint_as_float(0x4B000000u | (n & 2047u));   // 2^23 + (n mod 2^11), exact
         half[l] = n << 20;                                    // sign bit: the half turn
     }
-    // -2 ln u = -2 (e - 21) ln 2 + 2 ln r_j - 2 ln(1 + d)
-    const V d = vfma(vmake<V>(f), vmake<V>(lr), V::bc(-1.0f));
-    V p = vfma(d, V::bc(-0.4f), V::bc(0.5f));  // -2 x the series of ln(1 + d)/d, Horner form
-    p = vfma(d, p, V::bc(-2.0f / 3.0f));
-    p = vfma(d, p, V::bc(1.0f));
+    // -2 ln u = -2 (e - 21) ln 2 - 2 ln(1 + d), the first product exact but for the rest of ln 2
+    const V d = vmake<V>(f) - V::bc(1.0f);
+    V p = vfma(d, V::bc(0.14902374148368835f), V::bc(-0.25613221526145935f));
+    p = vfma(d, p, V::bc(0.26532062888145447f));
+    p = vfma(d, p, V::bc(-0.2839930057525635f));
+    p = vfma(d, p, V::bc(0.332167387008667f));
+    p = vfma(d, p, V::bc(-0.4000187814235687f));
+    p = vfma(d, p, V::bc(0.500031590461731f));
+    p = vfma(d, p, V::bc(-0.6666669249534607f));
+    p = vfma(d, p, V::bc(0.9999997615814209f));
     p = vfma(d, p, V::bc(-2.0f));
     const V em = vmake<V>(eb) - V::bc(12582912.0f);       // e - 21, exact
-    const V e2 = vfma(d, p, vfma(em, V::bc(-2.0f * 0.693147180559945f), vmake<V>(l2r)));  // >= 9.5e-7
+    const V e2 = vfma(em, V::bc(9.574836212777882e-07f), vfma(d, p, em * V::bc(-1.3862953186035156f)));  // >= 9.5e-7
     float rs[L];
 #pragma unroll
     for (int l = 0; l < L; ++l)

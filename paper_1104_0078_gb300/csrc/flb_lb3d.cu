@@ -12,11 +12,11 @@
 // Indices are 32-bit (N and the padded planes are < 2^31); population plane i
 // of N sites starts at fin + i*N.  The plain kernel runs seven 128-thread blocks
 // per SM (72 registers, no spills; six blocks at 80 registers and eight at 64,
-// spilling, measured slower): 3.71 ms at 512^3, 5.5 TB/s on its 152 B/site.  It is bound by
+// spilling, measured slower): 3.62 ms at 512^3, 5.6 TB/s on its 152 B/site.  It is bound by
 // instruction issue and by the L1's wavefronts together: 4.01 ms before sites away from
 // the box's y and z faces took one index for all planes (of pre-shifted plane
 // pointers) and the pair of sites the planes of mu between them once (3.82), and
-// before the angle of Box-Muller came from polynomials instead of gathers (3.71).
+// before Box-Muller came from polynomials instead of table gathers (3.62).
 // Marching z with the populations fetched one pair of planes ahead by cp.async took
 // 4.69 ms: latency is not what bounds it.  Noise order: bulk, 3c_x^2-c^2, c_y^2-c_z^2,
 // xy, yz, zx, three c^2 c_a ghosts, three c_a(c_b^2-c_g^2) ghosts, c^4,
