@@ -108,14 +108,14 @@ __device__ __forceinline__ void form_mu(const Psi3Args &a, int x0, int y0, int z
 // The output of a stage at (x, y, z) from the increment D and the noise increment
 // eta, pv the stage input there (Sec. V; operations and order as in
 // psi3_fv_tma_block).
+// e: the accumulator E there (later stages).
 template <bool FIRST>
-__device__ __forceinline__ void stage_out(const Psi3Args &a, int x, int y, int z, F1 pv, F1 D, F1 eta)
+__device__ __forceinline__ void stage_out(const Psi3Args &a, int x, int y, int z, F1 pv, F1 e, F1 D, F1 eta)
 {
     const Geom &g = a.g;
     const int si = x + g.nx * (y + g.ny * z);
     F1 out;
     if (!FIRST) {
-        const F1 e{a.E[si]};
         if (a.rk4 == 4) {
             out = vfma(D, 1.f / 6.f, e);
         } else if (a.rk4) {  // stages 2 and 3
@@ -212,6 +212,12 @@ __device__ __forceinline__ void cube_fv_stage(const Psi3Args &a, const float *mu
     constexpr int JN = (CZ + 2) * CP1;
     const Geom &g = a.g;
     const int nzt = min(CZ, g.nz - z0);
+    const int tx = threadIdx.x % CX, ty = (threadIdx.x / CX) % CY, zh = (threadIdx.x / (CX * CY)) * (CZ / 2);
+    const bool act = x0 + tx < g.nx && y0 + ty < g.ny && zh < nzt;
+    float e_pre[CZ / 2];  // a later stage's accumulator, in flight meanwhile
+#pragma unroll
+    for (int j = 0; j < CZ / 2; ++j)
+        e_pre[j] = !FIRST && act ? a.E[x0 + tx + g.nx * (y0 + ty + g.ny * min(z0 + zh + j, g.nz - 1))] : 0.f;
     if (!MU_IN) {
         form_mu<T, 2, W>(a, x0, y0, z0, nzt, smu);
         __syncthreads();
@@ -284,9 +290,8 @@ __device__ __forceinline__ void cube_fv_stage(const Psi3Args &a, const float *mu
     }
     __syncthreads();
     {  // output columns, planes zh .. zh + CZ/2 - 1 of the tile
-        const int tx = threadIdx.x % CX, ty = (threadIdx.x / CX) % CY, zh = (threadIdx.x / (CX * CY)) * (CZ / 2);
         const int x = x0 + tx, y = y0 + ty;
-        if (x >= g.nx || y >= g.ny || zh >= nzt) return;
+        if (!act) return;
         constexpr float DIV = Q15 ? 1.0f / 24.0f : 1.0f / 12.0f;
         int c = (tx + 1) + CW1 * (ty + 1) + CP1 * zh;
         Div3 d0, d1, n0, n1;
@@ -313,7 +318,7 @@ __device__ __forceinline__ void cube_fv_stage(const Psi3Args &a, const float *mu
             d1 = d2;
             if (zh + j >= nzt) break;
             const F1 pv{FIRST ? __ldg(a.psi + g.pidx32(x, y, z)) : 0.f};
-            stage_out<FIRST>(a, x, y, z, pv, D, eta);
+            stage_out<FIRST>(a, x, y, z, pv, F1{e_pre[j]}, D, eta);
         }
     }
 }
@@ -375,11 +380,16 @@ __global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
         }
     }
     pdl_wait();
-    if (!MU_IN) form_mu<T, 1, W>(a, x0, y0, z0, nzt, smu);
-    if (NOISE || !MU_IN) __syncthreads();
     const int tx = threadIdx.x % CX, ty = (threadIdx.x / CX) % CY, zh = (threadIdx.x / (CX * CY)) * (CZ / 2);
     const int x = x0 + tx, y = y0 + ty;
-    if (x >= g.nx || y >= g.ny || zh >= nzt) return;
+    const bool act = x < g.nx && y < g.ny && zh < nzt;
+    float e_pre[CZ / 2];  // a later stage's accumulator, in flight while mu is formed
+#pragma unroll
+    for (int j = 0; j < CZ / 2; ++j)
+        e_pre[j] = !FIRST && act ? a.E[x + g.nx * (y + g.ny * min(z0 + zh + j, g.nz - 1))] : 0.f;
+    if (!MU_IN) form_mu<T, 1, W>(a, x0, y0, z0, nzt, smu);
+    if (NOISE || !MU_IN) __syncthreads();
+    if (!act) return;
     const int Y = MU_IN ? g.px : CW1, Z = MU_IN ? g.px * g.py : CP1;
     const float *m = MU_IN ? ca.mu + g.pidx32(x, y, z0 + zh - 1) : smu + (tx + 1) + CW1 * (ty + 1) + CP1 * zh;
     Plane3 q0 = plane3<MU_IN>(m, Y), q1 = plane3<MU_IN>(m + Z, Y);
@@ -414,8 +424,8 @@ __global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
                     eta += sZ[l * ZN + c - kCubeL[l][0] - CW1 * kCubeL[l][1] - CP1 * kCubeL[l][2]] - sZ[l * ZN + c];
             }
         }
-        const F1 pv{FIRST ? __ldg(a.psi + pi) : 0.f};
-        stage_out<FIRST>(a, x, y, z, pv, F1{D}, F1{eta});
+        const F1 own{FIRST ? __ldg(a.psi + pi) : 0.f};
+        stage_out<FIRST>(a, x, y, z, own, F1{e_pre[j]}, F1{D}, F1{eta});
     }
 }
 

@@ -14,11 +14,12 @@
 //
 // What bounds them: the populations go through HBM twice read and once written
 // (108 B/site of the about 150 a step moves), but a large box is bound by
-// instruction issue (65-73% of the slots; 480 instructions per site in lb2_kernel,
-// 705 in the first stage, 235 in the second): a 2048^2 FD Heun step takes 233 us
-// (82 + 107 + 54 us; 383 us with one thread per site and one launch per field).  A small
+// instruction issue and L1 latency (65-73% of the slots; 480 instructions per site in
+// lb2_kernel, 705 in the first stage, 235 in the second): a 2048^2 FD Heun step takes
+// 213 us (383 us with one thread per site and one launch per field; 226 with a later
+// stage's velocities and accumulator loaded where they are used).  A small
 // one is bound by latency, so what counts is the number of launches and what each
-// has to wait for: 64^2 takes 7.9 us a step (28.8 us with eight launches; 15.7 us
+// has to wait for: 64^2 takes 7.6 us a step (28.8 us with eight launches; 15.7 us
 // with these three before programmatic dependent launch, with the noise drawn ahead of the
 // wait and the populations in flight while mu is formed).
 #include "flb_internal.cuh"
@@ -344,6 +345,24 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
         if (point(threadIdx.x, lx, ly))
             pull9((const T *)a.f, g.n, g.nx, g.ny, wrapi(x0 + lx, g.nx), wrapi(y0 + ly, g.ny), f0);
     }
+    // a later stage's velocities and accumulator, in flight while mu is formed
+    constexpr int J0 = (TX * TY + NT - 1) / NT;
+    float uxy[J1][2], e_pre[J0];
+    if (!FIRST) {
+#pragma unroll
+        for (int j = 0; j < J1; ++j) {
+            int lx, ly;
+            const bool in = advect && point((int)threadIdx.x + j * NT, lx, ly);
+            const int o = in ? (x0 + lx + GX) + g.px * (y0 + ly + GY) : 0;
+            uxy[j][0] = in ? __ldg(a.u + o) : 0.f;
+            uxy[j][1] = in ? __ldg(a.u + g.pn + o) : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < J0; ++j) {
+            const int k = (int)threadIdx.x + j * NT, x = x0 + k % TX, y = y0 + k / TX;
+            e_pre[j] = k < TX * TY && x < g.nx && y < g.ny ? a.E[x + g.nx * y] : 0.f;
+        }
+    }
     load_psi2<TX, TY, PH, NT>(g, a.psi, x0, y0, sps);
     __syncthreads();
     form_mu2<TX, TY, MH, NT>(sps, smu, a.A, a.B, a.K, a.lw);
@@ -376,10 +395,9 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
                 store_padded(a.u, g, x, y, 0, ux, 1);
                 store_padded(a.u + g.pn, g, x, y, 0, uy, 1);
             }
-        } else if (advect) {
-            const int o = (x + GX) + g.px * (y + GY);
-            ux = __ldg(a.u + o);
-            uy = __ldg(a.u + g.pn + o);
+        } else {
+            ux = uxy[j][0];
+            uy = uxy[j][1];
         }
         const float px = advect ? ux * ps : 0.f, py = advect ? uy * ps : 0.f;
         if (FV) {
@@ -402,7 +420,7 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
         return (1.f / 12.f) * (4.f * ax + dg);
     };
 #pragma unroll
-    for (int j = 0; j < (TX * TY + NT - 1) / NT; ++j) {
+    for (int j = 0; j < J0; ++j) {
         const int k = (int)threadIdx.x + j * NT;
         const int tx = k % TX, ty = k / TX, x = x0 + tx, y = y0 + ty;
         if (k >= TX * TY || x >= g.nx || y >= g.ny) continue;
@@ -434,16 +452,16 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
                 a.E[site] = ps + eta + D * (1.f / 6.f);
                 a.eta[site] = eta;
             } else if (a.stage == 4) {
-                out = a.E[site] + D * (1.f / 6.f);
+                out = e_pre[j] + D * (1.f / 6.f);
             } else {
                 out = a.base[(x + GX) + g.px * (y + GY)] + (a.stage == 2 ? 0.5f : 1.f) * (D + a.eta[site]);
-                a.E[site] += D * (1.f / 3.f);
+                a.E[site] = e_pre[j] + D * (1.f / 3.f);
             }
         } else if (FIRST) {
             out = ps + D + eta;
             if (a.integrator == FLB_HEUN) a.E[site] = ps + 0.5f * D + eta;
         } else {
-            out = a.E[site] + 0.5f * D;
+            out = e_pre[j] + 0.5f * D;
         }
         store_padded(a.out, g, x, y, 0, out, 3);
     }
