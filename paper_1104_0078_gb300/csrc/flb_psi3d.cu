@@ -34,7 +34,7 @@ struct TmaArgs {
 // 256 threads, each on point pairs (y, y + H/2) of every region in packed FP32 (F2)
 using StageV = F2;
 template <int STAGE, bool NOISE, bool RK, bool MU_IN, bool Q15 = false>
-__global__ void __launch_bounds__(stage_threads<StageV>(), 2) psi3_fv_tma_kernel(const __grid_constant__ CUtensorMap psi_map,
+__global__ void __launch_bounds__(block_threads<StageV, MU_IN>(), 2) psi3_fv_tma_kernel(const __grid_constant__ CUtensorMap psi_map,
                                                                    const __grid_constant__ CUtensorMap u_map,
                                                                    const __grid_constant__ CUtensorMap mu_map,
                                                                    const TmaArgs ta)
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(stage_threads<StageV>(), 2) psi3_fv_tma_kernel
 // batched: block b of the launch works on L.psi[b]; MU_IN: stage 1 reads mu of
 // psi^n from the replica's mu field (every replica's step formed it)
 template <int STAGE, bool NOISE, bool MU_IN = false, bool Q15 = false>
-__global__ void __launch_bounds__(stage_threads<StageV>(), 2) psi3_fv_tma_batch_kernel(const BatchLists L)
+__global__ void __launch_bounds__(block_threads<StageV, MU_IN>(), 2) psi3_fv_tma_batch_kernel(const BatchLists L)
 {
     extern __shared__ __align__(1024) float tsmem[];
     __shared__ Psi3Args sa;
@@ -74,18 +74,19 @@ static cudaError_t batch_psi(const BatchLists &L, bool heun, bool noise, bool mu
     const size_t sm = sizeof(float) * (size_t)fv_smem_floats<StageV>();
     const size_t smm = sizeof(float) * (size_t)fv_mu_smem_floats<StageV>();
     const size_t nb = sizeof(float) * FV_NOISE_FLOATS;
-    auto go = [&](auto kernel, size_t bytes) {
+    auto go = [&](auto kernel, size_t bytes, int nt) {
         cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (r != cudaSuccess) return r;
-        kernel<<<L.npsi, stage_threads<StageV>(), bytes, st>>>(L);
+        kernel<<<L.npsi, nt, bytes, st>>>(L);
         return cudaGetLastError();
     };
-    cudaError_t e = mu_in ? (noise ? go(psi3_fv_tma_batch_kernel<1, true, true, Q15>, smm + nb)
-                                   : go(psi3_fv_tma_batch_kernel<1, false, true, Q15>, smm))
-                          : (noise ? go(psi3_fv_tma_batch_kernel<1, true, false, Q15>, sm + nb)
-                                   : go(psi3_fv_tma_batch_kernel<1, false, false, Q15>, sm));
+    constexpr int n1 = block_threads<StageV, true>(), nn = block_threads<StageV, false>();
+    cudaError_t e = mu_in ? (noise ? go(psi3_fv_tma_batch_kernel<1, true, true, Q15>, smm + nb, n1)
+                                   : go(psi3_fv_tma_batch_kernel<1, false, true, Q15>, smm, n1))
+                          : (noise ? go(psi3_fv_tma_batch_kernel<1, true, false, Q15>, sm + nb, nn)
+                                   : go(psi3_fv_tma_batch_kernel<1, false, false, Q15>, sm, nn));
     if (e != cudaSuccess || !heun) return e;
-    return go(psi3_fv_tma_batch_kernel<2, false, false, Q15>, sm);
+    return go(psi3_fv_tma_batch_kernel<2, false, false, Q15>, sm, nn);
 }
 
 cudaError_t launch_batch_psi(const BatchLists &L, bool heun, bool noise, bool mu_in, bool q15, cudaStream_t st)
@@ -163,7 +164,7 @@ static cudaError_t launch_fv_tma(const Psi3Args &a, int q, int stage, bool noise
     auto go = [&](auto kernel, size_t bytes) {
         cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (r != cudaSuccess) return r;
-        return launch_pdl(kernel, grid, stage_threads<StageV>(), bytes, st, PDL_BLOCKS, pm, um, mm, ta);
+        return launch_pdl(kernel, grid, mu ? block_threads<StageV, true>() : block_threads<StageV, false>(), bytes, st, PDL_BLOCKS, pm, um, mm, ta);
     };
     const size_t smn = sm + sizeof(float) * FV_NOISE_FLOATS;
     const size_t smm = sizeof(float) * (size_t)fv_mu_smem_floats<StageV>(), smmn = smm + sizeof(float) * FV_NOISE_FLOATS;

@@ -109,10 +109,17 @@ __device__ __forceinline__ V mu_so_v(float A, float B, float k22, V ps, V n1, V 
     return vfma(l22, -k22, vfma((ps * ps) * B, ps, ps * A));
 }
 
-// Threads of a stage block: one output point per thread (F1: 512), or a pair of
+// Threads with output points: one point per thread (F1: 512), or a pair of
 // output rows y and y + TY/2 per thread in the lanes of packed FP32 (F2: 256).
 template <class V>
 __host__ __device__ constexpr int stage_threads() { return V::L == 1 ? PS_NT : PS_NT / 2; }
+// Threads of a block: with mu given (MU_IN) the flux region's 306 row pairs set the
+// pace, and 320 threads take one each: with 256, two warps worked 50 of them, noise and
+// all, in a second round while the others waited at the barrier (512^3 stage 1 2.27 ms, 2.10 with
+// 320; 384 threads 2.26).  Where the block forms mu (360 pairs) 320 and 384 threads
+// measured level with 256 (stage 2 1.42, 1.44, 1.42 ms).
+template <class V, bool MU_IN>
+__host__ __device__ constexpr int block_threads() { return V::L == 2 && MU_IN ? 320 : stage_threads<V>(); }
 
 // One block (tile bx, by; z chunk bz).  psi_map / u_map: tensor maps of the stage
 // input psi and of the velocity (kernel parameters or global memory); tsmem: the
@@ -163,7 +170,7 @@ __device__ __forceinline__ void psi3_fv_tma_block(const CUtensorMap *psi_map, co
                                                   float *tsmem, const CUtensorMap *mu_map = nullptr)
 {
     static_assert(!MU_IN || STAGE == 1, "mu of psi^n is the input of stage 1 only");
-    constexpr int L = V::L, NT = stage_threads<V>();
+    constexpr int L = V::L, NT = block_threads<V, MU_IN>(), NTO = stage_threads<V>();  // NTO: threads with output points
     constexpr int LO2 = (H2Y / 2) * TB_X, LO1 = (H1Y / 2) * TB_X, LO0 = (PS_TY / 2) * TB_X;  // lane 1's offsets
     constexpr int LR2 = L == 1 ? 0 : LO2, LR1 = L == 1 ? 0 : LO1, LR0 = L == 1 ? 0 : LO0;
     constexpr int HH2 = H2Y / L, HH1 = H1Y / L;  // rows of the mu and flux regions per lane
@@ -190,7 +197,7 @@ __device__ __forceinline__ void psi3_fv_tma_block(const CUtensorMap *psi_map, co
 #pragma unroll
     for (int l = 0; l < L; ++l) {
         yl[l] = y0 + ty + l * (PS_TY / 2);
-        act[l] = x < g.nx && yl[l] < g.ny;
+        act[l] = threadIdx.x < NTO && x < g.nx && yl[l] < g.ny;
         // the output column has no periodic image within 3 cells in x and y: its
         // interior planes are stored with one plain store
         inner[l] = x >= 3 && x < g.nx - 3 && yl[l] >= 3 && yl[l] < g.ny - 3;
@@ -217,8 +224,10 @@ __device__ __forceinline__ void psi3_fv_tma_block(const CUtensorMap *psi_map, co
 #pragma unroll
     for (int j = 0; j < SS1; ++j) {
         int lx, ly;
-        region_point(threadIdx.x + j * NT, H1X, HH1, lx, ly);
-        const bool ok = threadIdx.x + j * NT < H1X * HH1;
+        // the second round starts half a block on: the warps that have two mu pairs get one here
+        const int k = j == 0 ? threadIdx.x : (threadIdx.x + NT / 2) % NT + j * NT;
+        region_point(k, H1X, HH1, lx, ly);
+        const bool ok = k < H1X * HH1;
         p1[j] = ok ? (lx + 3) + TB_X * (ly + 2) : -1;
 #pragma unroll
         for (int l = 0; l < L; ++l)
@@ -441,7 +450,7 @@ __device__ __forceinline__ void psi3_fv_tma_block(const CUtensorMap *psi_map, co
         // (C) flux partials of plane q = p-2 SK (complete since the last barrier) at
         // the tile point; the output of plane q-1 completes
         const int q = p - 2 * SK;
-        if (q >= z0 - 1) {
+        if (q >= z0 - 1 && threadIdx.x < NTO) {
             const int c = (tx + 4) + TB_X * (ty + 1);  // the tile point (lane 0) in the flux plane
             const float *Jx = sJ + (q & 1) * 3 * TJ_N, *Jy = Jx + TJ_N, *Jz = Jy + TJ_N;
             const V hxy = (lds_v<V>(Jx, c + 1, LR0) - lds_v<V>(Jx, c - 1, LR0)) +
