@@ -553,6 +553,9 @@ LBArgs lb_args(const Rep &r, float *psi_n)
     return la;
 }
 
+// Noise of the psi equation: 0 none, 1, or 2 by the tables (FP16 storage: bm_eval).
+int noise_kind(const flb_params &p) { return p.kT > 0 && p.M > 0 ? (p.storage == FLB_F16_DEV ? 2 : 1) : 0; }
+
 // The Runge-Kutta stages of psi (3D) for the current step of replica r, advected
 // by the velocity in r.u.  They write only step scratch (psi*, E) and the other
 // psi buffer, so repeating them leaves the state unchanged (the autotuner relies
@@ -566,7 +569,7 @@ int launch_psi_stages(flb_handle *h, Rep &r)
     const LapW *lw = app_a_weights(r, lwv);
     float *psi_n = r.psi[r.pcur], *psi_np1 = r.psi[r.pcur ^ 1];
     const float *mu_n = (p.coupling & FLB_COUPLE_FORCE) && p.force_grad != FLB_FORCE_STRESS ? r.mu : nullptr;
-    const bool noisy = p.kT > 0 && p.M > 0;
+    const int noise = noise_kind(p);
     const bool heun = p.integrator == FLB_HEUN;
     const int advect = (p.coupling & FLB_COUPLE_ADVECT) ? 1 : 0;
     const PhiloxKey key = philox_key(p.seed);
@@ -576,21 +579,21 @@ int launch_psi_stages(flb_handle *h, Rep &r)
         const float *in[4] = {psi_n, r.psis, psi_np1, r.psis};
         float *out[4] = {r.psis, psi_np1, r.psis, psi_np1};
         for (int s = 0; s < 4; ++s)
-            FLB_TRY(launch_psi3(r.g, p.psi_scheme, r.q, s == 0 ? 1 : 2, s == 0 && noisy, in[s], r.u, out[s], r.E,
+            FLB_TRY(launch_psi3(r.g, p.psi_scheme, r.q, s == 0 ? 1 : 2, s == 0 ? noise : 0, in[s], r.u, out[s], r.E,
                                 (float)p.A, (float)p.B, (float)p.K, (float)p.M, (float)p.kT, advect, 0, key, r.step,
                                 zc, s + 1, psi_n, r.Dn, s == 0 ? mu_n : nullptr, h->status, st, lw));
         return FLB_OK;
     }
     if (r.fused && heun) {  // both stages in one launch (flb_set_psi_fused)
         FLB_TRY(launch_psi3_heun1(r.g, p.psi_scheme, psi_n, r.u, psi_np1, (float)p.A, (float)p.B, (float)p.K,
-                                  (float)p.M, (float)p.kT, advect, noisy, key, r.step, r.zc, st));
+                                  (float)p.M, (float)p.kT, advect, noise, key, r.step, r.zc, st));
         return FLB_OK;
     }
-    FLB_TRY(launch_psi3(r.g, p.psi_scheme, r.q, 1, noisy, psi_n, r.u, heun ? r.psis : psi_np1, r.E, (float)p.A,
+    FLB_TRY(launch_psi3(r.g, p.psi_scheme, r.q, 1, noise, psi_n, r.u, heun ? r.psis : psi_np1, r.E, (float)p.A,
                         (float)p.B, (float)p.K, (float)p.M, (float)p.kT, advect, heun ? 1 : 0, key, r.step, zc, 0,
                         nullptr, nullptr, mu_n, h->status, st, lw));
     if (heun)
-        FLB_TRY(launch_psi3(r.g, p.psi_scheme, r.q, 2, false, r.psis, r.u, psi_np1, r.E, (float)p.A, (float)p.B,
+        FLB_TRY(launch_psi3(r.g, p.psi_scheme, r.q, 2, 0, r.psis, r.u, psi_np1, r.E, (float)p.A, (float)p.B,
                             (float)p.K, (float)p.M, (float)p.kT, advect, 1, key, r.step, zc, 0, nullptr, nullptr,
                             nullptr, h->status, st, lw));
     return FLB_OK;
@@ -958,11 +961,12 @@ bool batch_mu_in(const flb_handle *h)
 int batch_capture(flb_handle *h)
 {
     if (h->b_exec) return FLB_OK;
-    bool ghost = false, force = false, noise = false;
+    bool ghost = false, force = false;
+    int noise = 0;
     for (const Rep &r : h->reps) {
         ghost |= r.gamma_g != 0.f;
         force |= (r.p.coupling & FLB_COUPLE_FORCE) != 0;
-        noise |= r.p.kT > 0 && r.p.M > 0;
+        noise = std::max(noise, noise_kind(r.p));
     }
     const flb_params &p0 = h->reps[0].p;
     const BatchLists L = batch_lists(h);
@@ -1701,11 +1705,11 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
     if ((h->mode == FLB_MODE_BATCHED || h->mode == FLB_MODE_PERSISTENT) && batch_supported(h)) {
         // one value for every replica, timed on the batched psi launches
         std::string all;
-        bool noise = false;
+        int noise = 0;
         int nzmax = 1;
         for (const Rep &r : h->reps) {
             all += rep_key(r) + ";";
-            noise |= r.p.kT > 0 && r.p.M > 0;
+            noise = std::max(noise, noise_kind(r.p));
             nzmax = std::max(nzmax, r.g.nz);
         }
         uint64_t hash = 1469598103934665603ull;  // FNV-1a over the replica keys

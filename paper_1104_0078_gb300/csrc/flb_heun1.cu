@@ -111,7 +111,7 @@ struct Heun1Args {
     int64_t step;
 };
 
-template <bool NOISE>
+template <int NOISE>
 __global__ void __launch_bounds__(HT_NT, 1) psi3_fv_heun1_kernel(const Heun1Args a)
 {
     extern __shared__ __align__(16) float hsm[];
@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(HT_NT, 1) psi3_fv_heun1_kernel(const Heun1Args
                 J[2 * Reg<4>::N + k] = mg * gz - u4[j][2] * pv;
                 if (NOISE) {
                     float Gn[4];
-                    normals<2, false, true>(a.key, a.step, (uint32_t)(id4[j] + zid), 1u, 0u, Gn, sdx);
+                    normals<2, false, true, NOISE == 2>(a.key, a.step, (uint32_t)(id4[j] + zid), 1u, 0u, Gn, sdx);
                     X[k] = Gn[0];
                     X[Reg<4>::N + k] = Gn[1];
                     X[2 * Reg<4>::N + k] = Gn[2];
@@ -364,7 +364,7 @@ __device__ __forceinline__ float adv_at(const float *Pm, const float *P0, const 
     return -0.5f * adv;
 }
 
-template <bool NOISE>
+template <int NOISE>
 __global__ void __launch_bounds__(HT_NT, 1) psi3_fd_heun1_kernel(const Heun1Args a)
 {
     static_assert(Reg<0>::S == 1, "one output point per thread");
@@ -453,8 +453,8 @@ __global__ void __launch_bounds__(HT_NT, 1) psi3_fd_heun1_kernel(const Heun1Args
                 if (NOISE) {
                     const uint32_t sid = (uint32_t)(id3[j] + zid);
                     float G[14];  // normals 0-12: block 0, and block 1's first three words
-                    normals<4>(a.key, a.step, sid, 1u, 0u, G);
-                    normals<3>(a.key, a.step, sid, 1u, 1u, G + 8);
+                    normals<4, false, false, NOISE == 2>(a.key, a.step, sid, 1u, 0u, G);
+                    normals<3, false, false, NOISE == 2>(a.key, a.step, sid, 1u, 1u, G + 8);
 #pragma unroll
                     for (int l = 0; l < 13; ++l) sZ[l * Reg<3>::N + k] = (l < 3 ? s1 : (l < 9 ? s2 : s3)) * G[l];
                 }
@@ -543,7 +543,7 @@ __global__ void __launch_bounds__(HT_NT, 1) psi3_fd_heun1_kernel(const Heun1Args
 size_t psi3_heun1_smem_bytes() { return sizeof(float) * (size_t)H1_SMEM_FLOATS; }
 
 cudaError_t launch_psi3_heun1(const Geom &g, int scheme, const float *psi, const float *u, float *out, float A, float B,
-                              float K, float M, float kT, int advect, bool noise, const PhiloxKey &key, int64_t step,
+                              float K, float M, float kT, int advect, int noise, const PhiloxKey &key, int64_t step,
                               int zc, cudaStream_t st)
 {
     Heun1Args a;
@@ -561,27 +561,22 @@ cudaError_t launch_psi3_heun1(const Geom &g, int scheme, const float *psi, const
     a.key = key;
     a.step = step;
     const dim3 grid((g.nx + HT_X - 1) / HT_X, (g.ny + HT_Y - 1) / HT_Y, (g.nz + zc - 1) / zc);
-    cudaError_t e;
+    auto go = [&](auto k, size_t smem) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        k<<<grid, HT_NT, smem, st>>>(a);
+        return cudaGetLastError();
+    };
     if (scheme == FLB_FD) {
         const size_t smem = sizeof(float) * (size_t)FD_SMEM_FLOATS;
-        const void *k = noise ? (const void *)psi3_fd_heun1_kernel<true> : (const void *)psi3_fd_heun1_kernel<false>;
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        if (noise) psi3_fd_heun1_kernel<true><<<grid, HT_NT, smem, st>>>(a);
-        else psi3_fd_heun1_kernel<false><<<grid, HT_NT, smem, st>>>(a);
-        return cudaGetLastError();
+        return noise == 2 ? go(psi3_fd_heun1_kernel<2>, smem)
+               : noise    ? go(psi3_fd_heun1_kernel<1>, smem)
+                          : go(psi3_fd_heun1_kernel<0>, smem);
     }
     const size_t smem = psi3_heun1_smem_bytes();
-    if (noise) {
-        e = cudaFuncSetAttribute(psi3_fv_heun1_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        psi3_fv_heun1_kernel<true><<<grid, HT_NT, smem, st>>>(a);
-    } else {
-        e = cudaFuncSetAttribute(psi3_fv_heun1_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        psi3_fv_heun1_kernel<false><<<grid, HT_NT, smem, st>>>(a);
-    }
-    return cudaGetLastError();
+    return noise == 2 ? go(psi3_fv_heun1_kernel<2>, smem)
+           : noise    ? go(psi3_fv_heun1_kernel<1>, smem)
+                      : go(psi3_fv_heun1_kernel<0>, smem);
 }
 
 }  // namespace flb

@@ -36,7 +36,7 @@ __global__ void eq_pop_kernel(Geom g, int q, float mun, PhiloxKey key, T *f)
     if (s >= g.n) return;
     float G[24];
     const int nb = (q + 7) / 8;
-    for (int b = 0; b < nb; ++b) normals<4>(key, 0, (uint32_t)s, 3u, (uint32_t)b, G + 8 * b);
+    for (int b = 0; b < nb; ++b) normals<4, false, false, sizeof(T) == 2>(key, 0, (uint32_t)s, 3u, (uint32_t)b, G + 8 * b);
     for (int i = 0; i < q; ++i) {
         const float v = sqrtf(mun * lattice_weight(q, i)) * G[i];
         if (sizeof(T) == 2) reinterpret_cast<__half *>(f)[(long long)i * g.n + s] = __float2half_rn(v);
@@ -45,6 +45,7 @@ __global__ void eq_pop_kernel(Geom g, int q, float mun, PhiloxKey key, T *f)
 }
 
 // X(q) for every mode of the FFT grid
+template <bool TABLE>
 __global__ void eq_modes_kernel(Geom g, LapW lw, double kT, double A, double K, PhiloxKey key, float2 *X)
 {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -58,7 +59,7 @@ __global__ void eq_modes_kernel(Geom g, LapW lw, double kT, double A, double K, 
     else
         L = lw.c0 + lw.c1 * 2.0 * (cx + cy) + lw.c2 * 4.0 * cx * cy;
     float Gq[2];
-    normals<1>(key, 0, (uint32_t)t, 4u, 0u, Gq);
+    normals<1, false, false, TABLE>(key, 0, (uint32_t)t, 4u, 0u, Gq);
     const float amp = t == 0 ? 0.f : (float)sqrt(kT / (A - K * L) / (double)g.n);
     X[t] = make_float2(amp * Gq[0], amp * Gq[1]);
 }
@@ -115,7 +116,8 @@ cudaError_t launch_equilibrium_start(const Geom &g, int q, int storage, const La
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     float2 *X = (float2 *)spare, *Y = X + g.n;  // 16 bytes per site of the spare buffer
-    eq_modes_kernel<<<nb, bs, 0, st>>>(g, lw, kT, A, K, key, X);
+    if (storage == FLB_F16_DEV) eq_modes_kernel<true><<<nb, bs, 0, st>>>(g, lw, kT, A, K, key, X);
+    else eq_modes_kernel<false><<<nb, bs, 0, st>>>(g, lw, kT, A, K, key, X);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const long long N = g.n, sxy = (long long)g.nx * g.ny;
     idft_axis_kernel<<<nb, bs, 0, st>>>(N, g.nx, 1, X, Y);

@@ -99,11 +99,104 @@ __device__ __forceinline__ u32x4 philox4x32_10_r0(u32x4 c, uint32_t a, uint32_t 
 // collide-stream 3.82 ms with both tables, 3.71 with the logarithm's, 3.62 with
 // none; the FD step at 160^3 467, 441 and 427 us.  (Fewer integer steps, funnel shifts
 // in place of the conversion and a mask: 3.63 ms, no gain.)
+// Runs with populations stored as FP16 deviations draw by the tables (bm_eval_table
+// below) in every kernel: a last bit of a normal moves roundings to 16 bits, and these
+// psi by up to 4e-4 of itself in 200 steps, where FP32 runs stay within 2e-6.  So an FP16 run
+// takes the same course, bit for bit, by either set of kernels:
+//  * ln u by the table-driven method of P. T. P. Tang (ACM TOMS 16(4), 1990): the bits
+//    of f select one of 32 cells; ln f = -ln r_j + ln(1 + d) with d = f r_j - 1
+//    formed by one FMA (|d| < 1/64) and ln(1 + d) by its series to d^5 (error < 3e-12),
+//    r_j near 1/(cell centre) and exactly 1 in the cell holding 1.
+//  * sin, cos of 2 pi v: v = j/64 + t_lo, the table of sin, cos(2 pi j/64) and the
+//    angle-addition formulas with sin b, cos b of b = 2 pi t_lo < 2 pi/64 by their
+//    series (to b^5 and b^4; error < 2e-9).
+// The tables are computed at compile time in double precision from the same series and
+// rounded to float.
 namespace bm {
 
+struct alignas(16) SinCos {
+    float s, c, ns, pad;  // sin, cos and -sin of 2 pi j/64
+};
+struct alignas(8) LogCell {
+    float r, l2r;  // r_j and 2 ln r_j
+};
+struct Tables {
+    SinCos sc[64];
+    LogCell lg[32];
+};
+
+constexpr double kPi = 3.14159265358979323846;
 constexpr uint32_t kSqrtHalfBits = 0x3F3504F3u;  // bits of sqrt(1/2) in binary32
 
+// sin and cos of x in [0, pi/2] by their Taylor series (x^31 terms: < 1e-25)
+constexpr double taylor_sin(double x)
+{
+    double term = x, sum = x;
+    for (int n = 1; n < 16; ++n) {
+        term *= -x * x / ((2.0 * n) * (2.0 * n + 1.0));
+        sum += term;
+    }
+    return sum;
+}
+constexpr double taylor_cos(double x)
+{
+    double term = 1.0, sum = 1.0;
+    for (int n = 1; n < 16; ++n) {
+        term *= -x * x / ((2.0 * n - 1.0) * (2.0 * n));
+        sum += term;
+    }
+    return sum;
+}
+// ln x for x in [0.5, 2] as 2 atanh((x - 1)/(x + 1)) (|s| <= 1/3; 40 terms)
+constexpr double series_log(double x)
+{
+    const double s = (x - 1.0) / (x + 1.0);
+    double p = s, sum = 0.0;
+    for (int n = 0; n < 40; ++n) {
+        sum += p / (2.0 * n + 1.0);
+        p *= s * s;
+    }
+    return 2.0 * sum;
+}
+// the binary32 value with bits b, for b in [0x3F000000, 0x40000000)
+constexpr double f32_of_bits(uint32_t b)
+{
+    return b < 0x3F800000u ? 0.5 * (1.0 + (double)(b - 0x3F000000u) / 8388608.0)
+                           : 1.0 + (double)(b - 0x3F800000u) / 8388608.0;
+}
+constexpr Tables make_tables()
+{
+    Tables T{};
+    for (int j = 0; j < 64; ++j) {
+        const int q = j / 16;  // quadrant of 2 pi j/64
+        const double x = 2.0 * kPi * (j % 16) / 64.0;
+        const double s = taylor_sin(x), c = taylor_cos(x);
+        const double sq[4] = {s, c, -s, -c}, cq[4] = {c, -s, -c, s};
+        T.sc[j].s = (float)sq[q];
+        T.sc[j].c = (float)cq[q];
+        T.sc[j].ns = -(float)sq[q];
+        T.sc[j].pad = 0.0f;
+    }
+    const int one = (int)((0x3F800000u - kSqrtHalfBits) >> 18);  // the cell holding 1
+    for (int j = 0; j < 32; ++j) {
+        if (j == one) {
+            T.lg[j].r = 1.0f;
+            T.lg[j].l2r = 0.0f;
+            continue;
+        }
+        const double lo = f32_of_bits(kSqrtHalfBits + ((uint32_t)j << 18));
+        const double hi = f32_of_bits(kSqrtHalfBits + ((uint32_t)(j + 1) << 18));
+        const float r = (float)(2.0 / (lo + hi));
+        T.lg[j].r = r;
+        T.lg[j].l2r = -2.0f * (float)(-series_log((double)r));  // -2 x (the binary32 -ln r_j)
+    }
+    return T;
+}
+
 }  // namespace bm
+
+// one copy per translation unit, read through the read-only cache
+static __device__ const bm::Tables kBM = bm::make_tables();
 
 // 1/sqrt(x) of a positive normal x: rsqrtf without its steps for subnormals (the same
 // approximation and bits)
@@ -174,6 +267,55 @@ __device__ __forceinline__ void bm_eval(const uint32_t *w, V sc, V &g0, V &g1)
     g1 = rad * s;
 }
 
+// The same by the tables.
+template <class V, bool SCALED = false>
+__device__ __forceinline__ void bm_eval_table(const uint32_t *w, V sc, V &g0, V &g1)
+{
+    constexpr int L = V::L;
+    float f[L], lr[L], l2r[L], eb[L], xm[L], sa[L], ca[L], nsa[L];
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+        const float fn = __uint2float_rn((w[l] >> 11) | 1u);  // 2k+1 < 2^21, exact
+        const int bits = __float_as_int(fn);
+        const int t = bits - (int)bm::kSqrtHalfBits;
+        const int e = t >> 23;                                // 2k+1 = 2^e f
+        f[l] = __int_as_float(bits - (e << 23));              // f in [sqrt(1/2), sqrt(2))
+        const float2 C = __ldg(reinterpret_cast<const float2 *>(&kBM.lg[(t >> 18) & 31]));  // (r_j, 2 ln r_j)
+        lr[l] = C.x;
+        l2r[l] = C.y;
+        eb[l] = __int_as_float(0x4B400000 + e - 21);          // 1.5 2^23 + (e - 21), exact
+        const uint32_t m = w[l] & 0xFFFu;
+        const float4 A = __ldg(reinterpret_cast<const float4 *>(&kBM.sc[m >> 6]));  // (sin, cos, -sin)(2 pi j/64)
+        sa[l] = A.x;
+        ca[l] = A.y;
+        nsa[l] = A.z;
+        xm[l] = __int_as_float(0x4B000000u | (m & 63u));      // 2^23 + (m mod 64), exact
+    }
+    // -2 ln u = -2 (e - 21) ln 2 + 2 ln r_j - 2 ln(1 + d)
+    const V d = vfma(vmake<V>(f), vmake<V>(lr), V::bc(-1.0f));
+    V p = vfma(d, V::bc(-0.4f), V::bc(0.5f));  // -2 x the series of ln(1 + d)/d, Horner form
+    p = vfma(d, p, V::bc(-2.0f / 3.0f));
+    p = vfma(d, p, V::bc(1.0f));
+    p = vfma(d, p, V::bc(-2.0f));
+    const V em = vmake<V>(eb) - V::bc(12582912.0f);       // e - 21, exact
+    const V e2 = vfma(d, p, vfma(em, V::bc(-2.0f * 0.693147180559945f), vmake<V>(l2r)));  // >= 9.5e-7
+    float rs[L];
+#pragma unroll
+    for (int l = 0; l < L; ++l) rs[l] = rsqrt_normal(e2.lane(l));
+    V rad = e2 * vmake<V>(rs);
+    if (SCALED) rad = rad * sc;
+    // sin, cos of 2 pi v by angle addition
+    const V x = vfma(vmake<V>(xm) - V::bc(8388608.0f), V::bc((float)(2.0 * bm::kPi / 4096.0)),
+                     V::bc((float)(bm::kPi / 4096.0)));
+    const V x2 = x * x;
+    const V cb = vfma(x2, vfma(x2, V::bc(1.0f / 24.0f), V::bc(-0.5f)), V::bc(1.0f));
+    const V sb = x * vfma(x2, vfma(x2, V::bc(1.0f / 120.0f), V::bc(-1.0f / 6.0f)), V::bc(1.0f));
+    const V s = vfma(vmake<V>(sa), cb, vmake<V>(ca) * sb);
+    const V c = vfma(vmake<V>(ca), cb, vmake<V>(nsa) * sb);
+    g0 = rad * c;
+    g1 = rad * s;
+}
+
 __device__ __forceinline__ uint32_t word(const u32x4 &r, int k) { return k == 0 ? r.x : k == 1 ? r.y : k == 2 ? r.z : r.w; }
 
 __device__ __forceinline__ u32x4 philox_ctr(int64_t step, uint32_t site, uint32_t stream, uint32_t block)
@@ -185,8 +327,8 @@ __device__ __forceinline__ u32x4 philox_ctr(int64_t step, uint32_t site, uint32_
 // Box-Muller pairs of the block's first NP words (normals 2k, 2k + 1 of a block
 // come from its word k), two words evaluated together in one packed register.
 // KEY_R0: form the round keys from K's round-0 keys (arguments in shared memory).
-// SCALED: every normal multiplied by sc.
-template <int NP, bool KEY_R0 = false, bool SCALED = false>
+// SCALED: every normal multiplied by sc.  TABLE: Box-Muller by the tables (FP16 storage).
+template <int NP, bool KEY_R0 = false, bool SCALED = false, bool TABLE = false>
 __device__ __forceinline__ void normals(const PhiloxKey &K, int64_t step, uint32_t site, uint32_t stream,
                                         uint32_t block, float *g, float sc = 1.0f)
 {
@@ -197,7 +339,8 @@ __device__ __forceinline__ void normals(const PhiloxKey &K, int64_t step, uint32
     for (int k = 0; k + 1 < NP; k += 2) {
         const uint32_t w[2] = {word(r, k), word(r, k + 1)};
         F2 c0, s0;
-        bm_eval<F2, SCALED>(w, F2::bc(sc), c0, s0);
+        if (TABLE) bm_eval_table<F2, SCALED>(w, F2::bc(sc), c0, s0);
+        else bm_eval<F2, SCALED>(w, F2::bc(sc), c0, s0);
         g[2 * k] = c0.v.x;
         g[2 * k + 1] = s0.v.x;
         g[2 * k + 2] = c0.v.y;
@@ -206,7 +349,8 @@ __device__ __forceinline__ void normals(const PhiloxKey &K, int64_t step, uint32
     if constexpr ((NP & 1) != 0) {
         const uint32_t w = word(r, NP - 1);
         F1 c0, s0;
-        bm_eval<F1, SCALED>(&w, F1{sc}, c0, s0);
+        if (TABLE) bm_eval_table<F1, SCALED>(&w, F1{sc}, c0, s0);
+        else bm_eval<F1, SCALED>(&w, F1{sc}, c0, s0);
         g[2 * NP - 2] = c0.v;
         g[2 * NP - 1] = s0.v;
     }
@@ -217,8 +361,8 @@ __device__ __forceinline__ void normals(const PhiloxKey &K, int64_t step, uint32
 // site (n has room for NB rounded up to even).  F2: the lanes are the two
 // sites; F1: the site's words are evaluated in pairs in one packed register.
 // A caller consumes one block's normals before drawing the next, so that at
-// most eight are live.
-template <int NB, bool KEY_R0, class V>
+// most eight are live.  TABLE: Box-Muller by the tables (FP16 storage).
+template <int NB, bool KEY_R0, bool TABLE = false, class V>
 __device__ __forceinline__ void lane_block(const PhiloxKey &K, int64_t step, const uint32_t *site, uint32_t b, V sc,
                                            V *n)
 {
@@ -234,14 +378,16 @@ __device__ __forceinline__ void lane_block(const PhiloxKey &K, int64_t step, con
 #pragma unroll
         for (int k = 0; k < NPAIR; ++k) {
             const uint32_t w[2] = {word(r[0], k), word(r[1], k)};
-            bm_eval<V, true>(w, sc, n[2 * k], n[2 * k + 1]);
+            if (TABLE) bm_eval_table<V, true>(w, sc, n[2 * k], n[2 * k + 1]);
+            else bm_eval<V, true>(w, sc, n[2 * k], n[2 * k + 1]);
         }
     } else {
 #pragma unroll
         for (int k = 0; k < NPAIR; k += 2) {
             const uint32_t w[2] = {word(r[0], k), word(r[0], k + 1)};
             F2 c0, s0;
-            bm_eval<F2, true>(w, F2::bc(sc.lane(0)), c0, s0);
+            if (TABLE) bm_eval_table<F2, true>(w, F2::bc(sc.lane(0)), c0, s0);
+            else bm_eval<F2, true>(w, F2::bc(sc.lane(0)), c0, s0);
             n[2 * k] = V::bc(c0.v.x);
             n[2 * k + 1] = V::bc(s0.v.x);
             if (k + 1 < NPAIR) {
@@ -568,9 +714,9 @@ cudaError_t encode_tensor_map_f32(CUtensorMap *map, const void *base, int rank, 
 // mu_in: every replica's step forms mu of psi^n, so FV stage 1 reads it (map_mu)
 // q15: D3Q15 replicas (collide-stream, velocity and the FV operators of D3Q15)
 cudaError_t launch_batch_step(const BatchLists &L, int storage, bool ghost, bool force, int scheme_fv, bool heun,
-                              bool noise, bool mu_in, bool q15, cudaStream_t st);
+                              int noise, bool mu_in, bool q15, cudaStream_t st);
 // the psi stage launches of a batched step alone (no state change: the autotuner times them)
-cudaError_t launch_batch_psi(const BatchLists &L, bool heun, bool noise, bool mu_in, bool q15, cudaStream_t st);
+cudaError_t launch_batch_psi(const BatchLists &L, bool heun, int noise, bool mu_in, bool q15, cudaStream_t st);
 
 // ---- persistent batched mode (flb_persist.cu) --------------------------------
 enum { PH_MU = 0, PH_LB = 1, PH_VEL = 2, PH_S1 = 3, PH_S2 = 4, PH_COUNT = 5 };
@@ -621,7 +767,7 @@ cudaError_t launch_vel2(const LBArgs &a, int storage, cudaStream_t s);  // of a 
 // every scheme and Laplacian); q: the lattice of the FV operators
 // (19 or 15); mu_in: the mu of the stage input on the interior and 2 ghost layers,
 // or null (stage 1 then forms it)
-cudaError_t launch_psi3(const Geom &g, int scheme, int q, int stage, bool noise, const float *psi, const float *u,
+cudaError_t launch_psi3(const Geom &g, int scheme, int q, int stage, int noise, const float *psi, const float *u,
                         float *out, float *E, float A, float B, float K, float M, float kT, int advect, int heun,
                         const PhiloxKey &key, int64_t step, int zc, int rk4, const float *base, float *Dn,
                         const float *mu_in, int *status, cudaStream_t st, const LapW *lw = nullptr);
@@ -633,7 +779,7 @@ cudaError_t launch_init_eq(const Geom &g, int q, int storage, const float *rho, 
                            cudaStream_t st);
 // both Heun stages of the FV psi step in one launch by halo recompute (flb_heun1.cu)
 cudaError_t launch_psi3_heun1(const Geom &g, int scheme, const float *psi, const float *u, float *out, float A, float B,
-                              float K, float M, float kT, int advect, bool noise, const PhiloxKey &key, int64_t step,
+                              float K, float M, float kT, int advect, int noise, const PhiloxKey &key, int64_t step,
                               int zc, cudaStream_t st);
 // equilibrium start (flb_init.cu): populations into f (the current buffer), psi
 // (padded) through an inverse DFT whose intermediates use `spare` (>= 16 bytes

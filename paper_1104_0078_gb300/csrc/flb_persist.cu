@@ -158,37 +158,37 @@ __global__ void __launch_bounds__(PB_NT, 2) persist_kernel(const PersistArgs P)
                 const CUtensorMap *pm = &r.map_psi[(int)(ds & 1)];
                 if (r.mu_in) {
                     if (r.noise)
-                        psi3_fv_tma_block<1, true, true, true, false, true, true>(pm, &r.map_u, spa, P.status, task.bx,
+                        psi3_fv_tma_block<1, 1, true, true, false, true, true>(pm, &r.map_u, spa, P.status, task.bx,
                                                                                  task.by, task.bz, tsmem, &r.map_mu);
                     else
-                        psi3_fv_tma_block<1, false, true, false, false, true, true>(pm, &r.map_u, spa, P.status, task.bx,
+                        psi3_fv_tma_block<1, 0, true, false, false, true, true>(pm, &r.map_u, spa, P.status, task.bx,
                                                                                    task.by, task.bz, tsmem, &r.map_mu);
                 } else if (r.noise) {
-                    psi3_fv_tma_block<1, true, true, true, false, false, true>(pm, &r.map_u, spa, P.status, task.bx,
+                    psi3_fv_tma_block<1, 1, true, true, false, false, true>(pm, &r.map_u, spa, P.status, task.bx,
                                                                               task.by, task.bz, tsmem);
                 } else {
-                    psi3_fv_tma_block<1, false, true, false, false, false, true>(pm, &r.map_u, spa, P.status, task.bx,
+                    psi3_fv_tma_block<1, 0, true, false, false, false, true>(pm, &r.map_u, spa, P.status, task.bx,
                                                                                 task.by, task.bz, tsmem);
                 }
             } else if (Q15) {
-                psi3_fv_tma_block<2, false, true, false, false, false, true>(&r.map_psis, &r.map_u, spa, P.status, task.bx,
+                psi3_fv_tma_block<2, 0, true, false, false, false, true>(&r.map_psis, &r.map_u, spa, P.status, task.bx,
                                                                             task.by, task.bz, tsmem);
             } else if (stage == 1) {
                 const CUtensorMap *pm = &r.map_psi[(int)(ds & 1)];
                 if (r.mu_in) {  // mu of psi^n from this step's mu tasks
                     if (r.noise)
-                        psi3_fv_tma_block<1, true, true, true, false, true>(pm, &r.map_u, spa, P.status, task.bx,
+                        psi3_fv_tma_block<1, 1, true, true, false, true>(pm, &r.map_u, spa, P.status, task.bx,
                                                                             task.by, task.bz, tsmem, &r.map_mu);
                     else
-                        psi3_fv_tma_block<1, false, true, false, false, true>(pm, &r.map_u, spa, P.status, task.bx,
+                        psi3_fv_tma_block<1, 0, true, false, false, true>(pm, &r.map_u, spa, P.status, task.bx,
                                                                               task.by, task.bz, tsmem, &r.map_mu);
                 } else if (r.noise) {
-                    psi3_fv_tma_block<1, true, true, true, false>(pm, &r.map_u, spa, P.status, task.bx, task.by, task.bz, tsmem);
+                    psi3_fv_tma_block<1, 1, true, true, false>(pm, &r.map_u, spa, P.status, task.bx, task.by, task.bz, tsmem);
                 } else {
-                    psi3_fv_tma_block<1, false, true, false, false>(pm, &r.map_u, spa, P.status, task.bx, task.by, task.bz, tsmem);
+                    psi3_fv_tma_block<1, 0, true, false, false>(pm, &r.map_u, spa, P.status, task.bx, task.by, task.bz, tsmem);
                 }
             } else {
-                psi3_fv_tma_block<2, false, true, false, false>(&r.map_psis, &r.map_u, spa, P.status, task.bx, task.by, task.bz, tsmem);
+                psi3_fv_tma_block<2, 0, true, false, false>(&r.map_psis, &r.map_u, spa, P.status, task.bx, task.by, task.bz, tsmem);
             }
         }
         __syncthreads();

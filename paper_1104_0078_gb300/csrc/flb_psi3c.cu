@@ -76,7 +76,7 @@ __device__ __forceinline__ Plane3 plane3(const float *p, int Y)
 
 // mu on the columns of a region (tile + H) from psi in global memory, planes
 // z0 - H .. z0 + nzt + H - 1, into smu [CZ + 2H][CY + 2H][CX + 2H].
-template <class T, int H, bool W>
+template <class T, int H, bool W, bool FD>
 __device__ __forceinline__ void form_mu(const Psi3Args &a, int x0, int y0, int z0, int nzt, float *smu)
 {
     FLB_TILE3(T);
@@ -95,11 +95,12 @@ __device__ __forceinline__ void form_mu(const Psi3Args &a, int x0, int y0, int z
 #pragma unroll
     for (int j = 0; j < CZ + 2 * H; ++j) {
         const Plane3 q2 = plane3<true>(p + min(j + 2, nzt + 2 * H + 1) * Z, Y);
-        const F1 n1 = q1.b + (q0.a + q2.a), n2 = q1.d + (q0.b + q2.b), n3 = q0.d + q2.d;
+        const F1 n1 = q1.b + (q0.a + q2.a), n2 = FD ? (q1.d + q0.b) + q2.b : q1.d + (q0.b + q2.b), n3 = q0.d + q2.d;
         const float ps = q1.a.v;
         smu[(j * WY + ly) * WX + lx] =
             W ? a.A * ps + a.B * ps * ps * ps - a.K * ((a.lw.c1 * n1.v + a.lw.c2 * n2.v) + (a.lw.c3 * n3.v + a.lw.c0 * ps))
-              : mu_so_v<F1>(a.A, a.B, k22, q1.a, n1, n2, n3).v;
+            : FD ? a.A * ps + a.B * ps * ps * ps - k22 * (6.f * n1.v + 3.f * n2.v + n3.v - 80.f * ps)
+                 : mu_so_v<F1>(a.A, a.B, k22, q1.a, n1, n2, n3).v;
         q0 = q1;
         q1 = q2;
     }
@@ -176,14 +177,14 @@ __device__ __forceinline__ F1 div_sum(const Div3 &below, const Div3 &own, const 
 }
 
 // shared memory of a block (floats)
-template <class T, bool NOISE, bool MU_IN>
+template <class T, int NOISE, bool MU_IN>
 __host__ __device__ constexpr int cube_fv_floats()
 {
     return (T::CZ + 2) * T::CP1 * (NOISE ? 6 : 3) + (MU_IN ? 0 : (T::CZ + 4) * T::CW2 * T::CH2);
 }
 
 // The noise of the block's nodes (tile + 1) into sX, [3][CZ + 2][CH1][CW1].
-template <class T>
+template <class T, int NOISE>
 __device__ __forceinline__ void cube_fv_noise(const Psi3Args &a, int x0, int y0, int z0, float *sX)
 {
     FLB_TILE3(T);
@@ -196,7 +197,7 @@ __device__ __forceinline__ void cube_fv_noise(const Psi3Args &a, int x0, int y0,
         if (x > g.nx || y > g.ny || z > g.nz) continue;
         float G[4];
         const uint32_t id = (uint32_t)(wrapi(x, g.nx) + g.nx * (wrapi(y, g.ny) + g.ny * wrapi(z, g.nz)));
-        normals<2, false, true>(a.key, a.step, id, 1u, 0u, G, sdx);
+        normals<2, false, true, NOISE == 2>(a.key, a.step, id, 1u, 0u, G, sdx);
         sX[k] = G[0];
         sX[JN + k] = G[1];
         sX[2 * JN + k] = G[2];
@@ -204,7 +205,7 @@ __device__ __forceinline__ void cube_fv_noise(const Psi3Args &a, int x0, int y0,
 }
 
 // The rest of a stage on the tile at (x0, y0, z0); the noise, if any, is in sX.
-template <class T, bool FIRST, bool NOISE, bool MU_IN, bool Q15, bool W>
+template <class T, bool FIRST, int NOISE, bool MU_IN, bool Q15, bool W>
 __device__ __forceinline__ void cube_fv_stage(const Psi3Args &a, const float *mu, int x0, int y0, int z0, float *sJ,
                                               const float *sX, float *smu)
 {
@@ -219,7 +220,7 @@ __device__ __forceinline__ void cube_fv_stage(const Psi3Args &a, const float *mu
     for (int j = 0; j < CZ / 2; ++j)
         e_pre[j] = !FIRST && act ? a.E[x0 + tx + g.nx * (y0 + ty + g.ny * min(z0 + zh + j, g.nz - 1))] : 0.f;
     if (!MU_IN) {
-        form_mu<T, 2, W>(a, x0, y0, z0, nzt, smu);
+        form_mu<T, 2, W, false>(a, x0, y0, z0, nzt, smu);
         __syncthreads();
     }
     {  // flux columns
@@ -323,7 +324,7 @@ __device__ __forceinline__ void cube_fv_stage(const Psi3Args &a, const float *mu
     }
 }
 
-template <class T, bool FIRST, bool NOISE, bool MU_IN, bool Q15, bool W>
+template <class T, bool FIRST, int NOISE, bool MU_IN, bool Q15, bool W>
 __global__ void __launch_bounds__(T::NT) psi3_fv_cube_kernel(const CubeArgs ca)
 {
     constexpr int JN = (T::CZ + 2) * T::CP1;
@@ -331,7 +332,7 @@ __global__ void __launch_bounds__(T::NT) psi3_fv_cube_kernel(const CubeArgs ca)
     float *sJ = csm, *sX = sJ + 3 * JN, *smu = sX + (NOISE ? 3 * JN : 0);  // smu: [CZ + 4][CH2][CW2] unless MU_IN
     const int x0 = blockIdx.x * T::CX, y0 = blockIdx.y * T::CY, z0 = blockIdx.z * T::CZ;
     pdl_trigger();
-    if (NOISE) cube_fv_noise<T>(ca.a, x0, y0, z0, sX);
+    if (NOISE) cube_fv_noise<T, NOISE>(ca.a, x0, y0, z0, sX);
     pdl_wait();
     cube_fv_stage<T, FIRST, NOISE, MU_IN, Q15, W>(ca.a, ca.mu, x0, y0, z0, sJ, sX, smu);
 }
@@ -345,7 +346,7 @@ __device__ constexpr int8_t kCubeL[13][3] = {{1, 0, 0},  {0, 1, 0},  {0, 0, 1}, 
                                              {1, 0, 1},  {1, 0, -1}, {0, 1, 1},  {0, 1, -1}, {1, 1, 1},
                                              {1, 1, -1}, {1, -1, 1}, {1, -1, -1}};
 
-template <class T, bool FIRST, bool NOISE, bool MU_IN, bool W>
+template <class T, bool FIRST, int NOISE, bool MU_IN, bool W>
 __global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
 {
     FLB_TILE3(T);
@@ -366,14 +367,14 @@ __global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
             const uint32_t id = (uint32_t)(wrapi(x, g.nx) + g.nx * (wrapi(y, g.ny) + g.ny * wrapi(z, g.nz)));
             if (ca.naive) {
                 float G[4];
-                normals<2>(a.key, a.step, id, 1u, 0u, G);
+                normals<2, false, false, NOISE == 2>(a.key, a.step, id, 1u, 0u, G);
 #pragma unroll
                 for (int l = 0; l < 3; ++l) sZ[l * ZN + k] = G[l];
             } else {
                 if (lx == CW1 - 1) continue;  // no half-link points to -x: the last column is not read
                 float G[14];
-                normals<4>(a.key, a.step, id, 1u, 0u, G);
-                normals<3>(a.key, a.step, id, 1u, 1u, G + 8);
+                normals<4, false, false, NOISE == 2>(a.key, a.step, id, 1u, 0u, G);
+                normals<3, false, false, NOISE == 2>(a.key, a.step, id, 1u, 1u, G + 8);
 #pragma unroll
                 for (int l = 0; l < 13; ++l) sZ[l * ZN + k] = (l < 3 ? ca.s1 : (l < 9 ? ca.s2 : ca.s3)) * G[l];
             }
@@ -387,7 +388,7 @@ __global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
 #pragma unroll
     for (int j = 0; j < CZ / 2; ++j)
         e_pre[j] = !FIRST && act ? a.E[x + g.nx * (y + g.ny * min(z0 + zh + j, g.nz - 1))] : 0.f;
-    if (!MU_IN) form_mu<T, 1, W>(a, x0, y0, z0, nzt, smu);
+    if (!MU_IN) form_mu<T, 1, W, true>(a, x0, y0, z0, nzt, smu);
     if (NOISE || !MU_IN) __syncthreads();
     if (!act) return;
     const int Y = MU_IN ? g.px : CW1, Z = MU_IN ? g.px * g.py : CP1;
@@ -398,7 +399,7 @@ __global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
         const int z = z0 + zh + j;
         if (zh + j >= nzt) break;
         const Plane3 q2 = plane3<MU_IN>(m + (j + 2) * Z, Y);
-        const float n1 = (q1.b + (q0.a + q2.a)).v, n2 = (q1.d + (q0.b + q2.b)).v, n3 = (q0.d + q2.d).v;
+        const float n1 = (q1.b + (q0.a + q2.a)).v, n2 = ((q1.d + q0.b) + q2.b).v, n3 = (q0.d + q2.d).v;
         float D = W ? a.M * ((a.lw.c1 * n1 + a.lw.c2 * n2) + (a.lw.c3 * n3 + a.lw.c0 * q1.a.v))
                     : a.M * ((1.0f / 22.0f) * (6.f * n1 + 3.f * n2 + n3 - 80.f * q1.a.v));
         q0 = q1;
@@ -419,9 +420,16 @@ __global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
                 eta = 0.5f * ca.sd * ((sZ[c + 1] - sZ[c - 1]) + (sZ[ZN + c + CW1] - sZ[ZN + c - CW1]) +
                                       (sZ[2 * ZN + c + CP1] - sZ[2 * ZN + c - CP1]));
             } else {
+                float own = 0.f, in0 = 0.f, up = 0.f, dn = 0.f;
 #pragma unroll
-                for (int l = 0; l < 13; ++l)
-                    eta += sZ[l * ZN + c - kCubeL[l][0] - CW1 * kCubeL[l][1] - CP1 * kCubeL[l][2]] - sZ[l * ZN + c];
+                for (int l = 0; l < 13; ++l) {
+                    own += sZ[l * ZN + c];
+                    const float v = sZ[l * ZN + c - kCubeL[l][0] - CW1 * kCubeL[l][1] - CP1 * kCubeL[l][2]];
+                    if (kCubeL[l][2] == 0) in0 += v;
+                    else if (kCubeL[l][2] > 0) up += v;
+                    else dn += v;
+                }
+                eta = (up + (in0 - own)) + dn;
             }
         }
         const F1 own{FIRST ? __ldg(a.psi + pi) : 0.f};
@@ -437,43 +445,55 @@ cudaError_t go(K k, const CubeArgs &ca, dim3 grid, int threads, int floats, cuda
     return e != cudaSuccess ? e : launch_pdl(k, grid, threads, smem, st, PDL_BLOCKS, ca);
 }
 
-template <class T, bool FIRST, bool NOISE, bool MU_IN, bool W>
+template <class T, bool FIRST, int NOISE, bool MU_IN, bool W>
 cudaError_t go_fd(const CubeArgs &ca, dim3 grid, cudaStream_t st)
 {
     const int zn = (T::CZ + 2) * T::CP1;
     return go(psi3_fd_cube_kernel<T, FIRST, NOISE, MU_IN, W>, ca, grid, T::NT,
               zn * ((MU_IN ? 0 : 1) + (NOISE ? (ca.naive ? 3 : 13) : 0)), st);
 }
-template <class T, bool FIRST, bool NOISE, bool MU_IN, bool Q15, bool W>
+template <class T, bool FIRST, int NOISE, bool MU_IN, bool Q15, bool W>
 cudaError_t go_fv(const CubeArgs &ca, dim3 grid, cudaStream_t st)
 {
     return go(psi3_fv_cube_kernel<T, FIRST, NOISE, MU_IN, Q15, W>, ca, grid, T::NT, cube_fv_floats<T, NOISE, MU_IN>(), st);
 }
 
-template <class T, bool W>
-cudaError_t fd_cube(const CubeArgs &ca, bool first, bool noise, dim3 g, cudaStream_t st)
+template <class T, bool MU_IN, bool W>
+cudaError_t first_fd(const CubeArgs &ca, int noise, dim3 g, cudaStream_t st)
 {
-    if (!first) return go_fd<T, false, false, false, W>(ca, g, st);
-    if (ca.mu) return noise ? go_fd<T, true, true, true, W>(ca, g, st) : go_fd<T, true, false, true, W>(ca, g, st);
-    return noise ? go_fd<T, true, true, false, W>(ca, g, st) : go_fd<T, true, false, false, W>(ca, g, st);
+    return noise == 2 ? go_fd<T, true, 2, MU_IN, W>(ca, g, st)
+           : noise    ? go_fd<T, true, 1, MU_IN, W>(ca, g, st)
+                      : go_fd<T, true, 0, MU_IN, W>(ca, g, st);
+}
+template <class T, bool MU_IN, bool Q15, bool W>
+cudaError_t first_fv(const CubeArgs &ca, int noise, dim3 g, cudaStream_t st)
+{
+    return noise == 2 ? go_fv<T, true, 2, MU_IN, Q15, W>(ca, g, st)
+           : noise    ? go_fv<T, true, 1, MU_IN, Q15, W>(ca, g, st)
+                      : go_fv<T, true, 0, MU_IN, Q15, W>(ca, g, st);
+}
+
+template <class T, bool W>
+cudaError_t fd_cube(const CubeArgs &ca, bool first, int noise, dim3 g, cudaStream_t st)
+{
+    if (!first) return go_fd<T, false, 0, false, W>(ca, g, st);
+    if (ca.mu) return first_fd<T, true, W>(ca, noise, g, st);
+    return first_fd<T, false, W>(ca, noise, g, st);
 }
 
 template <class T, bool Q15>
-cudaError_t fv_cube(const CubeArgs &ca, bool first, bool noise, dim3 g, cudaStream_t st)
+cudaError_t fv_cube(const CubeArgs &ca, bool first, int noise, dim3 g, cudaStream_t st)
 {
     const bool w = ca.a.lap_w;
-    if (!first) return w ? go_fv<T, false, false, false, Q15, true>(ca, g, st)
-                         : go_fv<T, false, false, false, Q15, false>(ca, g, st);
-    if (ca.mu) return noise ? go_fv<T, true, true, true, Q15, false>(ca, g, st)
-                            : go_fv<T, true, false, true, Q15, false>(ca, g, st);
-    if (w) return noise ? go_fv<T, true, true, false, Q15, true>(ca, g, st)
-                        : go_fv<T, true, false, false, Q15, true>(ca, g, st);
-    return noise ? go_fv<T, true, true, false, Q15, false>(ca, g, st)
-                 : go_fv<T, true, false, false, Q15, false>(ca, g, st);
+    if (!first) return w ? go_fv<T, false, 0, false, Q15, true>(ca, g, st)
+                         : go_fv<T, false, 0, false, Q15, false>(ca, g, st);
+    if (ca.mu) return first_fv<T, true, Q15, false>(ca, noise, g, st);
+    if (w) return first_fv<T, false, Q15, true>(ca, noise, g, st);
+    return first_fv<T, false, Q15, false>(ca, noise, g, st);
 }
 
 template <class T>
-cudaError_t tile_cube(const CubeArgs &ca, int scheme, int q, bool first, bool noise, cudaStream_t st)
+cudaError_t tile_cube(const CubeArgs &ca, int scheme, int q, bool first, int noise, cudaStream_t st)
 {
     const Geom &g = ca.a.g;
     const dim3 grid((g.nx + T::CX - 1) / T::CX, (g.ny + T::CY - 1) / T::CY, (g.nz + T::CZ - 1) / T::CZ);
@@ -495,7 +515,7 @@ bool wide_tile(const Geom &g)
 
 }  // namespace
 
-cudaError_t launch_psi3_cube(const Psi3Args &a, int scheme, int q, bool first, bool noise, const float *mu_in,
+cudaError_t launch_psi3_cube(const Psi3Args &a, int scheme, int q, bool first, int noise, const float *mu_in,
                              cudaStream_t st)
 {
     CubeArgs ca;

@@ -20,6 +20,8 @@
 // writes psi^{n+1} = E + D(psi*)/2 (the noise is held fixed over the step).
 #include <cudaTypedefs.h>
 
+#include <type_traits>
+
 #include "flb_psi3d.cuh"
 
 namespace flb {
@@ -33,7 +35,7 @@ struct TmaArgs {
 // the FV operators of D3Q15
 // 256 threads, each on point pairs (y, y + H/2) of every region in packed FP32 (F2)
 using StageV = F2;
-template <int STAGE, bool NOISE, bool RK, bool MU_IN, bool Q15 = false>
+template <int STAGE, int NOISE, bool RK, bool MU_IN, bool Q15 = false>
 __global__ void __launch_bounds__(block_threads<StageV, MU_IN>(), 2) psi3_fv_tma_kernel(const __grid_constant__ CUtensorMap psi_map,
                                                                    const __grid_constant__ CUtensorMap u_map,
                                                                    const __grid_constant__ CUtensorMap mu_map,
@@ -48,7 +50,7 @@ __global__ void __launch_bounds__(block_threads<StageV, MU_IN>(), 2) psi3_fv_tma
 
 // batched: block b of the launch works on L.psi[b]; MU_IN: stage 1 reads mu of
 // psi^n from the replica's mu field (every replica's step formed it)
-template <int STAGE, bool NOISE, bool MU_IN = false, bool Q15 = false>
+template <int STAGE, int NOISE, bool MU_IN = false, bool Q15 = false>
 __global__ void __launch_bounds__(block_threads<StageV, MU_IN>(), 2) psi3_fv_tma_batch_kernel(const BatchLists L)
 {
     extern __shared__ __align__(1024) float tsmem[];
@@ -69,7 +71,7 @@ cudaError_t launch_lb3_batch(const BatchLists &L, int storage, bool ghost, bool 
 cudaError_t launch_lb15_batch(const BatchLists &L, int storage, bool ghost, bool force, cudaStream_t st);
 
 template <bool Q15>
-static cudaError_t batch_psi(const BatchLists &L, bool heun, bool noise, bool mu_in, cudaStream_t st)
+static cudaError_t batch_psi(const BatchLists &L, bool heun, int noise, bool mu_in, cudaStream_t st)
 {
     const size_t sm = sizeof(float) * (size_t)fv_smem_floats<StageV>();
     const size_t smm = sizeof(float) * (size_t)fv_mu_smem_floats<StageV>();
@@ -81,21 +83,23 @@ static cudaError_t batch_psi(const BatchLists &L, bool heun, bool noise, bool mu
         return cudaGetLastError();
     };
     constexpr int n1 = block_threads<StageV, true>(), nn = block_threads<StageV, false>();
-    cudaError_t e = mu_in ? (noise ? go(psi3_fv_tma_batch_kernel<1, true, true, Q15>, smm + nb, n1)
-                                   : go(psi3_fv_tma_batch_kernel<1, false, true, Q15>, smm, n1))
-                          : (noise ? go(psi3_fv_tma_batch_kernel<1, true, false, Q15>, sm + nb, nn)
-                                   : go(psi3_fv_tma_batch_kernel<1, false, false, Q15>, sm, nn));
+    cudaError_t e = mu_in ? (noise == 2 ? go(psi3_fv_tma_batch_kernel<1, 2, true, Q15>, smm + nb, n1)
+                                 : noise ? go(psi3_fv_tma_batch_kernel<1, 1, true, Q15>, smm + nb, n1)
+                                         : go(psi3_fv_tma_batch_kernel<1, 0, true, Q15>, smm, n1))
+                          : (noise == 2 ? go(psi3_fv_tma_batch_kernel<1, 2, false, Q15>, sm + nb, nn)
+                                 : noise ? go(psi3_fv_tma_batch_kernel<1, 1, false, Q15>, sm + nb, nn)
+                                         : go(psi3_fv_tma_batch_kernel<1, 0, false, Q15>, sm, nn));
     if (e != cudaSuccess || !heun) return e;
-    return go(psi3_fv_tma_batch_kernel<2, false, false, Q15>, sm, nn);
+    return go(psi3_fv_tma_batch_kernel<2, 0, false, Q15>, sm, nn);
 }
 
-cudaError_t launch_batch_psi(const BatchLists &L, bool heun, bool noise, bool mu_in, bool q15, cudaStream_t st)
+cudaError_t launch_batch_psi(const BatchLists &L, bool heun, int noise, bool mu_in, bool q15, cudaStream_t st)
 {
     return q15 ? batch_psi<true>(L, heun, noise, mu_in, st) : batch_psi<false>(L, heun, noise, mu_in, st);
 }
 
 cudaError_t launch_batch_step(const BatchLists &L, int storage, bool ghost, bool force, int scheme_fv, bool heun,
-                              bool noise, bool mu_in, bool q15, cudaStream_t st)
+                              int noise, bool mu_in, bool q15, cudaStream_t st)
 {
     if (!scheme_fv) return cudaErrorNotSupported;
     cudaError_t e = q15 ? launch_lb15_batch(L, storage, ghost, force, st)
@@ -134,7 +138,7 @@ cudaError_t encode_tensor_map_f32(CUtensorMap *map, const void *base, int rank, 
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-static cudaError_t launch_fv_tma(const Psi3Args &a, int q, int stage, bool noise, const float *mu_in, int *status,
+static cudaError_t launch_fv_tma(const Psi3Args &a, int q, int stage, int noise, const float *mu_in, int *status,
                                  cudaStream_t st)
 {
     const Geom &g = a.g;
@@ -168,34 +172,28 @@ static cudaError_t launch_fv_tma(const Psi3Args &a, int q, int stage, bool noise
     };
     const size_t smn = sm + sizeof(float) * FV_NOISE_FLOATS;
     const size_t smm = sizeof(float) * (size_t)fv_mu_smem_floats<StageV>(), smmn = smm + sizeof(float) * FV_NOISE_FLOATS;
-    if (q == 15) {  // D3Q15 (the RK4 branches compiled into RK4 launches only, as below)
-        if (stage == 2) return a.rk4 ? go(psi3_fv_tma_kernel<2, false, true, false, true>, sm)
-                                     : go(psi3_fv_tma_kernel<2, false, false, false, true>, sm);
-        if (a.rk4) {
-            if (mu) return noise ? go(psi3_fv_tma_kernel<1, true, true, true, true>, smmn)
-                                 : go(psi3_fv_tma_kernel<1, false, true, true, true>, smm);
-            return noise ? go(psi3_fv_tma_kernel<1, true, true, false, true>, smn)
-                         : go(psi3_fv_tma_kernel<1, false, true, false, true>, sm);
-        }
-        if (mu) return noise ? go(psi3_fv_tma_kernel<1, true, false, true, true>, smmn)
-                             : go(psi3_fv_tma_kernel<1, false, false, true, true>, smm);
-        return noise ? go(psi3_fv_tma_kernel<1, true, false, false, true>, smn)
-                     : go(psi3_fv_tma_kernel<1, false, false, false, true>, sm);
-    }
-    if (stage == 2) return a.rk4 ? go(psi3_fv_tma_kernel<2, false, true, false>, sm)
-                                 : go(psi3_fv_tma_kernel<2, false, false, false>, sm);
-    if (mu) {
-        if (a.rk4) return noise ? go(psi3_fv_tma_kernel<1, true, true, true>, smmn)
-                                : go(psi3_fv_tma_kernel<1, false, true, true>, smm);
-        return noise ? go(psi3_fv_tma_kernel<1, true, false, true>, smmn)
-                     : go(psi3_fv_tma_kernel<1, false, false, true>, smm);
-    }
-    if (a.rk4) return noise ? go(psi3_fv_tma_kernel<1, true, true, false>, smn)
-                            : go(psi3_fv_tma_kernel<1, false, true, false>, sm);
-    return noise ? go(psi3_fv_tma_kernel<1, true, false, false>, smn) : go(psi3_fv_tma_kernel<1, false, false, false>, sm);
+    // one kernel per stage, RK4 or not (its branches cost registers), mu given or not,
+    // noise (0, 1, 2) and lattice
+    auto stage1 = [&](auto rk, auto mi, auto q15) {
+        constexpr bool RK = decltype(rk)::value, MU = decltype(mi)::value, Q15 = decltype(q15)::value;
+        const size_t bytes = MU ? smm : sm, bytes_n = MU ? smmn : smn;
+        return noise == 2 ? go(psi3_fv_tma_kernel<1, 2, RK, MU, Q15>, bytes_n)
+               : noise    ? go(psi3_fv_tma_kernel<1, 1, RK, MU, Q15>, bytes_n)
+                          : go(psi3_fv_tma_kernel<1, 0, RK, MU, Q15>, bytes);
+    };
+    auto lattice = [&](auto q15) {
+        constexpr bool Q15 = decltype(q15)::value;
+        using Yes = std::true_type;
+        using No = std::false_type;
+        if (stage == 2) return a.rk4 ? go(psi3_fv_tma_kernel<2, 0, true, false, Q15>, sm)
+                                     : go(psi3_fv_tma_kernel<2, 0, false, false, Q15>, sm);
+        if (a.rk4) return mu ? stage1(Yes(), Yes(), q15) : stage1(Yes(), No(), q15);
+        return mu ? stage1(No(), Yes(), q15) : stage1(No(), No(), q15);
+    };
+    return q == 15 ? lattice(std::true_type()) : lattice(std::false_type());
 }
 
-cudaError_t launch_psi3(const Geom &g, int scheme, int q, int stage, bool noise, const float *psi, const float *u,
+cudaError_t launch_psi3(const Geom &g, int scheme, int q, int stage, int noise, const float *psi, const float *u,
                         float *out, float *E, float A, float B, float K, float M, float kT, int advect, int heun,
                         const PhiloxKey &key, int64_t step, int zc, int rk4, const float *base, float *Dn,
                         const float *mu_in, int *status, cudaStream_t st, const LapW *lw)

@@ -33,7 +33,7 @@ struct Psi3Args {
 };
 
 // One stage by small tiles (flb_psi3c.cu).
-cudaError_t launch_psi3_cube(const Psi3Args &a, int scheme, int q, bool first, bool noise, const float *mu_in,
+cudaError_t launch_psi3_cube(const Psi3Args &a, int scheme, int q, bool first, int noise, const float *mu_in,
                              cudaStream_t st);
 
 // Point k of a W x H region (W >= 32): rows' first 32 columns first, then the
@@ -163,7 +163,7 @@ __host__ __device__ constexpr int block_threads() { return V::L == 2 && MU_IN ? 
 // (mu_map, valid to 2 ghost layers), written for the force of the same step.  Its
 // planes then come by TMA, like psi and u, into a third ring ([TY+4][TX+8], column
 // c <-> x = x0 - 4 + c, row r <-> y = y0 - 2 + r), and the block skips forming mu.
-template <int STAGE, bool NOISE, bool COH = false, bool KEY_R0 = false, bool RK = true, bool MU_IN = false,
+template <int STAGE, int NOISE, bool COH = false, bool KEY_R0 = false, bool RK = true, bool MU_IN = false,
           bool Q15 = false, class V = F1>
 __device__ __forceinline__ void psi3_fv_tma_block(const CUtensorMap *psi_map, const CUtensorMap *u_map,
                                                   const Psi3Args &a, int *status, int bx, int by, int bz,
@@ -434,7 +434,7 @@ __device__ __forceinline__ void psi3_fv_tma_block(const CUtensorMap *psi_map, co
 #pragma unroll
                         for (int l = 0; l < L; ++l) {
                             float Gn[4];
-                            normals<2, KEY_R0, true>(a.key, a.step, (uint32_t)(n1[j][l] + zid), 1u, 0u, Gn, sdx);
+                            normals<2, KEY_R0, true, NOISE == 2>(a.key, a.step, (uint32_t)(n1[j][l] + zid), 1u, 0u, Gn, sdx);
                             X[k + l * LR1] = Gn[0];
                             X[TJ_N + k + l * LR1] = Gn[1];
                             X[2 * TJ_N + k + l * LR1] = Gn[2];

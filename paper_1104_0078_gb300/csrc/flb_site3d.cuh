@@ -387,7 +387,7 @@ __device__ __forceinline__ void lb_sites_on(const LBArgs &a, const PL &P, int x,
         for (int l = 0; l < L; ++l) su[l] = (uint32_t)s[l];
         const V sc = vmake<V>(sq);
         V n[8];
-        lane_block<8, KEY_R0>(a.key, a.step, su, 0u, sc, n);  // normals 0-7
+        lane_block<8, KEY_R0, sizeof(T) == 2>(a.key, a.step, su, 0u, sc, n);  // normals 0-7
         const V m0 = n[0] * a.nq[0], m1 = n[1] * a.nq[1], m2 = n[2] * a.nq[2];
         const V t01 = m0 - m1;
         Qxx = Qxx + vfma(m1, 2.0f, m0);
@@ -398,7 +398,7 @@ __device__ __forceinline__ void lb_sites_on(const LBArgs &a, const PL &P, int x,
         Qxz = vfma(n[5], a.nq[5], Qxz);
         G10 = vfma(n[6], a.nq[6], G10);
         G11 = vfma(n[7], a.nq[7], G11);
-        lane_block<7, KEY_R0>(a.key, a.step, su, 1u, sc, n);  // normals 8-14
+        lane_block<7, KEY_R0, sizeof(T) == 2>(a.key, a.step, su, 1u, sc, n);  // normals 8-14
         G12 = vfma(n[0], a.nq[8], G12);
         G13 = vfma(n[1], a.nq[9], G13);
         G14 = vfma(n[2], a.nq[10], G14);

@@ -60,8 +60,8 @@ __device__ __forceinline__ void pull9(const T *__restrict__ f, long long n, int 
 template <int P>
 __device__ __forceinline__ float lap2(const float *f, int c, const LapW &w)
 {
-    const float n1 = (f[c + 1] + f[c - 1]) + (f[c + P] + f[c - P]);
-    const float n2 = (f[c + P + 1] + f[c - P - 1]) + (f[c - P + 1] + f[c + P - 1]);
+    const float n1 = f[c + 1] + f[c - 1] + f[c + P] + f[c - P];
+    const float n2 = f[c + P + 1] + f[c - P - 1] + f[c - P + 1] + f[c + P - 1];
     return (w.c1 * n1 + w.c2 * n2) + w.c0 * f[c];
 }
 
@@ -119,6 +119,9 @@ __device__ __forceinline__ void form_sigma2(const float *sps, float *sg, float A
         }
     }
 }
+
+// the links of D2Q9
+__device__ constexpr int8_t kLink9[8][2] = {{1, 0}, {-1, 0}, {0, 1}, {0, -1}, {1, 1}, {-1, -1}, {1, -1}, {-1, 1}};
 
 // Force density at offset c of the mu plane (pitch P; or of the three stress
 // planes of PN values): F = -psi grad mu with the central difference (kind 0) or
@@ -234,6 +237,91 @@ __device__ __forceinline__ void collide9(const LBArgs &a, const uint32_t *s, con
     store(8, (E7 - O7) * w2);
 }
 
+// The same for populations stored as FP16 deviations, one site, in the order of one
+// kernel per phase and one thread per site: a last bit here moves roundings to 16 bits and with
+// them psi by up to 4e-4 of itself in 200 steps (FP32 storage: 2e-6), so FP16 runs keep
+// that order, here and in psi2_kernel's F16 branches.  G: the site's unit normals.
+template <bool GHOST_RELAX>
+__device__ __forceinline__ void collide9_f16(const LBArgs &a, uint32_t site, const float *f, const float *G, float Fx,
+                                             float Fy)
+{
+    __half *fo = (__half *)a.fout;
+    const long long N = a.g.n;
+    float s[5], d[5];
+#pragma unroll
+    for (int p = 1; p <= 4; ++p) {
+        s[p] = f[2 * p - 1] + f[2 * p];
+        d[p] = f[2 * p - 1] - f[2 * p];
+    }
+    const float drho = f[0] + ((s[1] + s[2]) + (s[3] + s[4]));
+    const float jx = d[1] + (d[3] + d[4]);
+    const float jy = d[2] + (d[3] - d[4]);
+    const float third = drho * (1.0f / 3.0f);
+    const float Sxx = s[1] + (s[3] + s[4]) - third;
+    const float Syy = s[2] + (s[3] + s[4]) - third;
+    const float Sxy = s[3] - s[4];
+
+    const float rho = a.rho0 + drho;
+    const float irho = 1.0f / rho;
+    const float vx = (jx + 0.5f * Fx) * irho, vy = (jy + 0.5f * Fy) * irho;
+
+    const float ws = a.omega_s, wb = a.omega_b;
+    const float cs = 1.0f - 0.5f * ws, cb = 1.0f - 0.5f * wb;
+    const float Xxx = rho * vx * vx - Sxx, Xyy = rho * vy * vy - Syy;
+    const float trX2 = 0.5f * (Xxx + Xyy);
+    const float Txx = 2.f * vx * Fx, Tyy = 2.f * vy * Fy;
+    const float trT2 = 0.5f * (Txx + Tyy);
+    const float isoB = (wb - ws) * trX2 + (cb - cs) * trT2;
+    float Bxx = Sxx + ws * Xxx + cs * Txx + isoB;
+    float Byy = Syy + ws * Xyy + cs * Tyy + isoB;
+    float Bxy = Sxy + ws * (rho * vx * vy - Sxy) + cs * (vx * Fy + Fx * vy);
+    const float Ax = jx + Fx, Ay = jy + Fy;
+
+    float g6 = 0.f, g7 = 0.f, g8 = 0.f;
+    if (GHOST_RELAX) {
+        const float gg = a.gamma_g;
+        const float m6 = -(1.f / 3.f) * d[1] + (2.f / 3.f) * (d[3] + d[4]);
+        const float m7 = -(1.f / 3.f) * d[2] + (2.f / 3.f) * (d[3] - d[4]);
+        const float m8 = (2.f / 9.f) * f[0] - (4.f / 9.f) * (s[1] + s[2]) + (8.f / 9.f) * (s[3] + s[4]);
+        g6 = gg * m6 * 13.5f;          // 1/b = 27/2
+        g7 = gg * m7 * 13.5f;
+        g8 = gg * m8 * (81.f / 16.f);  // 1/b = 81/16
+    }
+    if (a.kT > 0.f) {
+        const float sq = sqrtf(3.0f * rho * a.kT);
+        float n[6];
+#pragma unroll
+        for (int t = 0; t < 6; ++t) n[t] = sq * a.namp[t] * G[t];
+        const float two9 = 2.0f / 9.0f;
+        Bxx += two9 * (n[0] + n[1]);
+        Byy += two9 * (n[0] - n[1]);
+        Bxy += (1.0f / 9.0f) * n[2];
+        g6 += n[3];
+        g7 += n[4];
+        g8 += n[5];
+    }
+    const float e0 = 1.5f * (Bxx + Byy);  // 9/2 trB/3
+    stp(fo + site, (4.f / 9.f) * (drho - e0 + (2.f / 9.f) * g8));
+    const float w1 = 1.f / 9.f, w2 = 1.f / 36.f;
+    float E, O;
+    E = drho + 4.5f * Bxx - e0 - (4.f / 9.f) * g8;
+    O = 3.f * Ax - (1.f / 3.f) * g6;
+    stp(fo + 1 * N + site, w1 * (E + O));
+    stp(fo + 2 * N + site, w1 * (E - O));
+    E = drho + 4.5f * Byy - e0 - (4.f / 9.f) * g8;
+    O = 3.f * Ay - (1.f / 3.f) * g7;
+    stp(fo + 3 * N + site, w1 * (E + O));
+    stp(fo + 4 * N + site, w1 * (E - O));
+    E = drho + 4.5f * (Bxx + Byy + 2.f * Bxy) - e0 + (8.f / 9.f) * g8;
+    O = 3.f * (Ax + Ay) + (2.f / 3.f) * (g6 + g7);
+    stp(fo + 5 * N + site, w2 * (E + O));
+    stp(fo + 6 * N + site, w2 * (E - O));
+    E = drho + 4.5f * (Bxx + Byy - 2.f * Bxy) - e0 + (8.f / 9.f) * g8;
+    O = 3.f * (Ax - Ay) + (2.f / 3.f) * (g6 - g7);
+    stp(fo + 7 * N + site, w2 * (E + O));
+    stp(fo + 8 * N + site, w2 * (E - O));
+}
+
 // V = F2: a thread works the sites (x, y) and (x, y + TY/2) in packed FP32.
 template <int TX, int TY, class V, typename T, bool GHOST_RELAX>
 __global__ void __launch_bounds__(TX *TY / V::L) lb2_kernel(const LBArgs a, const Psi2Args p)
@@ -255,8 +343,13 @@ __global__ void __launch_bounds__(TX *TY / V::L) lb2_kernel(const LBArgs a, cons
         s[l] = (uint32_t)(xc + g.nx * yc[l]);
     }
     pdl_trigger();
+    constexpr bool F16 = sizeof(T) == 2;
     V n[6];  // unit normals, drawn while the kernel before this one ends
-    if (a.kT > 0.f) lane_block<6, false>(a.key, a.step, s, 0u, V::bc(1.0f), n);
+    float G[6];
+    if (a.kT > 0.f) {
+        if constexpr (F16) normals<3, false, false, true>(a.key, a.step, s[0], 0u, 0u, G);
+        else lane_block<6, false>(a.key, a.step, s, 0u, V::bc(1.0f), n);
+    }
     pdl_wait();
     V f[9];  // in flight while mu is formed
     {
@@ -287,7 +380,15 @@ __global__ void __launch_bounds__(TX *TY / V::L) lb2_kernel(const LBArgs a, cons
                                Fx[l], Fy[l]);
         }
     }
-    collide9<V, T, GHOST_RELAX>(a, s, ok, f, n, vmake<V>(Fx), vmake<V>(Fy));
+    if constexpr (F16) {
+        static_assert(!F16 || L == 1, "one site per thread");
+        float f1[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) f1[i] = f[i].lane(0);
+        if (ok[0]) collide9_f16<GHOST_RELAX>(a, s[0], f1, G, Fx[0], Fy[0]);
+    } else {
+        collide9<V, T, GHOST_RELAX>(a, s, ok, f, n, vmake<V>(Fx), vmake<V>(Fy));
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -302,12 +403,13 @@ __global__ void __launch_bounds__(TX *TY / V::L) lb2_kernel(const LBArgs a, cons
 //       (1,0), (0,1), (1,1), (1,-1), a_l the Laplacian's axis and diagonal weights;
 //   FV: the divergence above of xi, two N(0, 2 kT M) per node;
 //   naive (Sec. III): (1/2) sum_a [xi_a(r + e_a) - xi_a(r - e_a)].
-// s1 holds u psi (FD) or J (FV) on tile + 1, sz the normals there.
+// s1 holds u (FD) or J (FV) on tile + 1, sz the normals there.
 // ---------------------------------------------------------------------------
 template <int TX, int TY, int NT, typename T, bool FV, bool FIRST, bool NOISE>
 __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
 {
     static_assert(FIRST || !NOISE, "the noise is drawn in the first stage");
+    constexpr bool F16 = sizeof(T) == 2;  // see collide9_f16
     constexpr int MH = FIRST || FV ? 2 : 1, PH = MH + 1;          // mu and psi regions: tile + MH, + PH
     constexpr int W1 = TX + 2, N1 = W1 * (TY + 2);
     constexpr int WM = TX + 2 * MH, NM = WM * (TY + 2 * MH), WP = TX + 2 * PH, NP = WP * (TY + 2 * PH);
@@ -333,7 +435,7 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
             int lx, ly;
             if (!point(k, lx, ly)) continue;
             float G[4];
-            normals<2>(a.key, a.step, (uint32_t)(wrapi(x0 + lx, g.nx) + g.nx * wrapi(y0 + ly, g.ny)), 1u, 0u, G);
+            normals<2, false, false, F16>(a.key, a.step, (uint32_t)(wrapi(x0 + lx, g.nx) + g.nx * wrapi(y0 + ly, g.ny)), 1u, 0u, G);
 #pragma unroll
             for (int t = 0; t < NZ; ++t) sz[t * N1 + k] = G[t];
         }
@@ -400,14 +502,25 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
             uy = uxy[j][1];
         }
         const float px = advect ? ux * ps : 0.f, py = advect ? uy * ps : 0.f;
-        if (FV) {
+        if (FV && F16) {
+            float gx = 0.f, gy = 0.f;
+#pragma unroll
+            for (int l = 0; l < 8; ++l) {
+                const float m = __fmul_rn(l < 4 ? 1.f / 9.f : 1.f / 36.f, smu[cm + kLink9[l][0] + WM * kLink9[l][1]]);
+                gx = __fmaf_rn((float)kLink9[l][0], m, gx);
+                gy = __fmaf_rn((float)kLink9[l][1], m, gy);
+            }
+            const float m3 = 3.f * a.M, jx = __fmul_rn(m3, gx), jy = __fmul_rn(m3, gy);
+            s1[k] = advect ? __fmaf_rn(-ux, ps, jx) : jx;
+            s1[N1 + k] = advect ? __fmaf_rn(-uy, ps, jy) : jy;
+        } else if (FV) {
             const float dx = smu[cm + 1] - smu[cm - 1], dy = smu[cm + WM] - smu[cm - WM];
             const float pp = smu[cm + 1 + WM], pm = smu[cm + 1 - WM], mp = smu[cm - 1 + WM], mm = smu[cm - 1 - WM];
             s1[k] = a.M * ((1.f / 12.f) * (4.f * dx + ((pp + pm) - (mp + mm)))) - px;
             s1[N1 + k] = a.M * ((1.f / 12.f) * (4.f * dy + ((pp - pm) + (mp - mm)))) - py;
         } else {
-            s1[k] = px;
-            s1[N1 + k] = py;
+            s1[k] = ux;
+            s1[N1 + k] = uy;
         }
     }
     __syncthreads();
@@ -425,16 +538,41 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
         const int tx = k % TX, ty = k / TX, x = x0 + tx, y = y0 + ty;
         if (k >= TX * TY || x >= g.nx || y >= g.ny) continue;
         const int c = (tx + 1) + W1 * (ty + 1);
+        const int cp = (tx + PH) + WP * (ty + PH);
         float D, eta = 0.f;
-        if (FV) {
+        if (FV && F16) {
+            const float *vy = s1 + N1;
+            float acc = 0.f;
+#pragma unroll
+            for (int l = 0; l < 8; ++l) {
+                const int o = c + kLink9[l][0] + W1 * kLink9[l][1];
+                const float cx = kLink9[l][0], cy = kLink9[l][1];
+                const float lx = __fadd_rn(s1[c], s1[o]), ly = __fadd_rn(vy[c], vy[o]);
+                acc = __fmaf_rn(l < 4 ? 1.f / 9.f : 1.f / 36.f, __fmaf_rn(cx, lx, cy * ly), acc);
+            }
+            D = __fmul_rn(3.f, acc);
+        } else if (FV) {
             D = div_fv(s1, c);
         } else {
-            const float *py = s1 + N1;
-            D = a.M * lap2<WM>(smu, (tx + MH) + WM * (ty + MH), a.lw) -
-                0.5f * ((s1[c + 1] - s1[c - 1]) + (py[c + W1] - py[c - W1]));
+            D = a.M * lap2<WM>(smu, (tx + MH) + WM * (ty + MH), a.lw);
+            if (advect) {
+                const float *v = s1 + N1;
+                float adv = s1[c + 1] * sps[cp + 1] - s1[c - 1] * sps[cp - 1];
+                adv += v[c + W1] * sps[cp + WP] - v[c - W1] * sps[cp - WP];
+                D -= 0.5f * adv;
+            }
         }
         if (NOISE) {
-            if (FV) {
+            if (FV && F16) {
+                const float *zx = sz, *zy = sz + N1;
+                const float ox = zx[c], oy = zy[c];
+                const float ax = ((ox + zx[c + 1]) - (ox + zx[c - 1])) + ((oy + zy[c + W1]) - (oy + zy[c - W1]));
+                const float dg = ((ox + zx[c + W1 + 1]) + (oy + zy[c + W1 + 1])) -
+                                 ((ox + zx[c - W1 - 1]) + (oy + zy[c - W1 - 1])) +
+                                 ((ox + zx[c - W1 + 1]) - (oy + zy[c - W1 + 1])) -
+                                 ((ox + zx[c + W1 - 1]) - (oy + zy[c + W1 - 1]));
+                eta = 3.f * a.amp[0] * ((1.f / 9.f) * ax + (1.f / 36.f) * dg);
+            } else if (FV) {
                 eta = a.amp[0] * div_fv(sz, c);
             } else if (a.scheme == FLB_NAIVE) {
                 eta = 0.5f * a.amp[0] * ((sz[c + 1] - sz[c - 1]) + (sz[N1 + c + W1] - sz[N1 + c - W1]));
@@ -444,7 +582,7 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
             }
         }
         const int site = x + g.nx * y;
-        const float ps = sps[(tx + PH) + WP * (ty + PH)];
+        const float ps = sps[cp];
         float out;
         if (a.integrator == FLB_RK4) {  // k_s = D_s + eta with eta fixed over the step
             if (FIRST) {
@@ -494,30 +632,30 @@ cudaError_t tile_psi2(const Psi2Args &a, cudaStream_t st)
 template <bool FV>
 cudaError_t scheme_psi2(const Psi2Args &a, int storage, bool noise, cudaStream_t st)
 {
-    if (a.stage > 1) return tile_psi2<float, FV, false, false>(a, st);  // reads no populations
-    if (storage == FLB_F16_DEV)
+    if (storage == FLB_F16_DEV) {
+        if (a.stage > 1) return tile_psi2<__half, FV, false, false>(a, st);
         return noise ? tile_psi2<__half, FV, true, true>(a, st) : tile_psi2<__half, FV, true, false>(a, st);
+    }
+    if (a.stage > 1) return tile_psi2<float, FV, false, false>(a, st);
     return noise ? tile_psi2<float, FV, true, true>(a, st) : tile_psi2<float, FV, true, false>(a, st);
 }
 
-template <int TX, int TY, class V>
-cudaError_t go_lb2(const LBArgs &a, const Psi2Args &p, int storage, cudaStream_t st)
+template <int TX, int TY, class V, typename T>
+cudaError_t go_lb2(const LBArgs &a, const Psi2Args &p, cudaStream_t st)
 {
     constexpr int NT = TX * TY / V::L;
     const dim3 grid((a.g.nx + TX - 1) / TX, (a.g.ny + TY - 1) / TY);
-    const bool gr = a.gamma_g != 0.0f;
-    if (storage == FLB_F16_DEV)
-        return gr ? launch_pdl(lb2_kernel<TX, TY, V, __half, true>, grid, NT, 0, st, PDL_BLOCKS2, a, p)
-                  : launch_pdl(lb2_kernel<TX, TY, V, __half, false>, grid, NT, 0, st, PDL_BLOCKS2, a, p);
-    return gr ? launch_pdl(lb2_kernel<TX, TY, V, float, true>, grid, NT, 0, st, PDL_BLOCKS2, a, p)
-              : launch_pdl(lb2_kernel<TX, TY, V, float, false>, grid, NT, 0, st, PDL_BLOCKS2, a, p);
+    return a.gamma_g != 0.0f ? launch_pdl(lb2_kernel<TX, TY, V, T, true>, grid, NT, 0, st, PDL_BLOCKS2, a, p)
+                             : launch_pdl(lb2_kernel<TX, TY, V, T, false>, grid, NT, 0, st, PDL_BLOCKS2, a, p);
 }
 
 }  // namespace
 
 cudaError_t launch_lb2(const LBArgs &a, const Psi2Args &p, int storage, cudaStream_t st)
 {
-    return small_box2(a.g) ? go_lb2<16, 8, F1>(a, p, storage, st) : go_lb2<32, 16, F2>(a, p, storage, st);
+    if (storage == FLB_F16_DEV)
+        return small_box2(a.g) ? go_lb2<16, 8, F1, __half>(a, p, st) : go_lb2<32, 8, F1, __half>(a, p, st);
+    return small_box2(a.g) ? go_lb2<16, 8, F1, float>(a, p, st) : go_lb2<32, 16, F2, float>(a, p, st);
 }
 
 cudaError_t launch_psi2(const Psi2Args &a, int storage, bool noise, cudaStream_t st)
