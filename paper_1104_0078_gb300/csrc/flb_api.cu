@@ -102,6 +102,11 @@ struct Rep {
     int fused = 0;   // single-pass Heun psi step (flb_set_psi_fused)
 };
 
+// Parts of the batched block lists: first entry and number of each.
+struct BatchSpan {
+    int mu = 0, nmu = 0, lb = 0, nlb = 0, psi = 0, npsi = 0;
+};
+
 struct Carver {
     char *base;
     size_t off = 0;
@@ -301,6 +306,7 @@ struct flb_handle {
     BatchRep *b_reps = nullptr;
     BatchBlock *b_mu = nullptr, *b_lb = nullptr, *b_psi = nullptr;
     int b_nmu = 0, b_nlb = 0, b_npsi = 0, b_npsi_cap = 0;
+    std::vector<BatchSpan> b_span;  // the lists' parts, one per replica group (batch_groups)
     long long *b_dstep = nullptr;
     std::vector<BatchRep> b_host;
     std::vector<BatchBlock> b_blocks_host;
@@ -367,8 +373,7 @@ size_t carve_all(flb_handle &h, char *base)
     for (Rep &r : h.reps) {
         if (r.dim != 3) continue;
         const Geom &g = r.g;
-        constexpr int E = 2 * MU3_HALO;
-        nmu += ((g.nx + E + MU_BX - 1) / MU_BX) * ((g.ny + E + MU_BY - 1) / MU_BY) * ((g.nz + E + MU_ZC - 1) / MU_ZC);
+        for_mu_blocks(g, [&](int, int, int) { ++nmu; });
         nlb += packed_blocks(pair_geom(g), LBB_NT);
         npsi += ((g.nx + PS_TX - 1) / PS_TX) * ((g.ny + PS_TY - 1) / PS_TY) * ((g.nz + PS_ZC_MIN - 1) / PS_ZC_MIN);
     }
@@ -834,39 +839,73 @@ void batch_depths(flb_handle *h)
     for (Rep &r : h->reps) r.bzc = r.btuned ? r.zc : split(r.g.nz, best);
 }
 
+// The replicas of a batched step in groups of about equal site counts (largest boxes dealt
+// first).  A group's kernels form a chain of their own in the graph, so the last
+// blocks of one group's kernel and the memory-bound velocity run beside the other group's work:
+// two groups took a step of 256 replicas of 16^3 to 48^3 from 1105 to 1086 us, of 160 of 30^3 from
+// 530 to 510, of 25 of 32^3 from 118 to 115 (three, four and eight groups: as two or
+// slower).  Below 600 thousand sites a kernel's own latency is what it costs, and twice as many
+// kernels are slower: 8 of 16^3 49.7 and 53.4 us, 2 of 48^3 62 and 66.
+std::vector<std::vector<int>> batch_groups(const flb_handle *h)
+{
+    const int n = (int)h->reps.size();
+    long long total = 0;
+    for (const Rep &r : h->reps) total += r.g.n;
+    const int G = n > 1 && total >= 600000 ? 2 : 1;
+    std::vector<int> order((size_t)n);
+    for (int r = 0; r < n; ++r) order[(size_t)r] = r;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return h->reps[(size_t)a].g.n > h->reps[(size_t)b].g.n; });
+    std::vector<std::vector<int>> groups((size_t)G);
+    std::vector<long long> sites((size_t)G, 0);
+    for (int r : order) {
+        const size_t k = (size_t)(std::min_element(sites.begin(), sites.end()) - sites.begin());
+        groups[k].push_back(r);
+        sites[k] += h->reps[(size_t)r].g.n;
+    }
+    for (auto &v : groups) std::sort(v.begin(), v.end());
+    return groups;
+}
+
 int batch_upload_lists(flb_handle *h)
 {
     batch_depths(h);
+    const std::vector<std::vector<int>> groups = batch_groups(h);
+    std::vector<BatchSpan> span(groups.size());
     std::vector<BatchBlock> &v = h->b_blocks_host;
     v.clear();
-    for (int r = 0; r < (int)h->reps.size(); ++r) {
-        const Geom &g = h->reps[(size_t)r].g;
-        constexpr int E = 2 * MU3_HALO;
-        for (int bz = 0; bz < (g.nz + E + MU_ZC - 1) / MU_ZC; ++bz)
-            for (int by = 0; by < (g.ny + E + MU_BY - 1) / MU_BY; ++by)
-                for (int bx = 0; bx < (g.nx + E + MU_BX - 1) / MU_BX; ++bx) v.push_back({r, bx, by, bz});
-    }
-    const size_t nmu = v.size();
-    for (int r = 0; r < (int)h->reps.size(); ++r)  // row-packed collide-stream / velocity blocks
-        for_packed_blocks(pair_geom(h->reps[(size_t)r].g), LBB_NT,
-                          [&](int x0, int y0, int z0) { v.push_back({r, x0, y0, z0}); });
-    const size_t nlb = v.size() - nmu;
-    for (int r = 0; r < (int)h->reps.size(); ++r) {
-        const Geom &g = h->reps[(size_t)r].g;
+    // one list after the other, its entries in group order; returns the list's length
+    auto list = [&](int BatchSpan::*first, int BatchSpan::*count, auto blocks) {
+        const size_t base = v.size();
+        for (size_t k = 0; k < groups.size(); ++k) {
+            span[k].*first = (int)(v.size() - base);
+            for (int r : groups[k]) blocks(r, h->reps[(size_t)r].g);
+            span[k].*count = (int)(v.size() - base) - span[k].*first;
+        }
+        return v.size() - base;
+    };
+    const size_t nmu = list(&BatchSpan::mu, &BatchSpan::nmu, [&](int r, const Geom &g) {
+        for_mu_blocks(g, [&](int k, int zb, int ze) { v.push_back({r, k, zb, ze}); });
+    });
+    const size_t nlb = list(&BatchSpan::lb, &BatchSpan::nlb, [&](int r, const Geom &g) {  // row-packed collide-stream / velocity blocks
+        for_packed_blocks(pair_geom(g), LBB_NT, [&](int x0, int y0, int z0) { v.push_back({r, x0, y0, z0}); });
+    });
+    const size_t npsi = list(&BatchSpan::psi, &BatchSpan::npsi, [&](int r, const Geom &g) {
         const int zc = h->reps[(size_t)r].bzc;
         for (int bz = 0; bz < (g.nz + zc - 1) / zc; ++bz)
             for (int by = 0; by < (g.ny + PS_TY - 1) / PS_TY; ++by)
                 for (int bx = 0; bx < (g.nx + PS_TX - 1) / PS_TX; ++bx) v.push_back({r, bx, by, bz});
-    }
-    const size_t npsi = v.size() - nmu - nlb;
+    });
     // longest z chunks first: the block scheduler then ends the launch on short
     // blocks instead of starting a long one last
     auto planes = [&](const BatchBlock &b) {
         const Rep &r = h->reps[(size_t)b.rep];
         return std::min(r.bzc, r.g.nz - b.bz * r.bzc);
     };
-    std::stable_sort(v.begin() + (std::ptrdiff_t)(nmu + nlb), v.end(),
-                     [&](const BatchBlock &a, const BatchBlock &b) { return planes(a) > planes(b); });
+    for (const BatchSpan &s : span) {
+        const auto p = v.begin() + (std::ptrdiff_t)(nmu + nlb + (size_t)s.psi);
+        std::stable_sort(p, p + s.npsi, [&](const BatchBlock &a, const BatchBlock &b) { return planes(a) > planes(b); });
+    }
+    h->b_span = span;
     if ((int)nmu != h->b_nmu || (int)nlb != h->b_nlb || (int)npsi > h->b_npsi_cap) return FLB_EINVAL;
     h->b_npsi = (int)npsi;
     int rc = cuerr(cudaMemcpyAsync(h->b_mu, v.data(), nmu * sizeof(BatchBlock), cudaMemcpyHostToDevice, h->st));
@@ -945,7 +984,7 @@ int batch_kernels_per_step(const flb_handle *h)
     bool force = false;
     for (const Rep &r : h->reps) force |= (r.p.coupling & FLB_COUPLE_FORCE) != 0;
     // mu (when any replica is forced), collide-stream, velocity, psi stage(s), step counter
-    return (force ? 1 : 0) + 1 + 1 + 1 + (p.integrator == FLB_HEUN ? 1 : 0) + 1;
+    return (int)h->b_span.size() * ((force ? 1 : 0) + 1 + 1 + 1 + (p.integrator == FLB_HEUN ? 1 : 0)) + 1;
 }
 
 // Every replica's step forms mu of psi^n for its force, so the batched FV
@@ -970,13 +1009,46 @@ int batch_capture(flb_handle *h)
     }
     const flb_params &p0 = h->reps[0].p;
     const BatchLists L = batch_lists(h);
-    // the kernels' attributes are set by one launch outside the capture on a zero-block list
+    const size_t G = h->b_span.size();
+    std::vector<cudaStream_t> side(G, h->st);
+    std::vector<cudaEvent_t> ev(G, nullptr);
+    auto drop = [&]() {
+        for (size_t k = 0; k < G; ++k) {
+            if (k && side[k] && side[k] != h->st) cudaStreamDestroy(side[k]);
+            if (ev[k]) cudaEventDestroy(ev[k]);
+        }
+    };
+    for (size_t k = 0; k < G; ++k)
+        if ((k && cudaStreamCreateWithFlags(&side[k], cudaStreamNonBlocking) != cudaSuccess) ||
+            cudaEventCreateWithFlags(&ev[k], cudaEventDisableTiming) != cudaSuccess) {
+            drop();
+            return FLB_ECUDA;
+        }
     cudaGraph_t gr = nullptr;
-    if (cudaStreamBeginCapture(h->st, cudaStreamCaptureModeRelaxed) != cudaSuccess) return FLB_ECUDA;
-    const cudaError_t e =
-        launch_batch_step(L, p0.storage, ghost, force, 1, p0.integrator == FLB_HEUN, noise, batch_mu_in(h),
-                          h->reps[0].q == 15, h->st);
+    if (cudaStreamBeginCapture(h->st, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
+        drop();
+        return FLB_ECUDA;
+    }
+    cudaError_t e = cudaEventRecord(ev[0], h->st);
+    for (size_t k = 0; k < G && e == cudaSuccess; ++k) {
+        const BatchSpan &s = h->b_span[k];
+        BatchLists P = L;
+        P.mu += s.mu;
+        P.lb += s.lb;
+        P.psi += s.psi;
+        P.nmu = s.nmu;
+        P.nlb = s.nlb;
+        P.npsi = s.npsi;
+        if (k) e = cudaStreamWaitEvent(side[k], ev[0], 0);
+        if (e == cudaSuccess)
+            e = launch_batch_step(P, p0.storage, ghost, force, 1, p0.integrator == FLB_HEUN, noise, batch_mu_in(h),
+                                  h->reps[0].q == 15, side[k]);
+        if (k && e == cudaSuccess) e = cudaEventRecord(ev[k], side[k]);
+    }
+    for (size_t k = 1; k < G && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(h->st, ev[k], 0);
+    if (e == cudaSuccess) e = launch_batch_advance(L, h->st);
     const cudaError_t e2 = cudaStreamEndCapture(h->st, &gr);
+    drop();
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (gr) cudaGraphDestroy(gr);
         return FLB_ECUDA;

@@ -99,15 +99,10 @@ __global__ void __launch_bounds__(MU_BX *MU_BY) mu3_kernel(const Geom g, const f
 // per SM (64^3 has 90 blocks of 16 planes).
 constexpr int MV_TX = 16, MV_TY = 8, MV_ZC = 16, MV_ZC_SMALL = 4;
 
-__global__ void __launch_bounds__(MV_TX *MV_TY) mu3_vec_kernel(const Geom g, const float *__restrict__ psi,
-                                                             float *__restrict__ mu, float A, float B, float K,
-                                                             int zc)
+// planes zb .. ze - 1 of the columns xs .. xs + 3 at y
+__device__ __forceinline__ void mu3_quad(const Geom &g, const float *__restrict__ psi, float *__restrict__ mu, float A,
+                                         float B, float K, int xs, int y, int zb, int ze)
 {
-    pdl_trigger();
-    pdl_wait();
-    const int xs = -4 + 4 * (int)(blockIdx.x * MV_TX + threadIdx.x);
-    const int y = (int)(blockIdx.y * MV_TY + threadIdx.y) - MU3_HALO;
-    const int zb = (int)blockIdx.z * zc - MU3_HALO, ze = min(zb + zc, g.nz + MU3_HALO);
     const int xl = g.nx + MU3_HALO;  // one past the last output column
     if (xs + 3 < -MU3_HALO || xs >= xl || y >= g.ny + MU3_HALO || zb >= ze) return;
     const bool lo = xs - 1 >= -MU3_HALO - 1, hi = xs + 4 <= xl;  // side cells some point needs
@@ -144,21 +139,39 @@ __global__ void __launch_bounds__(MV_TX *MV_TY) mu3_vec_kernel(const Geom g, con
     }
 }
 
+__global__ void __launch_bounds__(MV_TX *MV_TY) mu3_vec_kernel(const Geom g, const float *__restrict__ psi,
+                                                             float *__restrict__ mu, float A, float B, float K,
+                                                             int zc)
+{
+    pdl_trigger();
+    pdl_wait();
+    const int zb = (int)blockIdx.z * zc - MU3_HALO;
+    mu3_quad(g, psi, mu, A, B, K, -4 + 4 * (int)(blockIdx.x * MV_TX + threadIdx.x),
+             (int)(blockIdx.y * MV_TY + threadIdx.y) - MU3_HALO, zb, min(zb + zc, g.nz + MU3_HALO));
+}
+
 // ---- batched variants: block b of the launch works on L.mu[b] / L.lb[b] -------
-__global__ void __launch_bounds__(MU_BX *MU_BY) mu3_batch_kernel(const BatchLists L)
+// The fours of x of all rows of a box (mu_row_quads a row) form one list; entry b holds MUB_NT of
+// them from b.bx on and the planes b.by .. b.bz - 1.
+__global__ void __launch_bounds__(MUB_NT) mu3_batch_kernel(const BatchLists L)
 {
     const BatchBlock b = L.mu[blockIdx.x];
     const BatchRep &r = L.reps[b.rep];
     const int par = (int)(*L.dstep & 1);
-    if (r.lb.force_kind == 2) {  // stress form: sigma instead of mu
-        const Geom &g = r.lb.g;
-        const int x = b.bx * MU_BX + (int)threadIdx.x - 1, y = b.by * MU_BY + (int)threadIdx.y - 1;
-        const int zb = b.bz * MU_ZC - 1, ze = min(zb + MU_ZC, g.nz + 1);
-        if (x <= g.nx && y <= g.ny && zb < ze)
-            sigma3_column<false>(g, r.psi[par], const_cast<float *>(r.lb.sig), r.A, r.B, r.K, x, y, zb, ze);
+    const Geom &g = r.lb.g;
+    const int nq = mu_row_quads(g);
+    if (r.lb.force_kind == 2) {  // stress form: sigma instead of mu, one column after the other
+        const int zb = max(b.by, -1), ze = min(b.bz, g.nz + 1);
+        for (int j = 0; j < 4; ++j) {
+            const int p = j * MUB_NT + (int)threadIdx.x, k = b.bx + p / 4;
+            const int x = -4 + 4 * (k % nq) + p % 4, y = k / nq - MU3_HALO;
+            if (x >= -1 && x <= g.nx && y >= -1 && y <= g.ny && zb < ze)
+                sigma3_column<false>(g, r.psi[par], const_cast<float *>(r.lb.sig), r.A, r.B, r.K, x, y, zb, ze);
+        }
         return;
     }
-    mu3_block<MU3_HALO>(r.lb.g, r.psi[par], const_cast<float *>(r.lb.mu), r.A, r.B, r.K, b.bx, b.by, b.bz);
+    const int k = b.bx + (int)threadIdx.x;
+    mu3_quad(g, r.psi[par], const_cast<float *>(r.lb.mu), r.A, r.B, r.K, -4 + 4 * (k % nq), k / nq - MU3_HALO, b.by, b.bz);
 }
 
 // site pairs of the collide-stream's list, in packed FP32
@@ -211,7 +224,7 @@ cudaError_t launch_vel3(const LBArgs &a, int storage, cudaStream_t st)
 
 cudaError_t launch_mu3_batch(const BatchLists &L, cudaStream_t st)
 {
-    if (L.nmu > 0) mu3_batch_kernel<<<L.nmu, dim3(MU_BX, MU_BY, 1), 0, st>>>(L);
+    if (L.nmu > 0) mu3_batch_kernel<<<L.nmu, MUB_NT, 0, st>>>(L);
     return cudaGetLastError();
 }
 

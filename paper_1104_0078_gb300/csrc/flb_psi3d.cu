@@ -105,8 +105,11 @@ cudaError_t launch_batch_step(const BatchLists &L, int storage, bool ghost, bool
     cudaError_t e = q15 ? launch_lb15_batch(L, storage, ghost, force, st)
                         : launch_lb3_batch(L, storage, ghost, force, st);
     if (e != cudaSuccess) return e;
-    e = launch_batch_psi(L, heun, noise, mu_in, q15, st);
-    if (e != cudaSuccess) return e;
+    return launch_batch_psi(L, heun, noise, mu_in, q15, st);
+}
+
+cudaError_t launch_batch_advance(const BatchLists &L, cudaStream_t st)
+{
     advance_kernel<<<1, 1, 0, st>>>(const_cast<long long *>(L.dstep));
     return cudaGetLastError();
 }

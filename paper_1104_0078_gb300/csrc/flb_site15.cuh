@@ -239,9 +239,7 @@ __device__ __forceinline__ void vel15_site_on(const LBArgs &a, const PL &P, int 
     float Fx = 0.f, Fy = 0.f, Fz = 0.f;
     if (FORCE && (a.coupling & FLB_COUPLE_FORCE)) force3<COH>(a, x, y, z, Fx, Fy, Fz);
     const float irho = __fdividef(1.0f, a.rho0 + drho);
-    store_padded(a.u, g, x, y, z, (jx + 0.5f * Fx) * irho, 1);
-    store_padded(a.u + g.pn, g, x, y, z, (jy + 0.5f * Fy) * irho, 1);
-    store_padded(a.u + 2 * g.pn, g, x, y, z, (jz + 0.5f * Fz) * irho, 1);
+    store_velocity(a.u, g, x, y, z, (jx + 0.5f * Fx) * irho, (jy + 0.5f * Fy) * irho, (jz + 0.5f * Fz) * irho);
 }
 
 // The same with the populations pulled from the planes P.in (COH: loads through L2,

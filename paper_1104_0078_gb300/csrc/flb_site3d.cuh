@@ -513,9 +513,7 @@ __device__ __forceinline__ void vel3_sites(const LBArgs &a, const PL &P, int x, 
 #pragma unroll
     for (int l = 0; l < L; ++l) {
         if (l >= nl) break;
-        store_padded(a.u, g, x, y, zl[l], ux.lane(l), 1);
-        store_padded(a.u + g.pn, g, x, y, zl[l], uy.lane(l), 1);
-        store_padded(a.u + 2 * g.pn, g, x, y, zl[l], uz.lane(l), 1);
+        store_velocity(a.u, g, x, y, zl[l], ux.lane(l), uy.lane(l), uz.lane(l));
     }
 }
 

@@ -114,3 +114,27 @@ def test_read_of_a_large_field(shape):
     p, v = s.get_psi_u()
     assert np.array_equal(p, psi)
     assert np.array_equal(v, u)
+
+
+@pytest.mark.parametrize("q", [19, 15])
+@pytest.mark.parametrize("extra", [{}, dict(force_grad=3), dict(storage=F.FLB_F16_DEV), dict(coupling=2)])
+def test_batched_in_two_groups_equals_plain(q, extra):
+    # above 600 thousand sites a batched step runs as two chains of kernels; with boxes whose
+    # padded rows end within and at a group of four x
+    shapes = [(84, 84, 70), (60, 61, 37), (4, 5, 6), (17, 9, 5), (33, 7, 70)]
+    ds = [{**BASE, "q": q, "nx": nx, "ny": ny, "nz": nz, "seed": 40 + r, **extra}
+          for r, (nx, ny, nz) in enumerate(shapes)]
+    assert sum(nx * ny * nz for nx, ny, nz in shapes) >= 600000
+    runs = []
+    for mode in (F.FLB_MODE_PLAIN, F.FLB_MODE_BATCHED):
+        s = F.Solver([flb_params(d) for d in ds])
+        for r, d in enumerate(ds):
+            N = d["nx"] * d["ny"] * d["nz"]
+            s.set_fields(rep=r, psi=I.random_field(N, 0.05, 8 + r))
+            s.set_populations(weights_column(q) + I.random_deviations(q, N, 2e-3, 7 + r), rep=r)
+        s.set_mode(mode)
+        s.step(5)
+        runs.append([(s.get_populations(r), *s.get_psi_u(r)) for r in range(len(ds))])
+    for ra, rb in zip(*runs):
+        for a, b in zip(ra, rb):
+            assert np.array_equal(a, b)
