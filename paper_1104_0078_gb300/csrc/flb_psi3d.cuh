@@ -192,16 +192,13 @@ __device__ __forceinline__ void psi3_fv_tma_block(const CUtensorMap *psi_map, co
     const int z1 = min(z0 + a.zc, g.nz);
     const int x = x0 + tx;
     int yl[L];
-    bool act[L], inner[L];
-    int coff[L];
+    bool act[L];
+    Column3 col[L];
 #pragma unroll
     for (int l = 0; l < L; ++l) {
         yl[l] = y0 + ty + l * (PS_TY / 2);
         act[l] = threadIdx.x < NTO && x < g.nx && yl[l] < g.ny;
-        // the output column has no periodic image within 3 cells in x and y: its
-        // interior planes are stored with one plain store
-        inner[l] = x >= 3 && x < g.nx - 3 && yl[l] >= 3 && yl[l] < g.ny - 3;
-        coff[l] = (x + GX) + g.px * (yl[l] + GY);
+        col[l] = column3(g, x, yl[l]);
     }
     const float k22 = a.K * (1.0f / 22.0f);
     const float sdx = sqrtf(2.0f * a.kT * a.M);
@@ -537,10 +534,7 @@ __device__ __forceinline__ void psi3_fv_tma_block(const CUtensorMap *psi_map, co
                     const int si = x + g.nx * (yl[l] + g.ny * z);
                     if (wE) a.E[si] = Ew.lane(l);
                     if (wN) a.Dn[si] = Dn.lane(l);
-                    if (inner[l] && z >= 3 && z < g.nz - 3)
-                        a.out[coff[l] + g.px * g.py * (z + g.gz)] = out.lane(l);
-                    else
-                        store_padded(a.out, g, x, yl[l], z, out.lane(l), 3);
+                    store_column3(a.out, g, col[l], z, out.lane(l));
                 }
             }
         }
