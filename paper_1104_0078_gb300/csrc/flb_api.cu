@@ -1366,48 +1366,57 @@ int flb_set_populations(flb_handle *h, int32_t rep, const double *f)
 }
 
 // The values [0, n) of dev (n FP32 values on the device) as FP64: the first n0 to d0, the
-// rest to d1.  They come over in chunks of 16 MB into tmp, and from 2^21 values on host
-// threads (one per 2^19, at most 16) convert a chunk while the next is on its way; for fewer
-// their start costs more than they save.  psi and u of 100^3 take 1.2 ms (1.7 with the
-// copy first and then the conversion), of 160^3 2.9 (4.2).
+// rest to d1.  They come over in chunks of COPY_CHUNK values into tmp, a ring of COPY_RING
+// chunks (32 MB in all, which stays in the processor's cache and is not zeroed and faulted in for
+// the size of the box), and from 2^21 values on host threads (one per 2^19, at
+// most 16) convert a chunk while the next is on its way; for fewer their start costs more
+// than they save.  psi and u of 100^3 take 0.7 ms (1.6 with the copy first and then the
+// conversion), of 160^3 3.0 (4.1), of 512^3 54 to 66 in every run, where a stage of the
+// whole field took 42 to 590 from one run to the next.
+constexpr long long COPY_CHUNK = 1 << 21, COPY_RING = 4;
 static int copy_out(cudaStream_t st, const float *dev, long long n, float *tmp, double *d0, long long n0, double *d1)
 {
-    constexpr long long CHUNK = 1 << 22;
-    auto convert = [&](long long a, long long b) {
-        const long long m = std::min(b, n0);
-        for (long long s = a; s < m; ++s) d0[s] = (double)tmp[s];
-        for (long long s = std::max(a, n0); s < b; ++s) d1[s - n0] = (double)tmp[s];
-    };
+    const long long chunks = (n + COPY_CHUNK - 1) / COPY_CHUNK;
     const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
     const long long want = n < (1 << 21) ? 1 : std::min<long long>({n >> 19, (long long)hw, 16});
-    std::atomic<long long> ready{0};  // values in tmp; -1: give up
+    std::atomic<long long> ready{0};  // chunks that have come over; -1: give up
+    std::atomic<long long> done[COPY_RING] = {};  // shares that the threads have converted from each slot
     std::vector<std::thread> pool;
     long long nt = 0;
-    auto work = [&](long long t, long long of) {
-        for (long long a = 0; a < n; a += CHUNK) {
-            const long long b = std::min(a + CHUNK, n);
+    auto convert = [&](long long k, long long t) {  // share t of chunk k
+        const long long c0 = k * COPY_CHUNK, m = std::min(COPY_CHUNK, n - c0);
+        const long long a = c0 + m * t / want, b = c0 + m * (t + 1) / want, h = std::min(b, n0);
+        const float *src = tmp + (k % COPY_RING) * COPY_CHUNK - c0;
+        for (long long s = a; s < h; ++s) d0[s] = (double)src[s];
+        for (long long s = std::max(a, n0); s < b; ++s) d1[s - n0] = (double)src[s];
+    };
+    auto work = [&](long long t) {
+        for (long long k = 0; k < chunks; ++k) {
             long long r;
-            while ((r = ready.load(std::memory_order_acquire)) >= 0 && r < b) std::this_thread::yield();
+            while ((r = ready.load(std::memory_order_acquire)) >= 0 && r <= k) std::this_thread::yield();
             if (r < 0) return;
-            convert(a + (b - a) * t / of, a + (b - a) * (t + 1) / of);
+            convert(k, t);
+            done[k % COPY_RING].fetch_add(1, std::memory_order_release);
         }
     };
     if (want > 1) {
         try {
             pool.reserve((size_t)want);
-            for (; nt < want; ++nt) pool.emplace_back(work, nt, want);
-        } catch (...) {  // no more threads: the missing shares are converted below
+            for (; nt < want; ++nt) pool.emplace_back(work, nt);
+        } catch (...) {  // no more threads: the missing shares are converted here
         }
     }
     int rc = FLB_OK;
-    for (long long a = 0; a < n && rc == FLB_OK; a += CHUNK) {
-        const long long b = std::min(a + CHUNK, n);
-        rc = cuerr(cudaMemcpyAsync(tmp + a, dev + a, (size_t)(b - a) * 4, cudaMemcpyDeviceToHost, st));
+    for (long long k = 0; k < chunks && rc == FLB_OK; ++k) {
+        // the k / COPY_RING chunks that were in the slot are converted
+        while (done[k % COPY_RING].load(std::memory_order_acquire) < nt * (k / COPY_RING)) std::this_thread::yield();
+        const long long c0 = k * COPY_CHUNK;
+        rc = cuerr(cudaMemcpyAsync(tmp + (k % COPY_RING) * COPY_CHUNK, dev + c0,
+                                   (size_t)std::min(COPY_CHUNK, n - c0) * 4, cudaMemcpyDeviceToHost, st));
         if (rc == FLB_OK) rc = cuerr(cudaStreamSynchronize(st));
-        ready.store(rc == FLB_OK ? b : -1, std::memory_order_release);
+        ready.store(rc == FLB_OK ? k + 1 : -1, std::memory_order_release);
+        for (long long t = nt; t < want && rc == FLB_OK; ++t) convert(k, t);
     }
-    if (rc == FLB_OK)
-        for (long long t = nt; t < std::max<long long>(want, 1); ++t) work(t, std::max<long long>(want, 1));
     for (auto &th : pool) th.join();
     return rc;
 }
@@ -1424,7 +1433,8 @@ int flb_get_psi_u(flb_handle *h, int32_t rep, double *psi, double *u)
     const long long n0 = psi ? g.n : 0, n = n0 + (u ? r->dim * g.n : 0);
     const int rc = cuerr(launch_unpad(g, psi ? r->psi[r->pcur] : nullptr, u ? r->u : nullptr, r->dim, scratch, h->st));
     ++h->launches;
-    return rc == FLB_OK ? copy_out(h->st, scratch, n, h->host_stage((size_t)n), psi, n0, u) : rc;
+    return rc == FLB_OK ? copy_out(h->st, scratch, n, h->host_stage((size_t)std::min(n, COPY_RING * COPY_CHUNK)), psi, n0, u)
+                        : rc;
 }
 
 int flb_get_window(flb_handle *h, int32_t rep, int32_t x0, int32_t y0, int32_t z0, int32_t wx, int32_t wy,
