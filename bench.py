@@ -340,9 +340,9 @@ def path_variants(F, I, local, steps, peak, n=512, only=(), autotune=True):
     warm-up steps, inputs larger than L2 at the default n = 512: the FD psi
     scheme, the FP16 storage variant, the RK4 integrator, the stress-form force
     and the D3Q15 lattice (FD) on the n^3 quench; the quench with S(q) and the
-    dynamic S(q, tau) (8 lags) sampled every 10 steps; the per-site general
-    path of the paper's stencil studies: FD with the PK Laplacian, the naive
-    contrast scheme with the CD Laplacian, FV on D3Q15; the single-pass Heun
+    dynamic S(q, tau) (8 lags) sampled every 10 steps; the paper's
+    stencil studies: FD with the PK Laplacian, the naive contrast scheme with
+    the CD Laplacian, FV on D3Q15; the single-pass Heun
     step (both stages in one launch) of the FV and FD schemes; and the D2Q9 path on an
     (8n)^2 quench (same free energy, FD as in the 2D workload).  MLUPS and the
     fraction of the HBM roofline on the algorithmic bytes of that form."""

@@ -137,10 +137,9 @@ extern "C" {
  *                 noise follows it, so FLB_FD keeps the fluctuation-dissipation
  *                 theorem with any of them): FLB_LAP_SO (default), FLB_LAP_CD,
  *                 FLB_LAP_PK or FLB_LAP_LB; 2D takes SO or CD.
- * D3Q19 and D3Q15 with FLB_LAP_SO and FLB_FD or FLB_FV run the tiled 3D
- * kernels; every other 3D combination (another Laplacian, FLB_NAIVE) runs
- * one-thread-per-site stencil kernels that keep mu, the noise increment and
- * the FV flux in HBM, in FLB_MODE_PLAIN only.
+ * Every 3D combination runs fused kernels, one launch per Runge-Kutta stage;
+ * FLB_FV with FLB_LAP_SO also has the z-marching ones (see flb_set_tuning) and
+ * FLB_MODE_BATCHED and FLB_MODE_PERSISTENT.
  */
 typedef struct flb_params {
     int32_t dim, q;
@@ -293,12 +292,16 @@ int flb_set_mode(flb_handle *h, int32_t mode);
 int flb_set_wait_limit(flb_handle *h, double seconds);
 
 /*
- * Tiling of the 3D psi stage.  A psi block owns a 32 x 16 column of sites and
- * marches psi_zchunk planes of it in z (default 64).  Smaller chunks give more
- * blocks (small boxes fill the GPU) at the cost of recomputing the stencil halo
- * of 6 planes per chunk.  The choice changes no result bit: every site's
- * arithmetic is the same.  (A performance knob of this implementation; the
- * paper has no counterpart.)
+ * Tiling of the 3D psi stage (FLB_FV with FLB_LAP_SO; other combinations keep
+ * the value and make no use of it).  A psi block owns a 32 x 16 column of sites
+ * and marches psi_zchunk planes of it in z.  Smaller chunks give more blocks
+ * (small boxes fill the GPU) at the cost of recomputing the stencil halo of 6
+ * planes per chunk.  A replica that was neither set nor tuned reads 64 and takes
+ * what its size calls for: in FLB_MODE_PLAIN small 3D tiles below 1.3 million
+ * sites and an even split of the depth above, in the other modes even splits
+ * that fill the GPU with all replicas' blocks.  The choice changes no result
+ * bit: every site's arithmetic is the same.  (A performance knob of this
+ * implementation; the paper has no counterpart.)
  *
  * flb_get_tuning / flb_set_tuning read / set psi_zchunk of replica rep (-1 sets
  * every replica), 1 <= psi_zchunk <= 4096; EINVAL otherwise.  Setting it drops
@@ -307,7 +310,9 @@ int flb_set_wait_limit(flb_handle *h, double seconds);
  * flb_autotune times the candidates 4, 8, ... (up to the first value that
  * covers the box depth) on the handle's own buffers and keeps the fastest: in
  * FLB_MODE_PLAIN per distinct replica configuration (box, lattice, scheme,
- * integrator, noise, advection) on that replica's psi stages; in
+ * integrator, noise, advection) on that replica's psi stages, the small tiles
+ * included (a cached value is applied with the small tiles below 1.3 million
+ * sites); in
  * FLB_MODE_BATCHED and FLB_MODE_PERSISTENT one value for all replicas on the
  * batched psi launches, then, deepest boxes first, one value per distinct box
  * depth nz over the even splits ceil(nz / k), k = 1..16, the other depths held
@@ -320,8 +325,7 @@ int flb_set_wait_limit(flb_handle *h, double seconds);
  * timing (unless flags has FLB_TUNE_FORCE), new results are appended.  An
  * unreadable or unwritable file only disables the cache.  Synchronising; call
  * with the handle's device current and outside stream capture.  2D replicas and
- * the 3D combinations on one-thread-per-site kernels (see laplacian) are left as
- * they are.
+ * 3D combinations without the z-marching kernels are left as they are.
  */
 int flb_get_tuning(flb_handle *h, int32_t rep, int32_t *psi_zchunk);
 int flb_set_tuning(flb_handle *h, int32_t rep, int32_t psi_zchunk);

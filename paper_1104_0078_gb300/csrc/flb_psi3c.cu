@@ -17,10 +17,10 @@
 // psi, mu, u and E are read through L1 where they are used, without staging: what
 // bounds a small box is the latency of the chain, a large one instruction issue
 // (the FD noise above all: 13 normals on twice the sites).  Heun steps, 64^3 FV: 269 us
-// with one 64-plane chunk per column, 65.6 with the best chunk, 56 here; 32^3 FD
-// 213 (one thread block row marching), 50 with the best chunk, 37 here; 256^3 FD 1832 and 1770;
-// 96^3 FV with the Patra-Karttunen Laplacian 257 with one thread per site and a
-// launch per field, 128 here.
+// with one 64-plane chunk per column, 65.6 with the best chunk, 56 here (38 with the step's
+// launches overlapped); 32^3 FD 213 (one thread block row marching), 50 with the best chunk, 37
+// here (23); 256^3 FD 1832 and 1770 (1573 with the later Box-Muller); 96^3 FV with the
+// Patra-Karttunen Laplacian 257 with one thread per site and a launch per field, 128 here (112).
 //
 // The FV stages take the same explicitly rounded operations in the same order as
 // psi3_fv_tma_block (per-plane partial sums included), so a field has the same bits
