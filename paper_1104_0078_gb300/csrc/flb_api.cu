@@ -839,6 +839,14 @@ void batch_depths(flb_handle *h)
     for (Rep &r : h->reps) r.bzc = r.btuned ? r.zc : split(r.g.nz, best);
 }
 
+// Whether a batched step's kernels are long enough for overlapping them to pay.
+bool batch_large(const flb_handle *h)
+{
+    long long total = 0;
+    for (const Rep &r : h->reps) total += r.g.n;
+    return total >= 600000;
+}
+
 // The replicas of a batched step in groups of about equal site counts (largest boxes dealt
 // first).  A group's kernels form a chain of their own in the graph, so the last
 // blocks of one group's kernel and the memory-bound velocity run beside the other group's work:
@@ -849,9 +857,7 @@ void batch_depths(flb_handle *h)
 std::vector<std::vector<int>> batch_groups(const flb_handle *h)
 {
     const int n = (int)h->reps.size();
-    long long total = 0;
-    for (const Rep &r : h->reps) total += r.g.n;
-    const int G = n > 1 && total >= 600000 ? 2 : 1;
+    const int G = n > 1 && batch_large(h) ? 2 : 1;
     std::vector<int> order((size_t)n);
     for (int r = 0; r < n; ++r) order[(size_t)r] = r;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return h->reps[(size_t)a].g.n > h->reps[(size_t)b].g.n; });
@@ -975,6 +981,9 @@ BatchLists batch_lists(flb_handle *h)
     L.npsi = h->b_npsi;
     L.dstep = h->b_dstep;
     L.status = h->status;
+    // 25 replicas of 32^3 108.5 -> 104.8 us a step (D3Q15 102.7 -> 98.7), 8 of 52^3 165.3 -> 162.2; a
+    // graph of such launches costs more to start: 8 of 16^3 46.4 -> 50.2, 2 of 48^3 57.6 -> 61.6
+    L.pdl_max = batch_large(h) ? PDL_BLOCKS : 0;
     return L;
 }
 

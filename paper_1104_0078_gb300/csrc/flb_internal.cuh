@@ -797,6 +797,7 @@ struct BatchLists {
     int nmu, nlb, npsi;
     const long long *dstep;
     int *status;
+    long long pdl_max;  // launches of at most so many blocks overlap the one before (launch_pdl)
 };
 
 cudaError_t encode_tensor_map_f32(CUtensorMap *map, const void *base, int rank, const uint64_t *dims,
