@@ -292,14 +292,15 @@ int flb_set_mode(flb_handle *h, int32_t mode);
 int flb_set_wait_limit(flb_handle *h, double seconds);
 
 /*
- * Tiling of the 3D psi stage (FLB_FV with FLB_LAP_SO; other combinations keep
- * the value and make no use of it).  A psi block owns a 32 x 16 column of sites
+ * Tiling of the 3D psi stage (FLB_FV with FLB_LAP_SO, and the single-pass step of
+ * flb_set_psi_fused; other combinations keep the value and make no use of it).  A psi block owns a 32 x 16 column of sites
  * and marches psi_zchunk planes of it in z.  Smaller chunks give more blocks
  * (small boxes fill the GPU) at the cost of recomputing the stencil halo of 6
  * planes per chunk.  A replica that was neither set nor tuned reads 64 and takes
  * what its size calls for: in FLB_MODE_PLAIN small 3D tiles below 1.3 million
  * sites and an even split of the depth above, in the other modes even splits
- * that fill the GPU with all replicas' blocks.  The choice changes no result
+ * that fill the GPU with all replicas' blocks, as does the single-pass step with its
+ * own.  The choice changes no result
  * bit: every site's arithmetic is the same.  (A performance knob of this
  * implementation; the paper has no counterpart.)
  *
@@ -312,7 +313,8 @@ int flb_set_wait_limit(flb_handle *h, double seconds);
  * FLB_MODE_PLAIN per distinct replica configuration (box, lattice, scheme,
  * integrator, noise, advection) on that replica's psi stages, the small tiles
  * included (a cached value is applied with the small tiles below 1.3 million
- * sites); in
+ * sites), or on its single-pass step, which keeps a value of its own, where that is
+ * on; in
  * FLB_MODE_BATCHED and FLB_MODE_PERSISTENT one value for all replicas on the
  * batched psi launches, then, deepest boxes first, one value per distinct box
  * depth nz over the even splits ceil(nz / k), k = 1..16, the other depths held
@@ -325,7 +327,7 @@ int flb_set_wait_limit(flb_handle *h, double seconds);
  * timing (unless flags has FLB_TUNE_FORCE), new results are appended.  An
  * unreadable or unwritable file only disables the cache.  Synchronising; call
  * with the handle's device current and outside stream capture.  2D replicas and
- * 3D combinations without the z-marching kernels are left as they are.
+ * 3D combinations that make no use of the value are left as they are.
  */
 int flb_get_tuning(flb_handle *h, int32_t rep, int32_t *psi_zchunk);
 int flb_set_tuning(flb_handle *h, int32_t rep, int32_t psi_zchunk);
@@ -337,8 +339,8 @@ int flb_set_tuning(flb_handle *h, int32_t rep, int32_t psi_zchunk);
  * accumulator stay in shared memory and only psi^n and u are read.  The noise is
  * the two-stage form's (same counters), so both forms give the same step up to
  * FP32 rounding.  Applies to Heun with the SO Laplacian in plain mode: the FV
- * scheme on D3Q19, the FD scheme on either lattice; the z chunk is
- * flb_set_tuning's value.  Errors: EINVAL
+ * scheme on D3Q19, the FD scheme on either lattice; the z chunk is the value set
+ * by flb_set_tuning, or by flb_autotune while it is on.  Errors: EINVAL
  * (NULL handle), EUNSUPPORTED (on != 0 and some replica is not of that kind, or
  * the handle is not in plain mode).  Mode changes (flb_set_mode) turn it off. */
 int flb_set_psi_fused(flb_handle *h, int32_t on);

@@ -72,6 +72,12 @@ const double NORM9[6] = {4.0 / 9, 4.0 / 9, 1.0 / 9, 2.0 / 27, 2.0 / 27, 16.0 / 8
 constexpr long long WIN_MAX = 32768;  // sites of one flb_get_window call
 constexpr int RED_MAX_BLOCKS = 1024;
 
+// Planes per psi block of one form of the step, and whether they were set or tuned.
+struct Depth {
+    int zc = PS_ZC;
+    bool set = false;
+};
+
 struct Rep {
     flb_params p;
     Geom g;
@@ -94,12 +100,12 @@ struct Rep {
     int64_t step = 0;
     float omega_s = 0, omega_b = 0, gamma_g = 0;
     float namp[16] = {0};
-    int zc = PS_ZC;  // planes per psi block (3D), set by flb_set_tuning / flb_autotune
-    bool tuned = false;  // whether it was set (else auto_depth chooses)
+    Depth plain;         // planes per psi block (3D), set by flb_set_tuning / flb_autotune (else auto_depth chooses)
     bool cube = false;   // tuned: the small-tile kernels were faster than any chunk
     bool btuned = false; // whether it was set for the batched and persistent modes
-    int bzc = PS_ZC;     // planes per psi block in those modes: zc when set, else batch_depths()
+    int bzc = PS_ZC;     // planes per psi block in those modes: plain.zc when set, else batch_depths()
     int fused = 0;   // single-pass Heun psi step (flb_set_psi_fused)
+    Depth heun1;     // its depth (else heun1_depth chooses)
 };
 
 // Parts of the batched block lists: first entry and number of each.
@@ -189,26 +195,21 @@ const LapW *app_a_weights(const Rep &r, LapW &w)
     return &w;
 }
 
-// Planes per block of the z-marching psi kernel where neither the caller nor the
-// tuner has chosen, or 0 for the small-tile kernels.  Those are the faster ones up to
-// about 110^3 (a Heun step at 96^3: 123 against 132 us with the best chunk, at 128^3 239
-// against 230 us).  Above, the even split of the depth that costs least with two
-// blocks on each of 152 SMs, a chunk of zc planes taking zc + 8 plane times (its
-// pipeline fills): 128^3 16 planes, 160^3 27, 256 x 256 x 64 32, 512^3 64 (what the
-// tuner finds there); with 64 planes throughout those took 1.6, 1.16, 1.16 times as long.
-int auto_depth(const Geom &g)
+// The even split of a box's depth, into chunks of PS_ZC to `least` planes, that costs least with
+// `slots` blocks at a time on the chip, a chunk of zc planes taking zc + fill plane times
+// (its pipeline fills).
+int even_depth(const Geom &g, double slots, int fill, int least)
 {
-    if (g.n < 1300000) return 0;
     const double cols = (double)((g.nx + PS_TX - 1) / PS_TX) * ((g.ny + PS_TY - 1) / PS_TY);
     int best = PS_ZC;
     double cbest = 0.0;
     for (int k = 1; k <= g.nz; ++k) {
         const int zc = (g.nz + k - 1) / k;
         if (zc > PS_ZC) continue;
-        if (zc < 8) break;
-        double waves = cols * ((g.nz + zc - 1) / zc) / 304.0;
+        if (zc < least) break;
+        double waves = cols * ((g.nz + zc - 1) / zc) / slots;
         if (waves < 4.0) waves = std::ceil(waves);
-        const double cost = waves * (zc + 8);
+        const double cost = waves * (zc + fill);
         if (cbest == 0.0 || cost < cbest) {
             cbest = cost;
             best = zc;
@@ -217,13 +218,25 @@ int auto_depth(const Geom &g)
     return best;
 }
 
+// Planes per block of the z-marching psi kernel where neither the caller nor the
+// tuner has chosen, or 0 for the small-tile kernels.  Those are the faster ones up to
+// about 110^3 (a Heun step at 96^3: 123 against 132 us with the best chunk, at 128^3 239
+// against 230 us).  Above, the even split for two blocks on each of 152 SMs, 8 plane times
+// to fill the pipeline: 128^3 16 planes, 160^3 27, 256 x 256 x 64 32, 512^3 64 (what the
+// tuner finds there); with 64 planes throughout those took 1.6, 1.16, 1.16 times as long.
+int auto_depth(const Geom &g) { return g.n < 1300000 ? 0 : even_depth(g, 304.0, 8, 8); }
+
 // The same as it stands for replica r now.
 int psi_depth(const Rep &r)
 {
     if (!marching(r.p)) return 0;
-    if (!r.tuned) return auto_depth(r.g);
-    return r.cube ? 0 : r.zc;
+    if (!r.plain.set) return auto_depth(r.g);
+    return r.cube ? 0 : r.plain.zc;
 }
+
+// Planes per block of the single-pass step: the caller's or the tuner's, else the even
+// split for one block on each of 152 SMs.
+int heun1_depth(const Rep &r) { return r.heun1.set ? r.heun1.zc : even_depth(r.g, 152.0, 10, 4); }
 
 Geom make_geom(const flb_params &p)
 {
@@ -591,7 +604,7 @@ int launch_psi_stages(flb_handle *h, Rep &r)
     }
     if (r.fused && heun) {  // both stages in one launch (flb_set_psi_fused)
         FLB_TRY(launch_psi3_heun1(r.g, p.psi_scheme, psi_n, r.u, psi_np1, (float)p.A, (float)p.B, (float)p.K,
-                                  (float)p.M, (float)p.kT, advect, noise, key, r.step, r.zc, st));
+                                  (float)p.M, (float)p.kT, advect, noise, key, r.step, heun1_depth(r), st));
         return FLB_OK;
     }
     FLB_TRY(launch_psi3(r.g, p.psi_scheme, r.q, 1, noise, psi_n, r.u, heun ? r.psis : psi_np1, r.E, (float)p.A,
@@ -836,7 +849,7 @@ void batch_depths(flb_handle *h)
             best = target;
         }
     }
-    for (Rep &r : h->reps) r.bzc = r.btuned ? r.zc : split(r.g.nz, best);
+    for (Rep &r : h->reps) r.bzc = r.btuned ? r.plain.zc : split(r.g.nz, best);
 }
 
 // Whether a batched step's kernels are long enough for overlapping them to pay.
@@ -1760,25 +1773,20 @@ int flb_get_tuning(flb_handle *h, int32_t rep, int32_t *psi_zchunk)
 {
     Rep *r = get_rep(h, rep);
     if (!r || !psi_zchunk) return FLB_EINVAL;
-    *psi_zchunk = r->zc;
+    *psi_zchunk = r->fused ? r->heun1.zc : r->plain.zc;
     return FLB_OK;
 }
 
 int flb_set_tuning(flb_handle *h, int32_t rep, int32_t psi_zchunk)
 {
     if (!h || psi_zchunk < PS_ZC_MIN || psi_zchunk > 4096) return FLB_EINVAL;
-    if (rep == -1) {
-        for (Rep &r : h->reps) {
-            r.zc = psi_zchunk;
-            r.tuned = r.btuned = true;
-            r.cube = false;
-        }
-    } else {
-        Rep *r = get_rep(h, rep);
-        if (!r) return FLB_EINVAL;
-        r->zc = psi_zchunk;
-        r->tuned = r->btuned = true;
-        r->cube = false;
+    if (rep != -1 && !get_rep(h, rep)) return FLB_EINVAL;
+    for (size_t k = 0; k < h->reps.size(); ++k) {
+        Rep &r = h->reps[k];
+        if (rep != -1 && (size_t)rep != k) continue;
+        r.plain = r.heun1 = Depth{psi_zchunk, true};
+        r.btuned = true;
+        r.cube = false;
     }
     batch_reset(h);
     return FLB_OK;
@@ -1816,7 +1824,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
         for (Rep &r : h->reps) r.btuned = true;
         auto set_depth = [&](int nz, int zc) {
             for (Rep &r : h->reps)
-                if (r.g.nz == nz) r.zc = zc;
+                if (r.g.nz == nz) r.plain.zc = zc;
         };
         auto time_all = [&](float &t) {
             batch_reset(h);
@@ -1832,7 +1840,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
         };
         const auto it = cache.find(key);
         if (it != cache.end()) {
-            for (Rep &r : h->reps) r.zc = it->second;
+            for (Rep &r : h->reps) r.plain.zc = it->second;
             for (int nz : depths) {  // per-depth refinements, where tuned
                 const auto d = cache.find(std::string(key) + "|nz" + std::to_string(nz));
                 if (d != cache.end()) set_depth(nz, d->second);
@@ -1842,7 +1850,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
             float tbest = 0.f;
             int best = PS_ZC;
             for (int zc : zc_candidates(nzmax)) {
-                for (Rep &r : h->reps) r.zc = zc;
+                for (Rep &r : h->reps) r.plain.zc = zc;
                 float t = 0.f;
                 if ((rc = time_all(t)) != FLB_OK) return rc;
                 if (tbest == 0.f || t < tbest) {
@@ -1850,7 +1858,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
                     best = zc;
                 }
             }
-            for (Rep &r : h->reps) r.zc = best;
+            for (Rep &r : h->reps) r.plain.zc = best;
             append_cache(cache_path, key, best);
             // then each box depth on its own (the others held), over the chunk
             // sizes that split it evenly, ceil(nz / k); kept when 1% faster
@@ -1874,42 +1882,46 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
     } else {
         std::map<std::string, std::pair<int, bool>> done;
         for (Rep &r : h->reps) {
-            if (!marching(r.p)) continue;
-            const std::string key = "plain|" + dk + "|" + rep_key(r);
-            auto d = done.find(key);
+            if (!r.fused && !marching(r.p)) continue;
+            Depth &d = r.fused ? r.heun1 : r.plain;  // the single-pass step has a depth under either scheme
+            const std::string key = (r.fused ? "heun1|" : "plain|") + dk + "|" + rep_key(r);
+            const auto same = done.find(key);
             const auto it = cache.find(key);
-            if (d != done.end()) {
-                r.zc = d->second.first;
-                r.cube = d->second.second;
+            bool cube = false;
+            if (same != done.end()) {
+                d.zc = same->second.first;
+                cube = same->second.second;
             } else if (it != cache.end()) {
-                r.zc = it->second;
-                r.cube = auto_depth(r.g) == 0;
+                d.zc = it->second;
+                cube = !r.fused && auto_depth(r.g) == 0;
             } else {
-                float tbest = 0.f;
+                float t, tbest = 0.f;
                 int best = PS_ZC;
-                auto timed = [&](float &t) {
+                auto timed = [&]() {
                     t = time_launches(h, [&]() { return launch_psi_stages(h, r); }, reps);
                     return t >= 0.f;
                 };
-                r.tuned = true;
-                r.cube = false;
-                float t;
+                d.set = true;
+                if (!r.fused) r.cube = false;
                 for (int zc : zc_candidates(r.g.nz)) {
-                    r.zc = zc;
-                    if (!timed(t)) return FLB_ECUDA;
+                    d.zc = zc;
+                    if (!timed()) return FLB_ECUDA;
                     if (tbest == 0.f || t < tbest) {
                         tbest = t;
                         best = zc;
                     }
                 }
-                r.zc = best;
-                r.cube = true;  // the small tiles, where they are faster than any chunk
-                if (!timed(t)) return FLB_ECUDA;
-                r.cube = t < tbest;
+                d.zc = best;
+                if (!r.fused) {  // the small tiles, where they are faster than any chunk
+                    r.cube = true;
+                    if (!timed()) return FLB_ECUDA;
+                    cube = t < tbest;
+                }
                 append_cache(cache_path, key, best);
             }
-            r.tuned = true;
-            done[key] = {r.zc, r.cube};
+            d.set = true;
+            if (!r.fused) r.cube = cube;
+            done[key] = {d.zc, cube};
         }
     }
     batch_reset(h);

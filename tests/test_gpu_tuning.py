@@ -117,3 +117,23 @@ def test_tuning_argument_checks():
             s.set_tuning(bad)
     with pytest.raises(F.FlbError):
         s.set_tuning(8, rep=3)
+
+
+@pytest.mark.parametrize("q,scheme", [(19, 0), (15, 0), (19, 1)])
+def test_autotune_of_the_single_pass_step(tmp_path, q, scheme):
+    # the single-pass step has a depth under the FD scheme too, whose two-launch form has none
+    cache = str(tmp_path / "tune.txt")
+    p = flb_params(dict(RAGGED, q=q, scheme=scheme))
+    s = F.Solver(p)
+    assert s.get_tuning(0) == 64
+    s.set_psi_fused(True)
+    (chosen,) = s.autotune(cache=cache)
+    assert chosen in (4, 8, 16, 32)  # the candidates up to the first that covers 19 planes
+    lines = open(cache).read().splitlines()
+    assert len(lines) == 1 and lines[0].endswith(f"\t{chosen}")
+    s.set_psi_fused(False)
+    assert s.get_tuning(0) == 64     # the two-launch form keeps its own
+    s2 = F.Solver(p)
+    s2.set_psi_fused(True)
+    assert s2.autotune(cache=cache) == [chosen]
+    assert open(cache).read().splitlines() == lines
