@@ -852,25 +852,24 @@ void batch_depths(flb_handle *h)
     for (Rep &r : h->reps) r.bzc = r.btuned ? r.plain.zc : split(r.g.nz, best);
 }
 
-// Whether a batched step's kernels are long enough for overlapping them to pay.
-bool batch_large(const flb_handle *h)
-{
-    long long total = 0;
-    for (const Rep &r : h->reps) total += r.g.n;
-    return total >= 600000;
-}
-
 // The replicas of a batched step in groups of about equal site counts (largest boxes dealt
 // first).  A group's kernels form a chain of their own in the graph, so the last
 // blocks of one group's kernel and the memory-bound velocity run beside the other group's work:
 // two groups took a step of 256 replicas of 16^3 to 48^3 from 1105 to 1086 us, of 160 of 30^3 from
 // 530 to 510, of 25 of 32^3 from 118 to 115 (three, four and eight groups: as two or
-// slower).  Below 600 thousand sites a kernel's own latency is what it costs, and twice as many
-// kernels are slower: 8 of 16^3 49.7 and 53.4 us, 2 of 48^3 62 and 66.
+// slower).  The line at 600 thousand sites: one group against two, 16 of 32^3 (524 thousand) 79.9
+// and 80.9 us, 128 of 16^3 (524) 100.7 and 101.2, 4 of 52^3 (562) 94.6 and 94.3, but 20 of 32^3 (655) 93.5
+// and 91.7, 2 of 72^3 (746) 122.9 and 119.6, 200 of 16^3 (819) 151.3 and 143.7; far below it a
+// kernel's own latency is what it costs, and twice as many are slower: 8 of 16^3 49.7 and 53.4 us,
+// 2 of 48^3 62 and 66, 8 of 32^3 55.4 and 59.  The launches of a chain are made in plain
+// stream order: overlapping ones (launch_pdl) run in one of two states, fixed for a handle, in which 25
+// D3Q15 replicas of 32^3 take 96.6 or 115 us (25 of D3Q19 103 or 120.7), where these take 100.
 std::vector<std::vector<int>> batch_groups(const flb_handle *h)
 {
     const int n = (int)h->reps.size();
-    const int G = n > 1 && batch_large(h) ? 2 : 1;
+    long long total = 0;
+    for (const Rep &r : h->reps) total += r.g.n;
+    const int G = n > 1 && total >= 600000 ? 2 : 1;
     std::vector<int> order((size_t)n);
     for (int r = 0; r < n; ++r) order[(size_t)r] = r;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return h->reps[(size_t)a].g.n > h->reps[(size_t)b].g.n; });
@@ -994,9 +993,6 @@ BatchLists batch_lists(flb_handle *h)
     L.npsi = h->b_npsi;
     L.dstep = h->b_dstep;
     L.status = h->status;
-    // 25 replicas of 32^3 108.5 -> 104.8 us a step (D3Q15 102.7 -> 98.7), 8 of 52^3 165.3 -> 162.2; a
-    // graph of such launches costs more to start: 8 of 16^3 46.4 -> 50.2, 2 of 48^3 57.6 -> 61.6
-    L.pdl_max = batch_large(h) ? PDL_BLOCKS : 0;
     return L;
 }
 

@@ -155,10 +155,8 @@ __global__ void __launch_bounds__(MV_TX *MV_TY) mu3_vec_kernel(const Geom g, con
 // them from b.bx on and the planes b.by .. b.bz - 1.
 __global__ void __launch_bounds__(MUB_NT) mu3_batch_kernel(const BatchLists L)
 {
-    pdl_trigger();
     const BatchBlock b = L.mu[blockIdx.x];
     const BatchRep &r = L.reps[b.rep];
-    pdl_wait();
     const int par = (int)(*L.dstep & 1);
     const Geom &g = r.lb.g;
     const int nq = mu_row_quads(g);
@@ -181,10 +179,8 @@ template <typename T, bool FORCE>
 __global__ void __launch_bounds__(LBB_NT) vel3_batch_kernel(const BatchLists L)
 {
     __shared__ LBArgs sa;
-    pdl_trigger();
     const BatchBlock b = L.lb[blockIdx.x];
     batch_lb_args(L, L.reps[b.rep], sa);
-    pdl_wait();
     int x, y, zl[2], nl;
     if (packed_pair<LBB_NT>(sa.g, b.bx, b.by, b.bz, threadIdx.x, x, y, zl, nl))
         vel3_sites<F2, T, FORCE, false>(sa, PlanesFromBase<T>{(const T *)sa.fout, nullptr, sa.g.n}, x, y, zl, nl);
@@ -228,15 +224,21 @@ cudaError_t launch_vel3(const LBArgs &a, int storage, cudaStream_t st)
 
 cudaError_t launch_mu3_batch(const BatchLists &L, cudaStream_t st)
 {
-    return L.nmu > 0 ? launch_pdl(mu3_batch_kernel, L.nmu, MUB_NT, 0, st, L.pdl_max, L) : cudaSuccess;
+    if (L.nmu > 0) mu3_batch_kernel<<<L.nmu, MUB_NT, 0, st>>>(L);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_vel3_batch(const BatchLists &L, int storage, bool force, cudaStream_t st)
 {
     const dim3 block(LBB_NT);
-    auto go = [&](auto kernel) { return launch_pdl(kernel, L.nlb, block, 0, st, L.pdl_max, L); };
-    if (storage == FLB_F16_DEV) return force ? go(vel3_batch_kernel<__half, true>) : go(vel3_batch_kernel<__half, false>);
-    return force ? go(vel3_batch_kernel<float, true>) : go(vel3_batch_kernel<float, false>);
+    if (storage == FLB_F16_DEV) {
+        if (force) vel3_batch_kernel<__half, true><<<L.nlb, block, 0, st>>>(L);
+        else vel3_batch_kernel<__half, false><<<L.nlb, block, 0, st>>>(L);
+    } else {
+        if (force) vel3_batch_kernel<float, true><<<L.nlb, block, 0, st>>>(L);
+        else vel3_batch_kernel<float, false><<<L.nlb, block, 0, st>>>(L);
+    }
+    return cudaGetLastError();
 }
 
 }  // namespace flb

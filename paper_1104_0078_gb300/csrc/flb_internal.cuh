@@ -414,8 +414,8 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 // start, so that the next one's blocks may be scheduled as soon as its own leave
 // room, and pdl_wait before its first access to global memory, which returns when
 // the kernels before it in the stream have completed and their writes are visible.
-// What stands before pdl_wait (index arithmetic, random numbers) touches registers and
-// the block's own shared memory only.  A kernel that triggers also waits, so
+// What stands before pdl_wait (index arithmetic, random numbers) touches registers, the
+// block's own shared memory and the constant Box-Muller tables only.  A kernel that triggers also waits, so
 // completion stays in stream order however many launches overlap.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -797,7 +797,6 @@ struct BatchLists {
     int nmu, nlb, npsi;
     const long long *dstep;
     int *status;
-    long long pdl_max;  // launches of at most so many blocks overlap the one before (launch_pdl)
 };
 
 cudaError_t encode_tensor_map_f32(CUtensorMap *map, const void *base, int rank, const uint64_t *dims,

@@ -60,10 +60,8 @@ template <typename T, bool GHOST_RELAX, bool FORCE>
 __global__ void __launch_bounds__(LBB_NT, 7) lb15_batch_kernel(const BatchLists L)
 {
     __shared__ LBArgs sa;
-    pdl_trigger();
     const BatchBlock b = L.lb[blockIdx.x];
     batch_lb_args(L, L.reps[b.rep], sa);
-    pdl_wait();
     int x, y, zl[2], nl;
     if (!packed_pair<LBB_NT>(sa.g, b.bx, b.by, b.bz, threadIdx.x, x, y, zl, nl)) return;
     F2 Fx = F2::bc(0.f), Fy = F2::bc(0.f), Fz = F2::bc(0.f);
@@ -77,10 +75,8 @@ template <typename T, bool FORCE>
 __global__ void __launch_bounds__(LBB_NT) vel15_batch_kernel(const BatchLists L)
 {
     __shared__ LBArgs sa;
-    pdl_trigger();
     const BatchBlock b = L.lb[blockIdx.x];
     batch_lb_args(L, L.reps[b.rep], sa);
-    pdl_wait();
     int x, y, zl[2], nl;
     if (packed_pair<LBB_NT>(sa.g, b.bx, b.by, b.bz, threadIdx.x, x, y, zl, nl))
         for (int l = 0; l < nl; ++l) vel15_site<T, FORCE>(sa, x, y, zl[l]);
@@ -96,8 +92,7 @@ cudaError_t launch_lb15_batch(const BatchLists &L, int storage, bool ghost, bool
         const cudaError_t e = launch_mu3_batch(L, st);
         if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaSuccess;
-#define FLB_LB15B(T, G, F) e = launch_pdl(lb15_batch_kernel<T, G, F>, L.nlb, block, 0, st, L.pdl_max, L)
+#define FLB_LB15B(T, G, F) lb15_batch_kernel<T, G, F><<<L.nlb, block, 0, st>>>(L)
     if (storage == FLB_F16_DEV) {
         if (ghost) { if (force) FLB_LB15B(__half, true, true); else FLB_LB15B(__half, true, false); }
         else { if (force) FLB_LB15B(__half, false, true); else FLB_LB15B(__half, false, false); }
@@ -106,10 +101,16 @@ cudaError_t launch_lb15_batch(const BatchLists &L, int storage, bool ghost, bool
         else { if (force) FLB_LB15B(float, false, true); else FLB_LB15B(float, false, false); }
     }
 #undef FLB_LB15B
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    auto go = [&](auto kernel) { return launch_pdl(kernel, L.nlb, block, 0, st, L.pdl_max, L); };
-    if (storage == FLB_F16_DEV) return force ? go(vel15_batch_kernel<__half, true>) : go(vel15_batch_kernel<__half, false>);
-    return force ? go(vel15_batch_kernel<float, true>) : go(vel15_batch_kernel<float, false>);
+    if (storage == FLB_F16_DEV) {
+        if (force) vel15_batch_kernel<__half, true><<<L.nlb, block, 0, st>>>(L);
+        else vel15_batch_kernel<__half, false><<<L.nlb, block, 0, st>>>(L);
+    } else {
+        if (force) vel15_batch_kernel<float, true><<<L.nlb, block, 0, st>>>(L);
+        else vel15_batch_kernel<float, false><<<L.nlb, block, 0, st>>>(L);
+    }
+    return cudaGetLastError();
 }
 
 cudaError_t launch_lb15(const LBArgs &a, int storage, cudaStream_t st)

@@ -58,10 +58,8 @@ template <typename T, bool GHOST_RELAX, bool FORCE>
 __global__ void __launch_bounds__(LBB_NT, 7) lb3_batch_kernel(const BatchLists L)
 {
     __shared__ LBArgs sa;
-    pdl_trigger();
     const BatchBlock b = L.lb[blockIdx.x];
     batch_lb_args(L, L.reps[b.rep], sa);
-    pdl_wait();
     int x, y, zl[2], nl;
     if (!packed_pair<LBB_NT>(sa.g, b.bx, b.by, b.bz, threadIdx.x, x, y, zl, nl)) return;
     F2 Fx = F2::bc(0.f), Fy = F2::bc(0.f), Fz = F2::bc(0.f);
@@ -77,8 +75,7 @@ cudaError_t launch_lb3_batch(const BatchLists &L, int storage, bool ghost, bool 
         const cudaError_t e = launch_mu3_batch(L, st);
         if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaSuccess;
-#define FLB_LB3B(T, G, F) e = launch_pdl(lb3_batch_kernel<T, G, F>, L.nlb, block, 0, st, L.pdl_max, L)
+#define FLB_LB3B(T, G, F) lb3_batch_kernel<T, G, F><<<L.nlb, block, 0, st>>>(L)
     if (storage == FLB_F16_DEV) {
         if (ghost) { if (force) FLB_LB3B(__half, true, true); else FLB_LB3B(__half, true, false); }
         else { if (force) FLB_LB3B(__half, false, true); else FLB_LB3B(__half, false, false); }
@@ -87,6 +84,7 @@ cudaError_t launch_lb3_batch(const BatchLists &L, int storage, bool ghost, bool 
         else { if (force) FLB_LB3B(float, false, true); else FLB_LB3B(float, false, false); }
     }
 #undef FLB_LB3B
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_vel3_batch(L, storage, force, st);
 }

@@ -55,13 +55,11 @@ __global__ void __launch_bounds__(block_threads<StageV, MU_IN>(), 2) psi3_fv_tma
 {
     extern __shared__ __align__(1024) float tsmem[];
     __shared__ Psi3Args sa;
-    pdl_trigger();
     const BatchBlock b = L.psi[blockIdx.x];
     const BatchRep &r = L.reps[b.rep];
     const long long ds = *L.dstep;
     if (threadIdx.x == 0) psi_batch_args(r, ds, STAGE, sa);
     __syncthreads();
-    pdl_wait();
     const CUtensorMap *pm = STAGE == 1 ? &r.map_psi[(int)(ds & 1)] : &r.map_psis;
     psi3_fv_tma_block<STAGE, NOISE, false, true, false, MU_IN, Q15, StageV>(pm, &r.map_u, sa, L.status, b.bx, b.by, b.bz,
                                                                        tsmem, &r.map_mu);
@@ -81,7 +79,8 @@ static cudaError_t batch_psi(const BatchLists &L, bool heun, int noise, bool mu_
     auto go = [&](auto kernel, size_t bytes, int nt) {
         cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         if (r != cudaSuccess) return r;
-        return launch_pdl(kernel, L.npsi, nt, bytes, st, L.pdl_max, L);
+        kernel<<<L.npsi, nt, bytes, st>>>(L);
+        return cudaGetLastError();
     };
     constexpr int n1 = block_threads<StageV, true>(), nn = block_threads<StageV, false>();
     cudaError_t e = mu_in ? (noise == 2 ? go(psi3_fv_tma_batch_kernel<1, 2, true, Q15>, smm + nb, n1)
