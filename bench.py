@@ -42,7 +42,7 @@ def parse():
     ap.add_argument("--storage", choices=["f32", "f16"], default="f32")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
-    ap.add_argument("--no-autotune", action="store_true", help="keep the default psi tile depth (64 planes)")
+    ap.add_argument("--no-autotune", action="store_true", help="leave the psi tiles and depths to the rule by size")
     ap.add_argument("--variant-size", type=int, default=512,
                     help="edge of the cubic box of the path variants (2D variant: 8x this edge)")
     ap.add_argument("--variants", default="",
@@ -278,7 +278,8 @@ def ensemble_batched_vs_plain(F, I, steps, local, rank, autotune=True):
         s = F.Solver(ps, device=f"cuda:{local}")
         s.set_mode(mode)
         if autotune:
-            out[key + "_psi_zchunk"] = sorted(set(s.autotune()))
+            s.autotune()
+        out[key + "_psi_zchunk"] = sorted({s.get_psi_planes(r) for r in range(len(ps))})  # 0: small tiles
         s.step(3)
         s.synchronize()
         e0 = torch.cuda.Event(enable_timing=True)
@@ -316,7 +317,8 @@ def ensemble_d3q15(F, I, steps, local, rank, autotune=True):
         s = F.Solver(ps, device=f"cuda:{local}")
         s.set_mode(mode)
         if autotune:
-            out[key + "_psi_zchunk"] = sorted(set(s.autotune()))
+            s.autotune()
+        out[key + "_psi_zchunk"] = sorted({s.get_psi_planes(r) for r in range(len(ps))})  # 0: small tiles
         s.step(3)
         s.synchronize()
         e0 = torch.cuda.Event(enable_timing=True)
@@ -443,7 +445,9 @@ def run_ours(args):
     s = F.Solver(p, device=f"cuda:{local}")
     psi0 = I.uniform_field(N, -0.01, 0.01, replica_seeds(d["seed"], rank)[1])
     s.set_fields(psi=psi0)
-    zchunk = s.autotune()[0] if not args.no_autotune else s.get_tuning(0)
+    if not args.no_autotune:
+        s.autotune()
+    zchunk = s.get_psi_planes(0)
     s.set_sampling(10, 1)
     s.step(args.warmup)
     s.synchronize()

@@ -307,13 +307,15 @@ int flb_set_wait_limit(flb_handle *h, double seconds);
  * flb_get_tuning / flb_set_tuning read / set psi_zchunk of replica rep (-1 sets
  * every replica), 1 <= psi_zchunk <= 4096; EINVAL otherwise.  Setting it drops
  * the batched mode's captured graph, which the next batched flb_step rebuilds.
+ * flb_get_psi_planes gives what the next flb_step takes in the handle's present
+ * mode, set, tuned or chosen by size: planes per block, 0 for the small tiles (or a
+ * 2D replica); EINVAL for no such replica or a NULL pointer.
  *
  * flb_autotune times the candidates 4, 8, ... (up to the first value that
  * covers the box depth) on the handle's own buffers and keeps the fastest: in
  * FLB_MODE_PLAIN per distinct replica configuration (box, lattice, scheme,
- * integrator, noise, advection) on that replica's psi stages, the small tiles
- * included (a cached value is applied with the small tiles below 1.3 million
- * sites), or on its single-pass step, which keeps a value of its own, where that is
+ * integrator, noise, advection, mu given) on that replica's psi stages, the small
+ * tiles included, or on its single-pass step, which keeps a value of its own, where that is
  * on; in
  * FLB_MODE_BATCHED and FLB_MODE_PERSISTENT one value for all replicas on the
  * batched psi launches, then, deepest boxes first, one value per distinct box
@@ -322,8 +324,9 @@ int flb_set_wait_limit(flb_handle *h, double seconds);
  * timed launches write only step scratch and the spare psi buffer, so the state
  * (populations, psi, step counters, spectra) is unchanged.  cache_path (may be
  * NULL) names a text file of "key<TAB>planes" lines, keyed by the device name,
- * its SM count and the configuration (batched: one line for the shared value
- * and one per box depth): entries found there are applied without
+ * its SM count and the configuration (plain: "<TAB>1" follows where the small tiles
+ * were faster than any number of planes, else "<TAB>0"; batched: one line for the
+ * shared value and one per box depth): entries found there are applied without
  * timing (unless flags has FLB_TUNE_FORCE), new results are appended.  An
  * unreadable or unwritable file only disables the cache.  Synchronising; call
  * with the handle's device current and outside stream capture.  2D replicas and
@@ -331,6 +334,7 @@ int flb_set_wait_limit(flb_handle *h, double seconds);
  */
 int flb_get_tuning(flb_handle *h, int32_t rep, int32_t *psi_zchunk);
 int flb_set_tuning(flb_handle *h, int32_t rep, int32_t psi_zchunk);
+int flb_get_psi_planes(flb_handle *h, int32_t rep, int32_t *planes);
 
 /* Single-pass Heun (tuning flag, default off): with on != 0 every replica's psi
  * step runs both Runge-Kutta stages of Sec. V in one launch by halo recompute:

@@ -93,6 +93,7 @@ def load_library(path: str = LIB_PATH):
         "flb_set_mode": (c_int, [H, ctypes.c_int32]),
         "flb_get_tuning": (c_int, [H, ctypes.c_int32, P(ctypes.c_int32)]),
         "flb_set_tuning": (c_int, [H, ctypes.c_int32, ctypes.c_int32]),
+        "flb_get_psi_planes": (c_int, [H, ctypes.c_int32, P(ctypes.c_int32)]),
         "flb_set_psi_fused": (c_int, [H, ctypes.c_int32]),
         "flb_autotune": (c_int, [H, ctypes.c_char_p, ctypes.c_int32]),
         "flb_set_wait_limit": (c_int, [H, ctypes.c_double]),
@@ -301,6 +302,12 @@ class Solver:
 
     def set_tuning(self, psi_zchunk: int, rep: int = -1):
         _check(self.lib.flb_set_tuning(self.h, rep, int(psi_zchunk)), "flb_set_tuning")
+
+    def get_psi_planes(self, rep=0) -> int:
+        """Planes per psi block that the next step takes; 0: small tiles (flb_get_psi_planes)."""
+        v = ctypes.c_int32()
+        _check(self.lib.flb_get_psi_planes(self.h, rep, ctypes.byref(v)), "flb_get_psi_planes")
+        return int(v.value)
 
     def set_psi_fused(self, on=True):
         """Single-pass Heun psi step (flb_set_psi_fused)."""

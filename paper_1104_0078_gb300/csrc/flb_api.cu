@@ -571,6 +571,9 @@ LBArgs lb_args(const Rep &r, float *psi_n)
     return la;
 }
 
+// Whether a 3D step forms mu of psi^n for its force, so that psi stage 1 reads it.
+bool mu_given(const flb_params &p) { return (p.coupling & FLB_COUPLE_FORCE) && p.force_grad != FLB_FORCE_STRESS; }
+
 // Noise of the psi equation: 0 none, 1, or 2 by the tables (FP16 storage: bm_eval).
 int noise_kind(const flb_params &p) { return p.kT > 0 && p.M > 0 ? (p.storage == FLB_F16_DEV ? 2 : 1) : 0; }
 
@@ -586,7 +589,7 @@ int launch_psi_stages(flb_handle *h, Rep &r)
     LapW lwv{};
     const LapW *lw = app_a_weights(r, lwv);
     float *psi_n = r.psi[r.pcur], *psi_np1 = r.psi[r.pcur ^ 1];
-    const float *mu_n = (p.coupling & FLB_COUPLE_FORCE) && p.force_grad != FLB_FORCE_STRESS ? r.mu : nullptr;
+    const float *mu_n = mu_given(p) ? r.mu : nullptr;
     const int noise = noise_kind(p);
     const bool heun = p.integrator == FLB_HEUN;
     const int advect = (p.coupling & FLB_COUPLE_ADVECT) ? 1 : 0;
@@ -1696,18 +1699,25 @@ std::string device_key()
     return name + "|sm" + std::to_string(sms);
 }
 
+// What selects a replica's psi kernels: n the noise (2: by the tables of FP16 storage), m whether
+// the step gives stage 1 its mu.
 std::string rep_key(const Rep &r)
 {
     char b[160];
-    std::snprintf(b, sizeof b, "%dx%dx%d|q%d|s%d|i%d|n%d|a%d", r.g.nx, r.g.ny, r.g.nz, r.q, r.p.psi_scheme,
-                  r.p.integrator, (r.p.kT > 0 && r.p.M > 0) ? 1 : 0, (r.p.coupling & FLB_COUPLE_ADVECT) ? 1 : 0);
+    std::snprintf(b, sizeof b, "%dx%dx%d|q%d|s%d|i%d|n%d|a%d|m%d", r.g.nx, r.g.ny, r.g.nz, r.q, r.p.psi_scheme,
+                  r.p.integrator, noise_kind(r.p), (r.p.coupling & FLB_COUPLE_ADVECT) ? 1 : 0, mu_given(r.p) ? 1 : 0);
     return b;
 }
 
-// Tuning cache: one "key<TAB>planes" line per tuned configuration; later lines win.
-std::map<std::string, int> read_cache(const char *path)
+// Tuning cache: one "key<TAB>planes" line per tuned configuration, with "<TAB>1" where the
+// small tiles were faster than any number of planes (else "<TAB>0" or nothing); later lines win.
+struct Tuned {
+    int zc;
+    bool cube;
+};
+std::map<std::string, Tuned> read_cache(const char *path)
 {
-    std::map<std::string, int> m;
+    std::map<std::string, Tuned> m;
     if (!path) return m;
     FILE *f = std::fopen(path, "r");
     if (!f) return m;
@@ -1717,18 +1727,19 @@ std::map<std::string, int> read_cache(const char *path)
         if (!tab) continue;
         *tab = 0;
         const int v = std::atoi(tab + 1);
-        if (v >= PS_ZC_MIN && v <= 4096) m[line] = v;
+        const char *form = std::strchr(tab + 1, '\t');
+        if (v >= PS_ZC_MIN && v <= 4096) m[line] = {v, form && std::atoi(form + 1) == 1};
     }
     std::fclose(f);
     return m;
 }
 
-void append_cache(const char *path, const std::string &key, int zc)
+void append_cache(const char *path, const std::string &key, int zc, const char *form = "")
 {
     if (!path) return;
     FILE *f = std::fopen(path, "a");
     if (!f) return;
-    std::fprintf(f, "%s\t%d\n", key.c_str(), zc);
+    std::fprintf(f, "%s\t%d%s\n", key.c_str(), zc, form);
     std::fclose(f);
 }
 
@@ -1773,6 +1784,19 @@ int flb_get_tuning(flb_handle *h, int32_t rep, int32_t *psi_zchunk)
     return FLB_OK;
 }
 
+int flb_get_psi_planes(flb_handle *h, int32_t rep, int32_t *planes)
+{
+    Rep *r = get_rep(h, rep);
+    if (!r || !planes) return FLB_EINVAL;
+    if (h->mode != FLB_MODE_PLAIN && batch_supported(h)) {
+        batch_depths(h);
+        *planes = r->bzc;
+    } else {
+        *planes = r->fused ? heun1_depth(*r) : psi_depth(*r);
+    }
+    return FLB_OK;
+}
+
 int flb_set_tuning(flb_handle *h, int32_t rep, int32_t psi_zchunk)
 {
     if (!h || psi_zchunk < PS_ZC_MIN || psi_zchunk > 4096) return FLB_EINVAL;
@@ -1794,7 +1818,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
     int rc = take_status(h);
     if (rc != FLB_OK) return rc;
     const bool force = (flags & FLB_TUNE_FORCE) != 0;
-    const std::map<std::string, int> cache = force ? std::map<std::string, int>() : read_cache(cache_path);
+    const std::map<std::string, Tuned> cache = force ? std::map<std::string, Tuned>() : read_cache(cache_path);
     const std::string dk = device_key();
     const int reps = 3;
     if ((h->mode == FLB_MODE_BATCHED || h->mode == FLB_MODE_PERSISTENT) && batch_supported(h)) {
@@ -1836,10 +1860,10 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
         };
         const auto it = cache.find(key);
         if (it != cache.end()) {
-            for (Rep &r : h->reps) r.plain.zc = it->second;
+            for (Rep &r : h->reps) r.plain.zc = it->second.zc;
             for (int nz : depths) {  // per-depth refinements, where tuned
                 const auto d = cache.find(std::string(key) + "|nz" + std::to_string(nz));
-                if (d != cache.end()) set_depth(nz, d->second);
+                if (d != cache.end()) set_depth(nz, d->second.zc);
             }
         } else {
             // one value for every replica first
@@ -1876,7 +1900,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
             }
         }
     } else {
-        std::map<std::string, std::pair<int, bool>> done;
+        std::map<std::string, Tuned> done;
         for (Rep &r : h->reps) {
             if (!r.fused && !marching(r.p)) continue;
             Depth &d = r.fused ? r.heun1 : r.plain;  // the single-pass step has a depth under either scheme
@@ -1884,12 +1908,10 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
             const auto same = done.find(key);
             const auto it = cache.find(key);
             bool cube = false;
-            if (same != done.end()) {
-                d.zc = same->second.first;
-                cube = same->second.second;
-            } else if (it != cache.end()) {
-                d.zc = it->second;
-                cube = !r.fused && auto_depth(r.g) == 0;
+            if (same != done.end() || it != cache.end()) {
+                const Tuned &t = same != done.end() ? same->second : it->second;
+                d.zc = t.zc;
+                cube = t.cube;
             } else {
                 float t, tbest = 0.f;
                 int best = PS_ZC;
@@ -1913,7 +1935,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
                     if (!timed()) return FLB_ECUDA;
                     cube = t < tbest;
                 }
-                append_cache(cache_path, key, best);
+                append_cache(cache_path, key, best, r.fused ? "" : cube ? "\t1" : "\t0");
             }
             d.set = true;
             if (!r.fused) r.cube = cube;

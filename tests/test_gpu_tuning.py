@@ -137,3 +137,59 @@ def test_autotune_of_the_single_pass_step(tmp_path, q, scheme):
     s2.set_psi_fused(True)
     assert s2.autotune(cache=cache) == [chosen]
     assert open(cache).read().splitlines() == lines
+
+
+def _planes(s, fused=False):
+    s.set_psi_fused(fused)
+    return s.get_psi_planes(0)
+
+
+def test_cache_keeps_the_tuned_form(tmp_path):
+    # a cached handle runs the form that its line names, small tiles or planes, whatever its size
+    cache = tmp_path / "tune.txt"
+    p = flb_params(dict(RAGGED, scheme=1))
+    s = F.Solver(p)
+    assert s.get_psi_planes(0) == 0                          # by its size
+    (chosen,) = s.autotune(cache=str(cache))
+    key, planes, form = cache.read_text().rstrip("\n").split("\t")
+    assert int(planes) == chosen and form in "01"
+    assert s.get_psi_planes(0) == (0 if form == "1" else chosen)
+    for form, runs in (("0", 8), ("1", 0)):
+        cache.write_text(f"{key}\t8\t{form}\n")
+        s = F.Solver(p)
+        assert s.autotune(cache=str(cache)) == [8]
+        assert s.get_psi_planes(0) == runs
+    assert cache.read_text().count("\n") == 1               # both without timing
+    # the single-pass step is another configuration, and its tuning leaves the tiles as they are
+    s.set_psi_fused(True)
+    (one,) = s.autotune(cache=str(cache))
+    assert cache.read_text().count("\n") == 2
+    assert _planes(s, True) == one and _planes(s) == 0
+
+
+@pytest.mark.parametrize("other", [dict(storage=F.FLB_F16_DEV), dict(force_grad=F.FLB_FORCE_STRESS), dict(coupling=2)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_cache_separates_configurations_of_other_kernels(tmp_path, mode, other):
+    # FP16 storage draws by other normals, and without a given mu stage 1 is another kernel
+    cache = tmp_path / "tune.txt"
+    lines = []
+    for d in (dict(RAGGED, scheme=1), dict(RAGGED, scheme=1, **other)):
+        s = F.Solver(flb_params(d))
+        s.set_mode(mode)
+        s.autotune(cache=str(cache))
+        lines.append(cache.read_text().count("\n"))
+    assert lines[1] == 2 * lines[0]
+
+
+def test_planes_in_use():
+    s = F.Solver(flb_params(dict(RAGGED, scheme=1)))
+    assert s.get_psi_planes(0) == 0
+    s.set_tuning(7)
+    assert s.get_psi_planes(0) == 7
+    s.set_mode(F.FLB_MODE_BATCHED)
+    assert s.get_psi_planes(0) == 7
+    s = F.Solver(flb_params(dict(RAGGED, scheme=0)))
+    s.set_tuning(7)                                          # FD: the single-pass step's alone
+    assert _planes(s) == 0 and _planes(s, True) == 7
+    with pytest.raises(F.FlbError):
+        s.get_psi_planes(1)
