@@ -305,7 +305,10 @@ int flb_set_wait_limit(flb_handle *h, double seconds);
  * implementation; the paper has no counterpart.)
  *
  * flb_get_tuning / flb_set_tuning read / set psi_zchunk of replica rep (-1 sets
- * every replica), 1 <= psi_zchunk <= 4096; EINVAL otherwise.  Setting it drops
+ * every replica), 1 <= psi_zchunk <= 4096; EINVAL otherwise.  FLB_MODE_PLAIN, the
+ * single-pass step and the two other modes together have a value each: setting sets
+ * all three (the small tiles give way to blocks of that many planes), tuning and
+ * reading concern the present one.  Setting it drops
  * the batched mode's captured graph, which the next batched flb_step rebuilds.
  * flb_get_psi_planes gives what the next flb_step takes in the handle's present
  * mode, set, tuned or chosen by size: planes per block, 0 for the small tiles (or a

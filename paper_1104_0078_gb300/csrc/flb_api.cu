@@ -102,8 +102,8 @@ struct Rep {
     float namp[16] = {0};
     Depth plain;         // planes per psi block (3D), set by flb_set_tuning / flb_autotune (else auto_depth chooses)
     bool cube = false;   // tuned: the small-tile kernels were faster than any chunk
-    bool btuned = false; // whether it was set for the batched and persistent modes
-    int bzc = PS_ZC;     // planes per psi block in those modes: plain.zc when set, else batch_depths()
+    Depth batch;         // the same for the batched and persistent modes
+    int bzc = PS_ZC;     // planes per psi block in those modes: batch.zc when set, else batch_depths()
     int fused = 0;   // single-pass Heun psi step (flb_set_psi_fused)
     Depth heun1;     // its depth (else heun1_depth chooses)
 };
@@ -820,6 +820,9 @@ bool batch_supported(const flb_handle *h)
     return !h->reps.empty();
 }
 
+// Whether the present mode advances all replicas by the same launches.
+bool all_at_once(const flb_handle *h) { return h->mode != FLB_MODE_PLAIN && batch_supported(h); }
+
 // Planes per psi block of every replica in the batched and persistent modes: the
 // caller's or the tuner's, else even splits of the boxes' depths near one target, the one that
 // costs least when the whole list runs on two blocks for each of 152 SMs, a chunk of
@@ -852,7 +855,7 @@ void batch_depths(flb_handle *h)
             best = target;
         }
     }
-    for (Rep &r : h->reps) r.bzc = r.btuned ? r.plain.zc : split(r.g.nz, best);
+    for (Rep &r : h->reps) r.bzc = r.batch.set ? r.batch.zc : split(r.g.nz, best);
 }
 
 // The replicas of a batched step in groups of about equal site counts (largest boxes dealt
@@ -1780,7 +1783,7 @@ int flb_get_tuning(flb_handle *h, int32_t rep, int32_t *psi_zchunk)
 {
     Rep *r = get_rep(h, rep);
     if (!r || !psi_zchunk) return FLB_EINVAL;
-    *psi_zchunk = r->fused ? r->heun1.zc : r->plain.zc;
+    *psi_zchunk = (all_at_once(h) ? r->batch : r->fused ? r->heun1 : r->plain).zc;
     return FLB_OK;
 }
 
@@ -1788,7 +1791,7 @@ int flb_get_psi_planes(flb_handle *h, int32_t rep, int32_t *planes)
 {
     Rep *r = get_rep(h, rep);
     if (!r || !planes) return FLB_EINVAL;
-    if (h->mode != FLB_MODE_PLAIN && batch_supported(h)) {
+    if (all_at_once(h)) {
         batch_depths(h);
         *planes = r->bzc;
     } else {
@@ -1804,8 +1807,7 @@ int flb_set_tuning(flb_handle *h, int32_t rep, int32_t psi_zchunk)
     for (size_t k = 0; k < h->reps.size(); ++k) {
         Rep &r = h->reps[k];
         if (rep != -1 && (size_t)rep != k) continue;
-        r.plain = r.heun1 = Depth{psi_zchunk, true};
-        r.btuned = true;
+        r.plain = r.heun1 = r.batch = Depth{psi_zchunk, true};
         r.cube = false;
     }
     batch_reset(h);
@@ -1821,7 +1823,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
     const std::map<std::string, Tuned> cache = force ? std::map<std::string, Tuned>() : read_cache(cache_path);
     const std::string dk = device_key();
     const int reps = 3;
-    if ((h->mode == FLB_MODE_BATCHED || h->mode == FLB_MODE_PERSISTENT) && batch_supported(h)) {
+    if (all_at_once(h)) {
         // one value for every replica, timed on the batched psi launches
         std::string all;
         int noise = 0;
@@ -1841,10 +1843,10 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
         for (const Rep &r : h->reps) depths.push_back(r.g.nz);
         std::sort(depths.begin(), depths.end(), std::greater<int>());
         depths.erase(std::unique(depths.begin(), depths.end()), depths.end());
-        for (Rep &r : h->reps) r.btuned = true;
+        for (Rep &r : h->reps) r.batch.set = true;
         auto set_depth = [&](int nz, int zc) {
             for (Rep &r : h->reps)
-                if (r.g.nz == nz) r.plain.zc = zc;
+                if (r.g.nz == nz) r.batch.zc = zc;
         };
         auto time_all = [&](float &t) {
             batch_reset(h);
@@ -1860,7 +1862,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
         };
         const auto it = cache.find(key);
         if (it != cache.end()) {
-            for (Rep &r : h->reps) r.plain.zc = it->second.zc;
+            for (Rep &r : h->reps) r.batch.zc = it->second.zc;
             for (int nz : depths) {  // per-depth refinements, where tuned
                 const auto d = cache.find(std::string(key) + "|nz" + std::to_string(nz));
                 if (d != cache.end()) set_depth(nz, d->second.zc);
@@ -1870,7 +1872,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
             float tbest = 0.f;
             int best = PS_ZC;
             for (int zc : zc_candidates(nzmax)) {
-                for (Rep &r : h->reps) r.plain.zc = zc;
+                for (Rep &r : h->reps) r.batch.zc = zc;
                 float t = 0.f;
                 if ((rc = time_all(t)) != FLB_OK) return rc;
                 if (tbest == 0.f || t < tbest) {
@@ -1878,7 +1880,7 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
                     best = zc;
                 }
             }
-            for (Rep &r : h->reps) r.plain.zc = best;
+            for (Rep &r : h->reps) r.batch.zc = best;
             append_cache(cache_path, key, best);
             // then each box depth on its own (the others held), over the chunk
             // sizes that split it evenly, ceil(nz / k); kept when 1% faster

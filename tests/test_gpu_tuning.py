@@ -193,3 +193,28 @@ def test_planes_in_use():
     assert _planes(s) == 0 and _planes(s, True) == 7
     with pytest.raises(F.FlbError):
         s.get_psi_planes(1)
+
+
+def test_modes_keep_their_own_depth(tmp_path):
+    cache = tmp_path / "tune.txt"
+    p = flb_params(dict(RAGGED, scheme=1))
+
+    def tuned(mode):
+        s.set_mode(mode)
+        return s.autotune(cache=str(cache))
+
+    s = F.Solver(p)
+    tuned(F.FLB_MODE_PLAIN)
+    tuned(F.FLB_MODE_BATCHED)
+    lines = [l.split("\t")[0] for l in cache.read_text().splitlines()]
+    plain = [k for k in lines if k.startswith("plain|")]
+    assert len(plain) == 1 and len(lines) > 1
+    cache.write_text("".join(k + ("\t8\t0\n" if k in plain else "\t5\n") for k in lines))
+    s = F.Solver(p)
+    assert tuned(F.FLB_MODE_PLAIN) == [8]
+    assert tuned(F.FLB_MODE_BATCHED) == [5]
+    assert (s.get_tuning(0), s.get_psi_planes(0)) == (5, 5)
+    s.set_mode(F.FLB_MODE_PLAIN)
+    assert (s.get_tuning(0), s.get_psi_planes(0)) == (8, 8)
+    s.set_mode(F.FLB_MODE_PERSISTENT)
+    assert (s.get_tuning(0), s.get_psi_planes(0)) == (5, 5)
