@@ -1020,18 +1020,11 @@ bool batch_mu_in(const flb_handle *h)
     return true;
 }
 
-// Capture one batched step into a CUDA graph (once per handle).
-int batch_capture(flb_handle *h)
+// A CUDA graph of launch(lists, stream) for the lists of each replica group, the groups' launches in
+// chains of their own, and then last(lists, stream).
+template <class Launch, class Last>
+int batch_record(flb_handle *h, Launch &&launch, Last &&last, cudaGraph_t *graph, cudaGraphExec_t *exec)
 {
-    if (h->b_exec) return FLB_OK;
-    bool ghost = false, force = false;
-    int noise = 0;
-    for (const Rep &r : h->reps) {
-        ghost |= r.gamma_g != 0.f;
-        force |= (r.p.coupling & FLB_COUPLE_FORCE) != 0;
-        noise = std::max(noise, noise_kind(r.p));
-    }
-    const flb_params &p0 = h->reps[0].p;
     const BatchLists L = batch_lists(h);
     const size_t G = h->b_span.size();
     std::vector<cudaStream_t> side(G, h->st);
@@ -1064,26 +1057,45 @@ int batch_capture(flb_handle *h)
         P.nlb = s.nlb;
         P.npsi = s.npsi;
         if (k) e = cudaStreamWaitEvent(side[k], ev[0], 0);
-        if (e == cudaSuccess)
-            e = launch_batch_step(P, p0.storage, ghost, force, 1, p0.integrator == FLB_HEUN, noise, batch_mu_in(h),
-                                  h->reps[0].q == 15, side[k]);
+        if (e == cudaSuccess) e = launch(P, side[k]);
         if (k && e == cudaSuccess) e = cudaEventRecord(ev[k], side[k]);
     }
     for (size_t k = 1; k < G && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(h->st, ev[k], 0);
-    if (e == cudaSuccess) e = launch_batch_advance(L, h->st);
+    if (e == cudaSuccess) e = last(L, h->st);
     const cudaError_t e2 = cudaStreamEndCapture(h->st, &gr);
     drop();
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (gr) cudaGraphDestroy(gr);
         return FLB_ECUDA;
     }
-    if (cudaGraphInstantiate(&h->b_exec, gr, 0) != cudaSuccess) {
+    if (cudaGraphInstantiate(exec, gr, 0) != cudaSuccess) {
         cudaGraphDestroy(gr);
-        h->b_exec = nullptr;
+        *exec = nullptr;
         return FLB_ECUDA;
     }
-    h->b_graph = gr;
+    *graph = gr;
     return FLB_OK;
+}
+
+// Capture one batched step into a CUDA graph (once per handle).
+int batch_capture(flb_handle *h)
+{
+    if (h->b_exec) return FLB_OK;
+    bool ghost = false, force = false;
+    int noise = 0;
+    for (const Rep &r : h->reps) {
+        ghost |= r.gamma_g != 0.f;
+        force |= (r.p.coupling & FLB_COUPLE_FORCE) != 0;
+        noise = std::max(noise, noise_kind(r.p));
+    }
+    const flb_params &p0 = h->reps[0].p;
+    return batch_record(
+        h,
+        [&](const BatchLists &L, cudaStream_t st) {
+            return launch_batch_step(L, p0.storage, ghost, force, 1, p0.integrator == FLB_HEUN, noise, batch_mu_in(h),
+                                     h->reps[0].q == 15, st);
+        },
+        launch_batch_advance, &h->b_graph, &h->b_exec);
 }
 
 Rep *get_rep(flb_handle *h, int32_t rep)
@@ -1853,11 +1865,22 @@ int flb_autotune(flb_handle *h, const char *cache_path, int32_t flags)
             int e = batch_upload_lists(h);
             if (e == FLB_OK) e = batch_upload_table(h);
             if (e != FLB_OK) return e;
-            const BatchLists L = batch_lists(h);
+            auto stages = [&](const BatchLists &L, cudaStream_t st) {
+                return launch_batch_psi(L, heun, noise, batch_mu_in(h), h->reps[0].q == 15, st);
+            };
+            const int G = (int)h->b_span.size();
+            cudaGraph_t gr = nullptr;
+            cudaGraphExec_t ex = nullptr;
+            if (G > 1) {  // side by side, as in a step
+                e = batch_record(h, stages, [](const BatchLists &, cudaStream_t) { return cudaSuccess; }, &gr, &ex);
+                if (e != FLB_OK) return e;
+            }
             t = time_launches(h, [&]() {
-                h->launches += heun ? 2 : 1;
-                return cuerr(launch_batch_psi(L, heun, noise, batch_mu_in(h), h->reps[0].q == 15, h->st));
+                h->launches += G * (heun ? 2 : 1);
+                return cuerr(ex ? cudaGraphLaunch(ex, h->st) : stages(batch_lists(h), h->st));
             }, reps);
+            if (ex) cudaGraphExecDestroy(ex);
+            if (gr) cudaGraphDestroy(gr);
             return t < 0.f ? (int)FLB_ECUDA : (int)FLB_OK;
         };
         const auto it = cache.find(key);

@@ -218,3 +218,16 @@ def test_modes_keep_their_own_depth(tmp_path):
     assert (s.get_tuning(0), s.get_psi_planes(0)) == (8, 8)
     s.set_mode(F.FLB_MODE_PERSISTENT)
     assert (s.get_tuning(0), s.get_psi_planes(0)) == (5, 5)
+
+
+@pytest.mark.parametrize("integrator", [1, 2])
+def test_autotune_times_both_groups_of_a_large_ensemble(integrator):
+    # from 600 thousand sites on a step launches the stages of two groups of replicas; at a depth
+    # of 4 the chunks 4, 2 and 1 are timed, each in four runs
+    ps = [flb_params(dict(RAGGED, nx=320, ny=317, nz=4, scheme=1, integrator=integrator, seed=r)) for r in range(2)]
+    s = F.Solver(ps)
+    s.set_mode(F.FLB_MODE_BATCHED)
+    before = s.launch_count()
+    chosen = s.autotune()
+    assert set(chosen) <= {1, 2, 4}
+    assert s.launch_count() - before == 3 * 4 * integrator * 2
