@@ -64,8 +64,7 @@ __device__ __forceinline__ void mu3_block(const Geom &g, const float *__restrict
     mu3_column<false>(g, psi, mu, A, B, K, x, y, zb, ze, lw);
 }
 
-__global__ void __launch_bounds__(MU_BX *MU_BY) sigma3_kernel(const Geom g, const float *__restrict__ psi,
-                                                             float *__restrict__ sig, float A, float B, float K)
+__global__ void __launch_bounds__(MU_BX *MU_BY) sigma3_kernel(const Geom g, const float *psi, float *sig, float A, float B, float K)
 {
     pdl_trigger();
     pdl_wait();
@@ -79,8 +78,7 @@ __global__ void __launch_bounds__(MU_BX *MU_BY) sigma3_kernel(const Geom g, cons
 
 // W: the class weights lw of an App. A Laplacian (false: SO)
 template <bool W>
-__global__ void __launch_bounds__(MU_BX *MU_BY) mu3_kernel(const Geom g, const float *__restrict__ psi,
-                                                          float *__restrict__ mu, float A, float B, float K, const LapW lw)
+__global__ void __launch_bounds__(MU_BX *MU_BY) mu3_kernel(const Geom g, const float *psi, float *mu, float A, float B, float K, const LapW lw)
 {
     pdl_trigger();
     pdl_wait();
@@ -115,13 +113,13 @@ __device__ __forceinline__ void mu3_quad(const Geom &g, const float *__restrict_
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
             const int o = c + (r - 1) * Y;
-            const float4 q = __ldg(reinterpret_cast<const float4 *>(psi + o));
-            v[r][0] = lo ? __ldg(psi + o - 1) : 0.f;
+            const float4 q = *reinterpret_cast<const float4 *>(psi + o);
+            v[r][0] = lo ? psi[o - 1] : 0.f;
             v[r][1] = q.x;
             v[r][2] = q.y;
             v[r][3] = q.z;
             v[r][4] = q.w;
-            v[r][5] = hi ? __ldg(psi + o + 4) : 0.f;
+            v[r][5] = hi ? psi[o + 4] : 0.f;
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -139,8 +137,7 @@ __device__ __forceinline__ void mu3_quad(const Geom &g, const float *__restrict_
     }
 }
 
-__global__ void __launch_bounds__(MV_TX *MV_TY) mu3_vec_kernel(const Geom g, const float *__restrict__ psi,
-                                                             float *__restrict__ mu, float A, float B, float K,
+__global__ void __launch_bounds__(MV_TX *MV_TY) mu3_vec_kernel(const Geom g, const float *psi, float *mu, float A, float B, float K,
                                                              int zc)
 {
     pdl_trigger();

@@ -417,6 +417,11 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 // What stands before pdl_wait (index arithmetic, random numbers) touches registers, the
 // block's own shared memory and the constant Box-Muller tables only.  A kernel that triggers also waits, so
 // completion stays in stream order however many launches overlap.
+// Fields are read by plain loads, never __ldg or through a const __restrict__ parameter: those become
+// ld.global.nc, which takes the memory to be constant while the kernel runs, and here the launches in front
+// are still writing it.  Such a load may be made before the wait and may find an old value (of 60
+// runs of 8 steps of a 397 x 395 box, whose four or so launches in flight fit the chip together, up to all
+// differed from the first).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Each block's wait drops its SM's L1 contents, which a grid of many short blocks

@@ -51,22 +51,14 @@ struct CubeArgs {
     float sd;         // naive: sqrt(2 kT M)
 };
 
-// The value at p (global memory through the read-only path, or shared memory).
-template <bool GLOBAL>
-__device__ __forceinline__ F1 rd(const float *p)
-{
-    return F1{GLOBAL ? __ldg(p) : *p};
-}
-
 // Sums of one plane of a field at p (row pitch Y): the centre, the four in-plane faces,
 // the four in-plane diagonals.
 struct Plane3 {
     F1 a, b, d;
 };
-template <bool GLOBAL>
 __device__ __forceinline__ Plane3 plane3(const float *p, int Y)
 {
-    auto at = [&](int o) { return rd<GLOBAL>(p + o); };
+    auto at = [&](int o) { return F1{p[o]}; };
     Plane3 r;
     r.a = at(0);
     r.b = (at(-1) + at(1)) + (at(-Y) + at(Y));
@@ -89,12 +81,12 @@ __device__ __forceinline__ void form_mu(const Psi3Args &a, int x0, int y0, int z
     const int Y = g.px, Z = g.px * g.py;
     const float k22 = a.K * (1.0f / 22.0f);
     const float *p = a.psi + g.pidx32(x, y, z0 - H - 1);
-    Plane3 q0 = plane3<true>(p, Y), q1 = plane3<true>(p + Z, Y);
+    Plane3 q0 = plane3(p, Y), q1 = plane3(p + Z, Y);
     // planes past a ragged box repeat its last one (loads stay unconditional, so that
     // those of all planes are in flight together); what they form is not used
 #pragma unroll
     for (int j = 0; j < CZ + 2 * H; ++j) {
-        const Plane3 q2 = plane3<true>(p + min(j + 2, nzt + 2 * H + 1) * Z, Y);
+        const Plane3 q2 = plane3(p + min(j + 2, nzt + 2 * H + 1) * Z, Y);
         const F1 n1 = q1.b + (q0.a + q2.a), n2 = FD ? (q1.d + q0.b) + q2.b : q1.d + (q0.b + q2.b), n3 = q0.d + q2.d;
         const float ps = q1.a.v;
         smu[(j * WY + ly) * WX + lx] =
@@ -235,7 +227,7 @@ __device__ __forceinline__ void cube_fv_stage(const Psi3Args &a, const float *mu
 #pragma unroll
             for (int j = 0; j < CZ + 4; ++j) {
                 const float *m = m0 + (MU_IN ? min(j, nzt + 3) : j) * Z;
-                auto at = [&](int o) { return rd<MU_IN>(m + o); };
+                auto at = [&](int o) { return F1{m[o]}; };
                 const F1 mxp = at(1), mxm = at(-1), myp = at(Y), mym = at(-Y);
                 const F1 mpp = at(1 + Y), mpm = at(1 - Y), mmp = at(-1 + Y), mmm = at(-1 - Y);
                 const F1 ex = mxp - mxm, ey = myp - mym;
@@ -276,10 +268,10 @@ __device__ __forceinline__ void cube_fv_stage(const Psi3Args &a, const float *mu
                     F1 jx = gx * mg, jy = gy * mg, jz = gz * mg;
                     if (a.advect) {
                         const int o = pi + min(j - 2, nzt + 1) * pz;
-                        const F1 npv = rd<true>(a.psi + o) * -1.0f;
-                        jx = vfma(rd<true>(a.u + o), npv, jx);
-                        jy = vfma(rd<true>(a.u + g.pn + o), npv, jy);
-                        jz = vfma(rd<true>(a.u + 2 * g.pn + o), npv, jz);
+                        const F1 npv = F1{a.psi[o]} * -1.0f;
+                        jx = vfma(F1{a.u[o]}, npv, jx);
+                        jy = vfma(F1{a.u[g.pn + o]}, npv, jy);
+                        jz = vfma(F1{a.u[2 * g.pn + o]}, npv, jz);
                     }
                     float *J = sJ + (j - 2) * CP1 + k;
                     J[0] = jx.v;
@@ -318,7 +310,7 @@ __device__ __forceinline__ void cube_fv_stage(const Psi3Args &a, const float *mu
             d0 = d1;
             d1 = d2;
             if (zh + j >= nzt) break;
-            const F1 pv{FIRST ? __ldg(a.psi + g.pidx32(x, y, z)) : 0.f};
+            const F1 pv{FIRST ? a.psi[g.pidx32(x, y, z)] : 0.f};
             stage_out<FIRST>(a, x, y, z, pv, F1{e_pre[j]}, D, eta);
         }
     }
@@ -393,12 +385,12 @@ __global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
     if (!act) return;
     const int Y = MU_IN ? g.px : CW1, Z = MU_IN ? g.px * g.py : CP1;
     const float *m = MU_IN ? ca.mu + g.pidx32(x, y, z0 + zh - 1) : smu + (tx + 1) + CW1 * (ty + 1) + CP1 * zh;
-    Plane3 q0 = plane3<MU_IN>(m, Y), q1 = plane3<MU_IN>(m + Z, Y);
+    Plane3 q0 = plane3(m, Y), q1 = plane3(m + Z, Y);
 #pragma unroll
     for (int j = 0; j < CZ / 2; ++j) {
         const int z = z0 + zh + j;
         if (zh + j >= nzt) break;
-        const Plane3 q2 = plane3<MU_IN>(m + (j + 2) * Z, Y);
+        const Plane3 q2 = plane3(m + (j + 2) * Z, Y);
         const float n1 = (q1.b + (q0.a + q2.a)).v, n2 = ((q1.d + q0.b) + q2.b).v, n3 = (q0.d + q2.d).v;
         float D = W ? a.M * ((a.lw.c1 * n1 + a.lw.c2 * n2) + (a.lw.c3 * n3 + a.lw.c0 * q1.a.v))
                     : a.M * ((1.0f / 22.0f) * (6.f * n1 + 3.f * n2 + n3 - 80.f * q1.a.v));
@@ -408,9 +400,9 @@ __global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
         if (a.advect) {
             const int sy = g.px, sz = g.px * g.py;
             const float *u = a.u + pi, *v = u + g.pn, *w = v + g.pn, *p = a.psi + pi;
-            const float adv = (__ldg(u + 1) * __ldg(p + 1) - __ldg(u - 1) * __ldg(p - 1)) +
-                              (__ldg(v + sy) * __ldg(p + sy) - __ldg(v - sy) * __ldg(p - sy)) +
-                              (__ldg(w + sz) * __ldg(p + sz) - __ldg(w - sz) * __ldg(p - sz));
+            const float adv = (u[1] * p[1] - u[-1] * p[-1]) +
+                              (v[sy] * p[sy] - v[-sy] * p[-sy]) +
+                              (w[sz] * p[sz] - w[-sz] * p[-sz]);
             D -= 0.5f * adv;
         }
         float eta = 0.f;
@@ -432,7 +424,7 @@ __global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
                 eta = (up + (in0 - own)) + dn;
             }
         }
-        const F1 own{FIRST ? __ldg(a.psi + pi) : 0.f};
+        const F1 own{FIRST ? a.psi[pi] : 0.f};
         stage_out<FIRST>(a, x, y, z, own, F1{e_pre[j]}, F1{D}, F1{eta});
     }
 }

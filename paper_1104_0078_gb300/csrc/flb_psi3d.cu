@@ -44,6 +44,8 @@ __global__ void __launch_bounds__(block_threads<StageV, MU_IN>(), 2) psi3_fv_tma
     extern __shared__ __align__(1024) float tsmem[];
     pdl_trigger();
     pdl_wait();
+    // the fields were stored by threads of the launches in front and come by TMA
+    if (threadIdx.x == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
     psi3_fv_tma_block<STAGE, NOISE, false, false, RK, MU_IN, Q15, StageV>(&psi_map, &u_map, ta.a, ta.status, blockIdx.x,
                                                                      blockIdx.y, blockIdx.z, tsmem, &mu_map);
 }

@@ -15,15 +15,13 @@
 
 namespace flb {
 
-// Loads of fields written by earlier launches take the read-only path (COH
-// false).  Inside the persistent batched kernel a field may have been written
-// by another block of the same launch, so loads go to L2 (COH true): the
-// read-only path and L1 are not coherent within a launch.
+// Loads of fields written by earlier launches are plain ones (COH false; see launch_pdl).  Inside the
+// persistent batched kernel a field may have been written by another block of the same
+// launch, so loads go to L2 (COH true): L1 is not coherent within a launch.
 template <bool COH>
 __device__ __forceinline__ float ldf(const float *p)
 {
-    if (COH) return __ldcg(p);
-    return __ldg(p);
+    return COH ? __ldcg(p) : *p;
 }
 template <bool COH>
 __device__ __forceinline__ float ld3(const float *p, int i)

@@ -32,7 +32,7 @@ namespace {
 template <typename T>
 __device__ __forceinline__ float ldp(const T *p);
 template <>
-__device__ __forceinline__ float ldp<float>(const float *p) { return __ldg(p); }
+__device__ __forceinline__ float ldp<float>(const float *p) { return *p; }
 template <>
 __device__ __forceinline__ float ldp<__half>(const __half *p) { return __half2float(*p); }
 __device__ __forceinline__ void stp(float *p, float v) { *p = v; }
@@ -42,7 +42,7 @@ __device__ __forceinline__ void stp(__half *p, float v) { *p = __float2half_rn(v
 // (n sites each): fbar_i(r) = stored_i(r - c_i).  Planes: 0 rest; (1,2) +-x,
 // (3,4) +-y, (5,6) +-(1,1), (7,8) +-(1,-1).
 template <typename T>
-__device__ __forceinline__ void pull9(const T *__restrict__ f, long long n, int nx, int ny, int x, int y, float v[9])
+__device__ __forceinline__ void pull9(const T *f, long long n, int nx, int ny, int x, int y, float v[9])
 {
     const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
     const int r0 = nx * y, rm = nx * (y == 0 ? ny - 1 : y - 1), rp = nx * (y == ny - 1 ? 0 : y + 1);
@@ -69,7 +69,7 @@ __device__ __forceinline__ float lap2(const float *f, int c, const LapW &w)
 // Load the psi region tile + H (row pitch TX + 2H) of the block at (x0, y0); cells
 // past a ragged box's ghost frame repeat its last column or row and are not used.
 template <int TX, int TY, int H, int NT>
-__device__ __forceinline__ void load_psi2(const Geom &g, const float *__restrict__ psi, int x0, int y0, float *s)
+__device__ __forceinline__ void load_psi2(const Geom &g, const float *psi, int x0, int y0, float *s)
 {
     constexpr int W = TX + 2 * H, N = W * (TY + 2 * H);
 #pragma unroll
@@ -77,7 +77,7 @@ __device__ __forceinline__ void load_psi2(const Geom &g, const float *__restrict
         const int k = (int)threadIdx.x + j * NT;
         if (k < N) {
             const int x = min(x0 - H + k % W, g.nx + GX - 1), y = min(y0 - H + k / W, g.ny + GY - 1);
-            s[k] = __ldg(psi + (x + GX) + g.px * (y + GY));
+            s[k] = psi[(x + GX) + g.px * (y + GY)];
         }
     }
 }
@@ -457,8 +457,8 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
             int lx, ly;
             const bool in = advect && point((int)threadIdx.x + j * NT, lx, ly);
             const int o = in ? (x0 + lx + GX) + g.px * (y0 + ly + GY) : 0;
-            uxy[j][0] = in ? __ldg(a.u + o) : 0.f;
-            uxy[j][1] = in ? __ldg(a.u + g.pn + o) : 0.f;
+            uxy[j][0] = in ? a.u[o] : 0.f;
+            uxy[j][1] = in ? a.u[g.pn + o] : 0.f;
         }
 #pragma unroll
         for (int j = 0; j < J0; ++j) {

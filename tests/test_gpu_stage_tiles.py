@@ -138,3 +138,32 @@ def test_batched_in_two_groups_equals_plain(q, extra):
     for ra, rb in zip(*runs):
         for a, b in zip(ra, rb):
             assert np.array_equal(a, b)
+
+
+# boxes whose launches are small enough for several to be in flight together
+@pytest.mark.parametrize("d", [
+    dict(dim=2, q=9, nx=397, ny=395, scheme=0, gamma_ghost=0.3, gamma_bulk=-0.4),
+    dict(dim=2, q=9, nx=397, ny=395, scheme=1, gamma_ghost=0.3, force_grad=3),
+    dict(dim=2, q=9, nx=397, ny=395, scheme=0, gamma_ghost=0.3, storage=F.FLB_F16_DEV),
+    dict(dim=2, q=9, nx=420, ny=371, scheme=1, integrator=4),
+    dict(dim=2, q=9, nx=130, ny=95, scheme=0, gamma_ghost=0.3), dict(dim=2, q=9, nx=64, ny=64, scheme=1),
+    dict(nx=64, ny=40, nz=52, gamma_ghost=0.3), dict(nx=32, ny=32, nz=32, q=15), dict(nx=63, ny=33, nz=45, scheme=0),
+    dict(nx=48, ny=48, nz=48, q=15, scheme=0, gamma_ghost=0.3), dict(nx=48, ny=40, nz=37, integrator=4, force_grad=3),
+    dict(nx=48, ny=40, nz=37, laplacian=2), dict(nx=48, ny=40, nz=37, scheme=2, laplacian=1),
+    dict(nx=64, ny=40, nz=52, storage=F.FLB_F16_DEV), dict(nx=121, ny=120, nz=93), dict(nx=60, ny=60, nz=60, q=15, zc=8)])
+def test_overlapped_launches_give_the_same_steps(d):
+    # steps enqueued one behind the other, whose launches overlap, against steps waited for one by one
+    d = dict(BASE, **d)
+    s = F.Solver(flb_params(d))
+    _start(s, d)
+    if "zc" in d:
+        s.set_tuning(d["zc"])
+    start = s.get_state()
+    for _ in range(8):
+        s.step(1)
+        s.synchronize()
+    ref = s.get_state()
+    for k in range(30):
+        s.set_state(start)
+        s.step(8)
+        assert s.get_state() == ref, k
