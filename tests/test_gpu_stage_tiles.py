@@ -167,3 +167,28 @@ def test_overlapped_launches_give_the_same_steps(d):
         s.set_state(start)
         s.step(8)
         assert s.get_state() == ref, k
+
+
+@pytest.mark.parametrize("shape", [(47, 31), (397, 395)])
+@pytest.mark.parametrize("extra", [{}, dict(force_grad=3, gamma_ghost=0.3), dict(kT=0.0, coupling=0)])
+def test_2d_bulk_rate_matches_oracle(shape, extra):
+    # the trace relaxing at its own rate, one site a thread and two
+    d = dict(BASE, dim=2, q=9, nx=shape[0], ny=shape[1], scheme=0, gamma_bulk=-0.4)
+    d.update(extra)
+    _against_oracle(d, 8, 1e-5, 1e-5)
+
+
+@pytest.mark.parametrize("shape,chunks", [((129, 130, 131), 5), ((161, 160, 163), 9)])
+def test_read_reuses_its_ring(shape, chunks):
+    # psi and u of more than four chunks of 2^21 values: from the fifth on a chunk takes a slot whose
+    # values the threads have converted; psi ends and a component of u begins within a chunk
+    N = shape[0] * shape[1] * shape[2]
+    assert -(-4 * N // 2 ** 21) == chunks
+    s = F.Solver(flb_params(dict(BASE, nx=shape[0], ny=shape[1], nz=shape[2])))
+    psi = I.random_field(N, 0.05, 3)
+    u = np.stack([I.random_field(N, 1e-2, 4 + a) for a in range(3)])
+    s.set_fields(psi=psi, u=u)
+    for _ in range(3):
+        p, v = s.get_psi_u()
+        assert np.array_equal(p, psi)
+        assert np.array_equal(v, u)
