@@ -28,7 +28,7 @@ struct PlanesStride32 {
 };
 
 // Two sites per thread, (x, y, z) and (x, y, z + 1), as in the collide-stream.
-template <typename T, bool FORCE>
+template <typename T, bool FORCE, int LK>
 __global__ void __launch_bounds__(LB_BX *LB_BY, 10) vel3_kernel(const LBArgs a)
 {
     pdl_trigger();
@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(LB_BX *LB_BY, 10) vel3_kernel(const LBArgs a)
     if (x >= g.nx || y >= g.ny || z >= g.nz) return;
     const int nl = z + 1 < g.nz ? 2 : 1;
     const int zl[2] = {z, z + nl - 1};
-    vel3_sites<F2, T, FORCE, false>(a, PlanesStride32<T>{(const T *)a.fout, (int)g.n}, x, y, zl, nl);
+    vel3_sites<F2, T, FORCE, LK>(a, PlanesStride32<T>{(const T *)a.fout, (int)g.n}, x, y, zl, nl);
 }
 
 // mu = A psi + B psi^3 - K lap_SO psi on the interior and HALO ghost layers
@@ -52,19 +52,21 @@ __global__ void __launch_bounds__(LB_BX *LB_BY, 10) vel3_kernel(const LBArgs a)
 //   22 lap_SO psi(z) = 6 [b(z) + a(z-1) + a(z+1)] + 3 [d(z) + b(z-1) + b(z+1)]
 //                      + d(z-1) + d(z+1) - 80 a(z)
 // takes 9 loads per plane instead of 27.
-template <int HALO = 1>
+template <int HALO, int LK>
 __device__ __forceinline__ void mu3_block(const Geom &g, const float *__restrict__ psi, float *__restrict__ mu, float A,
-                                          float B, float K, int bx, int by, int bz, const LapW *lw = nullptr)
+                                          float B, float K, int bx, int by, int bz, const LapW *lw)
 {
     const int x = bx * MU_BX + (int)threadIdx.x - HALO;
     const int y = by * MU_BY + (int)threadIdx.y - HALO;
     const int zb = bz * MU_ZC - HALO;                       // first output plane
     const int ze = min(zb + MU_ZC, g.nz + HALO);            // one past the last
     if (x >= g.nx + HALO || y >= g.ny + HALO || zb >= ze) return;
-    mu3_column<false>(g, psi, mu, A, B, K, x, y, zb, ze, lw);
+    mu3_column<LK>(g, psi, mu, A, B, K, x, y, zb, ze, lw);
 }
 
-__global__ void __launch_bounds__(MU_BX *MU_BY) sigma3_kernel(const Geom g, const float *psi, float *sig, float A, float B, float K)
+template <int LK>
+__global__ void __launch_bounds__(MU_BX *MU_BY) sigma3_kernel(const Geom g, const float *psi, float *sig, float A,
+                                                             float B, float K)
 {
     pdl_trigger();
     pdl_wait();
@@ -73,19 +75,20 @@ __global__ void __launch_bounds__(MU_BX *MU_BY) sigma3_kernel(const Geom g, cons
     const int zb = blockIdx.z * MU_ZC - 1;
     const int ze = min(zb + MU_ZC, g.nz + 1);
     if (x > g.nx || y > g.ny || zb >= ze) return;
-    sigma3_column<false>(g, psi, sig, A, B, K, x, y, zb, ze);
+    sigma3_column<LK>(g, psi, sig, A, B, K, x, y, zb, ze);
 }
 
-// W: the class weights lw of an App. A Laplacian (false: SO)
-template <bool W>
-__global__ void __launch_bounds__(MU_BX *MU_BY) mu3_kernel(const Geom g, const float *psi, float *mu, float A, float B, float K, const LapW lw)
+// lw: the class weights of an App. A Laplacian
+template <int LK>
+__global__ void __launch_bounds__(MU_BX *MU_BY) mu3_kernel(const Geom g, const float *psi, float *mu, float A, float B,
+                                                          float K, const LapW lw)
 {
     pdl_trigger();
     pdl_wait();
-    mu3_block<MU3_HALO>(g, psi, mu, A, B, K, blockIdx.x, blockIdx.y, blockIdx.z, W ? &lw : nullptr);
+    mu3_block<MU3_HALO, LK>(g, psi, mu, A, B, K, blockIdx.x, blockIdx.y, blockIdx.z, &lw);
 }
 
-// The same field (SO stencil) with four consecutive x per thread: x = xs ..
+// mu with the SO stencil, four consecutive x per thread: x = xs ..
 // xs+3, xs = -4 + 4 i, so that xs is 16-byte aligned in the padded rows.  Per
 // plane a thread reads each of the rows y-1, y, y+1 as one 16-byte load and the
 // two cells beside it (3 x 3 loads for four points instead of 4 x 9), keeps the
@@ -163,7 +166,7 @@ __global__ void __launch_bounds__(MUB_NT) mu3_batch_kernel(const BatchLists L)
             const int p = j * MUB_NT + (int)threadIdx.x, k = b.bx + p / 4;
             const int x = -4 + 4 * (k % nq) + p % 4, y = k / nq - MU3_HALO;
             if (x >= -1 && x <= g.nx && y >= -1 && y <= g.ny && zb < ze)
-                sigma3_column<false>(g, r.psi[par], const_cast<float *>(r.lb.sig), r.A, r.B, r.K, x, y, zb, ze);
+                sigma3_column<LD_PLAIN>(g, r.psi[par], const_cast<float *>(r.lb.sig), r.A, r.B, r.K, x, y, zb, ze);
         }
         return;
     }
@@ -180,14 +183,14 @@ __global__ void __launch_bounds__(LBB_NT) vel3_batch_kernel(const BatchLists L)
     batch_lb_args(L, L.reps[b.rep], sa);
     int x, y, zl[2], nl;
     if (packed_pair<LBB_NT>(sa.g, b.bx, b.by, b.bz, threadIdx.x, x, y, zl, nl))
-        vel3_sites<F2, T, FORCE, false>(sa, PlanesFromBase<T>{(const T *)sa.fout, nullptr, sa.g.n}, x, y, zl, nl);
+        vel3_sites<F2, T, FORCE, LD_PLAIN>(sa, PlanesFromBase<T>{(const T *)sa.fout, nullptr, sa.g.n}, x, y, zl, nl);
 }
 
 cudaError_t launch_mu3(const Geom &g, const float *psi, float *mu, float A, float B, float K, cudaStream_t st,
                        const LapW *lw)
 {
     constexpr int E = 2 * MU3_HALO;
-    if (!lw && g.dim == 3) {  // threads for x = -4 .. nx + 1 in fours
+    if (!lw) {  // threads for x = -4 .. nx + 1 in fours
         const int nxt = (g.nx + 2 + 4 + 3) / 4;
         const int cols = ((nxt + MV_TX - 1) / MV_TX) * ((g.ny + E + MV_TY - 1) / MV_TY);
         const int zc = cols * ((g.nz + E + MV_ZC - 1) / MV_ZC) < 4 * 152 ? MV_ZC_SMALL : MV_ZC;
@@ -196,15 +199,16 @@ cudaError_t launch_mu3(const Geom &g, const float *psi, float *mu, float A, floa
     }
     const dim3 block(MU_BX, MU_BY, 1);
     const dim3 grid((g.nx + E + MU_BX - 1) / MU_BX, (g.ny + E + MU_BY - 1) / MU_BY, (g.nz + E + MU_ZC - 1) / MU_ZC);
-    return lw ? launch_pdl(mu3_kernel<true>, grid, block, 0, st, PDL_BLOCKS, g, psi, mu, A, B, K, *lw)
-              : launch_pdl(mu3_kernel<false>, grid, block, 0, st, PDL_BLOCKS, g, psi, mu, A, B, K, LapW{0.f, 0.f, 0.f, 0.f});
+    return launch_pdl(overlaps(grid, PDL_BLOCKS) ? mu3_kernel<LD_PLAIN> : mu3_kernel<LD_CONST>, grid, block, 0, st,
+                      PDL_BLOCKS, g, psi, mu, A, B, K, *lw);
 }
 
 cudaError_t launch_sigma3(const Geom &g, const float *psi, float *sig, float A, float B, float K, cudaStream_t st)
 {
     const dim3 block(MU_BX, MU_BY, 1);
     const dim3 grid((g.nx + 2 + MU_BX - 1) / MU_BX, (g.ny + 2 + MU_BY - 1) / MU_BY, (g.nz + 2 + MU_ZC - 1) / MU_ZC);
-    return launch_pdl(sigma3_kernel, grid, block, 0, st, PDL_BLOCKS, g, psi, sig, A, B, K);
+    return launch_pdl(overlaps(grid, PDL_BLOCKS) ? sigma3_kernel<LD_PLAIN> : sigma3_kernel<LD_CONST>, grid, block, 0, st,
+                      PDL_BLOCKS, g, psi, sig, A, B, K);
 }
 
 cudaError_t launch_vel3(const LBArgs &a, int storage, cudaStream_t st)
@@ -212,11 +216,10 @@ cudaError_t launch_vel3(const LBArgs &a, int storage, cudaStream_t st)
     const dim3 block(LB_BX, LB_BY, 1);
     const dim3 grid((a.g.nx + LB_BX - 1) / LB_BX, (a.g.ny + LB_BY - 1) / LB_BY, (a.g.nz + LB_BZ - 1) / LB_BZ);
     const bool force = (a.coupling & FLB_COUPLE_FORCE) != 0;
-    if (storage == FLB_F16_DEV)
-        return force ? launch_pdl(vel3_kernel<__half, true>, grid, block, 0, st, PDL_BLOCKS, a)
-                     : launch_pdl(vel3_kernel<__half, false>, grid, block, 0, st, PDL_BLOCKS, a);
-    return force ? launch_pdl(vel3_kernel<float, true>, grid, block, 0, st, PDL_BLOCKS, a)
-                 : launch_pdl(vel3_kernel<float, false>, grid, block, 0, st, PDL_BLOCKS, a);
+    auto go = [&](auto kernel) { return launch_pdl(kernel, grid, block, 0, st, PDL_BLOCKS, a); };
+    if (storage == FLB_F16_DEV) return force ? go(vel3_kernel<__half, true, LD_PLAIN>) : go(vel3_kernel<__half, false, LD_PLAIN>);
+    if (overlaps(grid, PDL_BLOCKS)) return force ? go(vel3_kernel<float, true, LD_PLAIN>) : go(vel3_kernel<float, false, LD_PLAIN>);
+    return force ? go(vel3_kernel<float, true, LD_CONST>) : go(vel3_kernel<float, false, LD_CONST>);
 }
 
 cudaError_t launch_mu3_batch(const BatchLists &L, cudaStream_t st)

@@ -421,7 +421,8 @@ __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_g
 // ld.global.nc, which takes the memory to be constant while the kernel runs, and here the launches in front
 // are still writing it.  Such a load may be made before the wait and may find an old value (of 60
 // runs of 8 steps of a 397 x 395 box, whose four or so launches in flight fit the chip together, up to all
-// differed from the first).
+// differed from the first).  A kernel may have an instance that reads so for the grids that do not
+// overlap.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Each block's wait drops its SM's L1 contents, which a grid of many short blocks
@@ -431,6 +432,8 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // 128^3 gains most (64^3: 59.0 -> 49.1 us); the 2D kernels, which read little twice,
 // gain up to larger grids (2048^2, 8192 blocks: 244 -> 233 us).
 constexpr long long PDL_BLOCKS = 16 * 152;
+// whether launch_pdl lets a grid overlap the launches in front of it
+inline bool overlaps(dim3 grid, long long max_blocks) { return (long long)grid.x * grid.y * grid.z <= max_blocks; }
 template <class... P, class... A>
 inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                               long long max_blocks, A &&...args)
@@ -444,7 +447,7 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
     c.dynamicSmemBytes = smem;
     c.stream = st;
     c.attrs = at;
-    c.numAttrs = (long long)grid.x * grid.y * grid.z <= max_blocks ? 1 : 0;
+    c.numAttrs = overlaps(grid, max_blocks) ? 1 : 0;
     return cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 

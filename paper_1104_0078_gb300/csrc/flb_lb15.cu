@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(LB_BX *LB_BY, 7) lb15_kernel(const LBArgs a, c
     const int nl = z + 1 < g.nz ? 2 : 1;
     const int zl[2] = {z, z + nl - 1};
     F2 Fx = F2::bc(0.f), Fy = F2::bc(0.f), Fz = F2::bc(0.f);
-    if (FORCE) force3v<false, F2, true>(a, x, y, zl, Fx, Fy, Fz);
+    if (FORCE) force3v<LD_PLAIN, F2, true>(a, x, y, zl, Fx, Fy, Fz);
     const bool inner = y > 0 && y < g.ny - 1 && z > 0 && z < g.nz - 2;  // the same for the whole warp
     lb15_sites_on<F2, T, GHOST_RELAX, false>(a, P, x, y, zl, nl, Fx, Fy, Fz, [&](F2 *f) {
         if (inner) {
@@ -65,8 +65,8 @@ __global__ void __launch_bounds__(LBB_NT, 7) lb15_batch_kernel(const BatchLists 
     int x, y, zl[2], nl;
     if (!packed_pair<LBB_NT>(sa.g, b.bx, b.by, b.bz, threadIdx.x, x, y, zl, nl)) return;
     F2 Fx = F2::bc(0.f), Fy = F2::bc(0.f), Fz = F2::bc(0.f);
-    if (FORCE && (sa.coupling & FLB_COUPLE_FORCE)) force3v<false, F2, true>(sa, x, y, zl, Fx, Fy, Fz);
-    lb15_sites<F2, T, GHOST_RELAX, false, true>(sa, PlanesFromBase<T>{(const T *)sa.fin, (T *)sa.fout, sa.g.n}, x, y,
+    if (FORCE && (sa.coupling & FLB_COUPLE_FORCE)) force3v<LD_PLAIN, F2, true>(sa, x, y, zl, Fx, Fy, Fz);
+    lb15_sites<F2, T, GHOST_RELAX, LD_PLAIN, true>(sa, PlanesFromBase<T>{(const T *)sa.fin, (T *)sa.fout, sa.g.n}, x, y,
                                                 zl, nl, Fx, Fy, Fz);
 }
 

@@ -30,7 +30,9 @@ namespace flb {
 // of Blackwell's packed FP32 registers (one issue slot for both sites' FP32
 // arithmetic).  A warp covers 32 consecutive x, so every population plane is
 // read and written in full rows.
-template <typename T, bool GHOST_RELAX, bool FORCE>
+// LK: how the populations are read (ld3): large boxes, whose launches do not overlap, through the read-only
+// path.
+template <typename T, bool GHOST_RELAX, bool FORCE, int LK>
 __global__ void __launch_bounds__(LB_BX *LB_BY, 7)
     lb3_kernel(const LBArgs a, const __grid_constant__ PlaneTable<T> P)
 {
@@ -44,11 +46,11 @@ __global__ void __launch_bounds__(LB_BX *LB_BY, 7)
     const int nl = z + 1 < g.nz ? 2 : 1;
     const int zl[2] = {z, z + nl - 1};  // a lane past the box repeats lane 0's site
     F2 Fx = F2::bc(0.f), Fy = F2::bc(0.f), Fz = F2::bc(0.f);
-    if (FORCE && (a.coupling & FLB_COUPLE_FORCE)) force3v<false, F2, true>(a, x, y, zl, Fx, Fy, Fz);
+    if (FORCE && (a.coupling & FLB_COUPLE_FORCE)) force3v<LK, F2, true>(a, x, y, zl, Fx, Fy, Fz);
     const bool inner = y > 0 && y < g.ny - 1 && z > 0 && z < g.nz - 2;  // the same for the whole warp
     lb_sites_on<F2, T, GHOST_RELAX, false>(a, P, x, y, zl, nl, Fx, Fy, Fz, [&](F2 *f) {
-        if (inner) pull_inner<T, 19>(P, g, x, y, z, f);
-        else pullv<T, false>(P, g, x, y, zl, f);
+        if (inner) pull_inner<T, 19, LK>(P, g, x, y, z, f);
+        else pullv<T, LK>(P, g, x, y, zl, f);
     });
 }
 
@@ -63,8 +65,8 @@ __global__ void __launch_bounds__(LBB_NT, 7) lb3_batch_kernel(const BatchLists L
     int x, y, zl[2], nl;
     if (!packed_pair<LBB_NT>(sa.g, b.bx, b.by, b.bz, threadIdx.x, x, y, zl, nl)) return;
     F2 Fx = F2::bc(0.f), Fy = F2::bc(0.f), Fz = F2::bc(0.f);
-    if (FORCE && (sa.coupling & FLB_COUPLE_FORCE)) force3v<false, F2, true>(sa, x, y, zl, Fx, Fy, Fz);
-    lb_sites<F2, T, GHOST_RELAX, false, true>(sa, PlanesFromBase<T>{(const T *)sa.fin, (T *)sa.fout, sa.g.n}, x, y,
+    if (FORCE && (sa.coupling & FLB_COUPLE_FORCE)) force3v<LD_PLAIN, F2, true>(sa, x, y, zl, Fx, Fy, Fz);
+    lb_sites<F2, T, GHOST_RELAX, LD_PLAIN, true>(sa, PlanesFromBase<T>{(const T *)sa.fin, (T *)sa.fout, sa.g.n}, x, y,
                                               zl, nl, Fx, Fy, Fz);
 }
 
@@ -89,21 +91,24 @@ cudaError_t launch_lb3_batch(const BatchLists &L, int storage, bool ghost, bool 
     return launch_vel3_batch(L, storage, force, st);
 }
 
+namespace {
+template <typename T, int LK>
+cudaError_t go_lb3(const LBArgs &a, dim3 grid, cudaStream_t st)
+{
+    const bool force = (a.coupling & FLB_COUPLE_FORCE) != 0;
+    auto go = [&](auto kernel) {
+        return launch_pdl(kernel, grid, dim3(LB_BX, LB_BY, 1), 0, st, PDL_BLOCKS, a, plane_table<T>(a.fin, a.fout, a.g, 19));
+    };
+    if (a.gamma_g != 0.0f) return force ? go(lb3_kernel<T, true, true, LK>) : go(lb3_kernel<T, true, false, LK>);
+    return force ? go(lb3_kernel<T, false, true, LK>) : go(lb3_kernel<T, false, false, LK>);
+}
+}  // namespace
+
 cudaError_t launch_lb3d(const LBArgs &a, int storage, cudaStream_t st)
 {
-    const dim3 block(LB_BX, LB_BY, 1);
     const dim3 grid((a.g.nx + LB_BX - 1) / LB_BX, (a.g.ny + LB_BY - 1) / LB_BY, (a.g.nz + LB_BZ - 1) / LB_BZ);
-    const bool gr = a.gamma_g != 0.0f;
-    const bool force = (a.coupling & FLB_COUPLE_FORCE) != 0;
-#define FLB_LB3(T, G, F) return launch_pdl(lb3_kernel<T, G, F>, grid, block, 0, st, PDL_BLOCKS, a, plane_table<T>(a.fin, a.fout, a.g, 19))
-    if (storage == FLB_F16_DEV) {
-        if (gr) { if (force) FLB_LB3(__half, true, true); else FLB_LB3(__half, true, false); }
-        else { if (force) FLB_LB3(__half, false, true); else FLB_LB3(__half, false, false); }
-    } else {
-        if (gr) { if (force) FLB_LB3(float, true, true); else FLB_LB3(float, true, false); }
-        else { if (force) FLB_LB3(float, false, true); else FLB_LB3(float, false, false); }
-    }
-#undef FLB_LB3
+    if (storage == FLB_F16_DEV) return go_lb3<__half, LD_PLAIN>(a, grid, st);
+    return overlaps(grid, PDL_BLOCKS) ? go_lb3<float, LD_PLAIN>(a, grid, st) : go_lb3<float, LD_CONST>(a, grid, st);
 }
 
 }  // namespace flb

@@ -12,7 +12,7 @@ namespace flb {
 // null): the class weights of an App. A Laplacian instead of SO's,
 // mu = A psi + B psi^3 - K [(c1 n1 + c2 n2) + (c3 n3 + c0 psi)] over the faces
 // n1, edges n2 and corners n3 of the 3 x 3 x 3 neighbourhood.
-template <bool COH = false>
+template <int LK = LD_PLAIN>
 __device__ __forceinline__ void mu3_column(const Geom &g, const float *__restrict__ psi, float *__restrict__ mu, float A,
                                            float B, float K, int x, int y, int zb, int ze, const LapW *lw = nullptr)
 {
@@ -21,9 +21,9 @@ __device__ __forceinline__ void mu3_column(const Geom &g, const float *__restric
     int c = g.pidx32(x, y, zb - 1);
     float a0 = 0.f, b0 = 0.f, d0 = 0.f, a1 = 0.f, b1 = 0.f, d1 = 0.f;  // planes p-2, p-1
     for (int p = zb - 1; p <= ze; ++p, c += Z) {
-        const float a2 = ldf<COH>(psi + c);
-        const float b2 = (ldf<COH>(psi + c - 1) + ldf<COH>(psi + c + 1)) + (ldf<COH>(psi + c - Y) + ldf<COH>(psi + c + Y));
-        const float d2 = (ldf<COH>(psi + c - 1 - Y) + ldf<COH>(psi + c + 1 - Y)) + (ldf<COH>(psi + c - 1 + Y) + ldf<COH>(psi + c + 1 + Y));
+        const float a2 = ldf<LK>(psi + c);
+        const float b2 = (ldf<LK>(psi + c - 1) + ldf<LK>(psi + c + 1)) + (ldf<LK>(psi + c - Y) + ldf<LK>(psi + c + Y));
+        const float d2 = (ldf<LK>(psi + c - 1 - Y) + ldf<LK>(psi + c + 1 - Y)) + (ldf<LK>(psi + c - 1 + Y) + ldf<LK>(psi + c + 1 + Y));
         if (p - 1 >= zb) {
             const float n1 = b1 + (a0 + a2), n2 = d1 + (b0 + b2), n3 = d0 + d2;
             mu[c - Z] = lw ? A * a1 + B * a1 * a1 * a1 - K * ((lw->c1 * n1 + lw->c2 * n2) + (lw->c3 * n3 + lw->c0 * a1))
@@ -39,7 +39,7 @@ __device__ __forceinline__ void mu3_column(const Geom &g, const float *__restric
 // - K psi lap_SO psi - K/2 |g|^2], g the central-difference gradient of psi.
 // Per plane a thread keeps the centre, the faces and the diagonals of psi (the
 // SO stencil, as in mu3_column) and the in-plane face differences.
-template <bool COH = false>
+template <int LK = LD_PLAIN>
 __device__ __forceinline__ void sigma3_column(const Geom &g, const float *__restrict__ psi, float *__restrict__ sig,
                                               float A, float B, float K, int x, int y, int zb, int ze)
 {
@@ -47,11 +47,11 @@ __device__ __forceinline__ void sigma3_column(const Geom &g, const float *__rest
     int c = g.pidx32(x, y, zb - 1);
     float a0 = 0.f, b0 = 0.f, d0 = 0.f, a1 = 0.f, b1 = 0.f, d1 = 0.f, gx1 = 0.f, gy1 = 0.f;
     for (int p = zb - 1; p <= ze; ++p, c += Z) {
-        const float a2 = ldf<COH>(psi + c);
-        const float xm = ldf<COH>(psi + c - 1), xp = ldf<COH>(psi + c + 1);
-        const float ym = ldf<COH>(psi + c - Y), yp = ldf<COH>(psi + c + Y);
+        const float a2 = ldf<LK>(psi + c);
+        const float xm = ldf<LK>(psi + c - 1), xp = ldf<LK>(psi + c + 1);
+        const float ym = ldf<LK>(psi + c - Y), yp = ldf<LK>(psi + c + Y);
         const float b2 = (xm + xp) + (ym + yp);
-        const float d2 = (ldf<COH>(psi + c - 1 - Y) + ldf<COH>(psi + c + 1 - Y)) + (ldf<COH>(psi + c - 1 + Y) + ldf<COH>(psi + c + 1 + Y));
+        const float d2 = (ldf<LK>(psi + c - 1 - Y) + ldf<LK>(psi + c + 1 - Y)) + (ldf<LK>(psi + c - 1 + Y) + ldf<LK>(psi + c + 1 + Y));
         if (p - 1 >= zb) {  // plane p-1: centre a1, gradient (gx1, gy1, gz)
             const float n1 = b1 + (a0 + a2), n2 = d1 + (b0 + b2), n3 = d0 + d2;
             const float lap = (6.f * n1 + 3.f * n2 + n3 - 80.f * a1) * (1.0f / 22.0f);

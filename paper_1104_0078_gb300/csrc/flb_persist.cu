@@ -120,9 +120,9 @@ __global__ void __launch_bounds__(PB_NT, 2) persist_kernel(const PersistArgs P)
             const int zb = task.bz * MU_ZC - MU3_HALO, ze = min(zb + MU_ZC, g.nz + MU3_HALO);
             if (x < g.nx + MU3_HALO && y < g.ny + MU3_HALO) {
                 if (r.lb.force_kind == 2)
-                    sigma3_column<true>(g, r.psi[ds & 1], const_cast<float *>(r.lb.sig), r.A, r.B, r.K, x, y, zb, ze);
+                    sigma3_column<LD_L2>(g, r.psi[ds & 1], const_cast<float *>(r.lb.sig), r.A, r.B, r.K, x, y, zb, ze);
                 else
-                    mu3_column<true>(g, r.psi[ds & 1], const_cast<float *>(r.lb.mu), r.A, r.B, r.K, x, y, zb, ze);
+                    mu3_column<LD_L2>(g, r.psi[ds & 1], const_cast<float *>(r.lb.mu), r.A, r.B, r.K, x, y, zb, ze);
             }
         } else if (task.phase == PH_LB || task.phase == PH_VEL) {
             lb_args_at(r, ds, sla);
@@ -133,21 +133,21 @@ __global__ void __launch_bounds__(PB_NT, 2) persist_kernel(const PersistArgs P)
                 if (!packed_site<PL_SITES>(sla.g, task.bx, task.by, task.bz, t + PB_NT * j, x, y, z)) continue;
                 if (task.phase == PH_LB) {
                     float Fx = 0.f, Fy = 0.f, Fz = 0.f;
-                    if (force) force3<true>(sla, x, y, z, Fx, Fy, Fz);
+                    if (force) force3<LD_L2>(sla, x, y, z, Fx, Fy, Fz);
                     if (Q15) {
-                        if (sla.gamma_g != 0.f) lb15_site<float, true, true, true>(sla, x, y, z, Fx, Fy, Fz);
-                        else lb15_site<float, false, true, true>(sla, x, y, z, Fx, Fy, Fz);
+                        if (sla.gamma_g != 0.f) lb15_site<float, true, LD_L2, true>(sla, x, y, z, Fx, Fy, Fz);
+                        else lb15_site<float, false, LD_L2, true>(sla, x, y, z, Fx, Fy, Fz);
                     } else if (sla.gamma_g != 0.f) {
-                        lb_site<float, true, true, true>(sla, x, y, z, Fx, Fy, Fz);
+                        lb_site<float, true, LD_L2, true>(sla, x, y, z, Fx, Fy, Fz);
                     } else {
-                        lb_site<float, false, true, true>(sla, x, y, z, Fx, Fy, Fz);
+                        lb_site<float, false, LD_L2, true>(sla, x, y, z, Fx, Fy, Fz);
                     }
                 } else if (Q15) {
-                    if (force) vel15_site<float, true, true>(sla, x, y, z);
-                    else vel15_site<float, false, true>(sla, x, y, z);
+                    if (force) vel15_site<float, true, LD_L2>(sla, x, y, z);
+                    else vel15_site<float, false, LD_L2>(sla, x, y, z);
                 } else {
-                    if (force) vel3_site<float, true, true>(sla, x, y, z);
-                    else vel3_site<float, false, true>(sla, x, y, z);
+                    if (force) vel3_site<float, true, LD_L2>(sla, x, y, z);
+                    else vel3_site<float, false, LD_L2>(sla, x, y, z);
                 }
             }
         } else {

@@ -338,8 +338,10 @@ __device__ constexpr int8_t kCubeL[13][3] = {{1, 0, 0},  {0, 1, 0},  {0, 0, 1}, 
                                              {1, 0, 1},  {1, 0, -1}, {0, 1, 1},  {0, 1, -1}, {1, 1, 1},
                                              {1, 1, -1}, {1, -1, 1}, {1, -1, -1}};
 
+// Without noise, 512 threads go three blocks an SM (40 registers; with 43 two, and at 512^3 a later
+// stage with another Laplacian takes 2.30 ms instead of 1.75).  0: no bound.
 template <class T, bool FIRST, int NOISE, bool MU_IN, bool W>
-__global__ void __launch_bounds__(T::NT) psi3_fd_cube_kernel(const CubeArgs ca)
+__global__ void __launch_bounds__(T::NT, NOISE == 0 && T::NT == 512 ? 3 : 0) psi3_fd_cube_kernel(const CubeArgs ca)
 {
     FLB_TILE3(T);
     constexpr int ZN = (CZ + 2) * CP1;

@@ -25,7 +25,7 @@
 namespace flb {
 
 // fbar_i(r) = stored_i(r - c_i) for the 15 planes of site (x, y, z).
-template <typename T, bool COH = false, class PL>
+template <typename T, int LK = LD_PLAIN, class PL>
 __device__ __forceinline__ void pull15(const PL &P, const Geom &g, int x, int y, int z, float f[15])
 {
     const int nx = g.nx, ny = g.ny, nz = g.nz;
@@ -35,21 +35,21 @@ __device__ __forceinline__ void pull15(const PL &P, const Geom &g, int x, int y,
     const int row = nx, pl = nx * ny;
     const int sY0 = row * y, sYm = row * ym, sYp = row * yp;
     const int sZ0 = pl * z, sZm = pl * zm, sZp = pl * zp;
-    f[0] = ld3<COH>(P.in(0), x + sY0 + sZ0);
-    f[1] = ld3<COH>(P.in(1), xm + sY0 + sZ0);
-    f[2] = ld3<COH>(P.in(2), xp + sY0 + sZ0);
-    f[3] = ld3<COH>(P.in(3), x + sYm + sZ0);
-    f[4] = ld3<COH>(P.in(4), x + sYp + sZ0);
-    f[5] = ld3<COH>(P.in(5), x + sY0 + sZm);
-    f[6] = ld3<COH>(P.in(6), x + sY0 + sZp);
-    f[7] = ld3<COH>(P.in(7), xm + sYm + sZm);    // (1,1,1)
-    f[8] = ld3<COH>(P.in(8), xp + sYp + sZp);
-    f[9] = ld3<COH>(P.in(9), xm + sYm + sZp);    // (1,1,-1)
-    f[10] = ld3<COH>(P.in(10), xp + sYp + sZm);
-    f[11] = ld3<COH>(P.in(11), xm + sYp + sZm);  // (1,-1,1)
-    f[12] = ld3<COH>(P.in(12), xp + sYm + sZp);
-    f[13] = ld3<COH>(P.in(13), xm + sYp + sZp);  // (1,-1,-1)
-    f[14] = ld3<COH>(P.in(14), xp + sYm + sZm);
+    f[0] = ld3<LK>(P.in(0), x + sY0 + sZ0);
+    f[1] = ld3<LK>(P.in(1), xm + sY0 + sZ0);
+    f[2] = ld3<LK>(P.in(2), xp + sY0 + sZ0);
+    f[3] = ld3<LK>(P.in(3), x + sYm + sZ0);
+    f[4] = ld3<LK>(P.in(4), x + sYp + sZ0);
+    f[5] = ld3<LK>(P.in(5), x + sY0 + sZm);
+    f[6] = ld3<LK>(P.in(6), x + sY0 + sZp);
+    f[7] = ld3<LK>(P.in(7), xm + sYm + sZm);    // (1,1,1)
+    f[8] = ld3<LK>(P.in(8), xp + sYp + sZp);
+    f[9] = ld3<LK>(P.in(9), xm + sYm + sZp);    // (1,1,-1)
+    f[10] = ld3<LK>(P.in(10), xp + sYp + sZm);
+    f[11] = ld3<LK>(P.in(11), xm + sYp + sZm);  // (1,-1,1)
+    f[12] = ld3<LK>(P.in(12), xp + sYm + sZp);
+    f[13] = ld3<LK>(P.in(13), xm + sYp + sZp);  // (1,-1,-1)
+    f[14] = ld3<LK>(P.in(14), xp + sYm + sZm);
 }
 
 // Mass deviation and momentum of 15 populations; sp/dp the pair sums and differences.
@@ -228,23 +228,23 @@ __device__ __forceinline__ void lb15_sites_on(const LBArgs &a, const PL &P, int 
 
 // u = (sum fbar c + F/2)/rho of the streamed state at (x, y, z), F this step's
 // force; P.in: the planes of a.fout.
-template <typename T, bool FORCE, bool COH = false, class PL>
+template <typename T, bool FORCE, int LK = LD_PLAIN, class PL>
 __device__ __forceinline__ void vel15_site_on(const LBArgs &a, const PL &P, int x, int y, int z)
 {
     const Geom &g = a.g;
     float f[15];
-    pull15<T, COH>(P, g, x, y, z, f);
+    pull15<T, LK>(P, g, x, y, z, f);
     float sp[8], dp[8], drho, jx, jy, jz;
     moments15(f, sp, dp, drho, jx, jy, jz);
     float Fx = 0.f, Fy = 0.f, Fz = 0.f;
-    if (FORCE && (a.coupling & FLB_COUPLE_FORCE)) force3<COH>(a, x, y, z, Fx, Fy, Fz);
+    if (FORCE && (a.coupling & FLB_COUPLE_FORCE)) force3<LK>(a, x, y, z, Fx, Fy, Fz);
     const float irho = __fdividef(1.0f, a.rho0 + drho);
     store_velocity(a.u, g, x, y, z, (jx + 0.5f * Fx) * irho, (jy + 0.5f * Fy) * irho, (jz + 0.5f * Fz) * irho);
 }
 
-// The same with the populations pulled from the planes P.in (COH: loads through L2,
+// The same with the populations pulled from the planes P.in (LK: loads through L2,
 // fields written in the same launch).
-template <class V, typename T, bool GHOST_RELAX, bool COH = false, bool KEY_R0 = false, class PL>
+template <class V, typename T, bool GHOST_RELAX, int LK = LD_PLAIN, bool KEY_R0 = false, class PL>
 __device__ __forceinline__ void lb15_sites(const LBArgs &a, const PL &P, int x, int y, const int *zl, int nl, V Fx,
                                            V Fy, V Fz)
 {
@@ -252,7 +252,7 @@ __device__ __forceinline__ void lb15_sites(const LBArgs &a, const PL &P, int x, 
     lb15_sites_on<V, T, GHOST_RELAX, KEY_R0>(a, P, x, y, zl, nl, Fx, Fy, Fz, [&](V *f) {
         float fl[L][15];
 #pragma unroll
-        for (int l = 0; l < L; ++l) pull15<T, COH>(P, a.g, x, y, zl[l], fl[l]);
+        for (int l = 0; l < L; ++l) pull15<T, LK>(P, a.g, x, y, zl[l], fl[l]);
 #pragma unroll
         for (int i = 0; i < 15; ++i) {
             float t[L];
@@ -265,18 +265,18 @@ __device__ __forceinline__ void lb15_sites(const LBArgs &a, const PL &P, int x, 
 
 // One site's collide-stream on the planes of a.fin and a.fout (the persistent
 // kernel, one site per thread).
-template <typename T, bool GHOST_RELAX, bool COH = false, bool KEY_R0 = false>
+template <typename T, bool GHOST_RELAX, int LK = LD_PLAIN, bool KEY_R0 = false>
 __device__ __forceinline__ void lb15_site(const LBArgs &a, int x, int y, int z, float Fx, float Fy, float Fz)
 {
-    lb15_sites<F1, T, GHOST_RELAX, COH, KEY_R0>(a, PlanesFromBase<T>{(const T *)a.fin, (T *)a.fout, a.g.n}, x, y,
+    lb15_sites<F1, T, GHOST_RELAX, LK, KEY_R0>(a, PlanesFromBase<T>{(const T *)a.fin, (T *)a.fout, a.g.n}, x, y,
                                                 &z, 1, F1{Fx}, F1{Fy}, F1{Fz});
 }
 
 // The velocity at one site on the planes of a.fout.
-template <typename T, bool FORCE, bool COH = false>
+template <typename T, bool FORCE, int LK = LD_PLAIN>
 __device__ __forceinline__ void vel15_site(const LBArgs &a, int x, int y, int z)
 {
-    vel15_site_on<T, FORCE, COH>(a, PlanesFromBase<T>{(const T *)a.fout, nullptr, a.g.n}, x, y, z);
+    vel15_site_on<T, FORCE, LK>(a, PlanesFromBase<T>{(const T *)a.fout, nullptr, a.g.n}, x, y, z);
 }
 
 }  // namespace flb

@@ -15,23 +15,25 @@
 
 namespace flb {
 
-// Loads of fields written by earlier launches are plain ones (COH false; see launch_pdl).  Inside the
-// persistent batched kernel a field may have been written by another block of the same
-// launch, so loads go to L2 (COH true): L1 is not coherent within a launch.
-template <bool COH>
+// Loads of fields written by earlier launches: plain ones, or LD_CONST's read-only ones (ld.global.nc) in a
+// launch that never overlaps those in front of it (see launch_pdl).  Inside the persistent
+// batched kernel a field may have been written by another block of the same launch, so
+// loads go to L2 (LD_L2): L1 is not coherent within a launch.
+enum { LD_PLAIN = 0, LD_L2 = 1, LD_CONST = 2 };
+template <int LK>
 __device__ __forceinline__ float ldf(const float *p)
 {
-    return COH ? __ldcg(p) : *p;
+    return LK == LD_L2 ? __ldcg(p) : LK == LD_CONST ? __ldg(p) : *p;
 }
-template <bool COH>
+template <int LK>
 __device__ __forceinline__ float ld3(const float *p, int i)
 {
-    return ldf<COH>(p + i);
+    return ldf<LK>(p + i);
 }
-template <bool COH>
+template <int LK>
 __device__ __forceinline__ float ld3(const __half *p, int i)
 {
-    return __half2float(COH ? __ldcg(p + i) : p[i]);
+    return __half2float(LK == LD_L2 ? __ldcg(p + i) : p[i]);
 }
 
 template <typename T>
@@ -97,7 +99,7 @@ inline PlaneTable<T> plane_table(const void *in, void *out, const Geom &g, int q
 // Pull of the 19 populations of the lanes' sites (x, y, zl[l]) from stored
 // post-collision planes P.in(i): fbar_i(r) = stored_i(r - c_i).  Lane l of f[i]
 // holds lane l's population i.
-template <typename T, bool COH, class V, class PL>
+template <typename T, int LK, class V, class PL>
 __device__ __forceinline__ void pullv(const PL &P, const Geom &g, int x, int y, const int *zl, V f[19])
 {
     constexpr int L = V::L;
@@ -117,7 +119,7 @@ __device__ __forceinline__ void pullv(const PL &P, const Geom &g, int x, int y, 
     float t[L];
 #define FLB_PULL(i, X, SY, SZ)                                                        \
     do {                                                                              \
-        for (int l = 0; l < L; ++l) t[l] = ld3<COH>(P.in(i), X + SY + SZ[l]); \
+        for (int l = 0; l < L; ++l) t[l] = ld3<LK>(P.in(i), X + SY + SZ[l]); \
         f[i] = vmake<V>(t);                                                           \
     } while (0)
     FLB_PULL(0, x, sY0, sZ0);
@@ -145,7 +147,7 @@ __device__ __forceinline__ void pullv(const PL &P, const Geom &g, int x, int y, 
 // The same for two lanes (x, y, z) and (x, y, z + 1) that touch no face of the box in y
 // or z: population i of site s comes from P.up(i)[s], but for the columns x = 0 and
 // x = nx - 1, whose neighbours beyond the face are a row's length on.
-template <typename T, int Q, class PL>
+template <typename T, int Q, int LK = LD_PLAIN, class PL>
 __device__ __forceinline__ void pull_inner(const PL &P, const Geom &g, int x, int y, int z, F2 f[Q])
 {
     int s0[2], sm[2], sp[2];
@@ -161,7 +163,7 @@ __device__ __forceinline__ void pull_inner(const PL &P, const Geom &g, int x, in
     for (int i = 0; i < Q; ++i) {
         const bool xi = i == 1 || i == 2 || (i >= 7 && i <= 14);  // c_x = +1 for the odd ones, -1 for the even (both lattices)
         const int *s = !xi ? s0 : (i & 1) ? sm : sp;
-        const float t[2] = {ld3<false>(P.up(i), s[0]), ld3<false>(P.up(i), s[1])};
+        const float t[2] = {ld3<LK>(P.up(i), s[0]), ld3<LK>(P.up(i), s[1])};
         f[i] = vmake<F2>(t);
     }
 }
@@ -171,7 +173,7 @@ __device__ __forceinline__ void pull_inner(const PL &P, const Geom &g, int x, in
 // F = -div sigma (stress form).  PAIR: lane 1 is the site above lane 0's (on the last
 // plane of an odd box a ghost site, whose value is not used), so that the two share
 // the loads of the planes between them.
-template <bool COH, class V, bool PAIR = false>
+template <int LK, class V, bool PAIR = false>
 __device__ __forceinline__ void force3v(const LBArgs &a, int x, int y, const int *zl, V &Fx, V &Fy, V &Fz)
 {
     constexpr int L = V::L;
@@ -183,7 +185,7 @@ __device__ __forceinline__ void force3v(const LBArgs &a, int x, int y, const int
     auto LD = [&](const float *base, int off) {
         float t[L];
 #pragma unroll
-        for (int l = 0; l < L; ++l) t[l] = ldf<COH>(base + pi[l] + off);
+        for (int l = 0; l < L; ++l) t[l] = ldf<LK>(base + pi[l] + off);
         return vmake<V>(t);
     };
     if (a.force_kind == 2) {
@@ -242,11 +244,11 @@ __device__ __forceinline__ void force3v(const LBArgs &a, int x, int y, const int
 }
 
 // One site's force (the persistent kernel, one site per thread).
-template <bool COH = false>
+template <int LK = LD_PLAIN>
 __device__ __forceinline__ void force3(const LBArgs &a, int x, int y, int z, float &Fx, float &Fy, float &Fz)
 {
     F1 X, Y, Z;
-    force3v<COH, F1>(a, x, y, &z, X, Y, Z);
+    force3v<LK, F1>(a, x, y, &z, X, Y, Z);
     Fx = X.v;
     Fy = Y.v;
     Fz = Z.v;
@@ -463,32 +465,32 @@ __device__ __forceinline__ void lb_sites_on(const LBArgs &a, const PL &P, int x,
 }
 
 // The same with the populations pulled from the planes P.in.
-template <class V, typename T, bool GHOST_RELAX, bool COH, bool KEY_R0, class PL>
+template <class V, typename T, bool GHOST_RELAX, int LK, bool KEY_R0, class PL>
 __device__ __forceinline__ void lb_sites(const LBArgs &a, const PL &P, int x, int y, const int *zl, int nl, V Fx,
                                          V Fy, V Fz)
 {
     lb_sites_on<V, T, GHOST_RELAX, KEY_R0>(a, P, x, y, zl, nl, Fx, Fy, Fz,
-                                           [&](V *f) { pullv<T, COH>(P, a.g, x, y, zl, f); });
+                                           [&](V *f) { pullv<T, LK>(P, a.g, x, y, zl, f); });
 }
 
 // One site on the planes of a.fin and a.fout (the persistent kernel, one site per thread).
-template <typename T, bool GHOST_RELAX, bool COH = false, bool KEY_R0 = false>
+template <typename T, bool GHOST_RELAX, int LK = LD_PLAIN, bool KEY_R0 = false>
 __device__ __forceinline__ void lb_site(const LBArgs &a, int x, int y, int z, float Fx, float Fy, float Fz)
 {
-    lb_sites<F1, T, GHOST_RELAX, COH, KEY_R0>(a, PlanesFromBase<T>{(const T *)a.fin, (T *)a.fout, a.g.n}, x, y, &z,
+    lb_sites<F1, T, GHOST_RELAX, LK, KEY_R0>(a, PlanesFromBase<T>{(const T *)a.fin, (T *)a.fout, a.g.n}, x, y, &z,
                                               1, F1{Fx}, F1{Fy}, F1{Fz});
 }
 
 // Velocity of the streamed state at the lanes' sites (x, y, zl[l]), the first
 // nl stored: u = (sum fbar c + F/2)/rho with fbar the populations the next step
 // pulls (a.fout) and F this step's force.  P.in: the planes of a.fout.
-template <class V, typename T, bool FORCE, bool COH, class PL>
+template <class V, typename T, bool FORCE, int LK, class PL>
 __device__ __forceinline__ void vel3_sites(const LBArgs &a, const PL &P, int x, int y, const int *zl, int nl)
 {
     constexpr int L = V::L;
     const Geom &g = a.g;
     V f[19];
-    pullv<T, COH>(P, g, x, y, zl, f);
+    pullv<T, LK>(P, g, x, y, zl, f);
     V sp[10], dp[10];
 #pragma unroll
     for (int p = 1; p <= 9; ++p) {
@@ -501,7 +503,7 @@ __device__ __forceinline__ void vel3_sites(const LBArgs &a, const PL &P, int x, 
     const V jy = dp[2] + (dp[4] - dp[5]) + (dp[8] + dp[9]);
     const V jz = dp[3] + (dp[6] - dp[7]) + (dp[8] - dp[9]);
     V Fx = V::bc(0.f), Fy = V::bc(0.f), Fz = V::bc(0.f);
-    if (FORCE && (a.coupling & FLB_COUPLE_FORCE)) force3v<COH>(a, x, y, zl, Fx, Fy, Fz);
+    if (FORCE && (a.coupling & FLB_COUPLE_FORCE)) force3v<LK>(a, x, y, zl, Fx, Fy, Fz);
     const V rho = drho + a.rho0;
     float ir[L];
 #pragma unroll
@@ -516,10 +518,10 @@ __device__ __forceinline__ void vel3_sites(const LBArgs &a, const PL &P, int x, 
 }
 
 // The same at one site on the planes of a.fout.
-template <typename T, bool FORCE, bool COH = false>
+template <typename T, bool FORCE, int LK = LD_PLAIN>
 __device__ __forceinline__ void vel3_site(const LBArgs &a, int x, int y, int z)
 {
-    vel3_sites<F1, T, FORCE, COH>(a, PlanesFromBase<T>{(const T *)a.fout, nullptr, a.g.n}, x, y, &z, 1);
+    vel3_sites<F1, T, FORCE, LK>(a, PlanesFromBase<T>{(const T *)a.fout, nullptr, a.g.n}, x, y, &z, 1);
 }
 
 }  // namespace flb
