@@ -429,8 +429,8 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // pays for over and over (a 512^3 step took 13.2 ms with every launch so made
 // and 10.2 ms with none), so a grid above max_blocks is launched in plain stream order (both
 // instructions then return at once).  16 blocks per SM is where a step of 64^3 to
-// 128^3 gains most (64^3: 59.0 -> 49.1 us); the 2D kernels, which read little twice,
-// gain up to larger grids (2048^2, 8192 blocks: 244 -> 233 us).
+// 128^3 gains most (64^3: 59.0 -> 49.1 us); the 2D kernels, which read little twice, gain at every size
+// (flb_step2d.cu).
 constexpr long long PDL_BLOCKS = 16 * 152;
 // whether launch_pdl lets a grid overlap the launches in front of it
 inline bool overlaps(dim3 grid, long long max_blocks) { return (long long)grid.x * grid.y * grid.z <= max_blocks; }

@@ -609,7 +609,10 @@ __global__ void __launch_bounds__(NT) psi2_kernel(const Psi2Args a)
 // Tiles: 32 x 16 where two blocks per SM of them cover the chip, else 16 x 8: a
 // small box then has four times the blocks, each with one point per thread, and its
 // latency is what a step costs.
-constexpr long long PDL_BLOCKS2 = 108 * 152;  // see launch_pdl
+// Every launch overlaps (launch_pdl): Heun steps, overlapped and in stream order, 256^2 11.2 and 16.6 us,
+// 1024^2 54.5 and 63.7, 2048^2 205 and 214, 2560^2 314 and 323, 3072^2 442 and 451, 4096^2, the largest box,
+// 768 and 777.
+constexpr long long PDL_ALWAYS = 1LL << 62;
 bool small_box2(const Geom &g) { return (long long)g.nx * g.ny < 304LL * 512; }
 
 template <int TX, int TY, int NT, typename T, bool FV, bool FIRST, bool NOISE>
@@ -620,7 +623,7 @@ cudaError_t go_psi2(const Psi2Args &a, cudaStream_t st)
     const bool stress = FIRST && (a.coupling & FLB_COUPLE_FORCE) && a.force_kind == 2;
     const size_t smem = sizeof(float) * (size_t)(NP + NM + (2 + (NOISE ? (FV ? 2 : 4) : 0)) * N1 + (stress ? 3 * NM : 0));
     const dim3 grid((a.g.nx + TX - 1) / TX, (a.g.ny + TY - 1) / TY);
-    return launch_pdl(psi2_kernel<TX, TY, NT, T, FV, FIRST, NOISE>, grid, NT, smem, st, PDL_BLOCKS2, a);
+    return launch_pdl(psi2_kernel<TX, TY, NT, T, FV, FIRST, NOISE>, grid, NT, smem, st, PDL_ALWAYS, a);
 }
 
 template <typename T, bool FV, bool FIRST, bool NOISE>
@@ -646,8 +649,8 @@ cudaError_t go_lb2(const LBArgs &a, const Psi2Args &p, cudaStream_t st)
 {
     constexpr int NT = TX * TY / V::L;
     const dim3 grid((a.g.nx + TX - 1) / TX, (a.g.ny + TY - 1) / TY);
-    return a.gamma_g != 0.0f ? launch_pdl(lb2_kernel<TX, TY, V, T, true>, grid, NT, 0, st, PDL_BLOCKS2, a, p)
-                             : launch_pdl(lb2_kernel<TX, TY, V, T, false>, grid, NT, 0, st, PDL_BLOCKS2, a, p);
+    return a.gamma_g != 0.0f ? launch_pdl(lb2_kernel<TX, TY, V, T, true>, grid, NT, 0, st, PDL_ALWAYS, a, p)
+                             : launch_pdl(lb2_kernel<TX, TY, V, T, false>, grid, NT, 0, st, PDL_ALWAYS, a, p);
 }
 
 }  // namespace
