@@ -7,7 +7,8 @@
 #include <new>
 #include <utility>
 #include <algorithm>
-#include <atomic>
+#include <condition_variable>
+#include <mutex>
 #include <cstdio>
 #include <functional>
 #include <map>
@@ -1407,16 +1408,19 @@ int flb_set_populations(flb_handle *h, int32_t rep, const double *f)
 // the size of the box), and from 2^21 values on host threads (one per 2^19, at
 // most 16) convert a chunk while the next is on its way; for fewer their start costs more
 // than they save.  psi and u of 100^3 take 0.7 ms (1.6 with the copy first and then the
-// conversion), of 160^3 3.0 (4.1), of 512^3 54 to 66 in every run, where a stage of the
-// whole field took 42 to 590 from one run to the next.
+// conversion), of 160^3 3.2 (4.1), of 256^3 10.3 (10.9), of 512^3 63 in every run, where a stage of the
+// whole field took 42 to 590 from one run to the next.  The threads sleep while a
+// chunk is on its way (spinning, 512^3 took 68 ms and 890 instead of 605 ms of processor time).
 constexpr long long COPY_CHUNK = 1 << 21, COPY_RING = 4;
 static int copy_out(cudaStream_t st, const float *dev, long long n, float *tmp, double *d0, long long n0, double *d1)
 {
     const long long chunks = (n + COPY_CHUNK - 1) / COPY_CHUNK;
     const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
     const long long want = n < (1 << 21) ? 1 : std::min<long long>({n >> 19, (long long)hw, 16});
-    std::atomic<long long> ready{0};  // chunks that have come over; -1: give up
-    std::atomic<long long> done[COPY_RING] = {};  // shares that the threads have converted from each slot
+    std::mutex mx;  // of the two counters
+    std::condition_variable came, freed;
+    long long ready = 0;              // chunks that have come over; -1: give up
+    long long done[COPY_RING] = {};  // shares that the threads have converted from each slot
     std::vector<std::thread> pool;
     long long nt = 0;
     auto convert = [&](long long k, long long t) {  // share t of chunk k
@@ -1428,11 +1432,15 @@ static int copy_out(cudaStream_t st, const float *dev, long long n, float *tmp, 
     };
     auto work = [&](long long t) {
         for (long long k = 0; k < chunks; ++k) {
-            long long r;
-            while ((r = ready.load(std::memory_order_acquire)) >= 0 && r <= k) std::this_thread::yield();
-            if (r < 0) return;
+            {
+                std::unique_lock<std::mutex> lock(mx);
+                came.wait(lock, [&]() { return ready < 0 || ready > k; });
+                if (ready < 0) return;
+            }
             convert(k, t);
-            done[k % COPY_RING].fetch_add(1, std::memory_order_release);
+            std::lock_guard<std::mutex> lock(mx);
+            ++done[k % COPY_RING];
+            freed.notify_one();
         }
     };
     if (want > 1) {
@@ -1444,13 +1452,19 @@ static int copy_out(cudaStream_t st, const float *dev, long long n, float *tmp, 
     }
     int rc = FLB_OK;
     for (long long k = 0; k < chunks && rc == FLB_OK; ++k) {
-        // the k / COPY_RING chunks that were in the slot are converted
-        while (done[k % COPY_RING].load(std::memory_order_acquire) < nt * (k / COPY_RING)) std::this_thread::yield();
+        {  // the k / COPY_RING chunks that were in the slot are converted
+            std::unique_lock<std::mutex> lock(mx);
+            freed.wait(lock, [&]() { return done[k % COPY_RING] >= nt * (k / COPY_RING); });
+        }
         const long long c0 = k * COPY_CHUNK;
         rc = cuerr(cudaMemcpyAsync(tmp + (k % COPY_RING) * COPY_CHUNK, dev + c0,
                                    (size_t)std::min(COPY_CHUNK, n - c0) * 4, cudaMemcpyDeviceToHost, st));
         if (rc == FLB_OK) rc = cuerr(cudaStreamSynchronize(st));
-        ready.store(rc == FLB_OK ? k + 1 : -1, std::memory_order_release);
+        {
+            std::lock_guard<std::mutex> lock(mx);
+            ready = rc == FLB_OK ? k + 1 : -1;
+        }
+        came.notify_all();
         for (long long t = nt; t < want && rc == FLB_OK; ++t) convert(k, t);
     }
     for (auto &th : pool) th.join();
