@@ -16,11 +16,11 @@
 //   out    the increment and the stage output.
 // psi, mu, u and E are read through L1 where they are used, without staging: what
 // bounds a small box is the latency of the chain, a large one instruction issue
-// (the FD noise above all: 13 normals on twice the sites).  Heun steps, 64^3 FV: 269 us
-// with one 64-plane chunk per column, 65.6 with the best chunk, 56 here (38 with the step's
-// launches overlapped); 32^3 FD 213 (one thread block row marching), 50 with the best chunk, 37
-// here (23); 256^3 FD 1832 and 1770 (1573 with the later Box-Muller); 96^3 FV with the
-// Patra-Karttunen Laplacian 257 with one thread per site and a launch per field, 128 here (112).
+// (the FD noise above all: 13 normals on twice the sites, 1036 instructions per site at 72% of the
+// slots; FV 707 and 452 at 64^3, at 52 and 43%).  Heun steps, marching with the best chunk and here, both in
+// stream order: 64^3 FV 65.6 and 56 us, 32^3 FD 50 and 37; with launches overlapped and the
+// polynomial normals 38.5 and 22.  96^3 FV with the Patra-Karttunen Laplacian 257 us with
+// one thread per site and a launch per field, 111 here.
 //
 // The FV stages take the same explicitly rounded operations in the same order as
 // psi3_fv_tma_block (per-plane partial sums included), so a field has the same bits

@@ -13,16 +13,14 @@
 //   psi2_kernel       a later stage: mu of the stage input, its increment, the output.
 //
 // What bounds them: the populations go through HBM twice read and once written
-// (108 B/site of the about 150 a step moves), but a large box is bound by
-// instruction issue and L1 latency (65-73% of the slots; 480 instructions per site in
-// lb2_kernel, 705 in the first stage, 235 in the second): a 2048^2 FD Heun step takes
-// 205 us (383 us with one thread per site and one launch per field; 226 with a later
-// stage's velocities and accumulator loaded where they are used, 213 with u psi in shared
-// memory instead of u).  A small
-// one is bound by latency, so what counts is the number of launches and what each
-// has to wait for: 64^2 takes 7.6 us a step (28.8 us with eight launches; 15.7 us
-// with these three before programmatic dependent launch, with the noise drawn ahead of the
-// wait and the populations in flight while mu is formed).
+// (108 B/site; a step moves 134 at 2048^2), but a large box is bound by
+// instruction issue (65% of the slots in lb2_kernel, 78 and 86% in the two stages; 454, 683 and 262
+// instructions per site): a 2048^2 FD Heun step takes 204 us (383 us with one thread per
+// site and one launch per field; 226 with a later stage's velocities and accumulator loaded
+// where they are used, 213 with u psi in shared memory instead of u).  A small one is bound by
+// latency, so what counts is the number of launches and what each has to wait for: 64^2
+// takes 7.7 us a step (28.8 us with eight launches; 14.4 with these three in stream
+// order).
 #include "flb_internal.cuh"
 
 namespace flb {
