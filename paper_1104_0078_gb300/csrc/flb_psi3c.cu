@@ -20,7 +20,7 @@
 // slots; FV 707 and 452 at 64^3, at 52 and 43%).  Heun steps, marching with the best chunk and here, both in
 // stream order: 64^3 FV 65.6 and 56 us, 32^3 FD 50 and 37; with launches overlapped and the
 // polynomial normals 38.5 and 22.  96^3 FV with the Patra-Karttunen Laplacian 257 us with
-// one thread per site and a launch per field, 111 here.
+// one thread per site and a launch per field, 109 here.
 //
 // The FV stages take the same explicitly rounded operations in the same order as
 // psi3_fv_tma_block (per-plane partial sums included), so a field has the same bits
